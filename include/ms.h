@@ -95,12 +95,11 @@ typedef struct ms_config {
     int32_t video_restart; /* ms_video_* only: 1 = every frame starts from n_initial instead of the
                               seed count carried from the previous frame */
     int32_t tc_shape;     /* BF16 form: warp arrangement of the shift kernel, the same arithmetic in
-                             each (results bit-identical). Mask warps x pixels each per tile, GEMM2
-                             issuers: 0 = 16 x 32, two (default); 1 = 16 x 32, one; 2 = 8 x 64,
-                             two; 3 = 8 x 64, one; 4 = two groups of 8 x 64 taking alternate
-                             tiles, two; 5 = the same groups, one; 6 = GEMM1 on 64-pixel units
-                             (four S buffers, six mask buffers), two groups of 8 x 32 taking
-                             alternate units, two issuers; 7 = as 6, one issuer */
+                             each (results bit-identical). Mask warps in
+                             groups that take the pixel tiles in turn, and S buffers: 0 = 8 in two
+                             groups, three (default); 1 = 16 in one, three; 2 = 4 in one, three;
+                             3 = 8 in one, three; 4 = 16 in two, three; 5 = 12 in three, three;
+                             6 = 16 in two, two; 7 = 8 in two, two */
     int32_t reserved[3];  /* zero */
 } ms_config;
 

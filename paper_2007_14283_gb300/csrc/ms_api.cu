@@ -209,9 +209,10 @@ Layout plan(int64_t np, int Dp, bool bf16) {
         bf16 ? n * Dp * sizeof(float) : 0,                    // 25 Xr (merge candidates in rank order)
         bf16 ? n : 0,                                         // 26 removed_r
         bf16 ? (n + 127) / 128 * 128 * 128 * (Dp / 16) : 0,  // 27 Ck (their BF16 split rows)
+        (n + kFinThreads - 1) / kFinThreads * kMoveWords * sizeof(uint32_t),  // 28 moving
     };
     size_t t = 0;
-    for (int i = 0; i < 28; ++i) {
+    for (int i = 0; i < 29; ++i) {
         L.off[i] = t;
         t += align_up(sizes[i]);
     }
@@ -344,6 +345,7 @@ ms_status ctx_alloc(const ms_config* cfg, int64_t max_pixels, cudaStream_t strea
     ctx->Xr = cfg->precision == MS_BF16 ? (float*)(b + L.off[25]) : nullptr;
     ctx->removed_r = cfg->precision == MS_BF16 ? (uint8_t*)(b + L.off[26]) : nullptr;
     ctx->Ck = cfg->precision == MS_BF16 ? (void*)(b + L.off[27]) : nullptr;
+    ctx->moving = (uint32_t*)(b + L.off[28]);
     ctx->round_log_cap = 64;
     ctx->round_log = new (std::nothrow) int64_t[ctx->round_log_cap * 4];
     if (!ctx->round_log) {
@@ -393,6 +395,7 @@ ms_status ctx_bind_finish(ms_ctx* ctx, cudaStream_t st, uint64_t frame_id, int64
     ctx->N_carry = n_start;
     ctx->max_draw = 0;
     ctx->phase = 0;
+    ctx->last_iters = 0;
     ctx->n_kept = 0;
     ctx->m_round = 0;
     const int64_t launches = ctx->stats.launches;
@@ -478,7 +481,11 @@ ms_status ms_iterate(ms_ctx* ctx, int32_t max_iter, int32_t* n_converged_out, in
     if (ctx->phase != 1) return set_error(MS_ERR_STATE, "no seed batch is pending");
     const int mi = max_iter > 0 ? max_iter : ctx->cfg.max_iter;
     const int64_t seed_iters0 = ctx->hc->seed_iters;
-    int t = 0, batch = 4;
+    // Iterations queued before the first look at the counters: as many as the
+    // last round took (rounds of a frame mostly take the same number; queued
+    // iterations after the stop return at once, but each is three launches).
+    int t = 0, batch = ctx->last_iters > 0 ? ctx->last_iters : 4;
+    batch = batch < 32 ? batch : 32;
     for (;;) {
         const int iters_before = ctx->hc->iters;
         int launched = 0;
@@ -501,8 +508,9 @@ ms_status ms_iterate(ms_ctx* ctx, int32_t max_iter, int32_t* n_converged_out, in
             }
         }
         if (ctx->hc->done || t >= mi) break;
-        batch = batch < 32 ? batch * 2 : 32;
+        batch = 4;
     }
+    ctx->last_iters = ctx->hc->iters;
     const DevCounters& h = *ctx->hc;
     ctx->phase = 2;
     ctx->stats.iters_total += h.iters;

@@ -40,8 +40,9 @@ struct ms_batch {
     ms::BPlan plan;
     int32_t* blk_off;         // [B + 2] block work list of the current merge/cover/label kernel
     int32_t* blk_split;       // [B + 2] block work list with the inner loop split (slices at [B + 1])
+    uint32_t* moving;         // per block of active seeds: masks of those still moving (ms_ctx::moving)
     int32_t* misc;            // [0] passes, [1] status, u64 at [2] band pairs, [4] tick, [6] shift ns, [8] shift
-                              // launches, [14] last phase tick, [16..31] eight phase sums (ns)
+                              // launches, [10] compaction ticket, [14] last phase tick, [16..31] eight phase sums (ns)
     float* P32;
     int32_t* pix;
     uint8_t* covered;
@@ -96,6 +97,8 @@ constexpr int kIT = 1024;   // ingest / selection threads
 constexpr int kMT = 128;    // merge threads
 constexpr int kVT = 64;     // vectors per shared tile
 constexpr int kPT = 256;    // pixel threads (cover, label)
+constexpr int kSlotPx = 8;  // pixels a selection thread looks at when giving out slots
+constexpr uint8_t kTaken = 2;  // covered[]: drawn by the running selection
 constexpr int kDefaultMaxPasses = 200000;  // loop guard: far above any real run (rounds x iterations)
 
 enum BlockSel { kSelDoneSeeds = 0, kSelDoneCands = 1, kSelDonePixels = 2, kSelAllPixels = 3 };
@@ -298,8 +301,8 @@ __global__ void k_b_labels_clear(const BFrame* __restrict__ frames, int32_t* con
 __global__ void __launch_bounds__(kIT)
 k_b_seed(const BFrame* __restrict__ frames, BState* states, const float* __restrict__ P32, int Dp,
          uint8_t* __restrict__ covered, float* __restrict__ X, int32_t* __restrict__ seed_pix,
-         int32_t* __restrict__ seed_order, int32_t* __restrict__ act0, uint8_t* __restrict__ sstate, int max_rounds,
-         int all_seeds) {
+         int32_t* __restrict__ seed_order, int32_t* __restrict__ act0, uint8_t* __restrict__ sstate,
+         int32_t* __restrict__ order_of, int max_rounds, int all_seeds) {
     __shared__ int32_t warp_excl[32];
     __shared__ int32_t s_total, s_cut;
     __shared__ int s_go;
@@ -351,15 +354,8 @@ k_b_seed(const BFrame* __restrict__ frames, BState* states, const float* __restr
         __syncthreads();
         const int32_t r = warp_excl[wid] + __popc(bal & ((1u << lane) - 1u));
         if (flag && taken + r < want) {
-            const int64_t slot = base + taken + r;
-            covered[base + p] = 1;
-            seed_pix[slot] = p;
-            seed_order[slot] = drawn + taken + r;
-            act0[slot] = (int32_t)slot;
-            sstate[slot] = kMoving;
-            const float4* src = reinterpret_cast<const float4*>(P32 + (base + p) * Dp);
-            float4* dst = reinterpret_cast<float4*>(X + slot * Dp);
-            for (int k = 0; k < Dp / 4; ++k) dst[k] = src[k];
+            covered[base + p] = kTaken;
+            order_of[base + p] = drawn + taken + r;
             if (taken + r == want - 1) s_cut = pos + 1;
         }
         __syncthreads();
@@ -371,6 +367,30 @@ k_b_seed(const BFrame* __restrict__ frames, BState* states, const float* __restr
             cursor = min(n, cursor + kIT);
         }
         __syncthreads();
+    }
+    // slots in pixel order (ms_seed.cu); each thread looks at kSlotPx pixels
+    int slots = 0;
+    for (int p0 = 0; p0 < n; p0 += kIT * kSlotPx) {
+        const int q0 = p0 + tid * kSlotPx;
+        unsigned took = 0;
+#pragma unroll
+        for (int k = 0; k < kSlotPx; ++k)
+            if (q0 + k < n && covered[base + q0 + k] == kTaken) took |= 1u << k;
+        int tot;
+        int64_t slot = base + slots + block_scan(__popc(took), &tot);
+        for (; took; took &= took - 1) {
+            const int p = q0 + __ffs(took) - 1;
+            covered[base + p] = 1;
+            seed_pix[slot] = p;
+            seed_order[slot] = order_of[base + p];
+            act0[slot] = (int32_t)slot;
+            sstate[slot] = kMoving;
+            const float4* src = reinterpret_cast<const float4*>(P32 + (base + p) * Dp);
+            float4* dst = reinterpret_cast<float4*>(X + slot * Dp);
+            for (int k = 0; k < Dp / 4; ++k) dst[k] = src[k];
+            ++slot;
+        }
+        slots += tot;
     }
     if (tid == 0) {
         DevCounters& dc = st.dc;
@@ -394,7 +414,8 @@ k_b_seed(const BFrame* __restrict__ frames, BState* states, const float* __restr
 }
 
 // ------------------------------------------------------------ iteration
-// Work split of this iteration over the iterating frames. Each frame is cut
+// Work split of this iteration over the iterating frames; seed_off counts
+// their blocks of kFinThreads active seeds. Each frame is cut
 // into seed tiles x pixel chunks by the single-frame rule (a target item count
 // spread over the frame's seed tiles, chunks whole pixel tiles). With
 // canon_target > 0 every frame gets that target, the one the single-frame path
@@ -444,7 +465,7 @@ __global__ void k_b_plan(const BFrame* __restrict__ frames, const BState* __rest
                 plan.chunks[f] = sp.chunks;
                 items = sp.tiles * sp.chunks;
             }
-            seeds = na;
+            seeds = (na + kFinThreads - 1) / kFinThreads;
         }
         int ti, ts;
         const int ei = block_scan(items, &ti);
@@ -466,88 +487,40 @@ __global__ void k_b_plan(const BFrame* __restrict__ frames, const BState* __rest
     }
 }
 
-// Warp-aggregated atomicAdd of 1 from every lane with flag set, grouped by
-// key (lanes of one warp may belong to different frames). Returns the old
-// value plus the lane's rank within its group.
-__device__ __forceinline__ int agg_inc(int32_t* ctr, bool flag, int key) {
-    const unsigned act = __ballot_sync(0xffffffffu, flag);
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned grp = __match_any_sync(0xffffffffu, flag ? key : -1 - (int)lane) & act;
-    int old = 0;
-    if (flag && lane == (unsigned)(__ffs(grp) - 1)) old = atomicAdd(ctr, __popc(grp));
-    old = __shfl_sync(0xffffffffu, old, flag ? __ffs(grp) - 1 : lane);
-    return old + __popc(grp & ((1u << lane) - 1u));
-}
-
-// Mean-shift update of every active seed of every iterating frame (Eq. 5
-// with the flat kernel): x <- normalise(window sum), converged when the FP64
-// step norm is below tol; seeds still moving go to the frame's next list.
+// Mean-shift update of every active seed of every iterating frame, a block of
+// kFinThreads seeds of one frame at a time: x <- normalise(window sum), and the
+// seeds still moving as masks for k_b_compact_check.
 template <int Dp>
-__global__ void __launch_bounds__(256)
-k_b_finalize(const BFrame* __restrict__ frames, BState* states, int B, BPlan plan, int32_t* act0, int32_t* act1,
-             unsigned long long* __restrict__ acc, float* __restrict__ X, uint8_t* __restrict__ sstate,
-             int32_t* __restrict__ support, double tol) {
+__global__ void __launch_bounds__(kFinThreads)
+k_b_finalize(const BFrame* __restrict__ frames, BState* states, int B, BPlan plan, const int32_t* __restrict__ act0,
+             const int32_t* __restrict__ act1, unsigned long long* __restrict__ acc, float* __restrict__ X,
+             uint8_t* __restrict__ sstate, int32_t* __restrict__ support, double tol, uint32_t* __restrict__ moving) {
     const int total = plan.seed_off[B];
-    const int stride = gridDim.x * blockDim.x;
-    for (int i0 = blockIdx.x * blockDim.x; i0 < total; i0 += stride) {
-        const int i = i0 + threadIdx.x;
-        const bool in = i < total;
-        int f = 0, slot = 0;
-        bool fail = false, conv = false, moving = false;
-        int32_t* a_out = nullptr;
-        if (in) {
-            f = locate(plan.seed_off, B, i);
-            const int pos = i - plan.seed_off[f];
-            const int64_t base = frames[f].pix0;
-            const bool odd = states[f].dc.iters & 1;
-            a_out = (odd ? act0 : act1) + base;
-            slot = ((odd ? act1 : act0) + base)[pos];
-            unsigned long long* a = acc + (int64_t)slot * (Dp + 1);
-            const long long cnt = (long long)a[Dp];
-            a[Dp] = 0ull;
-            double y[Dp];
-            double ss = 0.0;
-#pragma unroll
-            for (int k = 0; k < Dp; ++k) {
-                y[k] = (double)(long long)a[k] * (1.0 / 68719476736.0);  // fixed point, 2^-36 units
-                a[k] = 0ull;
-                ss += y[k] * y[k];
-            }
-            if (cnt == 0) {
-                fail = true;
-                sstate[slot] = kFailed;
-            } else {
-                const double inv = 1.0 / sqrt(ss);
-                float* x = X + (int64_t)slot * Dp;
-                double dd = 0.0;
-#pragma unroll
-                for (int k = 0; k < Dp; ++k) {
-                    const float xn = (float)(y[k] * inv);
-                    const double diff = (double)xn - (double)x[k];
-                    dd += diff * diff;
-                    x[k] = xn;
-                }
-                support[slot] = (int32_t)cnt;
-                if (sqrt(dd) < tol) {
-                    conv = true;
-                    sstate[slot] = kConverged;
-                } else {
-                    moving = true;
-                }
-            }
+    for (int blk = blockIdx.x; blk < total; blk += gridDim.x) {
+        const int f = locate(plan.seed_off, B, blk);
+        const int pos = (blk - plan.seed_off[f]) * kFinThreads + threadIdx.x;
+        DevCounters& dc = states[f].dc;
+        bool conv = false, fail = false, move = false;
+        if (pos < dc.n_active) {
+            const int slot = ((dc.iters & 1) ? act1 : act0)[frames[f].pix0 + pos];
+            move = finalize_seed<Dp>(acc + (int64_t)slot * (Dp + 1), X + (int64_t)slot * Dp, sstate + slot,
+                                     support + slot, tol, &conv, &fail);
         }
-        agg_inc(&states[f].dc.fail_total, fail, f);
-        agg_inc(&states[f].dc.conv_new, conv, f);
-        const int at = agg_inc(&states[f].dc.n_next, moving, f);
-        if (moving) a_out[at] = slot;
+        const int mc = __syncthreads_count(conv), mf = __syncthreads_count(fail), mm = __syncthreads_count(move);
+        const unsigned bal = __ballot_sync(0xffffffffu, move);
+        uint32_t* mv = moving + (int64_t)blk * kMoveWords;
+        if ((threadIdx.x & 31) == 0) mv[1 + (threadIdx.x >> 5)] = bal;
+        if (threadIdx.x == 0) {
+            mv[0] = (uint32_t)mm;
+            if (mc) atomicAdd(&dc.conv_new, mc);
+            if (mf) atomicAdd(&dc.fail_total, mf);
+            if (mm) atomicAdd(&dc.n_next, mm);
+        }
     }
 }
 
-// Early stopping per frame (Sec. 3.2.3).
-__global__ void k_b_check(BState* states, int B, double gamma, int max_iter) {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= B) return;
-    BState& st = states[f];
+// End of a frame's iteration, with the early stop (Sec. 3.2.3).
+__device__ void frame_check(BState& st, double gamma, int max_iter) {
     if (st.phase != kIterating) return;
     DevCounters& dc = st.dc;
     dc.seed_iters += dc.n_active;
@@ -563,6 +536,50 @@ __global__ void k_b_check(BState* states, int B, double gamma, int max_iter) {
         st.cands_total += dc.conv_total;
         st.dropped_total += (int64_t)dc.m_round - dc.conv_total;
     }
+}
+
+// Each frame's next active list: its moving seeds in the order of the current
+// list (k_compact_check's reasons). The last block to finish ends the
+// iteration of every frame.
+__global__ void __launch_bounds__(kFinThreads)
+k_b_compact_check(const BFrame* __restrict__ frames, BState* states, int B, BPlan plan, int32_t* act0, int32_t* act1,
+                  const uint32_t* __restrict__ moving, int* ticket, double gamma, int max_iter) {
+    __shared__ int s_sum[kFinThreads / 32];
+    __shared__ bool s_last;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int total = plan.seed_off[B];
+    for (int blk = blockIdx.x; blk < total; blk += gridDim.x) {
+        const int f = locate(plan.seed_off, B, blk);
+        const int b0 = plan.seed_off[f];
+        const bool odd = states[f].dc.iters & 1;
+        const int64_t base = frames[f].pix0;
+        int before = 0;
+        for (int b = b0 + threadIdx.x; b < blk; b += kFinThreads) before += (int)moving[(int64_t)b * kMoveWords];
+        for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+        __syncthreads();
+        if (lane == 0) s_sum[wid] = before;
+        __syncthreads();
+        before = 0;
+        const uint32_t* mv = moving + (int64_t)blk * kMoveWords;
+#pragma unroll
+        for (int w = 0; w < kFinThreads / 32; ++w) {
+            before += s_sum[w];
+            if (w < wid) before += __popc(mv[1 + w]);
+        }
+        const uint32_t bits = mv[1 + wid];
+        if ((bits >> lane) & 1u)
+            ((odd ? act0 : act1) + base)[before + __popc(bits & ((1u << lane) - 1u))] =
+                ((odd ? act1 : act0) + base)[(blk - b0) * kFinThreads + threadIdx.x];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+        if (s_last) *ticket = 0;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    for (int f = threadIdx.x; f < B; f += kFinThreads) frame_check(states[f], gamma, max_iter);
 }
 
 // ------------------------------------------------------------ merge
@@ -1102,7 +1119,7 @@ ms_status enqueue_body(ms_batch* b, cudaStream_t s, cudaGraphConditionalHandle h
     int64_t nl = 0;
 #define LAUNCHED(name) do { MS_LAUNCH(name); ++nl; } while (0)
     k_b_seed<<<B, kIT, 0, s>>>(b->frames, b->states, b->P32, Dp, b->covered, b->X, b->seed_pix, b->seed_order,
-                               b->act[0], b->sstate, b->cfg.max_rounds, b->cfg.all_seeds);
+                               b->act[0], b->sstate, b->cand_rank, b->cfg.max_rounds, b->cfg.all_seeds);
     LAUNCHED("k_b_seed");
     // Split 0 gives every frame the single-frame target (2 x grid), so each
     // frame's results equal a single-frame run's; split 1 shares
@@ -1121,7 +1138,7 @@ ms_status enqueue_body(ms_batch* b, cudaStream_t s, cudaGraphConditionalHandle h
     }
     ms_status st;
     if (b->tc)
-        st = launch_shift_tc_batch(b->pmap, b->pmap1, Dp, b->P32, b->X, b->acc, cf, b->frames, b->states, b->plan,
+        st = launch_shift_tc_batch(b->pmap, b->pmap1, Dp, b->X, b->acc, cf, b->frames, b->states, b->plan,
                                    b->act[0],
                                    b->act[1], B, b->misc + 1, (unsigned long long*)(b->misc + 2), b->tc_grid,
                                    b->tc_shape, s);
@@ -1138,11 +1155,12 @@ ms_status enqueue_body(ms_batch* b, cudaStream_t s, cudaGraphConditionalHandle h
         k_b_phase<<<1, 1, 0, s>>>(b->misc, kPhShift);
         LAUNCHED("k_b_phase");
     }
-    k_b_finalize<Dp><<<G, 256, 0, s>>>(b->frames, b->states, B, b->plan, b->act[0], b->act[1], b->acc, b->X,
-                                       b->sstate, b->support, b->cfg.tol);
+    k_b_finalize<Dp><<<G, kFinThreads, 0, s>>>(b->frames, b->states, B, b->plan, b->act[0], b->act[1], b->acc, b->X,
+                                               b->sstate, b->support, b->cfg.tol, b->moving);
     LAUNCHED("k_b_finalize");
-    k_b_check<<<(B + 255) / 256, 256, 0, s>>>(b->states, B, gamma, b->cfg.max_iter);
-    LAUNCHED("k_b_check");
+    k_b_compact_check<<<G, kFinThreads, 0, s>>>(b->frames, b->states, B, b->plan, b->act[0], b->act[1], b->moving,
+                                                b->misc + 10, gamma, b->cfg.max_iter);
+    LAUNCHED("k_b_compact_check");
     if (b->prof_phases) {
         k_b_phase<<<1, 1, 0, s>>>(b->misc, kPhFinalize);
         LAUNCHED("k_b_phase");
@@ -1441,7 +1459,8 @@ extern "C" ms_status ms_batch_create(const ms_config* cfg, int32_t B, const floa
         n * (Dp + 1) * 8, n * Dp * 4, n * 4, n * 4, n * 4, n, n * 4, n * kMergeCap * 4,
         (size_t)B * b->nblk_max * 4 + 4, b->tc ? (size_t)b->total_pk_rows * 128 * (Dp / 16) : 0, sizeof(int32_t*) * B,
         tcl ? (size_t)b->total_pk_rows * 128 * (Dp / 16) : 0, tcl ? n * sizeof(int2) : 0, sizeof(int32_t) * (B + 1) + 16,
-        n * Dp * 4, n, tcl ? (size_t)b->total_pk_rows * 128 * (Dp / 16) : 0};
+        n * Dp * 4, n, tcl ? (size_t)b->total_pk_rows * 128 * (Dp / 16) : 0,
+        (n / kFinThreads + B) * kMoveWords * sizeof(uint32_t)};
     const int NS = (int)(sizeof(sizes) / sizeof(sizes[0]));
     size_t offs[32], tot = 0;
     for (int i = 0; i < NS; ++i) {
@@ -1493,6 +1512,7 @@ extern "C" ms_status ms_batch_create(const ms_config* cfg, int32_t B, const floa
     b->Xr = (float*)(w + offs[28]);
     b->removed_r = (uint8_t*)(w + offs[29]);
     b->Ck = tcl ? (void*)(w + offs[30]) : nullptr;
+    b->moving = (uint32_t*)(w + offs[31]);
     ms_status s = cuda_check(cudaMallocHost((void**)&b->h_states, sizeof(BState) * B), "cudaMallocHost");
     if (s == MS_OK) s = cuda_check(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking), "cudaStreamCreate");
     if (s == MS_OK)

@@ -50,7 +50,7 @@ struct BPlan {
 
 // Tensor-core shift over all iterating frames (ms_shift_tc.cu).
 ms_status tc_batch_setup(int D);
-ms_status launch_shift_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, int D, const float* P32,
+ms_status launch_shift_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, int D,
                                 const float* X, unsigned long long* acc, float c_f, const BFrame* frames,
                                 const BState* states, BPlan plan, const int32_t* act0, const int32_t* act1, int nf,
                                 int* status, unsigned long long* band, int grid, int shape, cudaStream_t st);
@@ -158,5 +158,44 @@ __host__ __device__ inline int tc_tiles_per_chunk(int tiles, int n_ptiles, int t
     }
     return best;
 }
+
+#ifdef __CUDACC__
+// tc_tiles_per_chunk by a converged warp, a candidate per lane (the divisions
+// of one thread took 3.5 us at the start of every shift launch).
+__device__ inline int tc_tiles_per_chunk_warp(int tiles, int n_ptiles, int target, int grid) {
+    if (tiles <= 0 || n_ptiles <= 0) return 1;
+    const int lane = threadIdx.x & 31;
+    const unsigned T = (unsigned)tiles, P = (unsigned)n_ptiles, G = (unsigned)(grid > 0 ? grid : 1);
+    // lane 0: the plain rule; lanes 1..7: 2..8 waves
+    unsigned c = lane == 0 ? ((unsigned)target + T - 1) / T : (unsigned)(lane + 1) * G / T;
+    const bool valid = lane == 0 || (lane < 8 && grid > 0 && c >= 1);
+    c = c < 1 ? 1 : (c > P ? P : c);
+    const unsigned tpc = (P + c - 1) / c;
+    const unsigned long long items = (unsigned long long)T * ((P + tpc - 1) / tpc);
+    const unsigned long long waves =
+        items + G <= 0xffffffffull ? ((unsigned)items + G - 1) / G : (items + G - 1) / G;
+    unsigned long long key = valid ? (waves * (tpc + 2)) << 3 | (unsigned)lane : ~0ull;
+    for (int o = 4; o > 0; o >>= 1) {
+        const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, key, o);
+        key = k2 < key ? k2 : key;
+    }
+    key = __shfl_sync(0xffffffffu, key, 0);
+    return (int)__shfl_sync(0xffffffffu, tpc, (int)(key & 7));
+}
+
+// Item i of a frame's seed tiles x chunks, heaviest first: a seed tile's
+// windows lie mostly in the chunks around its own place in pixel order (both
+// run in pixel order), so the items go from that diagonal outwards, chunk
+// offsets 0, +1, -1, +2, ... Items are dealt to the CTAs in turn, so every CTA
+// gets its share of heavy ones.
+__device__ __forceinline__ void tc_item_place(int i, int tiles, int chunks, int* tile, int* chunk) {
+    const int delta = i / tiles, t = i - delta * tiles;
+    int ch = (int)((unsigned)(2 * t + 1) * (unsigned long long)chunks / (2u * (unsigned)tiles));
+    ch += (delta & 1) ? (delta + 1) / 2 : -(delta / 2);
+    ch = ch < 0 ? ch + chunks : (ch >= chunks ? ch - chunks : ch);
+    *tile = t;
+    *chunk = ch;
+}
+#endif
 
 }  // namespace ms

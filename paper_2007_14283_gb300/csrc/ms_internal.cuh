@@ -55,10 +55,15 @@ struct DevCounters {
     int32_t undecided;   // merge candidates still undecided
     int32_t n_uncovered; // foreground pixels not covered
     int32_t n_fg;        // foreground pixels
+    int32_t cursor_next; // seed-order position after the running selection
+    int32_t ticket;      // blocks of the running compaction that have finished
     int32_t pad;
     int64_t seed_iters;  // seed-iterations summed
     int64_t band_pairs;  // BF16 form: pairs rechecked in FP32
 };
+
+constexpr int kFinThreads = 256;                 // active seeds per finalize / compaction block
+constexpr int kMoveWords = 1 + kFinThreads / 32; // words of ms_ctx::moving per block
 
 // Work split of one shift iteration: seed tiles x pixel chunks.
 struct ShiftSplit {
@@ -119,7 +124,8 @@ struct ms_ctx {
     uint8_t* cand_state; // [n_pixels]
     int32_t* conf_deg;   // [n_pixels]
     int32_t* conf;       // [n_pixels * kMergeCap]
-    int32_t* block_tmp;  // ingest scan scratch
+    int32_t* block_tmp;  // ingest and seed-selection scan scratch
+    uint32_t* moving;    // per 256 active seeds: a count and eight 32-seed masks of those still moving
     ms::DevCounters* dc;
     ms::DevCounters* hc; // pinned host mirror
     int64_t* round_log;  // host [cap * 4]
@@ -133,6 +139,7 @@ struct ms_ctx {
     int64_t uncovered;
     int32_t n_kept;
     int32_t m_round;
+    int32_t last_iters;  // iterations of the frame's last round (0: none yet)
     ms_stats stats;
     // BF16 tensor-core form
     void* Pk;            // [n_pad, 64] bf16: [Ph | Pm | Pl | 0] per pixel

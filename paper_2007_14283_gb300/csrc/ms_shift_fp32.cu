@@ -15,12 +15,12 @@
 // totals do not depend on the order in which items finish: runs are
 // deterministic, and the finalize step reads one word per component.
 #include "ms_batch.cuh"
+#include "ms_device.cuh"
 
 namespace ms {
 namespace {
 
 constexpr float kFixScale = 68719476736.0f;      // 2^36
-constexpr double kFixInv = 1.0 / 68719476736.0;  // 2^-36
 
 // What a work item covers: a tile of the frame's active seeds and the pixel
 // rows [p_begin, p_end) of P32.
@@ -137,71 +137,69 @@ k_shift_fp32(const float* __restrict__ P32, const float* __restrict__ X, unsigne
 
 // Reads and clears each active seed's accumulators, moves the seed to
 // normalise(y) (FP32 state, computed from the exact sums in FP64) and tests
-// ||x' - x|| < tol in FP64.
+// ||x' - x|| < tol in FP64. The seeds still moving are left as masks for
+// k_compact_check.
 template <int Dp>
-__global__ void __launch_bounds__(256)
-k_finalize(unsigned long long* __restrict__ acc, const int32_t* __restrict__ active_in,
-           int32_t* __restrict__ active_out, float* __restrict__ X, uint8_t* __restrict__ sstate,
-           int32_t* __restrict__ support, double tol, DevCounters* dc) {
+__global__ void __launch_bounds__(kFinThreads)
+k_finalize(unsigned long long* __restrict__ acc, const int32_t* __restrict__ active_in, float* __restrict__ X,
+           uint8_t* __restrict__ sstate, int32_t* __restrict__ support, double tol, uint32_t* __restrict__ moving,
+           DevCounters* dc) {
     if (dc->done) return;
     const int n_active = dc->n_active;
     const int pos = blockIdx.x * blockDim.x + threadIdx.x;
-    bool conv = false, fail = false, moving = false;
-    int slot = -1;
+    if (blockIdx.x * blockDim.x >= n_active) return;
+    bool conv = false, fail = false, move = false;
     if (pos < n_active) {
-        slot = active_in[pos];
-        unsigned long long* a = acc + (int64_t)slot * (Dp + 1);
-        const long long cnt = (long long)a[Dp];
-        a[Dp] = 0ull;
-        double y[Dp];
-        double ss = 0.0;
-#pragma unroll
-        for (int k = 0; k < Dp; ++k) {
-            y[k] = (double)(long long)a[k] * kFixInv;
-            a[k] = 0ull;
-            ss += y[k] * y[k];
-        }
-        if (cnt == 0) {
-            fail = true;
-            sstate[slot] = kFailed;
-        } else {
-            const double inv = 1.0 / sqrt(ss);
-            float* x = X + (int64_t)slot * Dp;
-            double dd = 0.0;
-#pragma unroll
-            for (int k = 0; k < Dp; ++k) {
-                const float xn = (float)(y[k] * inv);
-                const double diff = (double)xn - (double)x[k];
-                dd += diff * diff;
-                x[k] = xn;
-            }
-            support[slot] = (int32_t)cnt;
-            if (sqrt(dd) < tol) {
-                conv = true;
-                sstate[slot] = kConverged;
-            } else {
-                moving = true;
-            }
-        }
+        const int slot = active_in[pos];
+        move = finalize_seed<Dp>(acc + (int64_t)slot * (Dp + 1), X + (int64_t)slot * Dp, sstate + slot, support + slot,
+                                 tol, &conv, &fail);
     }
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned mc = __ballot_sync(0xffffffffu, conv);
-    const unsigned mf = __ballot_sync(0xffffffffu, fail);
-    const unsigned mm = __ballot_sync(0xffffffffu, moving);
-    int base = 0;
-    if (lane == 0) {
-        if (mc) atomicAdd(&dc->conv_new, __popc(mc));
-        if (mf) atomicAdd(&dc->fail_total, __popc(mf));
-        if (mm) base = atomicAdd(&dc->n_next, __popc(mm));
+    const int mc = __syncthreads_count(conv), mf = __syncthreads_count(fail), mm = __syncthreads_count(move);
+    const unsigned bal = __ballot_sync(0xffffffffu, move);
+    uint32_t* mv = moving + (int64_t)blockIdx.x * kMoveWords;
+    if ((threadIdx.x & 31) == 0) mv[1 + (threadIdx.x >> 5)] = bal;
+    if (threadIdx.x == 0) {
+        mv[0] = (uint32_t)mm;
+        if (mc) atomicAdd(&dc->conv_new, mc);
+        if (mf) atomicAdd(&dc->fail_total, mf);
+        if (mm) atomicAdd(&dc->n_next, mm);
     }
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (moving) active_out[base + __popc(mm & ((1u << lane) - 1u))] = slot;
 }
 
-// Early stopping (Sec. 3.2.3): the round ends once more than gamma of its
-// seeds have converged, when none is still moving, or at max_iter.
-__global__ void k_round_check(DevCounters* dc, double gamma, int max_iter) {
+// The next active list: the moving seeds in the order of the current list (the
+// pixel order that the selection gave them; appending them as blocks finish
+// would mix the cells of an item's seeds). The last block to finish ends the
+// iteration. Early stopping (Sec. 3.2.3): the round ends once more than gamma
+// of its seeds have converged, when none is still moving, or at max_iter.
+__global__ void __launch_bounds__(kFinThreads)
+k_compact_check(const uint32_t* __restrict__ moving, const int32_t* __restrict__ active_in,
+                int32_t* __restrict__ active_out, DevCounters* dc, double gamma, int max_iter) {
     if (dc->done) return;
+    const int n_active = dc->n_active;
+    if (blockIdx.x * kFinThreads < n_active) {
+        __shared__ int s_sum[kFinThreads / 32];
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        int before = 0;
+        for (int b = threadIdx.x; b < (int)blockIdx.x; b += kFinThreads) before += (int)moving[(int64_t)b * kMoveWords];
+        for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+        if (lane == 0) s_sum[wid] = before;
+        __syncthreads();
+        before = 0;
+        const uint32_t* mv = moving + (int64_t)blockIdx.x * kMoveWords;
+#pragma unroll
+        for (int w = 0; w < kFinThreads / 32; ++w) {
+            before += s_sum[w];
+            if (w < wid) before += __popc(mv[1 + w]);
+        }
+        const uint32_t bits = mv[1 + wid];
+        if ((bits >> lane) & 1u)
+            active_out[before + __popc(bits & ((1u << lane) - 1u))] = active_in[blockIdx.x * kFinThreads + threadIdx.x];
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicAdd(&dc->ticket, 1) != (int)gridDim.x - 1) return;
+    dc->ticket = 0;
     dc->seed_iters += dc->n_active;
     dc->conv_total += dc->conv_new;
     dc->conv_new = 0;
@@ -219,7 +217,7 @@ ms_status shift_iteration_t(ms_ctx* ctx, int t, int max_iter, cudaEvent_t e0, cu
     int32_t* a_out = ctx->active[(t + 1) & 1];
     const float c = ceil_to_float(ctx->cfg.bandwidth_cos);
     const double gamma = ctx->cfg.all_seeds ? 1.0 : ctx->cfg.gamma;
-    const unsigned fin_blocks = (unsigned)((ctx->m_round + 255) / 256);
+    const unsigned fin_blocks = (unsigned)((ctx->m_round + kFinThreads - 1) / kFinThreads);
     if (e0) MS_CUDA(cudaEventRecord(e0, ctx->stream));
     if (ctx->cfg.precision == MS_BF16) {
         ms_status s = launch_shift_tc(ctx, a_in, ctx->tc_grid, 2 * ctx->tc_grid, nullptr);
@@ -235,11 +233,11 @@ ms_status shift_iteration_t(ms_ctx* ctx, int t, int max_iter, cudaEvent_t e0, cu
         MS_LAUNCH("k_shift_fp32");
     }
     if (e1) MS_CUDA(cudaEventRecord(e1, ctx->stream));
-    k_finalize<Dp><<<fin_blocks, 256, 0, ctx->stream>>>(ctx->acc, a_in, a_out, ctx->X, ctx->sstate,
-                                                        ctx->support, ctx->cfg.tol, ctx->dc);
+    k_finalize<Dp><<<fin_blocks, kFinThreads, 0, ctx->stream>>>(ctx->acc, a_in, ctx->X, ctx->sstate, ctx->support,
+                                                                ctx->cfg.tol, ctx->moving, ctx->dc);
     MS_LAUNCH("k_finalize");
-    k_round_check<<<1, 1, 0, ctx->stream>>>(ctx->dc, gamma, max_iter);
-    MS_LAUNCH("k_round_check");
+    k_compact_check<<<fin_blocks, kFinThreads, 0, ctx->stream>>>(ctx->moving, a_in, a_out, ctx->dc, gamma, max_iter);
+    MS_LAUNCH("k_compact_check");
     ctx->launches += 3;
     return MS_OK;
 }

@@ -7,37 +7,55 @@
 //          terms against a ones column, so S' = x.p - c up to the dropped
 //          terms (at most 3.04 * 2^-16 = 4.64e-5 for unit vectors: a BF16
 //          residual is at most 2^-8 of what it splits) and the tensor cores'
-//          FP32 accumulation (at most 51 * 2^-22 = 1.2e-5 even for an adder
-//          that truncates; measured <= 6e-6): 5.9e-5 < kBand.
-//   mask   a pair is in the window when S' >= 0 (sign bit clear). Pairs with
-//          |S'| < kBand = 2^-14 are re-decided with the same sequential FP32
-//          dot product as the FP32 form, against the pixel's exact FP32 value
-//          rebuilt from its BF16 parts in the shared-memory tile, so every
-//          decision equals the FP32 form's, whose dot product is within 1e-6
-//          of x.p. Whether a warp holds such a pair comes with the TMEM load
-//          of S' (tcgen05.ld.red min.abs: each lane's smallest |S'|), so the
-//          mask costs a byte permute and a logic op per two pixels and nothing
-//          else.
-//   GEMM2  Y += Mask . [Ph | Pm | Pl | 1]    (8 tcgen05 MMAs, mask exact in BF16;
-//          the ones column yields the window size)
-// The seed-by-pixel matrix lives only in TMEM and registers. After the item's last tile the Y sums are added to the per-seed
-// fixed-point accumulators shared with the FP32 form, and the same finalize
-// kernel normalises the seeds and tests convergence in FP64.
+//          FP32 accumulation (at most 51 * 2^-22 = 1.2e-5 for d = 16 even for
+//          an adder that truncates; measured <= 6e-6): 5.9e-5 < kBand.
+//   scan   every 32 x 32 piece of S' (32 seeds, 32 pixels) whose largest value
+//          is below -kBand = -2^-14 holds no pair of any window. That maximum
+//          comes with the TMEM load (tcgen05.ld.red max), so such a piece
+//          costs one load and one compare and has no further work.
+//   mask   the other pieces: a pair is in the window when S' >= 0 (sign bit
+//          clear). Pairs with |S'| < kBand are re-decided with the same
+//          sequential FP32 dot product as the FP32 form, against the pixel's
+//          exact FP32 value rebuilt from its BF16 parts in the shared-memory
+//          tile, so every decision equals the FP32 form's, whose dot product
+//          is within 1e-6 of x.p. Whether a warp holds such a pair comes with
+//          the second TMEM load (ld.red min.abs), so the mask costs a byte
+//          permute and a logic op per two pixels and nothing else.
+//   GEMM2  Y += Mask . [Ph | Pm | Pl | 1]    (mask exact in BF16; the ones
+//          column yields the window size), 2 tcgen05 MMAs for each 32-pixel
+//          piece that holds a mask, with the lanes (seeds) of pieces without
+//          one disabled. A skipped product would have added zeros, so the
+//          sums are those of the full product, bit for bit.
+// The seed-by-pixel matrix lives only in TMEM and registers. After the item's
+// last tile the Y sums are added to the per-seed fixed-point accumulators
+// shared with the FP32 form, and the same finalize kernel normalises the seeds
+// and tests convergence in FP64.
 //
-// Warp roles (608 threads, one CTA per SM): warps 0-15 build the mask, four
-// warps per 32-lane TMEM quadrant (warp w reaches lanes 32 * (w % 4) + 0..31),
-// 32 pixels each, and store it to TMEM, where GEMM2 reads it as its A operand;
-// warp 16 issues TMA loads of pixel tiles into an 11-stage ring; warp 17 owns
-// TMEM (512 columns: two S, one Y and three mask buffers) and issues GEMM1,
-// running ahead of the mask warps as far as the S buffers allow; warp 18
-// issues GEMM2 as each mask tile lands. The issuing warps run their loops with
-// all 32 lanes and let one elected lane issue each MMA and commit: a loop run
-// by lane 0 alone issues the MMAs about 1.5x slower. Seed operands (A1) and S
-// are double-buffered, masks triple-buffered (the mask warps would otherwise
-// wait for GEMM2's commit round trip), Y single (one item at a time; the next
-// item's first GEMM2 waits for the epilogue's read). All waits are bounded; a
-// timeout raises the CTA's abort flag, drains what is in flight, frees TMEM
-// and reports MS_ERR_TIMEOUT through the frame's status word.
+// What this rests on: a window is a small part of a frame (0.5% on 512 x 512
+// frames of 60 cells), and the active seeds of a round are kept in pixel order
+// (ms_seed.cu), so the 128 seeds of an item come from the same few cells, and
+// so do 128 consecutive pixels: on such a frame 22% of the 128 x 128 tiles hold a
+// pair of any window for 4096 active seeds (99% with the seeds in draw order).
+// One launch of 32768 seeds on a 512 x 512 frame: 0.56 ms against 1.06 ms for
+// the form that built every mask and ran every product; 4096 seeds: 0.10
+// against 0.149 ms. What bounds it now: the issuing and scanning warps' chains
+// per tile (about 400 clocks; the tensor pipe needs 256 of them), and tiles
+// that hold windows, whose S buffer stays taken through mask and GEMM2.
+//
+// Warp roles (one CTA per SM): the mask warps read S and build masks (each
+// reaches the TMEM lanes 32 * (warp % 4) + 0..31), in groups that take the
+// pixel tiles in turn; then a TMA producer (a ring of pixel tiles), the GEMM1
+// issuer, which owns TMEM (three S buffers and Y), and the GEMM2 issuer. A mask is written over the
+// columns of S it was made from, where GEMM2 reads it as its A operand: the
+// buffer is free for GEMM1 again once the tile's mask warps are done and its
+// GEMM2, if any, has completed. The
+// issuing warps run their loops with all 32 lanes and let one elected lane
+// issue each MMA and commit: a loop run by lane 0 alone issues the MMAs about
+// 1.5x slower. Seed operands (A1) are double-buffered, Y is single (one item
+// at a time; the next item's GEMM2 waits for the epilogue's read). All waits
+// are bounded; a timeout raises the CTA's abort flag, drains what is in
+// flight, frees TMEM and reports MS_ERR_TIMEOUT through the frame's status
+// word.
 #include <cudaTypedefs.h>
 
 #include "ms_batch.cuh"
@@ -51,70 +69,67 @@ namespace {
 
 using namespace tc;
 
-// Tile shape of a CTA (what the autotuner chooses among). Pixels arrive in
-// 128-pixel stages; GEMM1 scores BN of them at a time (a unit: BN = 128, one
-// unit per stage, two 128-column S buffers; BN = 64, two units per stage,
-// four 64-column S buffers), and the mask of a unit takes BN / 2 TMEM columns
-// (three or six mask buffers in 192 columns for d = 16, two or four in 128
-// for d = 32). MW mask warps form G
-// groups that take turns unit by unit (group k builds the masks of units u
-// with u % G == k); each warp builds the mask of 4 * BN / (MW / G) pixels of
-// its group's units. Then come the TMA producer, the GEMM1 issuer and NG2
-// GEMM2 issuers (NG2 = 2: alternate units, on two sub-partitions).
-template <int MW, int NG2, int G, int BN>
+// Warp arrangement of a CTA (what the autotuner chooses among). MW mask warps
+// form G groups that take the pixel tiles in turn (group k has the tiles g with
+// g % G == k); each warp of a group scans 128 / (MW / G / 4) pixels of its
+// tiles for its 32 seeds. NS S buffers of 128 TMEM columns let GEMM1 run ahead
+// of the groups.
+template <int MW, int G, int NS>
 struct TcShape {
-    static constexpr int kMaskWarps = MW;           // warps 0..MW-1 build the mask
     static constexpr int kGroups = G;
-    static constexpr int kGroupWarps = MW / G;      // mask warps per unit
-    static constexpr int kBN = BN;                  // pixels per unit
-    static constexpr int kUPS = 128 / BN;           // units per 128-pixel stage
-    static constexpr int kSBufs = 256 / BN;         // S buffers of BN columns
-    static constexpr int kPxPerWarp = 4 * BN / kGroupWarps;  // pixels of a unit per mask warp
-    static constexpr int kSub = kPxPerWarp / 32;    // 32-pixel TMEM loads per mask warp and unit
+    static constexpr int kGroupWarps = MW / G;      // mask warps per tile
+    static constexpr int kSBufs = NS;
+    static constexpr int kPxPerWarp = 4 * 128 / kGroupWarps;  // pixels of a tile per mask warp
+    static constexpr int kSub = kPxPerWarp / 32;    // 32-pixel pieces per mask warp and tile
     static constexpr int kWarpTma = MW;
     static constexpr int kWarpG1 = MW + 1;
-    static constexpr int kWarpG2 = MW + 2;          // first GEMM2 issuer
-    static constexpr int kG2 = NG2;
-    static constexpr int kThreads = (MW + 2 + NG2) * 32;
-    static_assert(BN == 128 || BN == 64, "GEMM1 unit of 128 or 64 pixels");
+    static constexpr int kWarpG2 = MW + 3;
+    static constexpr int kThreads = (MW + 4) * 32;
     static_assert(MW % G == 0 && kGroupWarps % 4 == 0 && kPxPerWarp % 32 == 0 && kPxPerWarp >= 32,
                   "each group's mask warps cover the four TMEM quadrants evenly");
-    static_assert(NG2 == 1 || NG2 == 2, "one or two GEMM2 issuers");
+    static_assert(NS == 2 || NS == 3, "two or three S buffers");
+    // a group that waits for tile g has seen tile g - G, so S buffer phases up
+    // to tile g - NS are over and the parity it waits for is the next one
+    static_assert(G <= NS, "a group's tiles are at most NS apart");
 };
 // Index = ms_config.tc_shape.
-using TcShape0 = TcShape<16, 2, 1, 128>;
-using TcShape1 = TcShape<16, 1, 1, 128>;
-using TcShape2 = TcShape<8, 2, 1, 128>;
-using TcShape3 = TcShape<8, 1, 1, 128>;
-using TcShape4 = TcShape<16, 2, 2, 128>;
-using TcShape5 = TcShape<16, 1, 2, 128>;
-using TcShape6 = TcShape<16, 2, 2, 64>;
-using TcShape7 = TcShape<16, 1, 2, 64>;
+using TcShape0 = TcShape<8, 2, 3>;
+using TcShape1 = TcShape<16, 1, 3>;
+using TcShape2 = TcShape<4, 1, 3>;
+using TcShape3 = TcShape<8, 1, 3>;
+using TcShape4 = TcShape<16, 2, 3>;
+using TcShape5 = TcShape<12, 3, 3>;
+using TcShape6 = TcShape<16, 2, 2>;
+using TcShape7 = TcShape<8, 2, 2>;
 constexpr int kTileBytes = 128 * 128;  // 128 rows x 128 bytes
 constexpr uint32_t kTmemCols = 512;
-constexpr int kMaxSBufs = 4, kMaxMBufs = 6;
-constexpr uint32_t kColS = 0;          // S accumulators, 256 columns
-constexpr uint32_t kColY = 256;        // Y accumulators: 64 columns per 16-dimensional half
-constexpr float kBand = 6.103515625e-05f;    // 2^-14
+constexpr int kMaxSBufs = 3;
+constexpr uint32_t kColS = 0;          // S accumulators (and the masks built in place), 384 columns
+constexpr uint32_t kColY = 384;        // Y accumulators: 64 columns per 16-dimensional half
 constexpr float kFixScale = 68719476736.0f;  // 2^36
 
 // Layout for embedding dimension D: 16, or 32 as two 16-dimensional halves,
 // each with its own seed-operand tile, pixel tile (a second Pk array) and Y
-// block; the mask buffers take the TMEM columns after Y.
+// block.
 template <int D>
 struct TcDim {
     static_assert(D == 16 || D == 32, "embedding dimension 16 or 32");
     static constexpr int kHalves = D / 16;
-    static constexpr int kStages = D == 16 ? 10 : 4;              // pixel-tile ring
+    static constexpr int kStages = D == 16 ? 10 : 4;              // pixel-tile ring, more than the S buffers
     static constexpr int kStageBytes = kHalves * kTileBytes;
+    // Half-width of the recheck band: above the score's bound (dropped terms
+    // 4.64e-5 and accumulation (3 * D + 3) * 2^-22 = 1.2e-5 or 2.4e-5).
+    static constexpr float kBand = D == 16 ? 6.103515625e-05f : 7.5e-05f;  // 2^-14 for d = 16
     static constexpr int kOffA1 = 0;                              // 2 items x kHalves x 16 KB
     static constexpr int kOffP = 2 * kHalves * kTileBytes;        // kStages stages
     static constexpr int kOffX = kOffP + kStages * kStageBytes;   // 2 x 128 x D floats: the item's seeds
     static constexpr int kOffBar = kOffX + 2 * 128 * D * 4;
-    static constexpr int kNumBars = 2 * kStages + 2 * kMaxSBufs + 2 * kMaxMBufs + 2 + 2 + 3;  // aux: GEMM1 + two GEMM2
-    static constexpr int kSmemBytes = kOffBar + kNumBars * 8 + 32 + 1024;  // + TMEM slot, flags, alignment slack
-    static constexpr uint32_t kColM = kColY + 64 * kHalves;       // mask buffers up to column 512
+    static constexpr int kNumBars = 3 * kStages + kMaxSBufs + 2 + 3;
+    static constexpr int kOffHit = (kOffBar + kNumBars * 8 + 15) / 16 * 16;  // kStages x 16 bytes
+    static constexpr int kSmemBytes = kOffHit + kStages * 16 + 32 + 1024;    // + TMEM slot, flags, alignment slack
     static_assert(kSmemBytes <= 227 * 1024, "shared memory budget");
+    static_assert(kStages % 2 == 0, "a GEMM1 issuer of alternate tiles has seen its stage's previous phase");
+    static_assert(kStages > kMaxSBufs, "GEMM1 of a tile never waits for a stage that its own GEMM2 order holds");
 };
 
 struct TcSplit {
@@ -129,7 +144,7 @@ __device__ __forceinline__ TcSplit tc_split(int n_active, int n_ptiles, int targ
         s.tpc = 1;
         return s;
     }
-    s.tpc = tc_tiles_per_chunk(s.tiles, n_ptiles, target, grid);
+    s.tpc = tc_tiles_per_chunk_warp(s.tiles, n_ptiles, target, grid);
     s.chunks = (n_ptiles + s.tpc - 1) / s.tpc;
     return s;
 }
@@ -149,8 +164,8 @@ __device__ __forceinline__ uint32_t sign_halves(uint32_t a, uint32_t b) {
 }
 
 // Row r of one 16-dimensional half of a seed operand tile:
-// [Xh | Xl | -c split | 0] for the first half, [Xh | Xl | 0 | 0] for the
-// second (the -c column is added once), 128-byte swizzle.
+// [Xh | Xl | -c split, 0 | unused] for the first half, [Xh | Xl | unused] for
+// the second (the -c column is added once), 128-byte swizzle.
 __device__ __forceinline__ void write_a1_half(uint8_t* A1, int r, const float* x, float c_f, bool with_c) {
     uint32_t wh[8], wl[8];
 #pragma unroll
@@ -159,18 +174,18 @@ __device__ __forceinline__ void write_a1_half(uint8_t* A1, int r, const float* x
         wh[k / 2] = pack_bf16(h0, h1);
         wl[k / 2] = pack_bf16(x[k] - h0, x[k + 1] - h1);
     }
-    const float c_hi = bf16_round(c_f);
-    const float c_mid = bf16_round(c_f - c_hi);
-    const float c_lo = (c_f - c_hi) - c_mid;
-    const uint32_t wc0 = with_c ? pack_bf16(-c_hi, -c_mid) : 0u, wc1 = with_c ? pack_bf16(-c_lo, 0.f) : 0u;
     *reinterpret_cast<uint4*>(A1 + sw128_offset(r, 0)) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
     *reinterpret_cast<uint4*>(A1 + sw128_offset(r, 1)) = make_uint4(wh[4], wh[5], wh[6], wh[7]);
     *reinterpret_cast<uint4*>(A1 + sw128_offset(r, 2)) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
     *reinterpret_cast<uint4*>(A1 + sw128_offset(r, 3)) = make_uint4(wl[4], wl[5], wl[6], wl[7]);
-    *reinterpret_cast<uint4*>(A1 + sw128_offset(r, 4)) = make_uint4(wc0, wc1, 0u, 0u);
-#pragma unroll
-    for (int cidx = 5; cidx < 8; ++cidx)
-        *reinterpret_cast<uint4*>(A1 + sw128_offset(r, cidx)) = make_uint4(0u, 0u, 0u, 0u);
+    if (with_c) {
+        const float c_hi = bf16_round(c_f);
+        const float c_mid = bf16_round(c_f - c_hi);
+        const float c_lo = (c_f - c_hi) - c_mid;
+        *reinterpret_cast<uint4*>(A1 + sw128_offset(r, 4)) =
+            make_uint4(pack_bf16(-c_hi, -c_mid), pack_bf16(-c_lo, 0.f), 0u, 0u);
+        *reinterpret_cast<uint4*>(A1 + sw128_offset(r, 5)) = make_uint4(0u, 0u, 0u, 0u);
+    }
 }
 
 // Row r of an item's seed operand (one 16 KB tile per 16-dimensional half)
@@ -219,7 +234,8 @@ struct TcSingleMap {
     }
     __device__ __forceinline__ int total() const { return sp.tiles * sp.chunks; }
     __device__ __forceinline__ TcItem item(int i) const {
-        const int t = i / sp.chunks, ch = i - t * sp.chunks;
+        int t, ch;
+        tc_item_place(i, sp.tiles, sp.chunks, &t, &ch);
         const int pt0 = ch * sp.tpc;
         TcItem it;
         it.active = active;
@@ -233,28 +249,6 @@ struct TcSingleMap {
         return it;
     }
 };
-
-// FP32 value of pixel row `row` of a 16-dimensional pixel stage, rebuilt
-// exactly from its three BF16 parts (h + m) + l: the split of an FP32 value
-// into three round-to-nearest BF16 terms is exact, and so is this sum.
-__device__ __forceinline__ void stage_pixel16(const uint8_t* stage, int row, float (&p)[16]) {
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-        const uint4 hv = *reinterpret_cast<const uint4*>(stage + sw128_offset(row, c));
-        const uint4 mv = *reinterpret_cast<const uint4*>(stage + sw128_offset(row, c + 2));
-        const uint4 lv = *reinterpret_cast<const uint4*>(stage + sw128_offset(row, c + 4));
-        const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w}, mw[4] = {mv.x, mv.y, mv.z, mv.w},
-                       lw[4] = {lv.x, lv.y, lv.z, lv.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            p[c * 8 + 2 * k] = __fadd_rn(__fadd_rn(__uint_as_float(hw[k] << 16), __uint_as_float(mw[k] << 16)),
-                                         __uint_as_float(lw[k] << 16));
-            p[c * 8 + 2 * k + 1] =
-                __fadd_rn(__fadd_rn(__uint_as_float(hw[k] & 0xFFFF0000u), __uint_as_float(mw[k] & 0xFFFF0000u)),
-                          __uint_as_float(lw[k] & 0xFFFF0000u));
-        }
-    }
-}
 
 // Dot product, in FP32 with one FMA per component in component order (the
 // FP32 form's dot_seq, bit for bit), of seed x (D floats in shared memory)
@@ -275,6 +269,9 @@ __device__ __forceinline__ float stage_dot(const uint8_t* stage, int row, const 
             const uint4 lv = *reinterpret_cast<const uint4*>(t + sw128_offset(row, c + 4));
             const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w}, mw[4] = {mv.x, mv.y, mv.z, mv.w},
                            lw[4] = {lv.x, lv.y, lv.z, lv.w};
+            const float4 x0 = *reinterpret_cast<const float4*>(x + 16 * hf + c * 8);
+            const float4 x1 = *reinterpret_cast<const float4*>(x + 16 * hf + c * 8 + 4);
+            const float xv[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const float p0 = __fadd_rn(__fadd_rn(__uint_as_float(hw[k] << 16), __uint_as_float(mw[k] << 16)),
@@ -282,8 +279,8 @@ __device__ __forceinline__ float stage_dot(const uint8_t* stage, int row, const 
                 const float p1 =
                     __fadd_rn(__fadd_rn(__uint_as_float(hw[k] & 0xFFFF0000u), __uint_as_float(mw[k] & 0xFFFF0000u)),
                               __uint_as_float(lw[k] & 0xFFFF0000u));
-                acc = fmaf(x[16 * hf + c * 8 + 2 * k], p0, acc);
-                acc = fmaf(x[16 * hf + c * 8 + 2 * k + 1], p1, acc);
+                acc = fmaf(xv[2 * k], p0, acc);
+                acc = fmaf(xv[2 * k + 1], p1, acc);
             }
         }
     }
@@ -291,26 +288,67 @@ __device__ __forceinline__ float stage_dot(const uint8_t* stage, int row, const 
 }
 
 // Warp-uniform bounded wait: every lane polls, all lanes get the same answer.
+// The first look has no time limit to set up: the issuing warps run one
+// dependent chain per tile, in which reading the clock before every wait cost
+// more than the wait (a wait on a completed phase took 190 clocks).
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort));
 }
+
+// Both of two waits; b1 is looked at only once b0's phase is over. (Two
+// independent try_waits may be resolved in either order: the first can be held
+// back until its phase completes while the second is answered at once.)
+__device__ __forceinline__ bool warp_wait2(uint64_t* b0, uint32_t p0, uint64_t* b1, uint32_t p1, volatile int* abort) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(b0, p0)) && __all_sync(0xffffffffu, mbar_try_wait(b1, p1))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(b0, p0, abort) && mbar_wait(b1, p1, abort));
+}
+
+// Bounded wait of a converged warp for four counters in shared memory to reach
+// n. Counters, not a barrier: the warps that wait for items may skip items in
+// which they have no tile, and a barrier's parity tells only two phases apart.
+__device__ __forceinline__ bool seq_wait4(volatile int* seq, int n, volatile int* abort) {
+    volatile int* mine = seq + (threadIdx.x & 3);
+    if (*mine < n) {
+        const long long t0 = clock64();
+        while (*mine < n) {
+            if (*abort) break;
+            if (clock64() - t0 > kWaitCycles) {
+                *abort = 1;
+                break;
+            }
+        }
+    }
+    const bool ok = __all_sync(0xffffffffu, *mine >= n);
+    __threadfence_block();
+    return ok;
+}
+
+// Position in a ring of N slots, with the parity of the current lap.
+template <int N>
+struct Ring {
+    int i = 0;
+    uint32_t par = 0;
+    __device__ __forceinline__ void advance(int by) {  // by <= N
+        i += by;
+        if (i >= N) {
+            i -= N;
+            par ^= 1u;
+        }
+    }
+};
 
 template <class Shape, int kD, bool kDebug, class Map>
 __global__ void __launch_bounds__(Shape::kThreads, 1)
 k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUtensorMap pmap1,
-           const float* __restrict__ P32, const float* __restrict__ X, unsigned long long* __restrict__ acc, float c_f,
-           Map map, int* status, unsigned long long* band_ctr, float* __restrict__ dbg_S, int64_t dbg_stride) {
+           const float* __restrict__ X, unsigned long long* __restrict__ acc, float c_f, Map map, int* status,
+           unsigned long long* band_ctr, float* __restrict__ dbg_S, int64_t dbg_stride) {
     using L = TcDim<kD>;
     constexpr int kHalves = L::kHalves, kStages = L::kStages, kStageBytes = L::kStageBytes;
-    constexpr uint32_t kColM = L::kColM;
-    constexpr int kGroups = Shape::kGroups, kGroupWarps = Shape::kGroupWarps;
-    constexpr int kBN = Shape::kBN, kUPS = Shape::kUPS, kSBufs = Shape::kSBufs;
-    constexpr int kMBufs = (int)(kTmemCols - kColM) / (kBN / 2);  // mask buffers of BN / 2 columns
-    static_assert(kMBufs >= 2 && kMBufs <= kMaxMBufs, "mask buffers");
+    constexpr int kGroups = Shape::kGroups, kGroupWarps = Shape::kGroupWarps, kSBufs = Shape::kSBufs;
     constexpr int kPxPerWarp = Shape::kPxPerWarp, kSub = Shape::kSub;
-    constexpr int kWarpTma = Shape::kWarpTma, kWarpG1 = Shape::kWarpG1, kWarpG2 = Shape::kWarpG2, kG2 = Shape::kG2;
-    // GEMM2 issuers commit a stage's release after their last unit of it.
-    constexpr int kEmptyArrivals = kUPS < kG2 ? kUPS : kG2;
+    constexpr float kBand = L::kBand;
+    constexpr int kWarpTma = Shape::kWarpTma, kWarpG1 = Shape::kWarpG1, kWarpG2 = Shape::kWarpG2;
     if (!map.init()) return;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -319,39 +357,30 @@ k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
     float* Xs = (float*)(smem + L::kOffX);        // [2][128][kD] seeds of an item (FP32 re-decisions)
     uint64_t* bars = (uint64_t*)(smem + L::kOffBar);
     uint64_t* full = bars;                        // [kStages] pixel tile landed
-    uint64_t* empty = full + kStages;             // [kStages] pixel tile consumed by GEMM2
-    uint64_t* s_full = empty + kStages;           // [kSBufs] GEMM1 of a unit done
-    uint64_t* s_empty = s_full + kMaxSBufs;       // [kSBufs] S read by the mask warps of the unit's group
-    uint64_t* m_full = s_empty + kMaxSBufs;       // [kMBufs] mask of a unit stored to TMEM by its group's warps
-    uint64_t* m_empty = m_full + kMaxMBufs;       // [kMBufs] mask consumed by GEMM2
-    uint64_t* a1_full = m_empty + kMaxMBufs;      // [2] seed operand written
-    uint64_t* d_full = a1_full + 2;               // Y of an item complete
-    uint64_t* d_empty = d_full + 1;               // Y read by the epilogue
-    uint64_t* aux = d_empty + 1;                  // [1 + kG2] drain barriers of the MMA issuers
-    uint32_t* tmem_slot = (uint32_t*)(bars + L::kNumBars);
+    uint64_t* done = full + kStages;              // [kStages] the tile's mask warps have read S and written their masks
+    uint64_t* empty = done + kStages;             // [kStages] pixel tile no longer needed
+    uint64_t* s_full = empty + kStages;           // [kSBufs] GEMM1 of a tile done
+    uint64_t* d_full = s_full + kMaxSBufs;        // Y of an item complete
+    uint64_t* d_empty = d_full + 1;               // Y read by the epilogue and set to zero
+    uint64_t* aux = d_empty + 1;                  // [3] drain barriers of the MMA issuers
+    uint8_t* hits = smem + L::kOffHit;            // [kStages][quadrant][piece] 1: a mask was written
+    uint32_t* tmem_slot = (uint32_t*)(hits + kStages * 16);
     volatile int* abort = (volatile int*)(tmem_slot + 1);
-    volatile int* g2_next = (volatile int*)(tmem_slot + 2);  // the next unit whose GEMM2 may be issued
+    volatile int* a1_seq = (volatile int*)(tmem_slot + 4);  // [4] items whose rows of A1 a lead warp has written
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], kEmptyArrivals);
+            mbar_init(&done[s], kGroupWarps);
+            mbar_init(&empty[s], 1);
         }
-        for (int b = 0; b < kSBufs; ++b) {
-            mbar_init(&s_full[b], 1);
-            mbar_init(&s_empty[b], kGroupWarps);
-        }
-        for (int b = 0; b < 2; ++b) mbar_init(&a1_full[b], 128);
-        for (int b = 0; b < kMBufs; ++b) {
-            mbar_init(&m_full[b], kGroupWarps);
-            mbar_init(&m_empty[b], 1);
-        }
-        mbar_init(d_full, kG2);  // every GEMM2 issuer commits at an item's end
+        for (int b = 0; b < kSBufs; ++b) mbar_init(&s_full[b], 1);
+        mbar_init(d_full, 1);
         mbar_init(d_empty, 128);
-        for (int k = 0; k <= kG2; ++k) mbar_init(&aux[k], 1);
+        for (int k = 0; k < 3; ++k) mbar_init(&aux[k], 1);
         *abort = 0;
-        *g2_next = 0;
+        for (int k = 0; k < 4; ++k) a1_seq[k] = 1;  // the first item's are written before the roles start
         fence_mbar_init();
     }
     if (warp == kWarpTma && lane == 0) {
@@ -362,23 +391,30 @@ k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
         tmem_alloc(tmem_slot, kTmemCols);
         tmem_relinquish();
     }
+    const int items = map.total();
+    if (warp < 4 && (int)blockIdx.x < items) {  // the first item's seeds, while the rest is set up
+        const TcItem ii = map.item(blockIdx.x);
+        const int pos = ii.seed0 + warp * 32 + lane;
+        write_seed_rows<kD>(A1, Xs, warp * 32 + lane, X, pos < ii.n_active ? ii.active[pos] : -1, c_f);
+        fence_proxy_async();
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const int items = map.total();
 
     if (warp == kWarpTma) {
         // ------------------------------------------------ TMA producer
-        // The three issuing warps run their loops with all 32 lanes (waits
-        // are warp-uniform) and one lane issues; see mma_bf16_warp.
+        // The issuing warps run their loops with all 32 lanes (waits are
+        // warp-uniform) and one lane issues; see mma_bf16_warp.
+        Ring<kStages> st;
         int g = 0;
         bool ok = true;
         for (int item = blockIdx.x; item < items && ok; item += gridDim.x) {
             const TcItem ii = map.item(item);
-            for (int pt = ii.pt0; pt < ii.pt1; ++pt, ++g) {
-                const int s = g % kStages;
-                if (g >= kStages && !(ok = warp_wait(&empty[s], ((g / kStages) - 1) & 1, abort))) break;
+            for (int pt = ii.pt0; pt < ii.pt1; ++pt, ++g, st.advance(1)) {
+                const int s = st.i;
+                if (g >= kStages && !(ok = warp_wait(&empty[s], st.par ^ 1u, abort))) break;
                 if (lane == 0) {
                     mbar_arrive_expect_tx(&full[s], kStageBytes);
                     tma_load_2d(Pst + s * kStageBytes, &pmap, 0, ii.pk_row0 + pt * 128, &full[s]);
@@ -390,139 +426,122 @@ k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
         }
         if (lane == 0 && *abort)
             for (int q = max(0, g - kStages); q < g; ++q) drain_wait(&full[q % kStages], (q / kStages) & 1);
-    } else if (warp == kWarpG1) {
-        // ------------------------------------------------ GEMM1 issuer
-        // Runs ahead of the mask warps as far as the S buffers allow.
-        // Descriptors are built once; moving an operand by b bytes adds b >> 4
-        // to the descriptor's start-address field (no carry: shared addresses
-        // stay below 2^18).
-        const uint64_t dA1 = desc_sw128(smem_u32(A1), 16, 1024);   // seed operand, K-major
-        const uint64_t dP1 = desc_sw128(smem_u32(Pst), 16, 1024);  // pixel tile, K-major
-        constexpr uint32_t id1 = idesc_bf16(128, kBN, 0, 0);
+    } else if (warp >= kWarpG1 && warp < kWarpG2) {
+        // ------------------------------------------------ GEMM1 issuers
+        // Two warps take alternate tiles (a warp's chain of waits, address
+        // arithmetic, issue and commit takes 400 clocks), up to kSBufs tiles
+        // ahead of the mask warps. The S buffer of tile g - kSBufs is free when
+        // its pixel stage is: its mask warps are done and its GEMM2, if any,
+        // has completed. Descriptors are built once; moving an operand by b
+        // bytes adds b >> 4 to the descriptor's start-address field (no carry:
+        // shared addresses stay below 2^18).
+        const int par = warp - kWarpG1;
+        const uint64_t dA1 = desc_sw128(smem_u32(A1), 16, 1024);           // seed operand, K-major
+        const uint64_t dP1 = desc_sw128(smem_u32(Pst), 16, 1024);          // pixel tile, K-major
+        constexpr uint32_t id1 = idesc_bf16(128, 128, 0, 0);
         constexpr uint64_t kT = kTileBytes >> 4;
-        constexpr uint64_t kU = (kBN * 128) >> 4;  // one unit of pixel rows
+        Ring<kStages> st, old;   // stages of tile g and of tile g - kSBufs
+        Ring<kSBufs> sb;
+        st.advance(par);
+        sb.advance(par);
+        old.advance((kSBufs ^ par) & 1);  // tile g - kSBufs of the warp's first g >= kSBufs
         bool ok = true;
-        int g = 0, it = 0;
+        int g = par, g0 = 0, it = 0;
         for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++it) {
             const TcItem ii = map.item(item);
-            if (!(ok = warp_wait(&a1_full[it & 1], (it >> 1) & 1, abort))) break;
+            const int g1 = g0 + ii.pt1 - ii.pt0;
+            if (g < g1 && !(ok = seq_wait4(a1_seq, it + 1, abort))) break;
             const uint64_t a = dA1 + (uint64_t)(it & 1) * kHalves * kT;
-            for (int pt = ii.pt0; pt < ii.pt1 && ok; ++pt, ++g) {
-                const int s = g % kStages;
-                if (!(ok = warp_wait(&full[s], (g / kStages) & 1, abort))) break;
-#pragma unroll
-                for (int hh = 0; hh < kUPS; ++hh) {
-                    const int u = g * kUPS + hh, b = u % kSBufs;
-                    if (u >= kSBufs && !(ok = warp_wait(&s_empty[b], ((u / kSBufs) - 1) & 1, abort))) break;
-                    tc_fence_after();
-                    const uint32_t tS = tmem + kColS + b * kBN;
-                    const uint64_t pb = dP1 + (uint64_t)s * kHalves * kT + hh * kU;
-                    mma_bf16_warp(tS, a, pb, id1, 0);            // Xh . Ph
-                    mma_bf16_warp(tS, a, pb + 2, id1, 1);        // Xh . Pm
-                    mma_bf16_warp(tS, a + 2, pb, id1, 1);        // Xl . Ph
-                    mma_bf16_warp(tS, a + 4, pb + 6, id1, 1);    // -c split . ones
-                    if (kHalves > 1) {                           // dimensions 16..31
-                        mma_bf16_warp(tS, a + kT, pb + kT, id1, 1);
-                        mma_bf16_warp(tS, a + kT, pb + kT + 2, id1, 1);
-                        mma_bf16_warp(tS, a + kT + 2, pb + kT, id1, 1);
-                    }
-                    mma_commit_warp(&s_full[b]);
-                }
+            for (; g < g1; g += 2, st.advance(2), sb.advance(2)) {
+                const bool reuse = g >= kSBufs;  // (the first tiles find their S buffers free)
+                if (!(ok = warp_wait2(&full[st.i], st.par, reuse ? &empty[old.i] : &full[st.i],
+                                      reuse ? old.par : st.par, abort)))
+                    break;
+                if (reuse) old.advance(2);
+                tc_fence_after();
+                const uint32_t tS = tmem + kColS + sb.i * 128;
+                const uint64_t pb = dP1 + (uint64_t)st.i * kHalves * kT;
+                mma_bf16_split3c_warp(tS, a, pb, id1);                            // Xh.Ph + Xh.Pm + Xl.Ph - c
+                if (kHalves > 1) mma_bf16_split3_warp(tS, a + kT, pb + kT, id1);  // dimensions 16..31
+                mma_commit_warp(&s_full[sb.i]);
             }
+            g0 = g1;
         }
         if (__any_sync(0xffffffffu, *abort)) {
-            mma_commit_warp(&aux[0]);
-            drain_wait(&aux[0], 0);
+            mma_commit_warp(&aux[par]);
+            drain_wait(&aux[par], 0);
         }
-    } else if (warp >= kWarpG2 && warp < kWarpG2 + kG2) {
-        // ------------------------------------------------ GEMM2 issuers
-        // Y += Mask . P as soon as a unit's mask is in TMEM; the pixel stage
-        // is released when the MMAs of its units complete. With two issuers,
-        // warps on different sub-partitions take alternate units, so neither
-        // sub-partition's mask warps carry all of GEMM2's issue cost. Y
-        // accumulates in unit order: a warp issues unit u only after unit u-1
-        // was issued (g2_next, with tcgen05 fences around the hand-over).
-        // Each warp commits the releases of the units it issued (a stage's
-        // release after its last unit of that stage), and every issuer commits
-        // d_full at an item's end (a commit covers only its own thread's MMAs).
-        const int par = warp - kWarpG2;
+    } else if (warp == kWarpG2) {
+        // ------------------------------------------------ GEMM2 issuer
+        // Y += Mask . P for the pieces that hold a mask; the pixel stage is
+        // released when those MMAs complete, or at once when there are none.
         const uint64_t dP2 = desc_sw128(smem_u32(Pst), kTileBytes, 1024);  // pixel tile, MN-major
         constexpr uint32_t id2 = idesc_bf16(128, 64, 0, 1);
         constexpr uint64_t kT = kTileBytes >> 4;
-        constexpr int kK2 = kBN / 16;  // K = 16 pixels per MMA
+        Ring<kStages> st;
+        Ring<kSBufs> sb;
         bool ok = true;
-        int g = 0, it = 0;
+        int it = 0;
         for (int item = blockIdx.x; item < items && ok; item += gridDim.x, ++it) {
             const TcItem ii = map.item(item);
-            for (int pt = ii.pt0; pt < ii.pt1 && ok; ++pt, ++g) {
-#pragma unroll
-                for (int hh = 0; hh < kUPS; ++hh) {
-                    const int u = g * kUPS + hh;
-                    if (u % kG2 != par) continue;
-                    const int s = g % kStages, mb = u % kMBufs;
-                    const bool first = pt == ii.pt0 && hh == 0;
-                    if (!(ok = warp_wait(&m_full[mb], (u / kMBufs) & 1, abort))) break;
-                    if (!(ok = warp_wait(&full[s], (g / kStages) & 1, abort))) break;
-                    if (first && it >= 1 && !(ok = warp_wait(d_empty, (it - 1) & 1, abort))) break;
-                    if constexpr (kG2 > 1) {
-                        const long long t0 = clock64();
-                        bool turn = true;
-                        while (*g2_next != u) {
-                            if (*abort || clock64() - t0 > kWaitCycles) {
-                                *abort = 1;
-                                turn = false;
-                                break;
-                            }
-                        }
-                        if (!(ok = __all_sync(0xffffffffu, turn))) break;
-                    }
+            if (!(ok = warp_wait(d_empty, it & 1, abort))) break;
+            for (int pt = ii.pt0; pt < ii.pt1; ++pt, st.advance(1), sb.advance(1)) {
+                if (!(ok = warp_wait(&done[st.i], st.par, abort))) break;
+                const uint4 hm = *reinterpret_cast<const uint4*>(hits + st.i * 16);
+                if (hm.x | hm.y | hm.z | hm.w) {
                     tc_fence_after();
-                    const uint32_t tM = tmem + kColM + mb * (kBN / 2);
+                    const uint32_t tM = tmem + kColS + sb.i * 128;
 #pragma unroll
-                    for (int hf = 0; hf < kHalves; ++hf) {
-                        const uint32_t tY = tmem + kColY + 64 * hf;
-                        const uint64_t pb = dP2 + (uint64_t)(s * kHalves + hf) * kT + hh * kK2 * 128;
+                    for (int pc = 0; pc < 4; ++pc) {
+                        const uint32_t byte = 0xffu << (8 * pc);
+                        if (!((hm.x | hm.y | hm.z | hm.w) & byte)) continue;
+                        const uint32_t off0 = (hm.x & byte) ? 0u : 0xffffffffu, off1 = (hm.y & byte) ? 0u : 0xffffffffu,
+                                       off2 = (hm.z & byte) ? 0u : 0xffffffffu, off3 = (hm.w & byte) ? 0u : 0xffffffffu;
 #pragma unroll
-                        for (int k = 0; k < kK2; ++k)
-                            mma_bf16_ts_warp(tY, tM + 8 * k, pb + k * 128, id2, (first && k == 0) ? 0u : 1u);
-                    }
-                    mma_commit_warp(&m_empty[mb]);
-                    if (hh >= kUPS - kG2) mma_commit_warp(&empty[s]);
-                    if constexpr (kG2 > 1) {  // one thread's MMAs execute in issue order: no hand-over
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) {
-                            __threadfence_block();
-                            *g2_next = u + 1;
+                        for (int hf = 0; hf < kHalves; ++hf) {
+                            const uint32_t tY = tmem + kColY + 64 * hf;
+                            const uint64_t pb = dP2 + (uint64_t)(st.i * kHalves + hf) * kT;
+                            mma_bf16_ts2_lanes_warp(tY, tM + 32 * pc, pb + 2 * pc * 128, id2, off0, off1, off2, off3);
                         }
                     }
+                    mma_commit_warp(&empty[st.i]);
+                } else if (lane == 0) {
+                    mbar_arrive(&empty[st.i]);
                 }
             }
             if (!ok) break;
             mma_commit_warp(d_full);
         }
         if (__any_sync(0xffffffffu, *abort)) {
-            mma_commit_warp(&aux[1 + par]);
-            drain_wait(&aux[1 + par], 0);
+            mma_commit_warp(&aux[2]);
+            drain_wait(&aux[2], 0);
         }
     } else {
         // ------------------------------------------------ mask warps
-        // Group grp of kGroups takes the units u with u % kGroups == grp; in a
+        // Group grp of kGroups takes the tiles g with g % kGroups == grp; in a
         // group, warp w reaches TMEM lanes 32 * (w % 4) + 0..31 (its seeds) and
-        // builds the mask of kPxPerWarp pixels of the unit, 32 at a time.
+        // scans kPxPerWarp pixels of the tile.
         const int grp = warp / kGroupWarps;
         const int q = warp & 3;                         // TMEM lane quadrant
         const int h = (warp % kGroupWarps) >> 2;        // which kPxPerWarp pixels of a tile
         const bool lead = warp < 4;                     // writes the seed operand and reads Y
         const int r = q * 32 + lane;                    // seed row
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-        // One group: the mask is stored once per tile. Two groups (64 pixels
-        // per warp): each 32-pixel part of the mask is stored as soon as it
-        // is built, which keeps fewer registers live.
-        constexpr bool kEarlyStore = kGroups > 1;
         long long band_local = 0;
-        int g = 0, it = 0;
-        int mbn = 0, mphn = 0;  // mask buffer of tile g and its phase, kept without divisions
+        int my = grp, g0 = 0, it = 0;
+        Ring<kStages> st;
+        Ring<kSBufs> sb;
+        Ring<kStages> old;  // stage of tile my - kSBufs, from the first such tile on
+        st.advance(grp);
+        sb.advance(grp);
+        old.advance((kGroups - kSBufs % kGroups + grp) % kGroups);
+        if (lead) {  // Y starts from zero
+#pragma unroll
+            for (int k = 0; k < 4 * kHalves; ++k) tmem_zero16(tmem + kColY + lane_base + 16 * k);
+            tmem_st_wait();
+            tc_fence_before();
+            mbar_arrive(d_empty);
+        }
         for (int item = blockIdx.x; item < items; item += gridDim.x, ++it) {
             if (__any_sync(0xffffffffu, *abort)) break;
             const TcItem ii = map.item(item);
@@ -530,15 +549,9 @@ k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
             const int pos = ii.seed0 + r;
             const int slot = pos < ii.n_active ? ii.active[pos] : -1;
             if (lead) {
-                // A1 for this item (first item only) and the next one; the next
-                // one's buffer was last read by the GEMM1s of item it-1, which
-                // completed before this warp observed s_full of that item's
-                // last tile (a commit covers every earlier MMA of its thread).
-                if (it == 0) {
-                    write_seed_rows<kD>(A1, Xs, r, X, slot, c_f);
-                    fence_proxy_async();
-                    mbar_arrive(&a1_full[0]);
-                }
+                // A1 for the next item (the first item's was written at the
+                // start). Its buffer was last read by the GEMM1s of item it-1,
+                // all complete before this warp saw that item's d_full.
                 const int nitem = item + gridDim.x;
                 if (nitem < items) {
                     const TcItem ni = map.item(nitem);
@@ -546,123 +559,176 @@ k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
                     write_seed_rows<kD>(A1 + ((it + 1) & 1) * kHalves * kTileBytes, Xs + ((it + 1) & 1) * 128 * kD, r, X,
                                         npos < ni.n_active ? ni.active[npos] : -1, c_f);
                     fence_proxy_async();
-                    mbar_arrive(&a1_full[(it + 1) & 1]);
+                    __syncwarp();
+                    if (lane == 0) {
+                        __threadfence_block();
+                        a1_seq[warp] = it + 2;
+                    }
                 }
             }
-            // The item's seeds in shared memory: written by the lead warps
-            // before their a1_full arrival (at the start of the previous item,
-            // after every mask warp had finished the item before it).
-            bool ok = warp_wait(&a1_full[it & 1], (it >> 1) & 1, abort);
+            bool ok = true;
             const float* xs = Xs + (it & 1) * 128 * kD + r * kD;
-            for (int pt = pt0; pt < pt1 && ok; ++pt, ++g) {
+            // my: the group's next tile, counted over all items
+            for (; my < g0 + pt1 - pt0 && ok; my += kGroups, st.advance(kGroups), sb.advance(kGroups)) {
+                const int pt = pt0 + my - g0, s = st.i;
+                // The buffer's previous phase has to be over before the parity
+                // of this tile's means anything. A group that took tile
+                // g - kSBufs (one group, or as many as buffers) knows; else the
+                // release of that tile says so (it comes before GEMM1 of this
+                // one, so the wait is over by then, and its barrier is not a
+                // phase ahead before this tile is done).
+                if constexpr (kGroups > 1 && kGroups != kSBufs) {
+                    const bool reuse = my >= kSBufs;
+                    if (!(ok = warp_wait2(reuse ? &empty[old.i] : &s_full[sb.i], reuse ? old.par : sb.par,
+                                          &s_full[sb.i], sb.par, abort)))
+                        break;
+                    if (reuse) old.advance(kGroups);
+                } else {
+                    if (!(ok = warp_wait(&s_full[sb.i], sb.par, abort))) break;
+                }
+                tc_fence_after();
+                const uint32_t tS = tmem + kColS + sb.i * 128 + lane_base + h * kPxPerWarp;
+                // Which pieces may hold a pair of a window (a NaN seed's scores
+                // are all NaN: not below the threshold). Their scores are
+                // loaded again below, so that none stays in registers here.
+                uint32_t need = 0u;
+                {
+                    float mx[kSub];
+                    uint32_t v[32];
 #pragma unroll
-                for (int hh = 0; hh < kUPS; ++hh) {
-                    const int u = g * kUPS + hh;  // unit: BN pixels of stage g
-                    const int mb = mbn, mph = mphn;
-                    if (++mbn == kMBufs) {
-                        mbn = 0;
-                        mphn ^= 1;
+                    for (int p = 0; p < kSub; ++p) tmem_ld32_max(tS + 32 * p, v, &mx[p]);
+                    tmem_ld_wait();
+                    bool near[kSub], any = false;
+#pragma unroll
+                    for (int p = 0; p < kSub; ++p) any |= near[p] = !(mx[p] < -kBand);
+                    if (__any_sync(0xffffffffu, any)) {
+#pragma unroll
+                        for (int p = 0; p < kSub; ++p)
+                            if (__any_sync(0xffffffffu, near[p])) need |= 1u << p;
                     }
-                    if (kGroups > 1 && u % kGroups != grp) continue;
-                    const int b = u % kSBufs;
-                    if (!(ok = warp_wait(&s_full[b], (u / kSBufs) & 1, abort))) break;
-                    tc_fence_after();
-                    uint32_t w[kEarlyStore ? 1 : kSub][16];
-                    bool staged = false;  // pixel stage known to be complete (band path)
-#pragma unroll
+                }
+                if (kDebug) {
                     for (int j = 0; j < kSub; ++j) {
-                        uint32_t (&wj)[16] = w[kEarlyStore ? 0 : j];
                         uint32_t v[32];
-                        float mn;
-                        tmem_ld32_minabs(tmem + kColS + b * kBN + lane_base + h * kPxPerWarp + j * 32, v, &mn);
+                        tmem_ld32(tS + j * 32, v);
                         tmem_ld_wait();
-                        if (j == kSub - 1) {  // S read: hand the buffer back to GEMM1
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(&s_empty[b]);
-                        }
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) wj[i] = ~sign_halves(v[2 * i], v[2 * i + 1]) & 0x3F803F80u;
-                        if (__any_sync(0xffffffffu, mn < kBand)) {
-                            // Re-decide near-boundary pairs with the FP32 form's dot
-                            // product against the exact FP32 pixel rebuilt from the
-                            // tile in shared memory. Bit masks keep register-array
-                            // indices static.
-                            const int s = g % kStages;
-                            if (!staged && !(ok = warp_wait(&full[s], (g / kStages) & 1, abort))) break;
-                            staged = true;
-                            const uint8_t* stage = Pst + s * kStageBytes;
-                            uint32_t bandm = 0;
+                        for (int i = 0; i < 32; ++i)
+                            dbg_S[(int64_t)r * dbg_stride + pt * 128 + h * kPxPerWarp + j * 32 + i] =
+                                __uint_as_float(v[i]);
+                    }
+                }
+                // The masks of those pieces. Pairs near the boundary are noted
+                // (bit 31 - i: pair i is near / S' < 0) and decided below, once
+                // for all pieces: a decision that differs from the sign is rare.
+                uint32_t hit = 0u, bandp = 0u;
+                uint32_t bandm[kSub], negm[kSub];
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) bandm |= (uint32_t)(fabsf(__uint_as_float(v[i])) < kBand) << i;
-                            uint32_t inm = 0, todo = bandm;
-                            while (todo) {
-                                const int i = __ffs(todo) - 1;
-                                todo &= todo - 1;
-                                const int row = hh * kBN + h * kPxPerWarp + j * 32 + i;
-                                if (pt * 128 + row < ii.n) {
-                                    ++band_local;
-                                    // xs: the seed (a padding row: zeros)
-                                    float d;
-                                    if constexpr (kD == 16) {
-                                        float x[16], pv[16];
+                for (int p = 0; p < kSub; ++p) bandm[p] = negm[p] = 0u;
+                while (need) {
+                    const int j = __ffs(need) - 1;
+                    need &= need - 1u;
+                    uint32_t v[32], w[16];
+                    float mn;
+                    tmem_ld32_minabs(tS + j * 32, v, &mn);
+                    tmem_ld_wait();
 #pragma unroll
-                                        for (int k = 0; k < 16; k += 4) {
-                                            const float4 t4 = *reinterpret_cast<const float4*>(xs + k);
-                                            x[k] = t4.x; x[k + 1] = t4.y; x[k + 2] = t4.z; x[k + 3] = t4.w;
-                                        }
-                                        stage_pixel16(stage, row, pv);
-                                        d = dot_seq<16>(x, pv);
-                                    } else {
-                                        d = stage_dot<kD>(stage, row, xs);
-                                    }
-                                    if (d >= c_f) inm |= 1u << i;
-                                }
+                    for (int i = 0; i < 16; ++i) w[i] = ~sign_halves(v[2 * i], v[2 * i + 1]) & 0x3F803F80u;
+                    tmem_st16(tS + j * 32, w);
+                    hit |= 1u << (8 * j);
+                    if (__any_sync(0xffffffffu, mn < kBand)) {
+                        uint32_t bm[4] = {0u, 0u, 0u, 0u}, nm[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {  // four chains of eight
+                                const uint32_t vi = v[8 * e + i];
+                                bm[e] = __funnelshift_l(__float_as_uint(fabsf(__uint_as_float(vi)) - kBand), bm[e], 1);
+                                nm[e] = __funnelshift_l(vi, nm[e], 1);
                             }
+                        const uint32_t b4 = (bm[0] << 24) | (bm[1] << 16) | (bm[2] << 8) | bm[3];
+                        const uint32_t n4 = (nm[0] << 24) | (nm[1] << 16) | (nm[2] << 8) | nm[3];
+#pragma unroll
+                        for (int p = 0; p < kSub; ++p)
+                            if (p == j) {
+                                bandm[p] = b4;
+                                negm[p] = n4;
+                            }
+                        bandp |= 1u << j;
+                    }
+                }
+                if (bandp) {
+                    // Re-decide near-boundary pairs with the FP32 form's dot
+                    // product against the exact FP32 pixel rebuilt from the
+                    // tile in shared memory. The tile and the item's seeds
+                    // landed long ago; these waits make them visible here (the
+                    // barrier cannot be a phase ahead: this tile is not done).
+                    ok = seq_wait4(a1_seq, it + 1, abort) && mbar_wait(&full[s], st.par, abort);
+                    if (!ok) *abort = 1;
+                    const uint8_t* stage = Pst + s * kStageBytes;
+                    uint32_t flip[kSub];
+                    bool flips = false;
+#pragma unroll
+                    for (int p = 0; p < kSub; ++p) {
+                        uint32_t todo = ok ? bandm[p] : 0u;
+                        flip[p] = 0u;
+                        while (todo) {
+                            const int i = __clz(todo);
+                            const uint32_t bit = 0x80000000u >> i;
+                            todo &= ~bit;
+                            const int row = h * kPxPerWarp + p * 32 + i;
+                            bool in = false;  // a padding pixel is in no window
+                            if (pt * 128 + row < ii.n) {
+                                ++band_local;
+                                in = stage_dot<kD>(stage, row, xs) >= c_f;  // xs: the seed (a padding row: zeros)
+                            }
+                            if (in == ((negm[p] & bit) != 0u)) flip[p] |= bit;
+                        }
+                        flips |= flip[p] != 0u;
+                    }
+                    __syncwarp();
+                    if (__any_sync(0xffffffffu, flips)) {
+#pragma unroll 1
+                        for (int j = 0; j < kSub; ++j) {
+                            if (!((bandp >> j) & 1u)) continue;
+                            uint32_t f = flip[0];
+#pragma unroll
+                            for (int p = 1; p < kSub; ++p)
+                                if (p == j) f = flip[p];
+                            uint32_t w[16];
+                            tmem_st_wait();
+                            tmem_ld16(tS + j * 32, w);
+                            tmem_ld_wait();
 #pragma unroll
                             for (int k = 0; k < 16; ++k) {
-                                const uint32_t bm = (bandm >> (2 * k)) & 3u;
-                                const uint32_t im = (inm >> (2 * k)) & 3u;
-                                const uint32_t clear = ((bm & 1u) ? 0x3F80u : 0u) | ((bm & 2u) ? 0x3F800000u : 0u);
-                                const uint32_t set = ((im & 1u) ? 0x3F80u : 0u) | ((im & 2u) ? 0x3F800000u : 0u);
-                                wj[k] = (wj[k] & ~clear) | set;
+                                if (f & (0x80000000u >> (2 * k))) w[k] ^= 0x3F80u;
+                                if (f & (0x40000000u >> (2 * k))) w[k] ^= 0x3F800000u;
                             }
-                        }
-                        if (kDebug) {
-#pragma unroll
-                            for (int i = 0; i < 32; ++i)
-                                dbg_S[(int64_t)r * dbg_stride + pt * 128 + hh * kBN + h * kPxPerWarp + j * 32 + i] =
-                                    __uint_as_float(v[i]);
-                        }
-                        if constexpr (kEarlyStore) {
-                            if (j == 0) {
-                                if (u >= kMBufs && !(ok = warp_wait(&m_empty[mb], mph ^ 1, abort))) break;
-                                tc_fence_after();
-                            }
-                            tmem_st16(tmem + kColM + mb * (kBN / 2) + lane_base + h * (kPxPerWarp / 2) + j * 16, wj);
+                            tmem_st16(tS + j * 32, w);
                         }
                     }
-                    if (!ok) break;
-                    if constexpr (!kEarlyStore) {
-                        if (u >= kMBufs && !(ok = warp_wait(&m_empty[mb], mph ^ 1, abort))) break;
-                        tc_fence_after();
-#pragma unroll
-                        for (int j = 0; j < kSub; ++j)
-                            tmem_st16(tmem + kColM + mb * (kBN / 2) + lane_base + h * (kPxPerWarp / 2) + j * 16, w[j]);
-                    }
-                    tmem_st_wait();
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&m_full[mb]);
+                    if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                }
+                if (hit) tmem_st_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    uint8_t* hw = hits + s * 16 + q * 4 + h * kSub;
+                    if constexpr (kSub == 1) *hw = (uint8_t)hit;
+                    else if constexpr (kSub == 2) *reinterpret_cast<uint16_t*>(hw) = (uint16_t)hit;
+                    else *reinterpret_cast<uint32_t*>(hw) = hit;
+                    mbar_arrive(&done[s]);
                 }
             }
             if (!ok) break;
+            g0 += pt1 - pt0;
             if (lead) {
                 if (!warp_wait(d_full, it & 1, abort)) break;
                 tc_fence_after();
                 // Y: per half [sum ph | sum pm | sum pl | count] (the count in
-                // half 0); Y is handed back after the last half's load, the
-                // sums go out as fixed-point reductions half by half
+                // half 0), set back to zero once read; Y is handed back after
+                // the last half, the sums go out as fixed-point reductions half
+                // by half
                 const uint32_t ty = tmem + kColY + lane_base;
                 bool live = false;
 #pragma unroll
@@ -681,7 +747,10 @@ k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
                     } else {
                         tmem_ld_wait();
                     }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) tmem_zero16(ty + 64 * hf + 16 * k);
                     if (hf == kHalves - 1) {
+                        tmem_st_wait();
                         tc_fence_before();
                         mbar_arrive(d_empty);
                     }
@@ -815,13 +884,13 @@ ms_status launch_shift_tc(ms_ctx* ctx, const int32_t* active, int grid, int targ
         if (ctx->Dp == 32) {
             if (dbg_S) return set_error(MS_ERR_INVALID_ARG, "the score dump is for d <= 16");
             k_shift_tc<Sh, 32, false, TcSingleMap><<<grid, Sh::kThreads, TcDim<32>::kSmemBytes, ctx->stream>>>(
-                ctx->pmap, ctx->pmap1, ctx->P32, ctx->X, ctx->acc, c, map, &ctx->dc->status, band, nullptr, 0);
+                ctx->pmap, ctx->pmap1, ctx->X, ctx->acc, c, map, &ctx->dc->status, band, nullptr, 0);
         } else if (dbg_S) {
             k_shift_tc<Sh, 16, true, TcSingleMap><<<grid, Sh::kThreads, TcDim<16>::kSmemBytes, ctx->stream>>>(
-                ctx->pmap, ctx->pmap1, ctx->P32, ctx->X, ctx->acc, c, map, &ctx->dc->status, band, dbg_S, ctx->n_pad);
+                ctx->pmap, ctx->pmap1, ctx->X, ctx->acc, c, map, &ctx->dc->status, band, dbg_S, ctx->n_pad);
         } else {
             k_shift_tc<Sh, 16, false, TcSingleMap><<<grid, Sh::kThreads, TcDim<16>::kSmemBytes, ctx->stream>>>(
-                ctx->pmap, ctx->pmap1, ctx->P32, ctx->X, ctx->acc, c, map, &ctx->dc->status, band, nullptr, 0);
+                ctx->pmap, ctx->pmap1, ctx->X, ctx->acc, c, map, &ctx->dc->status, band, nullptr, 0);
         }
         MS_LAUNCH("k_shift_tc");
         return MS_OK;
@@ -848,11 +917,13 @@ struct TcBatchMap {
         const int f = locate(plan.item_off, nf, i);
         const int local = i - plan.item_off[f];
         const int chunks = plan.chunks[f], tpc = plan.tpc[f];
-        const int t = local / chunks, ch = local - t * chunks;
+        const int n_active = states[f].dc.n_active;
+        int t, ch;
+        tc_item_place(local, (n_active + 127) / 128, chunks, &t, &ch);
         const BFrame& fr = frames[f];
         TcItem it;
         it.active = ((states[f].dc.iters & 1) ? act1 : act0) + fr.pix0;
-        it.n_active = states[f].dc.n_active;
+        it.n_active = n_active;
         it.seed0 = t * 128;
         it.pt0 = ch * tpc;
         it.pt1 = min(fr.n_ptiles, it.pt0 + tpc);
@@ -867,7 +938,7 @@ ms_status tc_batch_setup(int D) {
     return D == 32 ? allow_smem_all_shapes<TcBatchMap, 32>() : allow_smem_all_shapes<TcBatchMap, 16>();
 }
 
-ms_status launch_shift_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, int D, const float* P32,
+ms_status launch_shift_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, int D,
                                 const float* X, unsigned long long* acc, float c_f, const BFrame* frames,
                                 const BState* states, BPlan plan, const int32_t* act0, const int32_t* act1, int nf,
                                 int* status, unsigned long long* band, int grid, int shape, cudaStream_t st) {
@@ -883,10 +954,10 @@ ms_status launch_shift_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap
         using Sh = decltype(sh);
         if (D == 32)
             k_shift_tc<Sh, 32, false, TcBatchMap><<<grid, Sh::kThreads, TcDim<32>::kSmemBytes, st>>>(
-                pmap, pmap1, P32, X, acc, c_f, map, status, band, nullptr, 0);
+                pmap, pmap1, X, acc, c_f, map, status, band, nullptr, 0);
         else
             k_shift_tc<Sh, 16, false, TcBatchMap><<<grid, Sh::kThreads, TcDim<16>::kSmemBytes, st>>>(
-                pmap, pmap1, P32, X, acc, c_f, map, status, band, nullptr, 0);
+                pmap, pmap1, X, acc, c_f, map, status, band, nullptr, 0);
         MS_LAUNCH("k_shift_tc(batch)");
         return MS_OK;
     });

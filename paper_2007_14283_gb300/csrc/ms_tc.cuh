@@ -52,6 +52,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
+// The same without suspending.
+__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
 // Bounded wait for the phase with the given parity to complete. Returns false
 // (and raises *abort) on timeout, or at once when *abort is already raised.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
@@ -165,6 +177,15 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
         "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
         : "memory");
 }
+// Thread i of the warp writes zeros to row (lane base + i), columns
+// [col, col + 16).
+__device__ __forceinline__ void tmem_zero16(uint32_t taddr) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, "
+        "%1, %1, %1};" ::"r"(taddr),
+        "r"(0)
+        : "memory");
+}
 // Thread i of the warp writes r[0..7] to row (lane base + i), columns
 // [col, col + 8).
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
@@ -221,6 +242,54 @@ __device__ __forceinline__ void mma_bf16_ts_warp(uint32_t d_tmem, uint32_t a_tme
         "elect.sync _|e, 0xffffffff;\n\t"
         "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
         "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// mma_bf16_split3_warp without accumulation, and then D += Ac Bc (64 and 96
+// bytes after a0 and b0: a split constant against ones).
+__device__ __forceinline__ void mma_bf16_split3c_warp(uint32_t d_tmem, uint64_t a0, uint64_t b0, uint32_t idesc) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t.reg .b64 a1, b1, ac, bc;\n\t"
+        "add.u64 a1, %1, 2;\n\t"
+        "add.u64 b1, %2, 2;\n\t"
+        "add.u64 ac, %1, 4;\n\t"
+        "add.u64 bc, %2, 6;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, b1, %3, 1;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a1, %2, %3, 1;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], ac, bc, %3, 1;\n\t}" ::"r"(d_tmem),
+        "l"(a0), "l"(b0), "r"(idesc)
+        : "memory");
+}
+// The three products of a split score, D += A0 B0 + A0 B1 + A1 B0 (all from
+// shared memory; b1 and a1 lie 32 bytes after b0 and a0), issued by one elected
+// lane.
+__device__ __forceinline__ void mma_bf16_split3_warp(uint32_t d_tmem, uint64_t a0, uint64_t b0, uint32_t idesc) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t.reg .b64 a1, b1;\n\t"
+        "add.u64 a1, %1, 2;\n\t"
+        "add.u64 b1, %2, 2;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, 1;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, b1, %3, 1;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a1, %2, %3, 1;\n\t}" ::"r"(d_tmem),
+        "l"(a0), "l"(b0), "r"(idesc)
+        : "memory");
+}
+// Two K steps of D += A[tmem] * B (the second 8 TMEM columns of A and 2048
+// bytes of B further on) with output lanes disabled: bit i % 32 of off<i / 32>
+// set keeps row i of D as it is (A's rows there are not used).
+__device__ __forceinline__ void mma_bf16_ts2_lanes_warp(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc,
+                                                        uint32_t idesc, uint32_t off0, uint32_t off1, uint32_t off2,
+                                                        uint32_t off3) {
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t.reg .b64 b1;\n\t.reg .b32 a1;\n\t"
+        "add.u64 b1, %2, 128;\n\t"
+        "add.u32 a1, %1, 8;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%4, %5, %6, %7}, 1;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [a1], b1, %3, {%4, %5, %6, %7}, 1;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(off0), "r"(off1), "r"(off2), "r"(off3)
         : "memory");
 }
 __device__ __forceinline__ void mma_commit_warp(uint64_t* bar) {
