@@ -177,7 +177,7 @@ struct Layout {
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 
-Layout plan(int64_t np, int Dp, bool bf16) {
+Layout plan(int64_t np, int Dp) {
     Layout L;
     const size_t n = (size_t)(np > 0 ? np : 1);
     const size_t sizes[] = {
@@ -203,12 +203,12 @@ Layout plan(int64_t np, int Dp, bool bf16) {
         n * kMergeCap * sizeof(int32_t),  // 19 conf
         ((n + 1023) / 1024 + 1) * sizeof(int32_t),  // 20 block_tmp
         sizeof(DevCounters),              // 21 dc
-        bf16 ? (n + 127) / 128 * 128 * 128 * (Dp / 16) : 0,  // 22 Pk (one array per 16 dimensions)
-        bf16 ? (n + 127) / 128 * 128 * 128 * (Dp / 16) : 0,  // 23 Mk (labelling on the tensor cores)
-        bf16 ? n * sizeof(int2) + 16 : 0,                     // 24 label_fix + count
-        bf16 ? n * Dp * sizeof(float) : 0,                    // 25 Xr (merge candidates in rank order)
-        bf16 ? n : 0,                                         // 26 removed_r
-        bf16 ? (n + 127) / 128 * 128 * 128 * (Dp / 16) : 0,  // 27 Ck (their BF16 split rows)
+        (n + 127) / 128 * 128 * 128 * (Dp / 16),  // 22 Pk (one array per 16 dimensions)
+        (n + 127) / 128 * 128 * 128 * (Dp / 16),  // 23 Mk (labelling on the tensor cores)
+        n * sizeof(int2) + 16,                     // 24 label_fix + count
+        n * Dp * sizeof(float),                    // 25 Xr (merge candidates in rank order)
+        n,                                         // 26 removed_r
+        (n + 127) / 128 * 128 * 128 * (Dp / 16),  // 27 Ck (their BF16 split rows)
         (n + kFinThreads - 1) / kFinThreads * kMoveWords * sizeof(uint32_t),  // 28 moving
     };
     size_t t = 0;
@@ -283,7 +283,7 @@ ms_status ms_workspace_bytes(const ms_config* cfg, int64_t n_pixels, int64_t* by
     if (s != MS_OK) return s;
     if (!bytes_out || n_pixels < 0 || n_pixels >= (1LL << 24))
         return set_error(MS_ERR_INVALID_ARG, "n_pixels must be in [0, 2^24)");
-    *bytes_out = (int64_t)plan(n_pixels, padded_dim(cfg->dim), cfg->precision == MS_BF16).total;
+    *bytes_out = (int64_t)plan(n_pixels, padded_dim(cfg->dim)).total;
     return MS_OK;
 }
 
@@ -304,7 +304,7 @@ ms_status ctx_alloc(const ms_config* cfg, int64_t max_pixels, cudaStream_t strea
     ctx->num_sms = device_sms();
     ctx->shift_grid = ctx->num_sms * shift_blocks_per_sm();
     ctx->target_items = 2 * ctx->shift_grid;
-    const Layout L = plan(max_pixels, ctx->Dp, cfg->precision == MS_BF16);
+    const Layout L = plan(max_pixels, ctx->Dp);
     ctx->ws_bytes = L.total;
     cudaError_t e = workspace_malloc(&ctx->ws, L.total);
     if (e != cudaSuccess) {
@@ -339,12 +339,12 @@ ms_status ctx_alloc(const ms_config* cfg, int64_t max_pixels, cudaStream_t strea
     ctx->conf = (int32_t*)(b + L.off[19]);
     ctx->block_tmp = (int32_t*)(b + L.off[20]);
     ctx->dc = (DevCounters*)(b + L.off[21]);
-    ctx->Pk = cfg->precision == MS_BF16 ? (void*)(b + L.off[22]) : nullptr;
-    ctx->Mk = cfg->precision == MS_BF16 ? (void*)(b + L.off[23]) : nullptr;
-    ctx->label_fix = cfg->precision == MS_BF16 ? (int2*)(b + L.off[24]) : nullptr;
-    ctx->Xr = cfg->precision == MS_BF16 ? (float*)(b + L.off[25]) : nullptr;
-    ctx->removed_r = cfg->precision == MS_BF16 ? (uint8_t*)(b + L.off[26]) : nullptr;
-    ctx->Ck = cfg->precision == MS_BF16 ? (void*)(b + L.off[27]) : nullptr;
+    ctx->Pk = (void*)(b + L.off[22]);
+    ctx->Mk = (void*)(b + L.off[23]);
+    ctx->label_fix = (int2*)(b + L.off[24]);
+    ctx->Xr = (float*)(b + L.off[25]);
+    ctx->removed_r = (uint8_t*)(b + L.off[26]);
+    ctx->Ck = (void*)(b + L.off[27]);
     ctx->moving = (uint32_t*)(b + L.off[28]);
     ctx->round_log_cap = 64;
     ctx->round_log = new (std::nothrow) int64_t[ctx->round_log_cap * 4];
@@ -371,7 +371,7 @@ ms_status ctx_bind_async(ms_ctx* ctx, const float* d_emb, const uint8_t* d_mask,
     const cudaStream_t keep = ctx->stream;
     ctx->stream = st;
     ms_status s = launch_ingest(ctx);
-    if (s == MS_OK && ctx->cfg.precision == MS_BF16) s = tc_pack_async(ctx);
+    if (s == MS_OK) s = tc_pack_async(ctx);
     ctx->stream = keep;
     return s;
 }
@@ -387,7 +387,7 @@ ms_status ctx_bind_finish(ms_ctx* ctx, cudaStream_t st, uint64_t frame_id, int64
     ctx->uncovered = ctx->n;
     seed_order_params(ctx->n, ctx->cfg.seed, frame_id, &ctx->perm_a, &ctx->perm_b);
     ctx->n_pad = ctx->n > 0 ? (ctx->n + 127) / 128 * 128 : 0;
-    if (ctx->cfg.precision == MS_BF16 && ctx->n > 0) {
+    if (ctx->n > 0) {
         ms_status s = tc_finish(ctx);
         if (s != MS_OK) return s;
     }
@@ -497,6 +497,7 @@ ms_status ms_iterate(ms_ctx* ctx, int32_t max_iter, int32_t* n_converged_out, in
         }
         ms_status s = readback(ctx);
         if (s != MS_OK) return s;
+        if (ctx->hc->status & 2) return set_error(MS_ERR_TIMEOUT, "a bounded device wait in the shift gave up");
         if (ctx->prof) {
             // only launches that ran an iteration (the rest returned at once)
             const int real = ctx->hc->iters - iters_before;

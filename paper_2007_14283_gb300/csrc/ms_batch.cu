@@ -463,7 +463,7 @@ __global__ void k_b_plan(const BFrame* __restrict__ frames, const BState* __rest
                 const ShiftSplit sp = shift_split(na, fr.n, tf);
                 plan.tpc[f] = sp.chunk_len;
                 plan.chunks[f] = sp.chunks;
-                items = sp.tiles * sp.chunks;
+                items = (na + 127) / 128 * sp.chunks;
             }
             seeds = (na + kFinThreads - 1) / kFinThreads;
         }
@@ -706,100 +706,6 @@ __global__ void k_b_rank(const BFrame* __restrict__ frames, const BState* __rest
 
 template <int Dp>
 __global__ void __launch_bounds__(kMT)
-k_b_merge_old(const BFrame* __restrict__ frames, const BState* __restrict__ states, int B,
-              const int32_t* __restrict__ off, const float* __restrict__ X, const int32_t* __restrict__ cand,
-              const float* __restrict__ modes, float thr_f, double thr, uint8_t* __restrict__ cand_state,
-              const int32_t* __restrict__ cand_rank, uint8_t* __restrict__ removed_r) {
-    __shared__ __align__(16) float tile[kVT * Dp];
-    const int S = off[B + 1];
-    for (int bb = blockIdx.x; bb < off[B]; bb += gridDim.x) {
-        const int f = locate(off, B, bb);
-        const int lb = bb - off[f], sl = lb % S;
-        const int64_t base = frames[f].pix0;
-        const int k = states[f].dc.n_cand;
-        const int K_old = states[f].dc.n_kept;
-        const int a = (lb / S) * kMT + threadIdx.x;
-        const int lo = (int)((int64_t)sl * K_old / S), hi = (int)((int64_t)(sl + 1) * K_old / S);
-        float x[Dp];
-        if (a < k) ldv<Dp>(x, X + (int64_t)cand[base + a] * Dp);
-        bool removed = false;
-        for (int t0 = lo; t0 < hi; t0 += kVT) {
-            const int cnt = min(kVT, hi - t0);
-            __syncthreads();
-            for (int q = threadIdx.x; q < cnt * Dp; q += kMT) tile[q] = modes[(base + t0) * Dp + q];
-            __syncthreads();
-            if (a < k && !removed)
-                for (int j = 0; j < cnt; ++j)
-                    if (cos_at_least<Dp>(x, tile + j * Dp, thr_f, thr)) {
-                        removed = true;
-                        break;
-                    }
-        }
-        if (a < k && removed) {
-            cand_state[base + a] = kRemoved;
-            removed_r[base + cand_rank[base + a]] = 1;
-        }
-        __syncthreads();
-    }
-}
-
-template <int Dp>
-__global__ void __launch_bounds__(kMT)
-k_b_merge_pairs(const BFrame* __restrict__ frames, const BState* __restrict__ states, int B,
-                const int32_t* __restrict__ off, const float* __restrict__ Xr, const uint8_t* __restrict__ removed_r,
-                const int32_t* __restrict__ rank_cand, float thr_f, double thr, int32_t* __restrict__ conf_deg,
-                int32_t* __restrict__ conf) {
-    // Candidates are visited in rank order: thread t of a block takes rank
-    // r0 + t and compares it with every higher-priority candidate (rank < its
-    // own) in the block's slice of ranks, so neighbouring lanes stop at
-    // neighbouring ranks and only the k(k-1)/2 ordered pairs are tested. The
-    // positions come from Xr (rank order), so a tile is one contiguous block
-    // of rows, read as float4.
-    constexpr int kQ = kVT * Dp / 4;  // float4 per tile
-    __shared__ __align__(16) float tile[kVT * Dp];
-    __shared__ int32_t s_idx[kVT];
-    __shared__ uint8_t s_rem[kVT];
-    const int S = off[B + 1];
-    for (int bb = blockIdx.x; bb < off[B]; bb += gridDim.x) {
-        const int f = locate(off, B, bb);
-        const int lb = bb - off[f], sl = lb % S;
-        const int64_t base = frames[f].pix0;
-        const int k = states[f].dc.n_cand;
-        const int r0 = (lb / S) * kMT;
-        const int r = r0 + threadIdx.x;
-        const bool act = r < k && !removed_r[base + r];
-        const int a = act ? rank_cand[base + r] : -1;
-        const int lo = (int)((int64_t)sl * k / S);
-        const int hi = min((int)((int64_t)(sl + 1) * k / S), r0 + kMT - 1);
-        float x[Dp];
-        if (act) ldv<Dp>(x, Xr + (base + r) * Dp);
-        for (int t0 = lo; t0 < hi; t0 += kVT) {
-            const int cnt = min(kVT, hi - t0);
-            __syncthreads();
-            const float4* src = reinterpret_cast<const float4*>(Xr + (base + t0) * Dp);
-            for (int q = threadIdx.x; q < cnt * (Dp / 4) && q < kQ; q += kMT) reinterpret_cast<float4*>(tile)[q] = src[q];
-            for (int j = threadIdx.x; j < cnt; j += kMT) {
-                s_idx[j] = rank_cand[base + t0 + j];
-                s_rem[j] = removed_r[base + t0 + j];
-            }
-            __syncthreads();
-            if (act) {
-                const int jend = min(cnt, r - t0);
-                for (int j = 0; j < jend; ++j) {
-                    if (s_rem[j]) continue;
-                    if (cos_at_least<Dp>(x, tile + j * Dp, thr_f, thr)) {
-                        const int slot = atomicAdd(&conf_deg[base + a], 1);
-                        if (slot < kMergeCap) conf[(base + a) * kMergeCap + slot] = s_idx[j];
-                    }
-                }
-            }
-        }
-        __syncthreads();
-    }
-}
-
-template <int Dp>
-__global__ void __launch_bounds__(kMT)
 k_b_merge_resolve(const BFrame* __restrict__ frames, BState* states, int B, const int32_t* __restrict__ off,
                   const float* __restrict__ X, const int32_t* __restrict__ cand,
                   const int32_t* __restrict__ cand_rank, const int32_t* __restrict__ rank_cand, uint8_t* cand_state,
@@ -906,108 +812,6 @@ k_b_merge_append(const BFrame* __restrict__ frames, BState* states, const float*
     }
 }
 
-// Coverage for the frames whose round ended: FP32 decides, FP64 inside the band.
-// A block takes kPT * cov_per(Dp) consecutive pixels (1024 for d <= 16),
-// compacts the uncovered ones into a shared list (warp ballots and a prefix
-// over the block's warp-passes) and gives each thread up to cov_per of them,
-// so every tile of new modes read from memory is tested against all the
-// block's uncovered pixels at once.
-__host__ __device__ constexpr int cov_per(int Dp) { return Dp <= 16 ? 4 : 2; }
-
-template <int Dp>
-__global__ void __launch_bounds__(kPT)
-k_b_cover(const BFrame* __restrict__ frames, BState* states, int B, const int32_t* __restrict__ off, int d,
-          const float* __restrict__ P32, const int32_t* __restrict__ pix, uint8_t* __restrict__ covered,
-          const float* __restrict__ modes, float c_f, double c) {
-    __shared__ __align__(16) float tile[kVT * Dp];
-    constexpr int kCovPer = cov_per(Dp);
-    constexpr int kNW = kPT / 32 * kCovPer;  // warp-passes of a block
-    static_assert(kNW <= 32, "one warp scans the warp-pass counts");
-    __shared__ int32_t s_list[kPT * kCovPer];
-    __shared__ int32_t s_pos[kNW];
-    __shared__ int s_nact;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int bb = blockIdx.x; bb < off[B]; bb += gridDim.x) {
-        const int f = locate(off, B, bb);
-        const int lb = bb - off[f];
-        const BFrame& fr = frames[f];
-        BState& st = states[f];
-        const int64_t base = fr.pix0;
-        const int k0 = st.k0, k1 = st.dc.n_kept;
-        const int i0 = lb * kPT * kCovPer;
-        unsigned bal[kCovPer];
-#pragma unroll
-        for (int u = 0; u < kCovPer; ++u) {
-            const int i = i0 + u * kPT + threadIdx.x;
-            bal[u] = __ballot_sync(0xffffffffu, i < fr.n && covered[base + i] == 0);
-            if (lane == 0) s_pos[u * (kPT / 32) + warp] = __popc(bal[u]);
-        }
-        __syncthreads();
-        if (warp == 0) {
-            const int v = lane < kNW ? s_pos[lane] : 0;
-            int incl = v;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += t;
-            }
-            if (lane < kNW) s_pos[lane] = incl - v;
-            if (lane == 31) s_nact = incl;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < kCovPer; ++u)
-            if ((bal[u] >> lane) & 1u)
-                s_list[s_pos[u * (kPT / 32) + warp] + __popc(bal[u] & ((1u << lane) - 1u))] =
-                    i0 + u * kPT + threadIdx.x;
-        __syncthreads();
-        const int nact = s_nact;
-        if (nact == 0) continue;
-        int idx[kCovPer];
-        float p[kCovPer][Dp];
-        bool cov[kCovPer], band[kCovPer];
-#pragma unroll
-        for (int u = 0; u < kCovPer; ++u) {
-            const int e = threadIdx.x + u * kPT;
-            idx[u] = e < nact ? s_list[e] : -1;
-            if (idx[u] >= 0) ldv<Dp>(p[u], P32 + (base + idx[u]) * Dp);
-            cov[u] = band[u] = false;
-        }
-        for (int t0 = k0; t0 < k1; t0 += kVT) {
-            const int cnt = min(kVT, k1 - t0);
-            __syncthreads();
-            for (int q = threadIdx.x; q < cnt * Dp; q += kPT) tile[q] = modes[(base + t0) * Dp + q];
-            __syncthreads();
-#pragma unroll
-            for (int u = 0; u < kCovPer; ++u)
-                if (idx[u] >= 0 && !cov[u])
-                    for (int j = 0; j < cnt; ++j) {
-                        const float sc = dot_seq<Dp>(p[u], tile + j * Dp);
-                        if (sc >= c_f + kEpsF32) { cov[u] = true; break; }
-                        if (sc >= c_f - kEpsF32) band[u] = true;
-                    }
-        }
-        int newly = 0;
-#pragma unroll
-        for (int u = 0; u < kCovPer; ++u) {
-            if (idx[u] >= 0 && !cov[u] && band[u]) {
-                const float* e = fr.emb + (int64_t)pix[base + idx[u]] * d;
-                for (int j = k0; j < k1 && !cov[u]; ++j) {
-                    const float* m = modes + (base + j) * Dp;
-                    if (dot_seq<Dp>(p[u], m) >= c_f - kEpsF32 && cos64(e, m, d) >= c) cov[u] = true;
-                }
-            }
-            if (idx[u] >= 0 && cov[u]) {
-                covered[base + idx[u]] = 1;
-                ++newly;
-            }
-        }
-        // each warp's count of newly covered pixels
-        for (int o = 16; o > 0; o >>= 1) newly += __shfl_xor_sync(0xffffffffu, newly, o);
-        if (lane == 0 && newly) atomicSub(&st.dc.n_uncovered, newly);
-        __syncthreads();
-    }
-}
-
 __global__ void k_b_schedule(BState* states, int B, double P, double L, double H, int max_rounds, int all_seeds) {
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
     if (f >= B) return;
@@ -1057,54 +861,6 @@ __global__ void k_b_cond(const BState* __restrict__ states, int B, int* misc, in
     cudaGraphSetConditional(h, live ? 1u : 0u);
 }
 
-// ------------------------------------------------------------ labels
-template <int Dp>
-__global__ void __launch_bounds__(kPT)
-k_b_label(const BFrame* __restrict__ frames, const BState* __restrict__ states, int B,
-          const int32_t* __restrict__ off, int d, const float* __restrict__ P32, const int32_t* __restrict__ pix,
-          const float* __restrict__ modes, int32_t* const* __restrict__ labels) {
-    __shared__ __align__(16) float tile[kVT * Dp];
-    for (int bb = blockIdx.x; bb < off[B]; bb += gridDim.x) {
-        const int f = locate(off, B, bb);
-        const int lb = bb - off[f];
-        const BFrame& fr = frames[f];
-        const int64_t base = fr.pix0;
-        const int K = states[f].dc.n_kept;
-        const int i = lb * kPT + threadIdx.x;
-        const bool act = i < fr.n;
-        float p[Dp];
-        if (act) ldv<Dp>(p, P32 + (base + i) * Dp);
-        float b1 = -INFINITY, b2 = -INFINITY;
-        int best = -1;
-        for (int t0 = 0; t0 < K; t0 += kVT) {
-            const int cnt = min(kVT, K - t0);
-            __syncthreads();
-            for (int q = threadIdx.x; q < cnt * Dp; q += kPT) tile[q] = modes[(base + t0) * Dp + q];
-            __syncthreads();
-            if (act)
-                for (int j = 0; j < cnt; ++j) {
-                    const float s = dot_seq<Dp>(p, tile + j * Dp);
-                    if (s > b1) { b2 = b1; b1 = s; best = t0 + j; }
-                    else if (s > b2) b2 = s;
-                }
-        }
-        if (act) {
-            if (K > 1 && b1 - b2 <= 2.f * kEpsF32) {
-                const float* e = fr.emb + (int64_t)pix[base + i] * d;
-                double bc = -INFINITY;
-                for (int j = 0; j < K; ++j) {
-                    const float* m = modes + (base + j) * Dp;
-                    if (dot_seq<Dp>(p, m) < b1 - 2.f * kEpsF32) continue;
-                    const double cs = cos64(e, m, d);
-                    if (cs > bc) { bc = cs; best = j; }
-                }
-            }
-            labels[f][pix[base + i]] = best;
-        }
-        __syncthreads();
-    }
-}
-
 // ------------------------------------------------------------ host
 float ceil_f(double c) { return ceil_to_float(c); }
 
@@ -1143,8 +899,8 @@ ms_status enqueue_body(ms_batch* b, cudaStream_t s, cudaGraphConditionalHandle h
                                    b->act[1], B, b->misc + 1, (unsigned long long*)(b->misc + 2), b->tc_grid,
                                    b->tc_shape, s);
     else
-        st = launch_shift_fp32_batch(b->P32, b->X, b->acc, cf, Dp, b->frames, b->states, b->plan, b->act[0],
-                                     b->act[1], B, b->f32_grid, s);
+        st = launch_shift_f32_tc_batch(b->pmap, b->pmap1, Dp, b->X, b->acc, cf, b->frames, b->states, b->plan,
+                                       b->act[0], b->act[1], B, b->misc + 1, b->num_sms, s);
     if (st != MS_OK) return st;
     ++nl;
     if (b->prof) {
@@ -1183,21 +939,12 @@ ms_status enqueue_body(ms_batch* b, cudaStream_t s, cudaGraphConditionalHandle h
     k_b_rank_invert<Dp><<<G, kMT, 0, s>>>(b->frames, b->states, B, b->blk_off, b->cand_rank, b->cand, b->X,
                                           b->rank_cand, b->Xr);
     LAUNCHED("k_b_rank_invert");
-    if (b->Ck) {  // BF16 form: both contractions of the merge on the tensor cores
-        ms_status ms2 = launch_merge_tc_batch(b->cmap, b->cmap1, b->mmap, b->mmap1, b->Ck, b->total_pk_rows, Dp,
-                                              b->frames, b->states, B, (int)b->max_pk_rows, b->Xr, b->modes,
-                                              b->rank_cand, b->cand_state, b->removed_r, b->conf_deg, b->conf, mf,
-                                              b->cfg.merge_cos, b->blk_off, b->lsc, b->num_sms, b->misc + 1, s);
-        if (ms2 != MS_OK) return ms2;
-        nl += 4;
-    } else {
-        k_b_merge_old<Dp><<<G, kMT, 0, s>>>(b->frames, b->states, B, b->blk_split, b->X, b->cand, b->modes, mf,
-                                            b->cfg.merge_cos, b->cand_state, b->cand_rank, b->removed_r);
-        LAUNCHED("k_b_merge_old");
-        k_b_merge_pairs<Dp><<<G, kMT, 0, s>>>(b->frames, b->states, B, b->blk_split, b->Xr, b->removed_r,
-                                              b->rank_cand, mf, b->cfg.merge_cos, b->conf_deg, b->conf);
-        LAUNCHED("k_b_merge_pairs");
-    }
+    st = launch_merge_tc_batch(b->cmap, b->cmap1, b->mmap, b->mmap1, b->Ck, b->total_pk_rows, Dp, b->frames, b->states,
+                               B, (int)b->max_pk_rows, b->Xr, b->modes, b->rank_cand, b->cand_state, b->removed_r,
+                               b->conf_deg, b->conf, mf, b->cfg.merge_cos, b->blk_off, b->lsc, b->num_sms, b->misc + 1,
+                               s);
+    if (st != MS_OK) return st;
+    nl += 4;
     for (int sw = 0; sw < 8; ++sw) {
         k_b_merge_resolve<Dp><<<G, kMT, 0, s>>>(b->frames, b->states, B, b->blk_off, b->X, b->cand, b->cand_rank,
                                                 b->rank_cand, b->cand_state, b->conf_deg, b->conf, mf,
@@ -1214,22 +961,13 @@ ms_status enqueue_body(ms_batch* b, cudaStream_t s, cudaGraphConditionalHandle h
         k_b_phase<<<1, 1, 0, s>>>(b->misc, kPhMerge);
         LAUNCHED("k_b_phase");
     }
-    if (b->Mk) {  // BF16 form: the pixels against the new modes on the tensor cores
-        k_b_blocks<<<1, 32, 0, s>>>(b->frames, b->states, B, kSelDonePixels, 128, 0, b->blk_off);
-        LAUNCHED("k_b_blocks");
-        ms_status cs = launch_cover_tc_batch(b->pmap, b->mmap, b->pmap1, b->mmap1, b->Mk, b->total_pk_rows, Dp,
-                                             b->frames, b->states, B, (int)b->max_pk_rows,
-                                             b->modes, b->P32, b->pix, b->d, b->cfg.bandwidth_cos, b->covered,
-                                             b->blk_off, b->lsc, b->num_sms, b->misc + 1, s);
-        if (cs != MS_OK) return cs;
-        nl += 3;
-    } else {
-        k_b_blocks<<<1, 32, 0, s>>>(b->frames, b->states, B, kSelDonePixels, kPT * cov_per(Dp), 0, b->blk_off);
-        LAUNCHED("k_b_blocks");
-        k_b_cover<Dp><<<G, kPT, 0, s>>>(b->frames, b->states, B, b->blk_off, b->d, b->P32, b->pix, b->covered,
-                                        b->modes, (float)b->cfg.bandwidth_cos, b->cfg.bandwidth_cos);
-        LAUNCHED("k_b_cover");
-    }
+    k_b_blocks<<<1, 32, 0, s>>>(b->frames, b->states, B, kSelDonePixels, 128, 0, b->blk_off);
+    LAUNCHED("k_b_blocks");
+    st = launch_cover_tc_batch(b->pmap, b->mmap, b->pmap1, b->mmap1, b->Mk, b->total_pk_rows, Dp, b->frames, b->states,
+                               B, (int)b->max_pk_rows, b->modes, b->P32, b->pix, b->d, b->cfg.bandwidth_cos,
+                               b->covered, b->blk_off, b->lsc, b->num_sms, b->misc + 1, s);
+    if (st != MS_OK) return st;
+    nl += 3;
     if (b->prof_phases) {
         k_b_phase<<<1, 1, 0, s>>>(b->misc, kPhCover);
         LAUNCHED("k_b_phase");
@@ -1269,11 +1007,9 @@ ms_status enqueue_setup(ms_batch* b, cudaStream_t s) {
     MS_LAUNCH("k_b_scan");
     k_b_compact<<<gc, kIT, 0, s>>>(b->frames, (int)b->nblk_max, b->block_tmp, b->d, Dp, b->P32, b->pix, b->misc + 1);
     MS_LAUNCH("k_b_compact");
-    if (b->tc) {
-        const dim3 gp((unsigned)((b->max_pk_rows + 255) / 256), (unsigned)B);
-        k_b_pack<<<gp, 256, 0, s>>>(b->frames, b->P32, Dp, (int64_t)b->total_pk_rows, (uint4*)b->Pk);
-        MS_LAUNCH("k_b_pack");
-    }
+    const dim3 gp((unsigned)((b->max_pk_rows + 255) / 256), (unsigned)B);
+    k_b_pack<<<gp, 256, 0, s>>>(b->frames, b->P32, Dp, (int64_t)b->total_pk_rows, (uint4*)b->Pk);
+    MS_LAUNCH("k_b_pack");
     const dim3 gl((unsigned)((b->max_np + 255) / 256 < 1024 ? (b->max_np + 255) / 256 : 1024), (unsigned)B);
     k_b_labels_clear<<<gl, 256, 0, s>>>(b->frames, b->label_ptrs);
     MS_LAUNCH("k_b_labels_clear");
@@ -1294,17 +1030,9 @@ ms_status enqueue_label_tick(ms_batch* b, cudaStream_t s) {
 
 template <int Dp>
 ms_status enqueue_label(ms_batch* b, cudaStream_t s) {
-    if (b->Mk)  // BF16 form: the tensor-core kernel, same labels (exact FP64 argmax)
-        return launch_label_tc_batch(b->pmap, b->mmap, b->pmap1, b->mmap1, b->Mk, b->total_pk_rows, Dp, b->frames,
-                                     b->states, b->B, (int)b->max_pk_rows,
-                                     b->modes, b->P32, b->pix, b->d, b->label_ptrs, b->lsc, b->num_sms, b->misc + 1,
-                                     s);
-    k_b_blocks<<<1, 32, 0, s>>>(b->frames, b->states, b->B, kSelAllPixels, kPT, 0, b->blk_off);
-    MS_LAUNCH("k_b_blocks");
-    k_b_label<Dp><<<b->grid, kPT, 0, s>>>(b->frames, b->states, b->B, b->blk_off, b->d, b->P32, b->pix, b->modes,
-                                          b->label_ptrs);
-    MS_LAUNCH("k_b_label");
-    return MS_OK;
+    return launch_label_tc_batch(b->pmap, b->mmap, b->pmap1, b->mmap1, b->Mk, b->total_pk_rows, Dp, b->frames,
+                                 b->states, b->B, (int)b->max_pk_rows, b->modes, b->P32, b->pix, b->d, b->label_ptrs,
+                                 b->lsc, b->num_sms, b->misc + 1, s);
 }
 
 template <int Dp>
@@ -1351,7 +1079,7 @@ ms_status build_graph(ms_batch* b) {
     if (st2 != MS_OK) return st2;
     MS_CUDA(cudaGraphInstantiate(&b->exec, g, 0));
     b->body_launches = nl;
-    b->fixed_launches = (b->tc ? 5 : 4) + (b->Mk ? 4 : 2) + (b->prof_phases ? 3 : 0);  // set-up, then labelling
+    b->fixed_launches = 9 + (b->prof_phases ? 3 : 0);  // set-up, then labelling
     return MS_OK;
 }
 
@@ -1451,15 +1179,14 @@ extern "C" ms_status ms_batch_create(const ms_config* cfg, int32_t B, const floa
     b->max_pk_rows = (b->max_np + 127) / 128 * 128;
     b->nblk_max = (b->max_np + kIT - 1) / kIT;
     const int Dp = b->Dp;
-    const bool tcl = b->tc;  // labelling and coverage on the tensor cores
     const size_t n = (size_t)b->total_px;
     const size_t sizes[] = {
         sizeof(BFrame) * B, sizeof(BState) * B, sizeof(int32_t) * ((B + 1) * 4 + (B + 2) * 2), sizeof(b->h_misc),
         n * Dp * 4, n * 4, n, n * Dp * 4, n * 4, n * 4, n, n * 4, n * 4, n * 4,
         n * (Dp + 1) * 8, n * Dp * 4, n * 4, n * 4, n * 4, n, n * 4, n * kMergeCap * 4,
-        (size_t)B * b->nblk_max * 4 + 4, b->tc ? (size_t)b->total_pk_rows * 128 * (Dp / 16) : 0, sizeof(int32_t*) * B,
-        tcl ? (size_t)b->total_pk_rows * 128 * (Dp / 16) : 0, tcl ? n * sizeof(int2) : 0, sizeof(int32_t) * (B + 1) + 16,
-        n * Dp * 4, n, tcl ? (size_t)b->total_pk_rows * 128 * (Dp / 16) : 0,
+        (size_t)B * b->nblk_max * 4 + 4, (size_t)b->total_pk_rows * 128 * (Dp / 16), sizeof(int32_t*) * B,
+        (size_t)b->total_pk_rows * 128 * (Dp / 16), n * sizeof(int2), sizeof(int32_t) * (B + 1) + 16,
+        n * Dp * 4, n, (size_t)b->total_pk_rows * 128 * (Dp / 16),
         (n / kFinThreads + B) * kMoveWords * sizeof(uint32_t)};
     const int NS = (int)(sizeof(sizes) / sizeof(sizes[0]));
     size_t offs[32], tot = 0;
@@ -1503,15 +1230,15 @@ extern "C" ms_status ms_batch_create(const ms_config* cfg, int32_t B, const floa
     b->conf_deg = (int32_t*)(w + offs[20]);
     b->conf = (int32_t*)(w + offs[21]);
     b->block_tmp = (int32_t*)(w + offs[22]);
-    b->Pk = b->tc ? (void*)(w + offs[23]) : nullptr;
+    b->Pk = (void*)(w + offs[23]);
     b->label_ptrs = (int32_t**)(w + offs[24]);
-    b->Mk = tcl ? (void*)(w + offs[25]) : nullptr;
-    b->lsc.fix = tcl ? (int2*)(w + offs[26]) : nullptr;
+    b->Mk = (void*)(w + offs[25]);
+    b->lsc.fix = (int2*)(w + offs[26]);
     b->lsc.off = (int32_t*)(w + offs[27]);
     b->lsc.fix_count = b->lsc.off + (B + 1);
     b->Xr = (float*)(w + offs[28]);
     b->removed_r = (uint8_t*)(w + offs[29]);
-    b->Ck = tcl ? (void*)(w + offs[30]) : nullptr;
+    b->Ck = (void*)(w + offs[30]);
     b->moving = (uint32_t*)(w + offs[31]);
     ms_status s = cuda_check(cudaMallocHost((void**)&b->h_states, sizeof(BState) * B), "cudaMallocHost");
     if (s == MS_OK) s = cuda_check(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking), "cudaStreamCreate");
@@ -1523,20 +1250,20 @@ extern "C" ms_status ms_batch_create(const ms_config* cfg, int32_t B, const floa
                                        b->stream),
                        "copy label pointers");
     if (s == MS_OK) s = cuda_check(cudaStreamSynchronize(b->stream), "sync");
-    if (s == MS_OK && b->tc) s = tc_batch_setup(Dp);
-    if (s == MS_OK && b->tc) s = encode_pk_map(b->Pk, (int)b->total_pk_rows, &b->pmap);
-    if (s == MS_OK && b->tc)
+    if (s == MS_OK) s = b->tc ? tc_batch_setup(Dp, b->tc_shape) : f32_tc_setup(Dp);
+    if (s == MS_OK) s = encode_pk_map(b->Pk, (int)b->total_pk_rows, &b->pmap);
+    if (s == MS_OK)
         s = encode_pk_map(Dp == 32 ? (uint8_t*)b->Pk + (size_t)b->total_pk_rows * 128 : b->Pk, (int)b->total_pk_rows,
                           &b->pmap1);
-    if (s == MS_OK && tcl) s = encode_pk_map(b->Mk, (int)b->total_pk_rows, &b->mmap);
-    if (s == MS_OK && tcl) b->mmap1 = b->mmap;
-    if (s == MS_OK && tcl && Dp == 32)
+    if (s == MS_OK) s = encode_pk_map(b->Mk, (int)b->total_pk_rows, &b->mmap);
+    if (s == MS_OK) b->mmap1 = b->mmap;
+    if (s == MS_OK && Dp == 32)
         s = encode_pk_map((uint8_t*)b->Mk + (size_t)b->total_pk_rows * 128, (int)b->total_pk_rows, &b->mmap1);
-    if (s == MS_OK && tcl) s = encode_pk_map(b->Ck, (int)b->total_pk_rows, &b->cmap);
-    if (s == MS_OK && tcl) b->cmap1 = b->cmap;
-    if (s == MS_OK && tcl && Dp == 32)
+    if (s == MS_OK) s = encode_pk_map(b->Ck, (int)b->total_pk_rows, &b->cmap);
+    if (s == MS_OK) b->cmap1 = b->cmap;
+    if (s == MS_OK && Dp == 32)
         s = encode_pk_map((uint8_t*)b->Ck + (size_t)b->total_pk_rows * 128, (int)b->total_pk_rows, &b->cmap1);
-    if (s == MS_OK && tcl) s = label_tc_setup();
+    if (s == MS_OK) s = label_tc_setup();
     if (s == MS_OK) s = rebuild_graph(b);
     if (s != MS_OK) {
         free_batch(b);
@@ -1617,6 +1344,8 @@ extern "C" ms_status ms_batch_configure(ms_batch* b, int32_t batch_split, int32_
     b->split = batch_split;
     b->target_mult = target_mult;
     b->tc_shape = tc_shape;
+    if (b->tc)
+        if (ms_status st = tc_batch_setup(b->Dp, tc_shape); st != MS_OK) return st;
     return rebuild_graph(b);
 }
 

@@ -141,7 +141,7 @@ struct ms_ctx {
     int32_t m_round;
     int32_t last_iters;  // iterations of the frame's last round (0: none yet)
     ms_stats stats;
-    // BF16 tensor-core form
+    // tensor-core operands
     void* Pk;            // [n_pad, 64] bf16: [Ph | Pm | Pl | 0] per pixel
     int64_t n_pad;       // n rounded up to 128 (0 when n = 0)
     CUtensorMap pmap;    // TMA map of Pk: boxes of 128 rows x 128 bytes, 128-byte swizzle
@@ -149,9 +149,9 @@ struct ms_ctx {
     int tc_grid;         // persistent grid of the tensor-core shift kernel
     void* Mk;            // [n_pad, 64] bf16 split rows of the kept modes (labelling)
     int2* label_fix;     // [n] near-tie queue of the tensor-core labelling, then its count
-    float* Xr;           // BF16 form: [n, Dp] merge candidates' positions in rank order
-    uint8_t* removed_r;  // BF16 form: [n] candidates removed by an earlier mode, by rank
-    void* Ck;            // BF16 form: [n_pad, 64] bf16 split rows of Xr (a second array for Dp = 32)
+    float* Xr;           // [n, Dp] merge candidates' positions in rank order
+    uint8_t* removed_r;  // [n] candidates removed by an earlier mode, by rank
+    void* Ck;            // [n_pad, 64] bf16 split rows of Xr (a second array for Dp = 32)
     // measurement
     bool prof;
     cudaEvent_t ev[64];  // start/end pairs around shift launches of one batch
@@ -189,7 +189,7 @@ ms_status launch_merge_resolve(ms_ctx* ctx, int32_t k, int sweeps);
 ms_status launch_merge_sequential(ms_ctx* ctx, int32_t k);
 ms_status launch_merge_append(ms_ctx* ctx, int32_t k);
 ms_status launch_cover(ms_ctx* ctx, int32_t k0, int32_t k1);
-ms_status launch_label(ms_ctx* ctx, int32_t* d_labels);     // ms_label.cu
+ms_status launch_label(ms_ctx* ctx, int32_t* d_labels);     // ms_label_tc.cu
 ms_status launch_collect(ms_ctx* ctx);                      // ms_merge.cu
 int shift_blocks_per_sm();                                  // ms_shift_fp32.cu
 // Window sums of the seeds active[0..dc->n_active) into acc (fixed point), d = 16.
@@ -204,6 +204,8 @@ ms_status ctx_bind_async(ms_ctx* ctx, const float* d_emb, const uint8_t* d_mask,
 ms_status ctx_bind_finish(ms_ctx* ctx, cudaStream_t st, uint64_t frame_id, int64_t n_start);
 void ctx_free(ms_ctx* ctx);
 int64_t carried_n(const ms_ctx* ctx);   // the N a video carries into its next frame
+ms_status launch_shift_f32_tc(ms_ctx* ctx, const int32_t* active, float c);  // ms_shift_f32_tc.cu
+ms_status f32_tc_setup(int D);                              // its kernels' attributes
 ms_status launch_shift_tc(ms_ctx* ctx, const int32_t* active, int grid, int target_items, float* dbg_S);
 int tc_smem_bytes(int D);
 constexpr int kTcShapes = 8;  // values of ms_config.tc_shape (warp arrangements of k_shift_tc)

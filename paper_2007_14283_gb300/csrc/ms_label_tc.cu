@@ -1137,4 +1137,15 @@ ms_status launch_label_tc_batch(const CUtensorMap& pmap, const CUtensorMap& mmap
                                          P32, pix, d, labels, sc, grid, status, st);
 }
 
+ms_status launch_label(ms_ctx* ctx, int32_t* d_labels) {
+    MS_CUDA(cudaMemsetAsync(d_labels, 0xff, sizeof(int32_t) * (size_t)ctx->n_pixels, ctx->stream));
+    if (ctx->n == 0) return MS_OK;
+    LabelTcScratch sc{ctx->label_fix, (int*)(ctx->label_fix + ctx->n), nullptr};
+    const ms_status s = launch_label_tc_single(ctx->pmap, ctx->pmap1, ctx->Mk, ctx->n_pad, ctx->Dp, ctx->modes,
+                                               ctx->n_kept, (int)ctx->n, ctx->P32, ctx->pix, ctx->emb, ctx->d,
+                                               d_labels, sc, ctx->num_sms, &ctx->dc->status, ctx->stream);
+    ctx->launches += ctx->n_kept > 1 ? 3 : 2;
+    return s;
+}
+
 }  // namespace ms

@@ -223,14 +223,8 @@ ms_status shift_iteration_t(ms_ctx* ctx, int t, int max_iter, cudaEvent_t e0, cu
         ms_status s = launch_shift_tc(ctx, a_in, ctx->tc_grid, 2 * ctx->tc_grid, nullptr);
         if (s != MS_OK) return s;
     } else {
-        F32SingleMap map;
-        map.active = a_in;
-        map.dc = ctx->dc;
-        map.n = (int)ctx->n;
-        map.target = ctx->target_items;
-        k_shift_fp32<Dp, F32SingleMap><<<ctx->shift_grid, kShiftThreads, 0, ctx->stream>>>(ctx->P32, ctx->X,
-                                                                                         ctx->acc, c, map);
-        MS_LAUNCH("k_shift_fp32");
+        ms_status s = launch_shift_f32_tc(ctx, a_in, c);
+        if (s != MS_OK) return s;
     }
     if (e1) MS_CUDA(cudaEventRecord(e1, ctx->stream));
     k_finalize<Dp><<<fin_blocks, kFinThreads, 0, ctx->stream>>>(ctx->acc, a_in, ctx->X, ctx->sstate, ctx->support,
@@ -271,57 +265,6 @@ ms_status launch_window_sums_fp32(const float* P32, int32_t n, const int32_t* ac
     map.target = 2 * grid;
     k_shift_fp32<16, F32SingleMap><<<grid, kShiftThreads, 0, stream>>>(P32, X, acc, c, map);
     MS_LAUNCH("k_shift_fp32");
-    return MS_OK;
-}
-
-// Work items of every iterating frame (batched form): frame f contributes
-// item_off[f+1] - item_off[f] items, seed tiles of 256 x chunks of tpc[f] pixels.
-struct F32BatchMap {
-    const BFrame* frames;
-    const BState* states;
-    BPlan plan;
-    const int32_t* act0;
-    const int32_t* act1;
-    int nf;
-    int total_;
-    __device__ __forceinline__ bool init() {
-        total_ = plan.item_off[nf];
-        return total_ > 0;
-    }
-    __device__ __forceinline__ int total() const { return total_; }
-    __device__ __forceinline__ F32Item item(int i) const {
-        const int f = locate(plan.item_off, nf, i);
-        const int local = i - plan.item_off[f];
-        const int chunks = plan.chunks[f];
-        const int t = local / chunks, ch = local - t * chunks;
-        const BFrame& fr = frames[f];
-        F32Item it;
-        it.active = ((states[f].dc.iters & 1) ? act1 : act0) + fr.pix0;
-        it.n_active = states[f].dc.n_active;
-        it.seed0 = t * kSeedsPerTile;
-        const int64_t b = (int64_t)ch * plan.tpc[f];
-        it.p_begin = fr.pix0 + b;
-        it.p_end = fr.pix0 + min((int64_t)fr.n, b + plan.tpc[f]);
-        return it;
-    }
-};
-
-ms_status launch_shift_fp32_batch(const float* P32, const float* X, unsigned long long* acc, float c_f, int Dp,
-                                  const BFrame* frames, const BState* states, BPlan plan, const int32_t* act0,
-                                  const int32_t* act1, int nf, int grid, cudaStream_t st) {
-    F32BatchMap map;
-    map.frames = frames;
-    map.states = states;
-    map.plan = plan;
-    map.act0 = act0;
-    map.act1 = act1;
-    map.nf = nf;
-    map.total_ = 0;
-    if (Dp == 16)
-        k_shift_fp32<16, F32BatchMap><<<grid, kShiftThreads, 0, st>>>(P32, X, acc, c_f, map);
-    else
-        k_shift_fp32<32, F32BatchMap><<<grid, kShiftThreads, 0, st>>>(P32, X, acc, c_f, map);
-    MS_LAUNCH("k_shift_fp32(batch)");
     return MS_OK;
 }
 
