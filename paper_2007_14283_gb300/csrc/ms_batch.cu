@@ -42,7 +42,8 @@ struct ms_batch {
     int32_t* blk_split;       // [B + 2] block work list with the inner loop split (slices at [B + 1])
     uint32_t* moving;         // per block of active seeds: masks of those still moving (ms_ctx::moving)
     int32_t* misc;            // [0] passes, [1] status, u64 at [2] band pairs, [4] tick, [6] shift ns, [8] shift
-                              // launches, [10] compaction ticket, [14] last phase tick, [16..31] eight phase sums (ns)
+                              // launches, [10] compaction ticket, [11] passes in which
+                              // a round ended, [14] last phase tick, [16..31] eight phase sums (ns)
     float* P32;
     int32_t* pix;
     uint8_t* covered;
@@ -76,6 +77,7 @@ struct ms_batch {
     cudaGraph_t graph;
     cudaGraphExec_t exec;
     int64_t body_launches;    // kernels per pass of the loop body
+    int64_t round_launches;   // and of a pass in which a round ended
     int split;                // 0: each frame split as on its own; 1: work items shared by load
     int target_mult;          // shift work items per launch = target_mult x shift grid
     int tc_shape;             // warp arrangement of the tensor-core shift kernel (ms_config.tc_shape)
@@ -540,10 +542,11 @@ __device__ void frame_check(BState& st, double gamma, int max_iter) {
 
 // Each frame's next active list: its moving seeds in the order of the current
 // list (k_compact_check's reasons). The last block to finish ends the
-// iteration of every frame.
+// iteration of every frame and says whether a round ended (enqueue_round).
 __global__ void __launch_bounds__(kFinThreads)
 k_b_compact_check(const BFrame* __restrict__ frames, BState* states, int B, BPlan plan, int32_t* act0, int32_t* act1,
-                  const uint32_t* __restrict__ moving, int* ticket, double gamma, int max_iter) {
+                  const uint32_t* __restrict__ moving, int* ticket, double gamma, int max_iter,
+                  cudaGraphConditionalHandle rounds, int set_rounds) {
     __shared__ int s_sum[kFinThreads / 32];
     __shared__ bool s_last;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -579,7 +582,13 @@ k_b_compact_check(const BFrame* __restrict__ frames, BState* states, int B, BPla
     }
     __syncthreads();
     if (!s_last) return;
-    for (int f = threadIdx.x; f < B; f += kFinThreads) frame_check(states[f], gamma, max_iter);
+    int ended = 0;
+    for (int f = threadIdx.x; f < B; f += kFinThreads) {
+        frame_check(states[f], gamma, max_iter);
+        ended |= states[f].phase == kRoundDone;
+    }
+    ended = __syncthreads_or(ended);
+    if (set_rounds && threadIdx.x == 0) cudaGraphSetConditional(rounds, ended ? 1u : 0u);
 }
 
 // ------------------------------------------------------------ merge
@@ -812,8 +821,10 @@ k_b_merge_append(const BFrame* __restrict__ frames, BState* states, const float*
     }
 }
 
-__global__ void k_b_schedule(BState* states, int B, double P, double L, double H, int max_rounds, int all_seeds) {
+__global__ void k_b_schedule(BState* states, int B, double P, double L, double H, int max_rounds, int all_seeds,
+                             int* misc) {
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
+    if (f == 0) ++misc[11];
     if (f >= B) return;
     BState& st = states[f];
     if (st.phase != kRoundDone) return;
@@ -865,18 +876,24 @@ __global__ void k_b_cond(const BState* __restrict__ states, int B, int* misc, in
 float ceil_f(double c) { return ceil_to_float(c); }
 
 template <int Dp>
-ms_status enqueue_body(ms_batch* b, cudaStream_t s, cudaGraphConditionalHandle h, bool with_cond, int64_t* nlaunch) {
+ms_status enqueue_seed(ms_batch* b, cudaStream_t s) {
+    k_b_seed<<<b->B, kIT, 0, s>>>(b->frames, b->states, b->P32, Dp, b->covered, b->X, b->seed_pix, b->seed_order,
+                                  b->act[0], b->sstate, b->cand_rank, b->cfg.max_rounds, b->cfg.all_seeds);
+    MS_LAUNCH("k_b_seed");
+    return MS_OK;
+}
+
+#define LAUNCHED(name) do { MS_LAUNCH(name); ++nl; } while (0)
+// One iteration of every iterating frame. rounds: the handle that k_b_compact_check
+// sets when a frame's round ended (enqueue_round's graph node), if set_rounds.
+template <int Dp>
+ms_status enqueue_iteration(ms_batch* b, cudaStream_t s, cudaGraphConditionalHandle rounds, bool set_rounds,
+                            int64_t* nlaunch) {
     const int B = b->B;
     const float cf = ceil_f(b->cfg.bandwidth_cos);
-    const float mf = (float)b->cfg.merge_cos;
     const double gamma = b->cfg.all_seeds ? 1.0 : b->cfg.gamma;
-    const double L = b->cfg.L > 0.0 ? b->cfg.L : b->cfg.alpha / gamma;
     const int G = b->grid;
     int64_t nl = 0;
-#define LAUNCHED(name) do { MS_LAUNCH(name); ++nl; } while (0)
-    k_b_seed<<<B, kIT, 0, s>>>(b->frames, b->states, b->P32, Dp, b->covered, b->X, b->seed_pix, b->seed_order,
-                               b->act[0], b->sstate, b->cand_rank, b->cfg.max_rounds, b->cfg.all_seeds);
-    LAUNCHED("k_b_seed");
     // Split 0 gives every frame the single-frame target (2 x grid), so each
     // frame's results equal a single-frame run's; split 1 shares
     // target_mult x grid items across the iterating frames by their work.
@@ -885,7 +902,7 @@ ms_status enqueue_body(ms_batch* b, cudaStream_t s, cudaGraphConditionalHandle h
                                b->split ? 0 : 2 * grid_shift, b->tc ? 1 : 0, grid_shift);
     LAUNCHED("k_b_plan");
     if (b->prof_phases) {
-        k_b_phase<<<1, 1, 0, s>>>(b->misc, kPhSeed);
+        k_b_phase<<<1, 1, 0, s>>>(b->misc, kPhSeed);  // the loop's relaunch and the plan
         LAUNCHED("k_b_phase");
     }
     if (b->prof) {
@@ -915,12 +932,29 @@ ms_status enqueue_body(ms_batch* b, cudaStream_t s, cudaGraphConditionalHandle h
                                                b->sstate, b->support, b->cfg.tol, b->moving);
     LAUNCHED("k_b_finalize");
     k_b_compact_check<<<G, kFinThreads, 0, s>>>(b->frames, b->states, B, b->plan, b->act[0], b->act[1], b->moving,
-                                                b->misc + 10, gamma, b->cfg.max_iter);
+                                                b->misc + 10, gamma, b->cfg.max_iter, rounds, set_rounds ? 1 : 0);
     LAUNCHED("k_b_compact_check");
     if (b->prof_phases) {
         k_b_phase<<<1, 1, 0, s>>>(b->misc, kPhFinalize);
         LAUNCHED("k_b_phase");
     }
+    *nlaunch = nl;
+    return MS_OK;
+}
+
+// The end of a round for the frames that reached it: merge, coverage, N
+// schedule and the next round's seeds. It runs only in passes in which a round
+// ended (a conditional node of the graph): most passes are iterations, and its
+// 27 launches, each finding nothing to do, were most of a pass of small frames.
+template <int Dp>
+ms_status enqueue_round(ms_batch* b, cudaStream_t s, int64_t* nlaunch) {
+    const int B = b->B;
+    const float mf = (float)b->cfg.merge_cos;
+    const double gamma = b->cfg.all_seeds ? 1.0 : b->cfg.gamma;
+    const double L = b->cfg.L > 0.0 ? b->cfg.L : b->cfg.alpha / gamma;
+    const int G = b->grid;
+    int64_t nl = 0;
+    ms_status st;
     // merge chain for the frames whose round ended
     k_b_blocks<<<1, 32, 0, s>>>(b->frames, b->states, B, kSelDoneSeeds, 256, 0, b->blk_off);
     LAUNCHED("k_b_blocks");
@@ -973,21 +1007,36 @@ ms_status enqueue_body(ms_batch* b, cudaStream_t s, cudaGraphConditionalHandle h
         LAUNCHED("k_b_phase");
     }
     k_b_schedule<<<(B + 255) / 256, 256, 0, s>>>(b->states, B, b->cfg.P_target, L, b->cfg.H, b->cfg.max_rounds,
-                                                 b->cfg.all_seeds);
+                                                 b->cfg.all_seeds, b->misc);
     LAUNCHED("k_b_schedule");
-    if (with_cond) {
-        k_b_cond<<<1, 32, 0, s>>>(b->states, B, b->misc,
-                                  b->cfg.batch_max_passes > 0 ? b->cfg.batch_max_passes : kDefaultMaxPasses, h);
-        LAUNCHED("k_b_cond");
-    }
     if (b->prof_phases) {
         k_b_phase<<<1, 1, 0, s>>>(b->misc, kPhSchedule);
         LAUNCHED("k_b_phase");
     }
-#undef LAUNCHED
+    if ((st = enqueue_seed<Dp>(b, s)) != MS_OK) return st;
+    ++nl;
+    if (b->prof_phases) {
+        k_b_phase<<<1, 1, 0, s>>>(b->misc, kPhSeed);
+        LAUNCHED("k_b_phase");
+    }
     *nlaunch = nl;
     return MS_OK;
 }
+
+// The loop condition, last in the body.
+ms_status enqueue_cond(ms_batch* b, cudaStream_t s, cudaGraphConditionalHandle h, int64_t* nlaunch) {
+    int64_t nl = 0;
+    k_b_cond<<<1, 32, 0, s>>>(b->states, b->B, b->misc,
+                              b->cfg.batch_max_passes > 0 ? b->cfg.batch_max_passes : kDefaultMaxPasses, h);
+    LAUNCHED("k_b_cond");
+    if (b->prof_phases) {
+        k_b_phase<<<1, 1, 0, s>>>(b->misc, kPhSchedule);
+        LAUNCHED("k_b_phase");
+    }
+    *nlaunch = nl;
+    return MS_OK;
+}
+#undef LAUNCHED
 
 template <int Dp>
 ms_status enqueue_setup(ms_batch* b, cudaStream_t s) {
@@ -1013,6 +1062,7 @@ ms_status enqueue_setup(ms_batch* b, cudaStream_t s) {
     const dim3 gl((unsigned)((b->max_np + 255) / 256 < 1024 ? (b->max_np + 255) / 256 : 1024), (unsigned)B);
     k_b_labels_clear<<<gl, 256, 0, s>>>(b->frames, b->label_ptrs);
     MS_LAUNCH("k_b_labels_clear");
+    if (ms_status st = enqueue_seed<Dp>(b, s); st != MS_OK) return st;
     if (b->prof_phases) {
         k_b_phase<<<1, 1, 0, s>>>(b->misc, kPhSetup);
         MS_LAUNCH("k_b_phase");
@@ -1035,6 +1085,16 @@ ms_status enqueue_label(ms_batch* b, cudaStream_t s) {
                                  b->lsc, b->num_sms, b->misc + 1, s);
 }
 
+// The nodes that the next one captured on s would depend on.
+ms_status capture_deps(cudaStream_t s, std::vector<cudaGraphNode_t>* deps) {
+    cudaStreamCaptureStatus cs;
+    const cudaGraphNode_t* d = nullptr;
+    size_t nd = 0;
+    MS_CUDA(cudaStreamGetCaptureInfo(s, &cs, nullptr, nullptr, &d, nullptr, &nd));
+    deps->assign(d, d + nd);
+    return MS_OK;
+}
+
 template <int Dp>
 ms_status build_graph(ms_batch* b) {
     cudaGraph_t g = nullptr;
@@ -1044,13 +1104,7 @@ ms_status build_graph(ms_batch* b) {
     MS_CUDA(cudaStreamBeginCaptureToGraph(s, g, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
     ms_status st = enqueue_setup<Dp>(b, s);
     std::vector<cudaGraphNode_t> deps;
-    if (st == MS_OK) {
-        cudaStreamCaptureStatus cs;
-        const cudaGraphNode_t* d = nullptr;
-        size_t nd = 0;
-        st = cuda_check(cudaStreamGetCaptureInfo(s, &cs, nullptr, nullptr, &d, nullptr, &nd), "capture info");
-        if (st == MS_OK) deps.assign(d, d + nd);
-    }
+    if (st == MS_OK) st = capture_deps(s, &deps);
     cudaGraph_t tmp = nullptr;
     ms_status st2 = cuda_check(cudaStreamEndCapture(s, &tmp), "end capture (set-up)");
     if (st != MS_OK) return st;
@@ -1065,10 +1119,32 @@ ms_status build_graph(ms_batch* b) {
     cudaGraphNode_t cnode;
     MS_CUDA(cudaGraphAddNode(&cnode, g, deps.data(), nullptr, deps.size(), &cp));
     cudaGraph_t body = cp.conditional.phGraph_out[0];
+    // body: an iteration; if a round ended in it, the round's end; the condition
+    cudaGraphConditionalHandle hr;
+    MS_CUDA(cudaGraphConditionalHandleCreate(&hr, body, 0, cudaGraphCondAssignDefault));
+    int64_t nl = 0, nr = 0, nc = 0;
     MS_CUDA(cudaStreamBeginCaptureToGraph(s, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-    int64_t nl = 0;
-    st = enqueue_body<Dp>(b, s, h, true, &nl);
-    st2 = cuda_check(cudaStreamEndCapture(s, &tmp), "end capture (body)");
+    st = enqueue_iteration<Dp>(b, s, hr, true, &nl);
+    if (st == MS_OK) st = capture_deps(s, &deps);
+    st2 = cuda_check(cudaStreamEndCapture(s, &tmp), "end capture (iteration)");
+    if (st != MS_OK) return st;
+    if (st2 != MS_OK) return st2;
+    cudaGraphNodeParams rp = {};
+    rp.type = cudaGraphNodeTypeConditional;
+    rp.conditional.handle = hr;
+    rp.conditional.type = cudaGraphCondTypeIf;
+    rp.conditional.size = 1;
+    cudaGraphNode_t rnode;
+    MS_CUDA(cudaGraphAddNode(&rnode, body, deps.data(), nullptr, deps.size(), &rp));
+    MS_CUDA(cudaStreamBeginCaptureToGraph(s, rp.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                          cudaStreamCaptureModeRelaxed));
+    st = enqueue_round<Dp>(b, s, &nr);
+    st2 = cuda_check(cudaStreamEndCapture(s, &tmp), "end capture (round)");
+    if (st != MS_OK) return st;
+    if (st2 != MS_OK) return st2;
+    MS_CUDA(cudaStreamBeginCaptureToGraph(s, body, &rnode, nullptr, 1, cudaStreamCaptureModeRelaxed));
+    st = enqueue_cond(b, s, h, &nc);
+    st2 = cuda_check(cudaStreamEndCapture(s, &tmp), "end capture (condition)");
     if (st != MS_OK) return st;
     if (st2 != MS_OK) return st2;
     MS_CUDA(cudaStreamBeginCaptureToGraph(s, g, &cnode, nullptr, 1, cudaStreamCaptureModeRelaxed));
@@ -1078,8 +1154,9 @@ ms_status build_graph(ms_batch* b) {
     if (st != MS_OK) return st;
     if (st2 != MS_OK) return st2;
     MS_CUDA(cudaGraphInstantiate(&b->exec, g, 0));
-    b->body_launches = nl;
-    b->fixed_launches = 9 + (b->prof_phases ? 3 : 0);  // set-up, then labelling
+    b->body_launches = nl + nc;
+    b->round_launches = nr;
+    b->fixed_launches = 10 + (b->prof_phases ? 3 : 0);  // set-up, then labelling
     return MS_OK;
 }
 
@@ -1090,7 +1167,8 @@ ms_status enqueue_eager(ms_batch* b, int passes) {
     ms_status st = enqueue_setup<Dp>(b, b->stream);
     for (int p = 0; st == MS_OK && p < passes; ++p) {
         int64_t nl = 0;
-        st = enqueue_body<Dp>(b, b->stream, cudaGraphConditionalHandle{}, false, &nl);
+        st = enqueue_iteration<Dp>(b, b->stream, cudaGraphConditionalHandle{}, false, &nl);
+        if (st == MS_OK) st = enqueue_round<Dp>(b, b->stream, &nl);
     }
     if (st == MS_OK) st = enqueue_label<Dp>(b, b->stream);
     if (st == MS_OK) st = enqueue_label_tick(b, b->stream);
@@ -1424,7 +1502,8 @@ extern "C" ms_status ms_batch_stats(const ms_batch* b, int32_t frame, ms_stats* 
     out->workspace_bytes = (int64_t)b->ws_bytes;
     if (frame < 0) {
         const unsigned long long* m = reinterpret_cast<const unsigned long long*>(b->h_misc);
-        out->launches = (int64_t)b->h_misc[0] * b->body_launches + b->fixed_launches;
+        out->launches = (int64_t)b->h_misc[0] * b->body_launches + (int64_t)b->h_misc[11] * b->round_launches +
+                        b->fixed_launches;
         out->band_pairs = (int64_t)m[1];
         out->shift_ms = (double)m[3] * 1e-6;
         out->shift_launches = (int64_t)m[4];

@@ -62,7 +62,10 @@ struct DevCounters {
     int64_t band_pairs;  // BF16 form: pairs rechecked in FP32
 };
 
-constexpr int kFinThreads = 256;                 // active seeds per finalize / compaction block
+// Active seeds per finalize / compaction block. A seed's update is about 170 FP64
+// operations and an SM does two a clock, so few seeds per block, spread over
+// the SMs: 256 per block took 6 us for 256 seeds, 64 take 3.
+constexpr int kFinThreads = 64;
 constexpr int kMoveWords = 1 + kFinThreads / 32; // words of ms_ctx::moving per block
 
 // Work split of one shift iteration: seed tiles x pixel chunks.
@@ -125,7 +128,7 @@ struct ms_ctx {
     int32_t* conf_deg;   // [n_pixels]
     int32_t* conf;       // [n_pixels * kMergeCap]
     int32_t* block_tmp;  // ingest and seed-selection scan scratch
-    uint32_t* moving;    // per 256 active seeds: a count and eight 32-seed masks of those still moving
+    uint32_t* moving;    // per kFinThreads active seeds: a count and 32-seed masks of those still moving
     ms::DevCounters* dc;
     ms::DevCounters* hc; // pinned host mirror
     int64_t* round_log;  // host [cap * 4]
