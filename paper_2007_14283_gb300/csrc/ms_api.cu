@@ -209,7 +209,7 @@ Layout plan(int64_t np, int Dp) {
         n * Dp * sizeof(float),                    // 25 Xr (merge candidates in rank order)
         n,                                         // 26 removed_r
         (n + 127) / 128 * 128 * 128 * (Dp / 16),  // 27 Ck (their BF16 split rows)
-        (n + kFinThreads - 1) / kFinThreads * kMoveWords * sizeof(uint32_t),  // 28 moving
+        (n + kFinSeeds - 1) / kFinSeeds * sizeof(uint32_t),  // 28 moving
     };
     size_t t = 0;
     for (int i = 0; i < 29; ++i) {

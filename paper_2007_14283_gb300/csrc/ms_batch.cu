@@ -417,7 +417,7 @@ k_b_seed(const BFrame* __restrict__ frames, BState* states, const float* __restr
 
 // ------------------------------------------------------------ iteration
 // Work split of this iteration over the iterating frames; seed_off counts
-// their blocks of kFinThreads active seeds. Each frame is cut
+// their blocks of kFinSeeds active seeds. Each frame is cut
 // into seed tiles x pixel chunks by the single-frame rule (a target item count
 // spread over the frame's seed tiles, chunks whole pixel tiles). With
 // canon_target > 0 every frame gets that target, the one the single-frame path
@@ -467,7 +467,7 @@ __global__ void k_b_plan(const BFrame* __restrict__ frames, const BState* __rest
                 plan.chunks[f] = sp.chunks;
                 items = (na + 127) / 128 * sp.chunks;
             }
-            seeds = (na + kFinThreads - 1) / kFinThreads;
+            seeds = (na + kFinSeeds - 1) / kFinSeeds;
         }
         int ti, ts;
         const int ei = block_scan(items, &ti);
@@ -490,34 +490,37 @@ __global__ void k_b_plan(const BFrame* __restrict__ frames, const BState* __rest
 }
 
 // Mean-shift update of every active seed of every iterating frame, a block of
-// kFinThreads seeds of one frame at a time: x <- normalise(window sum), and the
+// kFinSeeds seeds of one frame at a time: x <- normalise(window sum), and the
 // seeds still moving as masks for k_b_compact_check.
 template <int Dp>
 __global__ void __launch_bounds__(kFinThreads)
 k_b_finalize(const BFrame* __restrict__ frames, BState* states, int B, BPlan plan, const int32_t* __restrict__ act0,
              const int32_t* __restrict__ act1, unsigned long long* __restrict__ acc, float* __restrict__ X,
-             uint8_t* __restrict__ sstate, int32_t* __restrict__ support, double tol, uint32_t* __restrict__ moving) {
+             uint8_t* __restrict__ sstate, int32_t* __restrict__ support, double tol, StepBand band,
+             uint32_t* __restrict__ moving) {
+    __shared__ uint32_t s_part[kFinThreads / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int total = plan.seed_off[B];
     for (int blk = blockIdx.x; blk < total; blk += gridDim.x) {
         const int f = locate(plan.seed_off, B, blk);
-        const int pos = (blk - plan.seed_off[f]) * kFinThreads + threadIdx.x;
+        const int pos = (blk - plan.seed_off[f]) * kFinSeeds + wid * 8 + (lane & 7);
         DevCounters& dc = states[f].dc;
-        bool conv = false, fail = false, move = false;
-        if (pos < dc.n_active) {
-            const int slot = ((dc.iters & 1) ? act1 : act0)[frames[f].pix0 + pos];
-            move = finalize_seed<Dp>(acc + (int64_t)slot * (Dp + 1), X + (int64_t)slot * Dp, sstate + slot,
-                                     support + slot, tol, &conv, &fail);
-        }
-        const int mc = __syncthreads_count(conv), mf = __syncthreads_count(fail), mm = __syncthreads_count(move);
-        const unsigned bal = __ballot_sync(0xffffffffu, move);
-        uint32_t* mv = moving + (int64_t)blk * kMoveWords;
-        if ((threadIdx.x & 31) == 0) mv[1 + (threadIdx.x >> 5)] = bal;
+        const bool live = pos < dc.n_active;
+        const int64_t slot = live ? ((dc.iters & 1) ? act1 : act0)[frames[f].pix0 + pos] : 0;
+        const SeedEnd e = finalize_seed<Dp>(live, acc + slot * (Dp + 1), X + slot * Dp, sstate + slot, support + slot,
+                                            tol, band);
+        const bool first = lane < 8;  // one lane per seed
+        const uint32_t mv = __ballot_sync(0xffffffffu, first && e.move);
+        if (lane == 0) s_part[wid] = mv;
+        const int mc = __syncthreads_count(first && e.conv), mf = __syncthreads_count(first && e.fail);
         if (threadIdx.x == 0) {
-            mv[0] = (uint32_t)mm;
+            const uint32_t m = s_part[0] | s_part[1] << 8 | s_part[2] << 16 | s_part[3] << 24;
+            moving[blk] = m;
             if (mc) atomicAdd(&dc.conv_new, mc);
             if (mf) atomicAdd(&dc.fail_total, mf);
-            if (mm) atomicAdd(&dc.n_next, mm);
+            if (m) atomicAdd(&dc.n_next, __popc(m));
         }
+        __syncthreads();
     }
 }
 
@@ -541,38 +544,29 @@ __device__ void frame_check(BState& st, double gamma, int max_iter) {
 }
 
 // Each frame's next active list: its moving seeds in the order of the current
-// list (k_compact_check's reasons). The last block to finish ends the
-// iteration of every frame and says whether a round ended (enqueue_round).
+// list (k_finalize's reasons), a warp for the seeds of one mask. The last block
+// to finish ends the iteration of every frame and says whether a round ended
+// (enqueue_round).
 __global__ void __launch_bounds__(kFinThreads)
 k_b_compact_check(const BFrame* __restrict__ frames, BState* states, int B, BPlan plan, int32_t* act0, int32_t* act1,
                   const uint32_t* __restrict__ moving, int* ticket, double gamma, int max_iter,
                   cudaGraphConditionalHandle rounds, int set_rounds) {
-    __shared__ int s_sum[kFinThreads / 32];
+    constexpr int kWarps = kFinThreads / 32;
     __shared__ bool s_last;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int total = plan.seed_off[B];
-    for (int blk = blockIdx.x; blk < total; blk += gridDim.x) {
+    for (int blk = blockIdx.x * kWarps + wid; blk < total; blk += gridDim.x * kWarps) {
         const int f = locate(plan.seed_off, B, blk);
         const int b0 = plan.seed_off[f];
         const bool odd = states[f].dc.iters & 1;
         const int64_t base = frames[f].pix0;
         int before = 0;
-        for (int b = b0 + threadIdx.x; b < blk; b += kFinThreads) before += (int)moving[(int64_t)b * kMoveWords];
+        for (int b = b0 + lane; b < blk; b += 32) before += __popc(moving[b]);
         for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
-        __syncthreads();
-        if (lane == 0) s_sum[wid] = before;
-        __syncthreads();
-        before = 0;
-        const uint32_t* mv = moving + (int64_t)blk * kMoveWords;
-#pragma unroll
-        for (int w = 0; w < kFinThreads / 32; ++w) {
-            before += s_sum[w];
-            if (w < wid) before += __popc(mv[1 + w]);
-        }
-        const uint32_t bits = mv[1 + wid];
+        const uint32_t bits = moving[blk];
         if ((bits >> lane) & 1u)
             ((odd ? act0 : act1) + base)[before + __popc(bits & ((1u << lane) - 1u))] =
-                ((odd ? act1 : act0) + base)[(blk - b0) * kFinThreads + threadIdx.x];
+                ((odd ? act1 : act0) + base)[(blk - b0) * kFinSeeds + lane];
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -929,7 +923,7 @@ ms_status enqueue_iteration(ms_batch* b, cudaStream_t s, cudaGraphConditionalHan
         LAUNCHED("k_b_phase");
     }
     k_b_finalize<Dp><<<G, kFinThreads, 0, s>>>(b->frames, b->states, B, b->plan, b->act[0], b->act[1], b->acc, b->X,
-                                               b->sstate, b->support, b->cfg.tol, b->moving);
+                                               b->sstate, b->support, b->cfg.tol, step_band(b->cfg.tol), b->moving);
     LAUNCHED("k_b_finalize");
     k_b_compact_check<<<G, kFinThreads, 0, s>>>(b->frames, b->states, B, b->plan, b->act[0], b->act[1], b->moving,
                                                 b->misc + 10, gamma, b->cfg.max_iter, rounds, set_rounds ? 1 : 0);
@@ -1265,7 +1259,7 @@ extern "C" ms_status ms_batch_create(const ms_config* cfg, int32_t B, const floa
         (size_t)B * b->nblk_max * 4 + 4, (size_t)b->total_pk_rows * 128 * (Dp / 16), sizeof(int32_t*) * B,
         (size_t)b->total_pk_rows * 128 * (Dp / 16), n * sizeof(int2), sizeof(int32_t) * (B + 1) + 16,
         n * Dp * 4, n, (size_t)b->total_pk_rows * 128 * (Dp / 16),
-        (n / kFinThreads + B) * kMoveWords * sizeof(uint32_t)};
+        (n / kFinSeeds + B) * sizeof(uint32_t)};
     const int NS = (int)(sizeof(sizes) / sizeof(sizes[0]));
     size_t offs[32], tot = 0;
     for (int i = 0; i < NS; ++i) {

@@ -6,6 +6,13 @@
 
 namespace ms {
 
+// Let the stream's next kernel start its blocks (launch_after): they run up to
+// their own grid_wait.
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Wait until the work ahead on the stream has ended and its writes are visible;
+// returns at once in a kernel that was launched the ordinary way.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Sequential FP32 dot product, k = 0..Dp-1, one fused multiply-add per term.
 template <int Dp>
 __device__ __forceinline__ float dot_seq(const float* a, const float* b) {
@@ -37,62 +44,115 @@ __device__ __forceinline__ bool cos_at_least(const float* a, const float* b, flo
     return cos64(a, b, Dp) >= thr;
 }
 
-// Mean-shift update of one seed (Eq. 5 with the flat kernel) from its window
-// sums (fixed point, 2^-36 units) and count, which are set back to zero: x <-
-// normalise(sum), *conv when the FP64 step norm is below tol, *fail when the
-// window is empty. True when the seed moves on.
+// Squared step norms that an FP32 evaluation settles: below `lo` the seed has
+// converged, from `hi` on it moves; between them FP64 decides. The FP32 value's
+// relative error is at most (d + 5) 2^-24 < 3e-6 (differences, products and
+// sums of non-negative terms each round once), the lines lie 1e-5 apart from
+// tol^2, and below 1e-30, where products underflow, FP64 always decides.
+struct StepBand {
+    float lo, hi;
+};
+inline StepBand step_band(double tol) {
+    const double t2 = tol * tol;
+    StepBand b;
+    b.lo = t2 < 1e-30 ? -1.0f : (float)(t2 * (1.0 - 1e-5));
+    b.hi = t2 < 1e-30 ? 1e-30f : (float)(t2 * (1.0 + 1e-5));
+    return b;
+}
+
+struct SeedEnd {
+    bool conv, fail, move;
+};
+
+// Mean-shift update (Eq. 5 with the flat kernel) of the 8 seeds of a warp, four
+// lanes a seed: lane 8 q + s holds dimensions [q Dp/4, (q+1) Dp/4) of seed s.
+// The seed's window sums (fixed point, 2^-36 units) and count are set back to
+// zero: x <- normalise(sum), conv when the FP64 step norm is below tol, fail
+// when the window is empty, move when the seed moves on (the same on all four
+// lanes); lanes that are not `live` only take part in the shuffles.
+// Bound by the FP64 pipe: a warp's FP64 instruction takes about 64 clocks here,
+// and one thread per seed was 219 of them (5.6 us a launch of few seeds). Four
+// lanes a seed, no scaling by 2^-36 (a power of two moves through every step of
+// the normalisation unchanged) and the step norm in FP32 outside the band leave
+// 78. The sums over dimensions pass from lane to lane in the order of the
+// dimensions, so every bit is that of one thread's loop.
 // Every load comes before the first store: a store between two loads of the
-// same array keeps them in order, and the 33 loads of a seed then cost a memory
-// round trip each (18 us a launch instead of 4).
+// same array keeps them in order, and each load then costs a memory round trip.
 template <int Dp>
-__device__ __forceinline__ bool finalize_seed(unsigned long long* a, float* x, uint8_t* state, int32_t* support,
-                                              double tol, bool* conv, bool* fail) {
-    long long sum[Dp + 1];
-    float4 x4[Dp / 4];
+__device__ __forceinline__ SeedEnd finalize_seed(bool live, unsigned long long* a, float* x, uint8_t* state,
+                                                 int32_t* support, double tol, StepBand band) {
+    constexpr int kPer = Dp / 4;
+    const int lane = threadIdx.x & 31, q = lane >> 3, sl = lane & 7;
+    long long sum[kPer], cnt = 0;
+    float4 xo[kPer / 4];
 #pragma unroll
-    for (int k = 0; k <= Dp; ++k) sum[k] = (long long)a[k];
+    for (int k = 0; k < kPer; ++k) sum[k] = 0;
 #pragma unroll
-    for (int k = 0; k < Dp / 4; ++k) x4[k] = reinterpret_cast<const float4*>(x)[k];
-    const long long cnt = sum[Dp];
-    double y[Dp];
-    double ss = 0.0;
+    for (int k = 0; k < kPer / 4; ++k) xo[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (live) {
 #pragma unroll
-    for (int k = 0; k < Dp; ++k) {
-        y[k] = (double)sum[k] * (1.0 / 68719476736.0);
-        ss += y[k] * y[k];
+        for (int k = 0; k < kPer; ++k) sum[k] = (long long)a[q * kPer + k];
+        if (q == 0) cnt = (long long)a[Dp];
+#pragma unroll
+        for (int k = 0; k < kPer / 4; ++k) xo[k] = reinterpret_cast<const float4*>(x)[q * (kPer / 4) + k];
     }
+    double y[kPer], ss = 0.0;
 #pragma unroll
-    for (int k = 0; k <= Dp; ++k) a[k] = 0ull;
-    if (cnt == 0) {
-        *fail = true;
-        *state = kFailed;
-        return false;
+    for (int k = 0; k < kPer; ++k) y[k] = (double)sum[k];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        double t = ss;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) t += y[k] * y[k];
+        ss = __shfl_sync(0xffffffffu, t, 8 * g + sl);
+    }
+    cnt = __shfl_sync(0xffffffffu, cnt, sl);
+    if (live) {
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) a[q * kPer + k] = 0ull;
+        if (q == 0) a[Dp] = 0ull;
     }
     const double inv = 1.0 / sqrt(ss);
-    double dd = 0.0;
+    float xn[kPer];
+    float dd32 = 0.f;
 #pragma unroll
-    for (int k = 0; k < Dp; k += 4) {
-        float4 xn;
-        xn.x = (float)(y[k] * inv);
-        xn.y = (float)(y[k + 1] * inv);
-        xn.z = (float)(y[k + 2] * inv);
-        xn.w = (float)(y[k + 3] * inv);
-        const float4 xo = x4[k / 4];
-        const double d0 = (double)xn.x - (double)xo.x, d1 = (double)xn.y - (double)xo.y,
-                     d2 = (double)xn.z - (double)xo.z, d3 = (double)xn.w - (double)xo.w;
-        dd += d0 * d0;
-        dd += d1 * d1;
-        dd += d2 * d2;
-        dd += d3 * d3;
-        reinterpret_cast<float4*>(x)[k / 4] = xn;
+    for (int k = 0; k < kPer; ++k) {
+        xn[k] = (float)(y[k] * inv);
+        const float d = xn[k] - reinterpret_cast<const float*>(xo)[k];
+        dd32 = fmaf(d, d, dd32);
     }
-    *support = (int32_t)cnt;
-    if (sqrt(dd) < tol) {
-        *conv = true;
-        *state = kConverged;
-        return false;
+    dd32 += __shfl_xor_sync(0xffffffffu, dd32, 8);
+    dd32 += __shfl_xor_sync(0xffffffffu, dd32, 16);
+    bool conv = dd32 <= band.lo;
+    const bool settled = conv || dd32 >= band.hi || cnt == 0;
+    if (__any_sync(0xffffffffu, live && !settled)) {
+        double dd = 0.0;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            double t = dd;
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) {
+                const double d = (double)xn[k] - (double)reinterpret_cast<const float*>(xo)[k];
+                t += d * d;
+            }
+            dd = __shfl_sync(0xffffffffu, t, 8 * g + sl);
+        }
+        conv = sqrt(dd) < tol;
     }
-    return true;
+    if (!live) return SeedEnd{false, false, false};
+    if (cnt == 0) {
+        if (q == 0) *state = kFailed;
+        return SeedEnd{false, true, false};
+    }
+#pragma unroll
+    for (int k = 0; k < kPer / 4; ++k)
+        reinterpret_cast<float4*>(x)[q * (kPer / 4) + k] =
+            make_float4(xn[4 * k], xn[4 * k + 1], xn[4 * k + 2], xn[4 * k + 3]);
+    if (q == 0) {
+        *support = (int32_t)cnt;
+        if (conv) *state = kConverged;
+    }
+    return SeedEnd{conv, false, !conv};
 }
 
 }  // namespace ms

@@ -56,17 +56,17 @@ struct DevCounters {
     int32_t n_uncovered; // foreground pixels not covered
     int32_t n_fg;        // foreground pixels
     int32_t cursor_next; // seed-order position after the running selection
-    int32_t ticket;      // blocks of the running compaction that have finished
+    int32_t ticket;      // finalize blocks of the running iteration that are done
     int32_t pad;
     int64_t seed_iters;  // seed-iterations summed
     int64_t band_pairs;  // BF16 form: pairs rechecked in FP32
 };
 
-// Active seeds per finalize / compaction block. A seed's update is about 170 FP64
-// operations and an SM does two a clock, so few seeds per block, spread over
-// the SMs: 256 per block took 6 us for 256 seeds, 64 take 3.
-constexpr int kFinThreads = 64;
-constexpr int kMoveWords = 1 + kFinThreads / 32; // words of ms_ctx::moving per block
+// Active seeds per finalize block, four lanes each: one warp for each of an
+// SM's FP64 pipes, so that few seeds spread over many SMs. (256 seeds a block
+// took 6 us for 256 seeds.)
+constexpr int kFinSeeds = 32;
+constexpr int kFinThreads = 4 * kFinSeeds;
 
 // Work split of one shift iteration: seed tiles x pixel chunks.
 struct ShiftSplit {
@@ -128,7 +128,7 @@ struct ms_ctx {
     int32_t* conf_deg;   // [n_pixels]
     int32_t* conf;       // [n_pixels * kMergeCap]
     int32_t* block_tmp;  // ingest and seed-selection scan scratch
-    uint32_t* moving;    // per kFinThreads active seeds: a count and 32-seed masks of those still moving
+    uint32_t* moving;    // per kFinSeeds (32) active seeds: the mask of those still moving
     ms::DevCounters* dc;
     ms::DevCounters* hc; // pinned host mirror
     int64_t* round_log;  // host [cap * 4]
@@ -181,6 +181,26 @@ cudaError_t scratch_malloc_async(void** p, size_t bytes, cudaStream_t st);
         ms_status _s = ::ms::cuda_check(cudaGetLastError(), what);    \
         if (_s != MS_OK) return _s;                                   \
     } while (0)
+
+// A launch that may start before the kernel ahead of it on the stream has
+// ended, from the moment all of that kernel's blocks have called grid_release
+// (or ended). The kernel calls grid_wait before it touches anything that
+// earlier work on the stream writes or reads.
+template <class... P, class... A>
+cudaError_t launch_after(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st,
+                         const A&... args) {
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 
 // Kernel launchers. Each enqueues on ctx->stream and returns MS_OK or MS_ERR_CUDA.
 ms_status launch_ingest(ms_ctx* ctx);                       // ms_ingest.cu

@@ -72,7 +72,7 @@ k_shift_f32_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__
     constexpr int kHalves = L::kHalves, kStages = L::kStages, kStageBytes = L::kStageBytes, kSBufs = L::kSBufs;
     constexpr float kBand = kScoreBand<kD>;
     constexpr uint32_t kCols = 128 * kSBufs;
-    if (!map.init()) return;
+    grid_release();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* A1 = smem + L::kOffA1;
@@ -110,7 +110,8 @@ k_shift_f32_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const int items = map.total();
+    grid_wait();
+    const int items = map.init() ? map.total() : 0;
 
     if (warp == kFWarpTma) {
         // ------------------------------------------------ TMA producer
@@ -388,15 +389,6 @@ struct FBatchMap {
     }
 };
 
-template <int D, class Map>
-ms_status f32_tc_launch(const CUtensorMap& pmap, const CUtensorMap& pmap1, const float* X, unsigned long long* acc,
-                        float c, const Map& map, int* status, int num_sms, cudaStream_t st) {
-    k_shift_f32_tc<D, Map><<<num_sms * FDim<D>::kCtas, kFThreads, FDim<D>::kSmemBytes, st>>>(pmap, pmap1, X, acc, c,
-                                                                                            map, status);
-    MS_LAUNCH("k_shift_f32_tc");
-    return MS_OK;
-}
-
 template <int D>
 ms_status f32_tc_allow() {
     MS_CUDA(cudaFuncSetAttribute(k_shift_f32_tc<D, FSingleMap>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -416,10 +408,14 @@ ms_status launch_shift_f32_tc(ms_ctx* ctx, const int32_t* active, float c) {
     map.dc = ctx->dc;
     map.n = (int)ctx->n;
     map.target = ctx->target_items;
-    return ctx->Dp == 32 ? f32_tc_launch<32>(ctx->pmap, ctx->pmap1, ctx->X, ctx->acc, c, map, &ctx->dc->status,
-                                             ctx->num_sms, ctx->stream)
-                         : f32_tc_launch<16>(ctx->pmap, ctx->pmap1, ctx->X, ctx->acc, c, map, &ctx->dc->status,
-                                             ctx->num_sms, ctx->stream);
+    int* status = &ctx->dc->status;
+    if (ctx->Dp == 32)
+        MS_CUDA(launch_after(k_shift_f32_tc<32, FSingleMap>, ctx->num_sms * FDim<32>::kCtas, kFThreads,
+                             FDim<32>::kSmemBytes, ctx->stream, ctx->pmap, ctx->pmap1, ctx->X, ctx->acc, c, map, status));
+    else
+        MS_CUDA(launch_after(k_shift_f32_tc<16, FSingleMap>, ctx->num_sms * FDim<16>::kCtas, kFThreads,
+                             FDim<16>::kSmemBytes, ctx->stream, ctx->pmap, ctx->pmap1, ctx->X, ctx->acc, c, map, status));
+    return MS_OK;
 }
 
 ms_status launch_shift_f32_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, int Dp, const float* X,
@@ -434,8 +430,14 @@ ms_status launch_shift_f32_tc_batch(const CUtensorMap& pmap, const CUtensorMap& 
     map.act1 = act1;
     map.nf = nf;
     map.total_ = 0;
-    return Dp == 32 ? f32_tc_launch<32>(pmap, pmap1, X, acc, c, map, status, num_sms, st)
-                    : f32_tc_launch<16>(pmap, pmap1, X, acc, c, map, status, num_sms, st);
+    if (Dp == 32)
+        k_shift_f32_tc<32, FBatchMap><<<num_sms * FDim<32>::kCtas, kFThreads, FDim<32>::kSmemBytes, st>>>(
+            pmap, pmap1, X, acc, c, map, status);
+    else
+        k_shift_f32_tc<16, FBatchMap><<<num_sms * FDim<16>::kCtas, kFThreads, FDim<16>::kSmemBytes, st>>>(
+            pmap, pmap1, X, acc, c, map, status);
+    MS_LAUNCH("k_shift_f32_tc(batch)");
+    return MS_OK;
 }
 
 }  // namespace ms

@@ -214,7 +214,7 @@ k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
     constexpr int kPxPerWarp = Shape::kPxPerWarp, kSub = Shape::kSub;
     constexpr float kBand = kScoreBand<kD>;
     constexpr int kWarpTma = Shape::kWarpTma, kWarpG1 = Shape::kWarpG1, kWarpG2 = Shape::kWarpG2;
-    if (!map.init()) return;
+    grid_release();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* A1 = smem + L::kOffA1;               // [item buffer][half] 16 KB tiles
@@ -256,7 +256,8 @@ k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
         tmem_alloc(tmem_slot, kTmemCols);
         tmem_relinquish();
     }
-    const int items = map.total();
+    grid_wait();
+    const int items = map.init() ? map.total() : 0;
     if (warp < 4 && (int)blockIdx.x < items) {  // the first item's seeds, while the rest is set up
         const TcItem ii = map.item(blockIdx.x);
         const int pos = ii.seed0 + warp * 32 + lane;
@@ -742,16 +743,18 @@ ms_status launch_shift_tc(ms_ctx* ctx, const int32_t* active, int grid, int targ
         using Sh = decltype(sh);
         if (ctx->Dp == 32) {
             if (dbg_S) return set_error(MS_ERR_INVALID_ARG, "the score dump is for d <= 16");
-            k_shift_tc<Sh, 32, false, TcSingleMap><<<grid, Sh::kThreads, TcDim<32>::kSmemBytes, ctx->stream>>>(
-                ctx->pmap, ctx->pmap1, ctx->X, ctx->acc, c, map, &ctx->dc->status, band, nullptr, 0);
+            MS_CUDA(launch_after(k_shift_tc<Sh, 32, false, TcSingleMap>, grid, Sh::kThreads, TcDim<32>::kSmemBytes,
+                                 ctx->stream, ctx->pmap, ctx->pmap1, ctx->X, ctx->acc, c, map, &ctx->dc->status, band,
+                                 nullptr, 0));
         } else if (dbg_S) {
             MS_CUDA(cudaFuncSetAttribute(k_shift_tc<Sh, 16, true, TcSingleMap>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, TcDim<16>::kSmemBytes));
             k_shift_tc<Sh, 16, true, TcSingleMap><<<grid, Sh::kThreads, TcDim<16>::kSmemBytes, ctx->stream>>>(
                 ctx->pmap, ctx->pmap1, ctx->X, ctx->acc, c, map, &ctx->dc->status, band, dbg_S, ctx->n_pad);
         } else {
-            k_shift_tc<Sh, 16, false, TcSingleMap><<<grid, Sh::kThreads, TcDim<16>::kSmemBytes, ctx->stream>>>(
-                ctx->pmap, ctx->pmap1, ctx->X, ctx->acc, c, map, &ctx->dc->status, band, nullptr, 0);
+            MS_CUDA(launch_after(k_shift_tc<Sh, 16, false, TcSingleMap>, grid, Sh::kThreads, TcDim<16>::kSmemBytes,
+                                 ctx->stream, ctx->pmap, ctx->pmap1, ctx->X, ctx->acc, c, map, &ctx->dc->status, band,
+                                 nullptr, 0));
         }
         MS_LAUNCH("k_shift_tc");
         return MS_OK;
