@@ -969,10 +969,9 @@ ms_status enqueue_round(ms_batch* b, cudaStream_t s, int64_t* nlaunch) {
     LAUNCHED("k_b_rank_invert");
     st = launch_merge_tc_batch(b->cmap, b->cmap1, b->mmap, b->mmap1, b->Ck, b->total_pk_rows, Dp, b->frames, b->states,
                                B, (int)b->max_pk_rows, b->Xr, b->modes, b->rank_cand, b->cand_state, b->removed_r,
-                               b->conf_deg, b->conf, mf, b->cfg.merge_cos, b->blk_off, b->lsc, b->num_sms, b->misc + 1,
-                               s);
+                               b->conf_deg, b->conf, mf, b->cfg.merge_cos, b->blk_off, b->num_sms, b->misc + 1, s);
     if (st != MS_OK) return st;
-    nl += 4;
+    nl += 3;
     for (int sw = 0; sw < 8; ++sw) {
         k_b_merge_resolve<Dp><<<G, kMT, 0, s>>>(b->frames, b->states, B, b->blk_off, b->X, b->cand, b->cand_rank,
                                                 b->rank_cand, b->cand_state, b->conf_deg, b->conf, mf,
@@ -993,9 +992,9 @@ ms_status enqueue_round(ms_batch* b, cudaStream_t s, int64_t* nlaunch) {
     LAUNCHED("k_b_blocks");
     st = launch_cover_tc_batch(b->pmap, b->mmap, b->pmap1, b->mmap1, b->Mk, b->total_pk_rows, Dp, b->frames, b->states,
                                B, (int)b->max_pk_rows, b->modes, b->P32, b->pix, b->d, b->cfg.bandwidth_cos,
-                               b->covered, b->blk_off, b->lsc, b->num_sms, b->misc + 1, s);
+                               b->covered, b->blk_off, b->num_sms, b->misc + 1, s);
     if (st != MS_OK) return st;
-    nl += 3;
+    nl += 2;
     if (b->prof_phases) {
         k_b_phase<<<1, 1, 0, s>>>(b->misc, kPhCover);
         LAUNCHED("k_b_phase");

@@ -93,14 +93,14 @@ ms_status launch_label_tc_single(const CUtensorMap& pmap, const CUtensorMap& pma
 ms_status launch_cover_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, void* Mk, int64_t n_pad, int Dp,
                                  const float* modes, int k0, int k1, int n, const float* P32, const int32_t* pix,
                                  const float* emb, int d, double c, uint8_t* covered, int* n_uncovered,
-                                 LabelTcScratch sc, int grid, int* status, cudaStream_t st);
+                                 int grid, int* status, cudaStream_t st);
 // The same for the frames of a batch whose round ended (tile_off: their pixel
 // tiles, from k_b_blocks with 128 pixels per block).
 ms_status launch_cover_tc_batch(const CUtensorMap& pmap, const CUtensorMap& mmap, const CUtensorMap& pmap1,
                                 const CUtensorMap& mmap1, void* Mk, int64_t mk_rows, int Dp, const BFrame* frames,
                                 BState* states, int B, int max_pk_rows, const float* modes, const float* P32,
                                 const int32_t* pix, int d, double c, uint8_t* covered, const int32_t* tile_off,
-                                LabelTcScratch sc, int grid, int* status, cudaStream_t st);
+                                int grid, int* status, cudaStream_t st);
 // The merge's two contractions on the tensor cores for the frames whose round
 // ended (tile_off: their candidates in blocks of 128): the candidates in rank
 // order (Xr, packed into Ck) against their earlier modes (Mk), then against
@@ -111,14 +111,12 @@ ms_status launch_merge_tc_batch(const CUtensorMap& cmap, const CUtensorMap& cmap
                                 const CUtensorMap& mmap1, void* Ck, int64_t rows, int Dp, const BFrame* frames,
                                 BState* states, int B, int max_pk_rows, const float* Xr, const float* modes,
                                 const int32_t* rank_cand, uint8_t* cand_state, uint8_t* removed_r, int32_t* conf_deg,
-                                int32_t* conf, float thr_f, double thr, const int32_t* tile_off, LabelTcScratch sc,
-                                int grid, int* status, cudaStream_t st);
+                                int32_t* conf, float thr_f, double thr, const int32_t* tile_off, int grid, int* status, cudaStream_t st);
 // The same for one frame: k candidates (Xr, packed into Ck) against its K_old
 // earlier modes (Mk), then against one another.
 ms_status launch_merge_tc_single(void* Ck, void* Mk, int64_t n_pad, int Dp, int k, int K_old, const float* Xr,
                                  const float* modes, const int32_t* rank_cand, uint8_t* cand_state, uint8_t* removed_r,
-                                 int32_t* conf_deg, int32_t* conf, float thr_f, double thr, LabelTcScratch sc,
-                                 int grid, int* status, cudaStream_t st);
+                                 int32_t* conf_deg, int32_t* conf, float thr_f, double thr, int grid, int* status, cudaStream_t st);
 ms_status launch_label_tc_batch(const CUtensorMap& pmap, const CUtensorMap& mmap, const CUtensorMap& pmap1,
                                 const CUtensorMap& mmap1, void* Mk, int64_t mk_rows, int Dp, const BFrame* frames,
                                 const BState* states, int B, int max_pk_rows, const float* modes, const float* P32,

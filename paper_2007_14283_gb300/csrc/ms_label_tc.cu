@@ -9,11 +9,11 @@
 // with p = Ph + Pm + Pl and m = Mh + Mm + Ml the exact BF16 splits of the FP32
 // vectors, so |S - p.m| <= LbDim<D>::kEps (the bound is derived there).
 // Sixteen warps read S from TMEM, one pixel per lane and 32 mode columns per
-// warp, and keep the best and second-best score of each pixel. A pixel whose
-// best leads its second by more than 2 * kEps has the exact FP64 argmax as its
-// winner; the others (near-ties) are queued and re-decided by k_label_fix
-// exactly as the FP32 form decides them: FP32 scores over all modes, then
-// FP64 among those within 2 * kEpsF32 of the best.
+// warp, and keep the best two modes of each pixel and its third score. A pixel
+// whose best leads its second by more than kTie has the exact FP64 argmax as its
+// winner; a near-tie of two is decided on the spot, one of three or more is
+// queued for k_label_fix, both exactly as FP32 scores over all modes, then FP64
+// among those within 2 * kEpsF32 of the best, decide it.
 //
 // Warp roles (576 threads, one CTA per SM): warps 0-15 read S (warp w reaches
 // TMEM lanes 32 * (w % 4) + 0..31); warp 16 issues TMA loads (the item's pixel
@@ -55,8 +55,9 @@ struct LbDim {
     static constexpr int kStages = D == 16 ? 8 : 4;                        // mode-tile ring
     static constexpr int kOffA = 0;                                        // 2 pixel tiles per half
     static constexpr int kOffB = 2 * kHalves * kLTile;                     // kStages mode tiles per half
-    static constexpr int kOffX = kOffB + kStages * kHalves * kLTile;       // exchange: [4][128] x (b1, i1, b2)
-    static constexpr int kOffBar = kOffX + 4 * 128 * 12;
+    static constexpr int kOffX = kOffB + kStages * kHalves * kLTile;       // 2 exchanges: [4][128] x (b1, i1, b2, i2, b3)
+    static constexpr int kExchange = 4 * 128 * 20;
+    static constexpr int kOffBar = kOffX + 2 * kExchange;
     static constexpr int kNumBars = 2 * 2 + 2 * kStages + 2 * kLSBufs + 2;
     static constexpr int kSmemBytes = kOffBar + kNumBars * 8 + 16 + 1024;
     static constexpr float kEps = D == 16 ? 6e-5f : 7e-5f;
@@ -205,7 +206,13 @@ struct LbOut {
     uint8_t* cand_state;
     int32_t* conf_deg;
     int32_t* conf;
-    double thr;
+    double thr;            // merge_cos; coverage: c
+    // exact decisions: the pixels' FP32 rows, the modes (all frames) and the
+    // raw embeddings (single form; the batch takes its frames') of d values
+    const float* P32;
+    const float* modes;
+    const float* emb1;
+    int d;
 };
 
 // What k_label_tc's score readers do with a row's scores.
@@ -216,18 +223,39 @@ enum LbMode {
     kLbPairs = 3,   // every column ranked above the row at or above merge_cos (conflict lists)
 };
 
-// kMode = kLbLabel: labelling (best and second-best mode of every pixel).
+// The exact decision between modes i < j of a pixel (k_label_fix's, for two):
+// the larger FP32 score, or the larger FP64 cosine of the raw embedding when
+// the scores are within 2 kEpsF32 of one another, i on ties.
+template <int Dp>
+__device__ __noinline__ int better_mode(const float* p, const float* M, const float* em, int d, int i, int j) {
+    const float* a = M + (int64_t)i * Dp;
+    const float* b = M + (int64_t)j * Dp;
+    float pv[Dp];
+#pragma unroll
+    for (int k = 0; k < Dp; ++k) pv[k] = p[k];
+    const float sa = dot_seq<Dp>(pv, a), sb = dot_seq<Dp>(pv, b), best = fmaxf(sa, sb);
+    if (sa < best - 2.f * kEpsF32) return j;
+    if (sb < best - 2.f * kEpsF32) return i;
+    return cos64(em, b, d) > cos64(em, a, d) ? j : i;
+}
+
+// kMode = kLbLabel: labelling. The best two modes of every pixel and the third
+// score; a best two within 2 kEpsTc of one another, the third not, are decided
+// here by the exact test of the two (K = 11,500 modes: 1% of the pixels, which
+// took a scan of all modes each, 735 us of a frame's 1030 us of labelling).
 // kMode = kLbCover: coverage of the OSOP stop rule against the modes [k0, K):
-// an uncovered pixel whose best score clears c by kEpsTc is covered; one
-// within kEpsTc of c is queued for the FP32 form's exact test.
+// an uncovered pixel whose best score clears c by kEpsTc is covered; a score
+// within kEpsTc of c takes the exact test of that pixel and mode.
 // kMode = kLbOld, kLbPairs: the merge's two contractions, rows being the
 // candidates in rank order. A score farther than kDelta = kEpsTc + 2e-6 from
 // merge_cos decides the pair as the exact test does (kEpsTc bounds the split
 // score, 2e-6 the gap between x.m and the FP64 cosine of near-unit FP32
 // vectors); nearer ones take the exact test itself (cos_at_least). kLbOld:
-// a candidate within merge_cos of an earlier mode is removed; near ones are
-// queued for k_merge_old_fix. kLbPairs: every candidate ranked above the row
+// a candidate within merge_cos of an earlier mode is removed. kLbPairs: every candidate ranked above the row
 // that is not removed and within merge_cos joins the row's conflict list.
+// The exact tests run in the reader's warp, whose S buffer is free again by
+// then, on the columns in doubt alone. Queued rows that a second kernel tested
+// against every mode took 30 us (coverage) and 49 us (merge) a launch.
 // pmap / mmap: the pixel and mode split rows (dimensions 0-15); pmap1 /
 // mmap1: dimensions 16-31 (D = 32 only).
 template <class Map, int kMode, int kD>
@@ -238,16 +266,17 @@ k_label_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
     using L = LbDim<kD>;
     constexpr int kHalves = L::kHalves, kLStages = L::kStages;
     constexpr float kEpsTc = L::kEps;
-    constexpr float kDelta = L::kEps + 2e-6f;
+    constexpr float kDelta = kMode == kLbCover ? L::kEps : L::kEps + 2e-6f;
+    // Labelling: a mode whose score is farther than this below the best is not
+    // among those the exact decision compares (2 kEps of score error, 2 kEpsF32
+    // of its FP32 scores, 2 kEpsF32 of its own band, and rounding here).
+    constexpr float kTie = 2.f * L::kEps + 5.f * kEpsF32;
     constexpr bool kCover = kMode == kLbCover || kMode == kLbOld;  // best column against a threshold
     if (!map.init()) return;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* Ab = smem + L::kOffA;
     uint8_t* Bst = smem + L::kOffB;
-    float* xb1 = (float*)(smem + L::kOffX);        // [4][128]
-    int* xi1 = (int*)(xb1 + 4 * 128);              // [4][128]
-    float* xb2 = (float*)(xi1 + 4 * 128);          // [4][128]
     uint64_t* bars = (uint64_t*)(smem + L::kOffBar);
     uint64_t* a_full = bars;                       // [2]
     uint64_t* a_empty = a_full + 2;                // [2]
@@ -377,20 +406,30 @@ k_label_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
         const int h = warp >> 2;                 // which 32 columns of a mode tile
         const int r = q * 32 + lane;             // pixel row of the tile
         const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-        int g = 0;
+        int g = 0, ix = 0;
         for (int item = blockIdx.x; item < items; item += gridDim.x) {
             const LbItem ii = map.item(item);
             const int nmt = (ii.K - ii.k0 + 127) / 128;
             if (kMode != kLbLabel && nmt <= 0) continue;
+            // Exchange buffers by turns: a slice's warps go on to the next item
+            // while the first slice's decide this one, and write this buffer
+            // again only after the barrier of the item between.
+            float* xb1 = (float*)(smem + L::kOffX + (ix & 1) * L::kExchange);  // [4][128]
+            int* xi1 = (int*)(xb1 + 4 * 128);
+            float* xb2 = (float*)(xi1 + 4 * 128);
+            int* xi2 = (int*)(xb2 + 4 * 128);
+            float* xb3 = (float*)(xi2 + 4 * 128);
+            ++ix;
             bool ok = true;
-            float b1 = -INFINITY, b2 = -INFINITY;
-            int i1 = -1;
+            float b1 = -INFINITY, b2 = -INFINITY, b3 = -INFINITY;
+            int i1 = -1, i2 = -1;
             // merge rows: the candidate's rank, its frame's row base, and
             // whether it takes part (a candidate removed by an earlier mode
-            // needs no conflict list)
+            // needs no conflict list); coverage: the pixel, if uncovered
             const int mi = ii.pt * 128 + r;
-            const int64_t mbase = (kMode == kLbPairs && out.frames) ? out.frames[ii.frame].pix0 : 0;
-            const bool mrow = kMode == kLbPairs && mi < ii.n && !out.removed_r[mbase + mi];
+            const int64_t mbase = (kMode != kLbLabel && out.frames) ? out.frames[ii.frame].pix0 : 0;
+            const bool mrow = kMode != kLbLabel && mi < ii.n &&
+                              !(kMode == kLbCover ? out.covered : out.removed_r)[mbase + mi];
             int ma = -1;  // the row's candidate index, read when first needed
             for (int mt = 0; mt < nmt; ++mt, ++g) {
                 const int b = g % kLSBufs;
@@ -419,8 +458,38 @@ k_label_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
 #pragma unroll
                     for (int j = 1; j < 32; ++j) m = fmaxf(m, __uint_as_float(v[j]));
                 }
-                if (kCover) {
-                    b1 = fmaxf(b1, m);
+                if constexpr (kCover) {
+                    // b1: the best score that needs no exact test, +inf once
+                    // an exact test has passed
+                    const float lo = out.c_f - kDelta, hi = out.c_f + kDelta;
+                    const bool doubt = mrow && m >= lo && m < hi && b1 < hi;
+                    if (m >= hi) b1 = fmaxf(b1, m);
+                    if (__any_sync(0xffffffffu, doubt) && doubt) {
+                        uint32_t near = 0;
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) near |= (uint32_t)(__uint_as_float(v[j]) >= lo) << j;
+                        float xr[kD];
+                        const float* row = (kMode == kLbCover ? out.P32 : out.Xr) + (mbase + mi) * kD;
+#pragma unroll
+                        for (int k = 0; k < kD; ++k) xr[k] = row[k];
+                        for (; near; near &= near - 1) {
+                            const float* mode = out.modes + (mbase + col0 + __ffs(near) - 1) * kD;
+                            bool hit;
+                            if (kMode == kLbCover) {
+                                const float sc = dot_seq<kD>(xr, mode);
+                                hit = sc >= out.c_f + kEpsF32;
+                                if (!hit && sc >= out.c_f - kEpsF32)
+                                    hit = cos64((out.frames ? out.frames[ii.frame].emb : out.emb1) +
+                                                    (int64_t)out.pix[mbase + mi] * out.d, mode, out.d) >= out.thr;
+                            } else {
+                                hit = cos_at_least<kD>(xr, mode, out.c_f, out.thr);
+                            }
+                            if (hit) {
+                                b1 = INFINITY;
+                                break;
+                            }
+                        }
+                    }
                     continue;
                 }
                 if constexpr (kMode == kLbPairs) {
@@ -458,19 +527,36 @@ k_label_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
                     }
                     continue;
                 }
-                // A column can change the best two only if it beats the
-                // second best; in increasing column order a tie keeps the
-                // lower index as the best.
-                if (__any_sync(0xffffffffu, m > b2)) {
+                // Only columns within kTie of the best so far can take part in
+                // the decision; of those the best two and the third score are
+                // kept. A slice mostly holds one of them or none.
+                const float tie = fmaxf(b1, m) - kTie;
+                if (__any_sync(0xffffffffu, m >= tie)) {
+                    uint32_t near = 0;
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const float sc = __uint_as_float(v[j]);
-                        if (sc > b1) {
-                            b2 = b1;
-                            b1 = sc;
-                            i1 = col0 + j;
-                        } else if (sc > b2) {
-                            b2 = sc;
+                    for (int j = 0; j < 32; ++j) near |= (uint32_t)(__uint_as_float(v[j]) >= tie) << j;
+                    const bool single = __popc(near) <= 1;
+                    if (near && single) {
+                        const int c = col0 + __ffs(near) - 1;
+                        const bool first = m > b1, second = m > b2;
+                        b3 = second ? b2 : fmaxf(b3, m);
+                        i2 = first ? i1 : second ? c : i2;
+                        b2 = first ? b1 : second ? m : b2;
+                        i1 = first ? c : i1;
+                        b1 = first ? m : b1;
+                    }
+                    if (__any_sync(0xffffffffu, !single)) {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) {
+                            const float sc = __uint_as_float(v[j]);
+                            if (!single && sc > b3) {
+                                const bool first = sc > b1, second = sc > b2;
+                                b3 = second ? b2 : sc;
+                                i2 = first ? i1 : second ? col0 + j : i2;
+                                b2 = first ? b1 : second ? sc : b2;
+                                i1 = first ? col0 + j : i1;
+                                b1 = first ? sc : b1;
+                            }
                         }
                     }
                 }
@@ -481,6 +567,10 @@ k_label_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
             xb1[h * 128 + r] = b1;
             xi1[h * 128 + r] = i1;
             xb2[h * 128 + r] = b2;
+            if (kMode == kLbLabel) {
+                xi2[h * 128 + r] = i2;
+                xb3[h * 128 + r] = b3;
+            }
             uint32_t any_bad;
             asm volatile(
                 "{\n\t.reg .pred p, q;\n\t"
@@ -495,59 +585,55 @@ k_label_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
                 const float B1 = fmaxf(fmaxf(xb1[r], xb1[128 + r]), fmaxf(xb1[256 + r], xb1[384 + r]));
                 const int i = ii.pt * 128 + r;
                 const int64_t base = out.frames ? out.frames[ii.frame].pix0 : 0;
-                if (i < ii.n && !out.removed_r[base + i]) {
-                    if (B1 >= out.c_f + kDelta) {
-                        out.removed_r[base + i] = 1;
-                        out.cand_state[base + out.rank_cand[base + i]] = kRemoved;
-                    } else if (B1 >= out.c_f - kDelta) {
-                        const int slot = atomicAdd(out.fix_count, 1);
-                        out.fix[slot] = make_int2(ii.frame, i);
-                    }
+                if (B1 >= out.c_f + kDelta && mrow) {
+                    out.removed_r[base + i] = 1;
+                    out.cand_state[base + out.rank_cand[base + i]] = kRemoved;
                 }
             } else if (kMode == kLbCover && h == 0) {
                 const float B1 = fmaxf(fmaxf(xb1[r], xb1[128 + r]), fmaxf(xb1[256 + r], xb1[384 + r]));
                 const int i = ii.pt * 128 + r;
                 const int64_t base = out.frames ? out.frames[ii.frame].pix0 : 0;
-                bool newly = false;
-                if (i < ii.n && !out.covered[base + i]) {
-                    if (B1 >= out.c_f + kEpsTc) {
-                        out.covered[base + i] = 1;
-                        newly = true;
-                    } else if (B1 >= out.c_f - kEpsTc) {
-                        const int slot = atomicAdd(out.fix_count, 1);
-                        out.fix[slot] = make_int2(ii.frame, i);
-                    }
-                }
+                const bool newly = mrow && B1 >= out.c_f + kDelta;
+                if (newly) out.covered[base + i] = 1;
                 const unsigned nb = __ballot_sync(0xffffffffu, newly);
                 if (lane == 0 && nb)
                     atomicSub(out.states ? &out.states[ii.frame].dc.n_uncovered : out.n_uncovered, __popc(nb));
             } else if (kMode == kLbLabel && h == 0) {
-                float B1 = xb1[r], B2 = xb2[r];
-                int I1 = xi1[r];
+                float B1 = xb1[r], B2 = xb2[r], B3 = xb3[r];
+                int I1 = xi1[r], I2 = xi2[r];
 #pragma unroll
                 for (int k = 1; k < 4; ++k) {
-                    const float c1 = xb1[k * 128 + r], c2 = xb2[k * 128 + r];
-                    const int ci = xi1[k * 128 + r];
-                    if (c1 > B1 || (c1 == B1 && ci >= 0 && (I1 < 0 || ci < I1))) {
-                        B2 = fmaxf(B1, fmaxf(B2, c2));
-                        B1 = c1;
-                        I1 = ci;
-                    } else {
-                        B2 = fmaxf(B2, fmaxf(c1, c2));
+                    const float cb[2] = {xb1[k * 128 + r], xb2[k * 128 + r]};
+                    const int ci[2] = {xi1[k * 128 + r], xi2[k * 128 + r]};
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        const bool first = cb[t] > B1, second = cb[t] > B2;
+                        B3 = second ? B2 : fmaxf(B3, cb[t]);
+                        I2 = first ? I1 : second ? ci[t] : I2;
+                        B2 = first ? B1 : second ? cb[t] : B2;
+                        I1 = first ? ci[t] : I1;
+                        B1 = first ? cb[t] : B1;
                     }
+                    B3 = fmaxf(B3, xb3[k * 128 + r]);
                 }
                 const int i = ii.pt * 128 + r;
                 if (i < ii.n) {
                     const int64_t base = out.frames ? out.frames[ii.frame].pix0 : 0;
-                    int32_t* lab = out.labels ? out.labels[ii.frame] : out.labels1;
-                    lab[out.pix[base + i]] = I1;
-                    if (ii.K > 1 && !(B1 - B2 > 2.f * kEpsTc)) {
-                        const int slot = atomicAdd(out.fix_count, 1);
-                        out.fix[slot] = make_int2(ii.frame, i);
+                    int32_t* lab = (out.labels ? out.labels[ii.frame] : out.labels1) + out.pix[base + i];
+                    if (ii.K > 1 && !(B1 - B2 > kTie)) {
+                        if (B1 - B3 > kTie) {
+                            I1 = better_mode<kD>(out.P32 + (base + i) * kD, out.modes + base * kD,
+                                                 (out.frames ? out.frames[ii.frame].emb : out.emb1) +
+                                                     (int64_t)out.pix[base + i] * out.d,
+                                                 out.d, min(I1, I2), max(I1, I2));
+                        } else {
+                            const int slot = atomicAdd(out.fix_count, 1);
+                            out.fix[slot] = make_int2(ii.frame, i);
+                        }
                     }
+                    *lab = I1;
                 }
             }
-            asm volatile("bar.sync 1, %0;" ::"n"(kLEpi * 32) : "memory");
         }
     }
     tc_fence_before();
@@ -615,6 +701,7 @@ __global__ void k_label_fix(const int2* __restrict__ fix, const int* __restrict_
 // (so a mode is read from L2 once per 64 pixels instead of once per pixel).
 // Scores, thresholds and the FP64 tie-break are those of k_label_fix.
 constexpr int kFixPix = 64, kFixQ = 4, kFixTile = 128;
+constexpr int kFixFew = 8;  // pixels per block up to which a block takes one at a time
 template <int Dp>
 __global__ void __launch_bounds__(kFixPix * kFixQ)
 k_label_fix_tiled(const int2* __restrict__ fix, const int* __restrict__ fix_count, const float* __restrict__ P32,
@@ -625,6 +712,66 @@ k_label_fix_tiled(const int2* __restrict__ fix, const int* __restrict__ fix_coun
     __shared__ double rc[kFixQ][kFixPix];
     __shared__ int ri[kFixQ][kFixPix];
     const int cnt = *fix_count;
+    // Few pixels: a block each, its threads over the modes. A block of 64
+    // pixels passes the modes in 2 K / 128 dependent steps, 551 us for K =
+    // 11,500 however few the pixels; alone they took 98 us there. 64 pixels in
+    // 551 us are 14 alone in 40 us each: the line lies at 8 a block.
+    if (cnt <= kFixFew * (int)gridDim.x) {
+        constexpr int kT = kFixPix * kFixQ, kW = kT / 32;
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        float* rb1 = &rb[0][0];
+        double* rc1 = &rc[0][0];
+        int* ri1 = &ri[0][0];
+        for (int e = blockIdx.x; e < cnt; e += gridDim.x) {
+            const int i = fix[e].y;
+            float pv[Dp];
+#pragma unroll
+            for (int k = 0; k < Dp; ++k) pv[k] = P32[(int64_t)i * Dp + k];
+            float b1 = -INFINITY;
+#pragma unroll 2
+            for (int j = threadIdx.x; j < K; j += kT) b1 = fmaxf(b1, dot_seq<Dp>(pv, M + (int64_t)j * Dp));
+            for (int o = 16; o > 0; o >>= 1) b1 = fmaxf(b1, __shfl_xor_sync(0xffffffffu, b1, o));
+            __syncthreads();
+            if (lane == 0) rb1[wid] = b1;
+            __syncthreads();
+#pragma unroll
+            for (int w = 0; w < kW; ++w) b1 = fmaxf(b1, rb1[w]);
+            const float* em = emb + (int64_t)pix[i] * d;
+            double bc = -INFINITY;
+            int best = K;
+#pragma unroll 2
+            for (int j = threadIdx.x; j < K; j += kT) {
+                if (dot_seq<Dp>(pv, M + (int64_t)j * Dp) < b1 - 2.f * kEpsF32) continue;
+                const double cs = cos64(em, M + (int64_t)j * Dp, d);
+                if (cs > bc) {
+                    bc = cs;
+                    best = j;
+                }
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                const double ob = __shfl_xor_sync(0xffffffffu, bc, o);
+                const int oi = __shfl_xor_sync(0xffffffffu, best, o);
+                if (ob > bc || (ob == bc && oi < best)) {
+                    bc = ob;
+                    best = oi;
+                }
+            }
+            if (lane == 0) {
+                rc1[wid] = bc;
+                ri1[wid] = best;
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                for (int w = 1; w < kW; ++w)
+                    if (rc1[w] > bc || (rc1[w] == bc && ri1[w] < best)) {
+                        bc = rc1[w];
+                        best = ri1[w];
+                    }
+                if (best < K) labels[pix[i]] = best;
+            }
+        }
+        return;
+    }
     const int pl = threadIdx.x % kFixPix, q = threadIdx.x / kFixPix;
     for (int g0 = blockIdx.x * kFixPix; g0 < cnt; g0 += gridDim.x * kFixPix) {
         const int e = g0 + pl;
@@ -718,129 +865,31 @@ __global__ void k_pack_modes_range(const float* __restrict__ modes, int k0, int 
     pack_mode<Dp>(modes + (int64_t)r * Dp, Mk, r, half_rows);
 }
 
-// Coverage of the queued pixels (tensor-core score within kEpsTc of c),
-// decided exactly as the FP32 form decides it: one warp per pixel, lanes over
-// the new modes; a mode covers the pixel when its FP32 score clears c by
-// kEpsF32, or is within kEpsF32 of c and the FP64 cosine of the raw embedding
-// reaches c.
-template <int Dp>
-__global__ void k_cover_fix(const int2* __restrict__ fix, const int* __restrict__ fix_count,
-                            const float* __restrict__ P32, const float* __restrict__ modes, int k0, int k1,
-                            const int32_t* __restrict__ pix, const float* __restrict__ emb, int d, float c_f, double c,
-                            uint8_t* __restrict__ covered, int* __restrict__ n_uncovered) {
-    const int lane = threadIdx.x & 31;
-    const int wpb = blockDim.x >> 5;
-    const int cnt = *fix_count;
-    for (int e = blockIdx.x * wpb + (threadIdx.x >> 5); e < cnt; e += gridDim.x * wpb) {
-        const int i = fix[e].y;
-        float pv[Dp];
-#pragma unroll
-        for (int k = 0; k < Dp; ++k) pv[k] = P32[(int64_t)i * Dp + k];
-        const float* em = emb + (int64_t)pix[i] * d;
-        bool cov = false;
-        for (int j = k0 + lane; j < k1 && !cov; j += 32) {
-            const float* m = modes + (int64_t)j * Dp;
-            const float sc = dot_seq<Dp>(pv, m);
-            cov = sc >= c_f + kEpsF32 || (sc >= c_f - kEpsF32 && cos64(em, m, d) >= c);
-        }
-        if (__any_sync(0xffffffffu, cov) && lane == 0) {
-            covered[i] = 1;
-            atomicSub(n_uncovered, 1);
-        }
-    }
-}
-
 // The batch form of k_pack_modes_range: every frame whose round ended packs
-// its new modes [k0, n_kept) at its Mk rows; clears the recheck queue.
+// its new modes [k0, n_kept) at its Mk rows.
 template <int Dp>
 __global__ void k_pack_modes_new_batch(const BFrame* __restrict__ frames, const BState* __restrict__ states,
-                                       const float* __restrict__ modes, uint4* __restrict__ Mk, int64_t half_rows,
-                                       int* fix_count) {
+                                       const float* __restrict__ modes, uint4* __restrict__ Mk, int64_t half_rows) {
     const BFrame& fr = frames[blockIdx.y];
     const BState& st = states[blockIdx.y];
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *fix_count = 0;
     if (st.phase != kRoundDone) return;
     const int r = st.k0 + blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= st.dc.n_kept) return;
     pack_mode<Dp>(modes + (fr.pix0 + r) * Dp, Mk, fr.pk_row0 + r, half_rows);
 }
 
-// k_cover_fix for the batch: queued (frame, foreground index) pairs, each
-// against its frame's new modes.
-template <int Dp>
-__global__ void k_cover_fix_batch(const int2* __restrict__ fix, const int* __restrict__ fix_count,
-                                  const float* __restrict__ P32, const float* __restrict__ modes,
-                                  const BFrame* __restrict__ frames, BState* states, const int32_t* __restrict__ pix,
-                                  int d, float c_f, double c, uint8_t* __restrict__ covered) {
-    const int lane = threadIdx.x & 31;
-    const int wpb = blockDim.x >> 5;
-    const int cnt = *fix_count;
-    for (int e = blockIdx.x * wpb + (threadIdx.x >> 5); e < cnt; e += gridDim.x * wpb) {
-        const int2 fi = fix[e];
-        const int f = fi.x, i = fi.y;
-        const BFrame& fr = frames[f];
-        const int64_t base = fr.pix0;
-        const int k0 = states[f].k0, k1 = states[f].dc.n_kept;
-        float pv[Dp];
-#pragma unroll
-        for (int k = 0; k < Dp; ++k) pv[k] = P32[(base + i) * Dp + k];
-        const float* em = fr.emb + (int64_t)pix[base + i] * d;
-        bool cov = false;
-        for (int j = k0 + lane; j < k1 && !cov; j += 32) {
-            const float* m = modes + (base + j) * Dp;
-            const float sc = dot_seq<Dp>(pv, m);
-            cov = sc >= c_f + kEpsF32 || (sc >= c_f - kEpsF32 && cos64(em, m, d) >= c);
-        }
-        if (__any_sync(0xffffffffu, cov) && lane == 0) {
-            covered[base + i] = 1;
-            atomicSub(&states[f].dc.n_uncovered, 1);
-        }
-    }
-}
-
 // The candidates of every frame whose round ended, in rank order (Xr), as
-// BF16 split rows at the frame's Pk row offsets; clears the recheck queue.
+// BF16 split rows at the frame's Pk row offsets.
 template <int Dp>
 __global__ void k_pack_cands_batch(const BFrame* __restrict__ frames, const BState* __restrict__ states,
-                                   const float* __restrict__ Xr, uint4* __restrict__ Ck, int64_t half_rows,
-                                   int* fix_count) {
+                                   const float* __restrict__ Xr, uint4* __restrict__ Ck, int64_t half_rows) {
     const BFrame& fr = frames[blockIdx.y];
     const BState& st = states[blockIdx.y];
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *fix_count = 0;
     if (st.phase != kRoundDone) return;
     const int k = st.dc.n_cand;
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= (k + 127) / 128 * 128) return;
     pack_mode<Dp>(r < k ? Xr + (fr.pix0 + r) * Dp : nullptr, Ck, fr.pk_row0 + r, half_rows);
-}
-
-// Candidates queued by the tensor-core test against earlier modes (score
-// within kDelta of merge_cos), decided exactly as k_b_merge_old decides: one
-// warp per candidate, lanes over the frame's earlier modes.
-// One frame: frames and states are nullptr, the frame's earlier modes are K1.
-template <int Dp>
-__global__ void k_merge_old_fix_batch(const int2* __restrict__ fix, const int* __restrict__ fix_count,
-                                      const float* __restrict__ Xr, const float* __restrict__ modes,
-                                      const BFrame* __restrict__ frames, const BState* __restrict__ states, int K1,
-                                      const int32_t* __restrict__ rank_cand, float thr_f, double thr,
-                                      uint8_t* __restrict__ cand_state, uint8_t* __restrict__ removed_r) {
-    const int lane = threadIdx.x & 31;
-    const int wpb = blockDim.x >> 5;
-    const int cnt = *fix_count;
-    for (int e = blockIdx.x * wpb + (threadIdx.x >> 5); e < cnt; e += gridDim.x * wpb) {
-        const int2 fi = fix[e];
-        const int64_t base = frames ? frames[fi.x].pix0 : 0;
-        const int K = states ? states[fi.x].dc.n_kept : K1;
-        float x[Dp];
-#pragma unroll
-        for (int k = 0; k < Dp; ++k) x[k] = Xr[(base + fi.y) * Dp + k];
-        bool hit = false;
-        for (int j = lane; j < K && !hit; j += 32) hit = cos_at_least<Dp>(x, modes + (base + j) * Dp, thr_f, thr);
-        if (__any_sync(0xffffffffu, hit) && lane == 0) {
-            removed_r[base + fi.y] = 1;
-            cand_state[base + rank_cand[base + fi.y]] = kRemoved;
-        }
-    }
 }
 
 // One frame's k candidates (rank order, Xr) as BF16 split rows [0, kp).
@@ -887,9 +936,8 @@ ms_status label_tc_setup_dim() {
 template <int Dp>
 ms_status merge_tc_single(void* Ck, void* Mk, int64_t n_pad, int k, int K_old, const float* Xr, const float* modes,
                           const int32_t* rank_cand, uint8_t* cand_state, uint8_t* removed_r, int32_t* conf_deg,
-                          int32_t* conf, float thr_f, double thr, LabelTcScratch sc, int grid, int* status,
+                          int32_t* conf, float thr_f, double thr, int grid, int* status,
                           cudaStream_t st) {
-    MS_CUDA(cudaMemsetAsync(sc.fix_count, 0, sizeof(int), st));
     const int kp = (k + 127) / 128 * 128;
     k_pack_cands_single<Dp><<<(kp + 255) / 256, 256, 0, st>>>(Xr, k, kp, (uint4*)Ck, n_pad);
     MS_LAUNCH("k_pack_cands_single");
@@ -902,9 +950,8 @@ ms_status merge_tc_single(void* Ck, void* Mk, int64_t n_pad, int k, int K_old, c
     if (Dp == 32 && (s = encode_pk_map((uint8_t*)Ck + n_pad * 128, (int)n_pad, &cmap1)) != MS_OK) return s;
     if (Dp == 32 && (s = encode_pk_map((uint8_t*)Mk + n_pad * 128, (int)n_pad, &mmap1)) != MS_OK) return s;
     LbOut out{};
-    out.fix = sc.fix;
-    out.fix_count = sc.fix_count;
     out.c_f = thr_f;
+    out.modes = modes;
     out.Xr = Xr;
     out.removed_r = removed_r;
     out.rank_cand = rank_cand;
@@ -917,9 +964,6 @@ ms_status merge_tc_single(void* Ck, void* Mk, int64_t n_pad, int k, int K_old, c
         k_label_tc<LbSingleMerge, kLbOld, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(cmap, mmap, cmap1, mmap1,
                                                                                             om, out, status);
         MS_LAUNCH("k_label_tc(merge, earlier modes)");
-        k_merge_old_fix_batch<Dp><<<grid, 256, 0, st>>>(sc.fix, sc.fix_count, Xr, modes, nullptr, nullptr, K_old,
-                                                        rank_cand, thr_f, thr, cand_state, removed_r);
-        MS_LAUNCH("k_merge_old_fix");
     }
     LbSingleMerge pm{k, 0, 1};
     k_label_tc<LbSingleMerge, kLbPairs, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(cmap, cmap, cmap1, cmap1,
@@ -933,16 +977,15 @@ ms_status merge_tc_batch(const CUtensorMap& cmap, const CUtensorMap& cmap1, cons
                          const CUtensorMap& mmap1, void* Ck, int64_t rows, const BFrame* frames, BState* states, int B,
                          int max_pk_rows, const float* Xr, const float* modes, const int32_t* rank_cand,
                          uint8_t* cand_state, uint8_t* removed_r, int32_t* conf_deg, int32_t* conf, float thr_f,
-                         double thr, const int32_t* tile_off, LabelTcScratch sc, int grid, int* status,
+                         double thr, const int32_t* tile_off, int grid, int* status,
                          cudaStream_t st) {
     const dim3 gp((unsigned)((max_pk_rows + 255) / 256), (unsigned)B);
-    k_pack_cands_batch<Dp><<<gp, 256, 0, st>>>(frames, states, Xr, (uint4*)Ck, rows, sc.fix_count);
+    k_pack_cands_batch<Dp><<<gp, 256, 0, st>>>(frames, states, Xr, (uint4*)Ck, rows);
     MS_LAUNCH("k_pack_cands_batch");
     LbOut out{};
     out.frames = frames;
-    out.fix = sc.fix;
-    out.fix_count = sc.fix_count;
     out.c_f = thr_f;
+    out.modes = modes;
     out.Xr = Xr;
     out.removed_r = removed_r;
     out.rank_cand = rank_cand;
@@ -954,9 +997,6 @@ ms_status merge_tc_batch(const CUtensorMap& cmap, const CUtensorMap& cmap1, cons
     k_label_tc<LbBatchOld, kLbOld, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(cmap, mmap, cmap1, mmap1, om,
                                                                                      out, status);
     MS_LAUNCH("k_label_tc(merge, earlier modes)");
-    k_merge_old_fix_batch<Dp><<<grid, 256, 0, st>>>(sc.fix, sc.fix_count, Xr, modes, frames, states, 0, rank_cand,
-                                                    thr_f, thr, cand_state, removed_r);
-    MS_LAUNCH("k_merge_old_fix_batch");
     LbBatchPairs pm{frames, states, tile_off, B, 0};
     k_label_tc<LbBatchPairs, kLbPairs, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(cmap, cmap, cmap1, cmap1,
                                                                                          pm, out, status);
@@ -968,29 +1008,33 @@ template <int Dp>
 ms_status cover_tc_batch(const CUtensorMap& pmap, const CUtensorMap& mmap, const CUtensorMap& pmap1,
                          const CUtensorMap& mmap1, void* Mk, int64_t mk_rows, const BFrame* frames, BState* states,
                          int B, int max_pk_rows, const float* modes, const float* P32, const int32_t* pix, int d,
-                         double c, uint8_t* covered, const int32_t* tile_off, LabelTcScratch sc, int grid, int* status,
+                         double c, uint8_t* covered, const int32_t* tile_off, int grid, int* status,
                          cudaStream_t st) {
     const dim3 gp((unsigned)((max_pk_rows + 255) / 256), (unsigned)B);
-    k_pack_modes_new_batch<Dp><<<gp, 256, 0, st>>>(frames, states, modes, (uint4*)Mk, mk_rows, sc.fix_count);
+    k_pack_modes_new_batch<Dp><<<gp, 256, 0, st>>>(frames, states, modes, (uint4*)Mk, mk_rows);
     MS_LAUNCH("k_pack_modes_new_batch");
     const float c_f = (float)c;
     LbBatchCover map{frames, states, tile_off, B, 0};
-    LbOut out{nullptr, nullptr, frames, pix, sc.fix, sc.fix_count, covered, nullptr, c_f, states};
+    LbOut out{};
+    out.frames = frames;
+    out.pix = pix;
+    out.covered = covered;
+    out.c_f = c_f;
+    out.states = states;
+    out.thr = c;
+    out.P32 = P32;
+    out.modes = modes;
+    out.d = d;
     k_label_tc<LbBatchCover, kLbCover, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(pmap, mmap, pmap1, mmap1, map,
                                                                                        out, status);
     MS_LAUNCH("k_label_tc(cover, batch)");
-    k_cover_fix_batch<Dp><<<grid, 256, 0, st>>>(sc.fix, sc.fix_count, P32, modes, frames, states, pix, d, c_f, c,
-                                                covered);
-    MS_LAUNCH("k_cover_fix_batch");
     return MS_OK;
 }
 
 template <int Dp>
 ms_status cover_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, void* Mk, int64_t n_pad,
                           const float* modes, int k0, int k1, int n, const float* P32, const int32_t* pix,
-                          const float* emb, int d, double c, uint8_t* covered, int* n_uncovered, LabelTcScratch sc,
-                          int grid, int* status, cudaStream_t st) {
-    MS_CUDA(cudaMemsetAsync(sc.fix_count, 0, sizeof(int), st));
+                          const float* emb, int d, double c, uint8_t* covered, int* n_uncovered, int grid, int* status, cudaStream_t st) {
     k_pack_modes_range<Dp><<<(k1 - k0 + 255) / 256, 256, 0, st>>>(modes, k0, k1, (uint4*)Mk, n_pad);
     MS_LAUNCH("k_pack_modes_range");
     CUtensorMap mmap, mmap1;
@@ -1001,13 +1045,19 @@ ms_status cover_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, voi
     LbSingle map{n, k1};
     map.k0 = k0;
     const float c_f = (float)c;
-    LbOut out{nullptr, nullptr, nullptr, pix, sc.fix, sc.fix_count, covered, n_uncovered, c_f, nullptr};
+    LbOut out{};
+    out.pix = pix;
+    out.covered = covered;
+    out.n_uncovered = n_uncovered;
+    out.c_f = c_f;
+    out.thr = c;
+    out.P32 = P32;
+    out.modes = modes;
+    out.emb1 = emb;
+    out.d = d;
     k_label_tc<LbSingle, kLbCover, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(pmap, mmap, pmap1, mmap1, map, out,
                                                                                    status);
     MS_LAUNCH("k_label_tc(cover)");
-    k_cover_fix<Dp><<<grid, 256, 0, st>>>(sc.fix, sc.fix_count, P32, modes, k0, k1, pix, emb, d, c_f, c, covered,
-                                          n_uncovered);
-    MS_LAUNCH("k_cover_fix");
     return MS_OK;
 }
 
@@ -1027,7 +1077,15 @@ ms_status label_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, voi
     mmap1 = mmap;
     if (Dp == 32 && (s = encode_pk_map((uint8_t*)Mk + n_pad * 128, (int)n_pad, &mmap1)) != MS_OK) return s;
     LbSingle map{n, K};
-    LbOut out{nullptr, labels, nullptr, pix, sc.fix, sc.fix_count, nullptr, nullptr, 0.f, nullptr};
+    LbOut out{};
+    out.labels1 = labels;
+    out.pix = pix;
+    out.fix = sc.fix;
+    out.fix_count = sc.fix_count;
+    out.P32 = P32;
+    out.modes = modes;
+    out.emb1 = emb;
+    out.d = d;
     k_label_tc<LbSingle, kLbLabel, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(pmap, mmap, pmap1, mmap1, map,
                                                                                     out, status);
     MS_LAUNCH("k_label_tc");
@@ -1051,7 +1109,15 @@ ms_status label_tc_batch(const CUtensorMap& pmap, const CUtensorMap& mmap, const
     k_label_items<<<1, 32, 0, st>>>(frames, B, sc.off, sc.fix_count);
     MS_LAUNCH("k_label_items");
     LbBatch map{frames, states, sc.off, B, 0};
-    LbOut out{labels, nullptr, frames, pix, sc.fix, sc.fix_count, nullptr, nullptr, 0.f, nullptr};
+    LbOut out{};
+    out.labels = labels;
+    out.frames = frames;
+    out.pix = pix;
+    out.fix = sc.fix;
+    out.fix_count = sc.fix_count;
+    out.P32 = P32;
+    out.modes = modes;
+    out.d = d;
     k_label_tc<LbBatch, kLbLabel, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(pmap, mmap, pmap1, mmap1, map,
                                                                                    out, status);
     MS_LAUNCH("k_label_tc(batch)");
@@ -1072,47 +1138,45 @@ ms_status launch_merge_tc_batch(const CUtensorMap& cmap, const CUtensorMap& cmap
                                 const CUtensorMap& mmap1, void* Ck, int64_t rows, int Dp, const BFrame* frames,
                                 BState* states, int B, int max_pk_rows, const float* Xr, const float* modes,
                                 const int32_t* rank_cand, uint8_t* cand_state, uint8_t* removed_r, int32_t* conf_deg,
-                                int32_t* conf, float thr_f, double thr, const int32_t* tile_off, LabelTcScratch sc,
-                                int grid, int* status, cudaStream_t st) {
+                                int32_t* conf, float thr_f, double thr, const int32_t* tile_off, int grid, int* status, cudaStream_t st) {
     return Dp == 32 ? merge_tc_batch<32>(cmap, cmap1, mmap, mmap1, Ck, rows, frames, states, B, max_pk_rows, Xr, modes,
-                                         rank_cand, cand_state, removed_r, conf_deg, conf, thr_f, thr, tile_off, sc,
+                                         rank_cand, cand_state, removed_r, conf_deg, conf, thr_f, thr, tile_off,
                                          grid, status, st)
                     : merge_tc_batch<16>(cmap, cmap1, mmap, mmap1, Ck, rows, frames, states, B, max_pk_rows, Xr, modes,
-                                         rank_cand, cand_state, removed_r, conf_deg, conf, thr_f, thr, tile_off, sc,
+                                         rank_cand, cand_state, removed_r, conf_deg, conf, thr_f, thr, tile_off,
                                          grid, status, st);
 }
 
 ms_status launch_merge_tc_single(void* Ck, void* Mk, int64_t n_pad, int Dp, int k, int K_old, const float* Xr,
                                  const float* modes, const int32_t* rank_cand, uint8_t* cand_state, uint8_t* removed_r,
-                                 int32_t* conf_deg, int32_t* conf, float thr_f, double thr, LabelTcScratch sc,
-                                 int grid, int* status, cudaStream_t st) {
+                                 int32_t* conf_deg, int32_t* conf, float thr_f, double thr, int grid, int* status, cudaStream_t st) {
     if (k <= 0) return MS_OK;
     return Dp == 32 ? merge_tc_single<32>(Ck, Mk, n_pad, k, K_old, Xr, modes, rank_cand, cand_state, removed_r,
-                                          conf_deg, conf, thr_f, thr, sc, grid, status, st)
+                                          conf_deg, conf, thr_f, thr,  grid, status, st)
                     : merge_tc_single<16>(Ck, Mk, n_pad, k, K_old, Xr, modes, rank_cand, cand_state, removed_r,
-                                          conf_deg, conf, thr_f, thr, sc, grid, status, st);
+                                          conf_deg, conf, thr_f, thr,  grid, status, st);
 }
 
 ms_status launch_cover_tc_batch(const CUtensorMap& pmap, const CUtensorMap& mmap, const CUtensorMap& pmap1,
                                 const CUtensorMap& mmap1, void* Mk, int64_t mk_rows, int Dp, const BFrame* frames,
                                 BState* states, int B, int max_pk_rows, const float* modes, const float* P32,
                                 const int32_t* pix, int d, double c, uint8_t* covered, const int32_t* tile_off,
-                                LabelTcScratch sc, int grid, int* status, cudaStream_t st) {
+                                int grid, int* status, cudaStream_t st) {
     return Dp == 32 ? cover_tc_batch<32>(pmap, mmap, pmap1, mmap1, Mk, mk_rows, frames, states, B, max_pk_rows, modes,
-                                         P32, pix, d, c, covered, tile_off, sc, grid, status, st)
+                                         P32, pix, d, c, covered, tile_off,  grid, status, st)
                     : cover_tc_batch<16>(pmap, mmap, pmap1, mmap1, Mk, mk_rows, frames, states, B, max_pk_rows, modes,
-                                         P32, pix, d, c, covered, tile_off, sc, grid, status, st);
+                                         P32, pix, d, c, covered, tile_off,  grid, status, st);
 }
 
 ms_status launch_cover_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, void* Mk, int64_t n_pad, int Dp,
                                  const float* modes, int k0, int k1, int n, const float* P32, const int32_t* pix,
                                  const float* emb, int d, double c, uint8_t* covered, int* n_uncovered,
-                                 LabelTcScratch sc, int grid, int* status, cudaStream_t st) {
+                                 int grid, int* status, cudaStream_t st) {
     if (n == 0 || k1 <= k0) return MS_OK;
     return Dp == 32 ? cover_tc_single<32>(pmap, pmap1, Mk, n_pad, modes, k0, k1, n, P32, pix, emb, d, c, covered,
-                                          n_uncovered, sc, grid, status, st)
+                                          n_uncovered,  grid, status, st)
                     : cover_tc_single<16>(pmap, pmap1, Mk, n_pad, modes, k0, k1, n, P32, pix, emb, d, c, covered,
-                                          n_uncovered, sc, grid, status, st);
+                                          n_uncovered,  grid, status, st);
 }
 
 ms_status launch_label_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, void* Mk, int64_t n_pad, int Dp,

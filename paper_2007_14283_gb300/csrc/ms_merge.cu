@@ -222,11 +222,10 @@ ms_status merge_prepare_t(ms_ctx* ctx, int32_t k) {
     MS_CUDA(cudaMemsetAsync(ctx->removed_r, 0, (size_t)k, ctx->stream));
     k_rank_invert_xr<Dp><<<g256, 256, 0, ctx->stream>>>(ctx->cand_rank, k, ctx->cand, ctx->X, ctx->rank_cand, ctx->Xr);
     MS_LAUNCH("k_rank_invert_xr");
-    LabelTcScratch sc{ctx->label_fix, (int*)(ctx->label_fix + ctx->n), nullptr};
     const ms_status s = launch_merge_tc_single(ctx->Ck, ctx->Mk, ctx->n_pad, Dp, k, ctx->n_kept, ctx->Xr, ctx->modes,
                                                ctx->rank_cand, ctx->cand_state, ctx->removed_r, ctx->conf_deg,
-                                               ctx->conf, thr_f, thr, sc, ctx->num_sms, &ctx->dc->status, ctx->stream);
-    ctx->launches += 4 + (ctx->n_kept > 0 ? 2 : 0);
+                                               ctx->conf, thr_f, thr, ctx->num_sms, &ctx->dc->status, ctx->stream);
+    ctx->launches += 4 + (ctx->n_kept > 0 ? 1 : 0);
     return s;
 }
 
@@ -300,12 +299,11 @@ ms_status launch_merge_append(ms_ctx* ctx, int32_t k) {
 
 ms_status launch_cover(ms_ctx* ctx, int32_t k0, int32_t k1) {
     if (k1 <= k0 || ctx->n == 0) return MS_OK;
-    LabelTcScratch sc{ctx->label_fix, (int*)(ctx->label_fix + ctx->n), nullptr};
     const ms_status s = launch_cover_tc_single(ctx->pmap, ctx->pmap1, ctx->Mk, ctx->n_pad, ctx->Dp, ctx->modes, k0, k1,
                                                (int)ctx->n, ctx->P32, ctx->pix, ctx->emb, ctx->d,
-                                               ctx->cfg.bandwidth_cos, ctx->covered, &ctx->dc->n_uncovered, sc,
+                                               ctx->cfg.bandwidth_cos, ctx->covered, &ctx->dc->n_uncovered,
                                                ctx->num_sms, &ctx->dc->status, ctx->stream);
-    ctx->launches += 3;
+    ctx->launches += 2;
     return s;
 }
 
