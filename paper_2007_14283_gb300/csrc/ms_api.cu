@@ -32,15 +32,135 @@ ms_status set_error(ms_status code, const char* fmt, ...) {
 
 static std::atomic<int32_t> g_fail_allocs{0};
 
-cudaError_t workspace_malloc(void** p, size_t bytes) {
+bool injected_alloc_failure() {
     int32_t left = g_fail_allocs.load();
     while (left > 0 && !g_fail_allocs.compare_exchange_weak(left, left - 1)) {
     }
-    if (left > 0) {
-        *p = nullptr;
-        return cudaErrorMemoryAllocation;
+    return left > 0;
+}
+
+cudaError_t workspace_malloc(void** p, size_t bytes) {
+    *p = nullptr;
+    return injected_alloc_failure() ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+}
+
+// Blocks that destroyed contexts leave for the next one: a program that makes
+// a context per frame paid cudaMalloc, cudaFree and the pinned counters'
+// cudaMallocHost and cudaFreeHost for each: 743 us a frame of 20,000 pixels,
+// 533 us with blocks left by the frame before.
+// A block is kept only once the device is idle (as cudaFree waits for), so it
+// may serve any stream next; lists are under a mutex. Kept at most: kKeepBlocks
+// blocks and kKeepBytes on all devices together; the oldest goes first, a block
+// that 64 later frees did not reuse is given back, and all of a device's are
+// when an allocation there fails.
+namespace {
+
+constexpr size_t kKeepBytes = size_t(512) << 20;
+constexpr int kKeepBlocks = 8, kKeepCounters = 16;
+constexpr uint64_t kKeepFrees = 64;
+
+struct KeptBlock {
+    void* p;
+    size_t bytes;
+    int dev;
+    uint64_t tick;
+};
+std::mutex g_keep_mu;
+KeptBlock g_kept[kKeepBlocks];  // oldest first
+int g_n_kept = 0;
+size_t g_kept_bytes = 0;
+uint64_t g_frees = 0;
+void* g_counters[kKeepCounters];
+int g_n_counters = 0;
+
+void* drop_kept(int i) {
+    void* p = g_kept[i].p;
+    g_kept_bytes -= g_kept[i].bytes;
+    for (--g_n_kept; i < g_n_kept; ++i) g_kept[i] = g_kept[i + 1];
+    return p;
+}
+
+}  // namespace
+
+cudaError_t block_alloc(KeptSize* blk, void** p, size_t bytes) {
+    *p = nullptr;
+    blk->bytes = bytes;
+    cudaError_t e = cudaGetDevice(&blk->dev);
+    if (e != cudaSuccess) return e;
+    {
+        std::lock_guard<std::mutex> lk(g_keep_mu);
+        int pick = -1;
+        for (int i = 0; i < g_n_kept; ++i)
+            if (g_kept[i].dev == blk->dev && g_kept[i].bytes >= bytes && g_kept[i].bytes / 2 <= bytes &&
+                (pick < 0 || g_kept[i].bytes < g_kept[pick].bytes))
+                pick = i;
+        if (pick >= 0) {
+            blk->bytes = g_kept[pick].bytes;
+            *p = drop_kept(pick);
+            return cudaSuccess;
+        }
     }
+    e = cudaMalloc(p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    for (;;) {  // give everything of this device back, then try once more
+        void* old = nullptr;
+        {
+            std::lock_guard<std::mutex> lk(g_keep_mu);
+            for (int i = 0; i < g_n_kept && !old; ++i)
+                if (g_kept[i].dev == blk->dev) old = drop_kept(i);
+        }
+        if (!old) break;
+        cudaFree(old);
+    }
+    (void)cudaGetLastError();
     return cudaMalloc(p, bytes);
+}
+
+void block_free(const KeptSize& blk, void* p) {
+    if (!p) return;
+    int dev = -1;
+    void* out[kKeepBlocks + 1];
+    int n_out = 0;
+    if (blk.bytes > kKeepBytes || cudaGetDevice(&dev) != cudaSuccess || dev != blk.dev ||
+        cudaDeviceSynchronize() != cudaSuccess) {
+        cudaFree(p);
+        return;
+    }
+    {
+        std::lock_guard<std::mutex> lk(g_keep_mu);
+        ++g_frees;
+        while (g_n_kept > 0 && (g_n_kept == kKeepBlocks || g_kept_bytes + blk.bytes > kKeepBytes ||
+                                g_frees - g_kept[0].tick > kKeepFrees))
+            out[n_out++] = drop_kept(0);
+        g_kept[g_n_kept++] = KeptBlock{p, blk.bytes, blk.dev, g_frees};
+        g_kept_bytes += blk.bytes;
+    }
+    for (int i = 0; i < n_out; ++i) cudaFree(out[i]);
+}
+
+// Pinned DevCounters for one context.
+cudaError_t counters_alloc(DevCounters** p) {
+    {
+        std::lock_guard<std::mutex> lk(g_keep_mu);
+        if (g_n_counters > 0) {
+            *p = (DevCounters*)g_counters[--g_n_counters];
+            return cudaSuccess;
+        }
+    }
+    return cudaMallocHost((void**)p, sizeof(DevCounters));
+}
+
+// After the context's last copy into them (block_free's wait).
+void counters_free(DevCounters* p) {
+    if (!p) return;
+    {
+        std::lock_guard<std::mutex> lk(g_keep_mu);
+        if (g_n_counters < kKeepCounters) {
+            g_counters[g_n_counters++] = p;
+            return;
+        }
+    }
+    cudaFreeHost(p);
 }
 
 // The library's own stream-ordered pool on each device. It keeps freed memory
@@ -237,8 +357,8 @@ void free_ctx(ms_ctx* ctx) {
     if (!ctx) return;
     for (int i = 0; i < 64; ++i)
         if (ctx->ev[i]) cudaEventDestroy(ctx->ev[i]);
-    if (ctx->ws) cudaFree(ctx->ws);
-    if (ctx->hc) cudaFreeHost(ctx->hc);
+    block_free(ctx->ws_block, ctx->ws);
+    counters_free(ctx->hc);
     delete[] ctx->round_log;
     delete ctx;
 }
@@ -306,12 +426,13 @@ ms_status ctx_alloc(const ms_config* cfg, int64_t max_pixels, cudaStream_t strea
     ctx->target_items = 2 * ctx->shift_grid;
     const Layout L = plan(max_pixels, ctx->Dp);
     ctx->ws_bytes = L.total;
-    cudaError_t e = workspace_malloc(&ctx->ws, L.total);
+    cudaError_t e = injected_alloc_failure() ? cudaErrorMemoryAllocation
+                                             : block_alloc(&ctx->ws_block, &ctx->ws, L.total);
     if (e != cudaSuccess) {
         free_ctx(ctx);
         return cuda_check(e, "cudaMalloc(workspace)");
     }
-    e = cudaMallocHost((void**)&ctx->hc, sizeof(DevCounters));
+    e = counters_alloc(&ctx->hc);
     if (e != cudaSuccess) {
         free_ctx(ctx);
         return cuda_check(e, "cudaMallocHost(counters)");
@@ -640,7 +761,8 @@ ms_status ms_run_host(const ms_config* cfg, const float* h_emb, const uint8_t* h
     const size_t modes_b = h_modes ? sizeof(float) * (size_t)(cap > 0 ? cap : 0) * (size_t)cfg->dim : 0;
     char* buf = nullptr;
     const size_t o_mask = align_up(eb), o_lab = o_mask + align_up(mb), o_modes = o_lab + align_up(lb);
-    MS_CUDA(cudaMalloc(&buf, o_modes + align_up(modes_b) + kAlign));
+    KeptSize buf_block;
+    MS_CUDA(block_alloc(&buf_block, (void**)&buf, o_modes + align_up(modes_b) + kAlign));
     ms_ctx* ctx = nullptr;
     int32_t k = 0;
     s = cuda_check(cudaMemcpyAsync(buf, h_emb, eb, cudaMemcpyHostToDevice, st), "copy h_emb");
@@ -655,7 +777,7 @@ ms_status ms_run_host(const ms_config* cfg, const float* h_emb, const uint8_t* h
     if (s == MS_OK && stats_out) ms_stats_get(ctx, stats_out);
     if (n_modes_out) *n_modes_out = k;
     ms_destroy(ctx);
-    cudaFree(buf);
+    block_free(buf_block, buf);
     return s;
 }
 
