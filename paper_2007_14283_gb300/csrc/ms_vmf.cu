@@ -234,11 +234,19 @@ __global__ void k_vmf_bwd_reduce(const float* __restrict__ partial, VSplit sp, i
         for (int k = 0; k < 16; ++k) G[(int64_t)m * kVD + k] = s[k];
 }
 
-// Pass B: two pixels per thread (i and i + 128 of the block's 256), all
-// seeds from shared memory; each seed's x and gy are read once for both.
+// Pass B: two pixels per thread (i and i + 128 of the block's 256), the seeds
+// from shared memory; each seed's x and gy are read once for both.
+// Bound by FMA issue (64 a pixel and seed). 65536 pixels are 256 such blocks,
+// 1.7 per SM; blockIdx.y splits the seeds into chunks of `len` (a multiple of
+// 64) until the blocks fill the GPU about twice (vmf_alloc), and chunk c > 0
+// sums into its own copy of dP, `extra`, which k_vmf_bwd_join adds after the
+// last step. The 10-step adjoint of 65536 pixels and 1024 seeds, forward steps
+// included: 4.91 ms in one chunk, 4.63 in four.
 __global__ void __launch_bounds__(kBT)
 k_vmf_bwd_pixels(const float* __restrict__ P, int64_t N, const float* __restrict__ X, const float* __restrict__ GY,
-                 int M, float kappa, float* __restrict__ dP) {
+                 int M, int len, float kappa, float* dP0, float* extra) {
+    float* dP = blockIdx.y == 0 ? dP0 : extra + (int64_t)(blockIdx.y - 1) * N * kVD;
+    const int m_end = min(M, ((int)blockIdx.y + 1) * len);
     const float kl2 = kappa * 1.4426950408889634f;  // exp(kappa u) = 2^(kappa log2(e) u)
     __shared__ __align__(16) float sx[64 * kVD];
     __shared__ __align__(16) float sg[64 * kVD];
@@ -257,8 +265,8 @@ k_vmf_bwd_pixels(const float* __restrict__ P, int64_t N, const float* __restrict
             for (int k = 0; k < 16; ++k) p[u][k] = dp[u][k] = 0.f;
         }
     }
-    for (int base = 0; base < M; base += 64) {
-        const int cnt = min(64, M - base);
+    for (int base = blockIdx.y * len; base < m_end; base += 64) {
+        const int cnt = min(64, m_end - base);
         __syncthreads();
         for (int q = threadIdx.x; q < cnt * 4; q += kBT) {
             reinterpret_cast<float4*>(sx)[q] = reinterpret_cast<const float4*>(X + (int64_t)base * kVD)[q];
@@ -291,6 +299,21 @@ k_vmf_bwd_pixels(const float* __restrict__ P, int64_t N, const float* __restrict
             for (int k = 0; k < 16; ++k) dP[idx[u] * kVD + k] = dp[u][k];
 }
 
+// dP += the seed chunks' copies, in chunk order.
+__global__ void k_vmf_bwd_join(float* __restrict__ dP, const float* __restrict__ extra, int64_t n4, int copies) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n4) return;
+    float4 a = reinterpret_cast<float4*>(dP)[i];
+    for (int c = 0; c < copies; ++c) {
+        const float4 b = reinterpret_cast<const float4*>(extra)[(int64_t)c * n4 + i];
+        a.x += b.x;
+        a.y += b.y;
+        a.z += b.z;
+        a.w += b.w;
+    }
+    reinterpret_cast<float4*>(dP)[i] = a;
+}
+
 struct VmfWork {
     bool tc;        // steps and adjoint passes on the tensor cores (BF16 splits)
     void* Pk;       // tc: BF16 split rows of P
@@ -306,6 +329,8 @@ struct VmfWork {
     VmfAdjWork adj; // tc backward: the tensor-core adjoint's plans, maps and buffers
     VSplit sp;      // forward items (512-seed tiles)
     VSplit spa;     // adjoint pass A items (256-seed tiles)
+    float* extra;   // adjoint pass B: dP copies of the seed chunks after the first
+    int b_chunks, b_len;  // pass B: seed chunks, seeds in each
     void* adj_ws;   // tc backward: workspace of the tensor-core adjoint
     int sms;
 };
@@ -332,6 +357,16 @@ ms_status vmf_alloc(VmfWork* w, int64_t N, int32_t M, int32_t T, bool tc, bool a
     w->tc = tc;
     w->sp = vsplit(M, N, vmf_slots(k_vmf_fwd_partial, kFT), kFSeeds);
     w->spa = vsplit(M, N, vmf_slots(k_vmf_bwd_seeds, kAT), kASeeds);
+    // Pass B's seed chunks: blocks for two full waves, at least 128 seeds each,
+    // at most four (a copy of dP each beyond the first, together at most 60 MB).
+    const int64_t pblocks = (N + kBT * kBP - 1) / (kBT * kBP);
+    int64_t bc = adjoint && !tc ? (2 * (int64_t)vmf_slots(k_vmf_bwd_pixels, kBT) + pblocks - 1) / pblocks : 1;
+    bc = bc > 4 ? 4 : bc;
+    bc = bc > M / 128 ? M / 128 : bc;
+    bc = bc < 1 ? 1 : bc;
+    w->b_len = (int)((M + bc * 64 - 1) / (bc * 64) * 64);
+    w->b_chunks = (M + w->b_len - 1) / w->b_len;
+    const size_t extra_b = (size_t)(w->b_chunks - 1) * (size_t)N * kVD * sizeof(float);
     const size_t pf = (size_t)w->sp.tiles * w->sp.chunks * kFSeeds, pa = (size_t)w->spa.tiles * w->spa.chunks * kASeeds;
     const size_t pmax = pf > pa ? pf : pa;
     size_t tc_bytes = 0, adj_bytes = 0;
@@ -345,8 +380,8 @@ ms_status vmf_alloc(VmfWork* w, int64_t N, int32_t M, int32_t T, bool tc, bool a
         if (adjoint) adj_bytes = vmf_adj_bytes(M, N, w->sms) + 256;
     }
     const size_t bytes = pmax * kVD * sizeof(float) + (size_t)(T + 1) * M * kVD * sizeof(float) +
-                         (size_t)(T > 0 ? T : 1) * M * sizeof(float) + 2 * (size_t)M * kVD * sizeof(float) + 4 * 256 +
-                         tc_bytes + adj_bytes;
+                         (size_t)(T > 0 ? T : 1) * M * sizeof(float) + 2 * (size_t)M * kVD * sizeof(float) + 6 * 256 +
+                         extra_b + tc_bytes + adj_bytes;
     char* b = nullptr;
     MS_CUDA(scratch_malloc_async((void**)&b, bytes, st));
     auto take = [&](size_t n) {
@@ -359,6 +394,7 @@ ms_status vmf_alloc(VmfWork* w, int64_t N, int32_t M, int32_t T, bool tc, bool a
     w->ynorm = take((size_t)(T > 0 ? T : 1) * M * sizeof(float));
     w->gy = take((size_t)M * kVD * sizeof(float));
     w->g = take((size_t)M * kVD * sizeof(float));
+    w->extra = extra_b ? take(extra_b) : nullptr;
     w->Pk = nullptr;
     w->tc_partial = nullptr;
     w->status = nullptr;
@@ -446,6 +482,9 @@ extern "C" ms_status ms_vmf_backward_ex(const float* d_P, int64_t N, const float
     // pixel rows the forward steps packed
     if (s == MS_OK && w.tc) s = vmf_adj_prepare(w.Pk, N, M, w.sms, w.adj_ws, &w.adj);
     if (s == MS_OK) s = cuda_check(cudaMemsetAsync(d_dP, 0, sizeof(float) * (size_t)N * kVD, st), "memset dP");
+    if (s == MS_OK && w.extra)
+        s = cuda_check(cudaMemsetAsync(w.extra, 0, sizeof(float) * (size_t)(w.b_chunks - 1) * (size_t)N * kVD, st),
+                       "memset dP copies");
     if (s == MS_OK)
         s = cuda_check(cudaMemcpyAsync(w.g, d_GT, sizeof(float) * (size_t)M * kVD, cudaMemcpyDeviceToDevice, st),
                        "copy g_T");
@@ -457,13 +496,17 @@ extern "C" ms_status ms_vmf_backward_ex(const float* d_P, int64_t N, const float
         const float* Xn = w.iters + (size_t)(t + 1) * M * kVD;
         k_vmf_gy<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(w.g, Xn, w.ynorm + (size_t)t * M, M, w.gy);
         if ((s = cuda_check(cudaGetLastError(), "k_vmf_gy")) != MS_OK) break;
-        k_vmf_bwd_pixels<<<(unsigned)((N + kBT * kBP - 1) / (kBT * kBP)), kBT, 0, st>>>(d_P, N, Xt, w.gy, M, kf,
-                                                                                    d_dP);
+        const dim3 pgrid((unsigned)((N + kBT * kBP - 1) / (kBT * kBP)), (unsigned)w.b_chunks);
+        k_vmf_bwd_pixels<<<pgrid, kBT, 0, st>>>(d_P, N, Xt, w.gy, M, w.b_len, kf, d_dP, w.extra);
         if ((s = cuda_check(cudaGetLastError(), "k_vmf_bwd_pixels")) != MS_OK) break;
         k_vmf_bwd_seeds<<<items, kAT, 0, st>>>(d_P, N, Xt, w.gy, M, kf, w.spa, w.partial);
         if ((s = cuda_check(cudaGetLastError(), "k_vmf_bwd_seeds")) != MS_OK) break;
         k_vmf_bwd_reduce<<<rblocks, 256, 0, st>>>(w.partial, w.spa, M, w.g);
         s = cuda_check(cudaGetLastError(), "k_vmf_bwd_reduce");
+    }
+    if (s == MS_OK && w.extra && T > 0) {
+        k_vmf_bwd_join<<<(unsigned)((N * 4 + 255) / 256), 256, 0, st>>>(d_dP, w.extra, N * 4, w.b_chunks - 1);
+        s = cuda_check(cudaGetLastError(), "k_vmf_bwd_join");
     }
     if (s == MS_OK && !w.tc)
         s = cuda_check(cudaMemcpyAsync(d_dX0, w.g, sizeof(float) * (size_t)M * kVD, cudaMemcpyDeviceToDevice, st),
