@@ -198,20 +198,29 @@ cudaError_t scratch_malloc_async(void** p, size_t bytes, cudaStream_t st);
 // A launch that may start before the kernel ahead of it on the stream has
 // ended, from the moment all of that kernel's blocks have called grid_release
 // (or ended). The kernel calls grid_wait before it touches anything that
-// earlier work on the stream writes or reads.
+// earlier work on the stream writes or reads; what that work writes is not read
+// through `const __restrict__` pointers, whose loads may move above the wait.
+// Pays where kernels are short or end in few blocks (the shift loop, the smooth
+// kernel's tensor-core steps: 1650 -> 1515 us for 50021 pixels, 900 seeds, 8 steps);
+// kernels that fill one wave of resident blocks each got slower with it (the FP32
+// smooth kernel's forward 1.12 -> 1.37 ms) and are launched the ordinary way.
+// A kernel that takes TMEM calls grid_release only once it holds it: a later
+// kernel's block that got there first would wait for it forever.
 template <class... P, class... A>
-cudaError_t launch_after(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t st,
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st,
                          const A&... args) {
     cudaLaunchAttribute at = {};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool plain = cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
     cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = plain ? 0 : 1;  // a captured launch keeps its full dependency
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 

@@ -149,7 +149,7 @@ k_shift_fp32(const float* __restrict__ P32, const float* __restrict__ X, unsigne
 // ordinary launches, 14.6 ms now; a 64 x 64 FP32 frame 3.25 and 2.69 ms.
 template <int Dp>
 __global__ void __launch_bounds__(kFinThreads)
-k_finalize(unsigned long long* __restrict__ acc, const int32_t* __restrict__ active_in,
+k_finalize(unsigned long long* __restrict__ acc, const int32_t* active_in,
            int32_t* __restrict__ active_out, float* __restrict__ X, uint8_t* __restrict__ sstate,
            int32_t* __restrict__ support, double tol, StepBand band, uint32_t* __restrict__ moving, DevCounters* dc,
            double gamma, int max_iter) {

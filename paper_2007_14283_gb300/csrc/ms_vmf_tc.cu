@@ -32,7 +32,7 @@
 // MMAs and TMA loads in flight, frees TMEM and sets *status.
 #include <cudaTypedefs.h>
 
-#include "ms_internal.cuh"
+#include "ms_device.cuh"
 #include "ms_tc.cuh"
 
 namespace ms {
@@ -108,7 +108,7 @@ __device__ __forceinline__ bool vwarp_wait(uint64_t* bar, uint32_t parity, volat
 // partial[item][r][k] = sum over the item's pixel chunk of w p_k for seed
 // 128 t + r. k2 = kappa log2(e) (folded into the seed operand).
 __global__ void __launch_bounds__(kVThreads, 1)
-k_vmf_tc(const __grid_constant__ CUtensorMap pmap, const float* __restrict__ X, float k2, VmfTcMap map,
+k_vmf_tc(const __grid_constant__ CUtensorMap pmap, const float* X, float k2, VmfTcMap map,
          float* __restrict__ partial, int* status) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -155,6 +155,8 @@ k_vmf_tc(const __grid_constant__ CUtensorMap pmap, const float* __restrict__ X, 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    grid_release();  // TMEM is held
+    grid_wait();
     const int items = map.items();
 
     if (warp == kVWarpTma) {
@@ -342,8 +344,10 @@ k_vmf_tc(const __grid_constant__ CUtensorMap pmap, const float* __restrict__ X, 
 // x'_m = y_m / |y_m| with y_m the chunks' partial sums added in chunk order;
 // |y_m| kept for the adjoint. Sixteen threads per seed, one per component. A
 // raised status poisons the outputs (NaN).
-__global__ void k_vmf_tc_reduce(const float* __restrict__ partial, VmfTcMap map, const int* __restrict__ status,
-                                float* __restrict__ Xn, float* __restrict__ ynorm) {
+__global__ void k_vmf_tc_reduce(const float* partial, VmfTcMap map, const int* status, float* __restrict__ Xn,
+                                float* __restrict__ ynorm) {
+    grid_wait();
+    grid_release();
     const int gid = blockIdx.x * blockDim.x + threadIdx.x;
     const int m = gid >> 4, k = gid & 15;
     const bool live = m < map.M;
@@ -408,10 +412,8 @@ ms_status vmf_tc_step(const CUtensorMap& map, const float* Xt, int32_t M, float 
     mp.chunks = plan.chunks;
     mp.tpc = plan.tpc;
     const float k2 = (float)((double)kappa * 1.4426950408889634);  // kappa log2(e)
-    k_vmf_tc<<<(unsigned)plan.grid, kVThreads, kVSmemBytes, st>>>(map, Xt, k2, mp, partial, status);
-    MS_LAUNCH("k_vmf_tc");
-    k_vmf_tc_reduce<<<(unsigned)((M * 16 + 255) / 256), 256, 0, st>>>(partial, mp, status, Xn, ynorm);
-    MS_LAUNCH("k_vmf_tc_reduce");
+    MS_CUDA(launch_after(k_vmf_tc, (unsigned)plan.grid, kVThreads, kVSmemBytes, st, map, Xt, k2, mp, partial, status));
+    MS_CUDA(launch_after(k_vmf_tc_reduce, (unsigned)((M * 16 + 255) / 256), 256, 0, st, partial, mp, status, Xn, ynorm));
     return MS_OK;
 }
 

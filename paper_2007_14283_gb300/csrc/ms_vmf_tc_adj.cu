@@ -48,7 +48,7 @@
 // MMAs and TMA loads in flight, frees TMEM and sets *status.
 #include <cudaTypedefs.h>
 
-#include "ms_internal.cuh"
+#include "ms_device.cuh"
 #include "ms_tc.cuh"
 
 namespace ms {
@@ -212,6 +212,8 @@ k_vmf_adj_tc(const __grid_constant__ CUtensorMap rmap0, const __grid_constant__ 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    grid_release();  // TMEM is held
+    grid_wait();
     const int items = map.items;
 
     if (warp == kAdjWarpTma) {
@@ -444,10 +446,12 @@ __global__ void k_vmf_adj_sum(const float* __restrict__ partial, int64_t rows, i
 // exactly; rows >= M are zero (and carry the constant). A raised status
 // poisons g (NaN).
 __global__ void __launch_bounds__(256)
-k_vmf_adj_link(const float* __restrict__ partial, int chunks, const float* __restrict__ g_in,
-               const float* __restrict__ x_s, const float* __restrict__ x_prev, const float* __restrict__ yn_prev,
-               int M, int Mp, float k2, float kappa, const int* __restrict__ status, float* __restrict__ g_out,
-               uint16_t* __restrict__ Vk, uint16_t* __restrict__ Gk, uint16_t* __restrict__ Gak) {
+k_vmf_adj_link(const float* partial, int chunks, const float* g_in, const float* x_s, const float* x_prev,
+               const float* yn_prev, int M, int Mp, float k2, float kappa, const int* status,
+               float* __restrict__ g_out, uint16_t* __restrict__ Vk, uint16_t* __restrict__ Gk,
+               uint16_t* __restrict__ Gak) {
+    grid_wait();
+    grid_release();
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int m = (int)(gid >> 4), k = (int)(gid & 15);
     if (m >= Mp) return;  // never splits a row: Mp is a multiple of 128
@@ -611,19 +615,16 @@ ms_status vmf_adj_backward(VmfAdjWork* w, const float* iters, const float* ynorm
     MS_LAUNCH("k_vmf_adj_link");
     for (int t = T - 1; t >= 0; --t) {
         // pass B: dL/dp over every seed, added to the chunk slots
-        k_vmf_adj_tc<true><<<(unsigned)w->pb.grid, kAdjThreads, kAdjSmemBytes, st>>>(
-            w->pk_rows, w->pk_rows, w->v_cols, w->g_cols, mb, w->partial_b, t < T - 1 ? 1 : 0, status);
-        MS_LAUNCH("k_vmf_adj_tc(pixels)");
+        MS_CUDA(launch_after(k_vmf_adj_tc<true>, (unsigned)w->pb.grid, kAdjThreads, kAdjSmemBytes, st, w->pk_rows,
+                             w->pk_rows, w->v_cols, w->g_cols, mb, w->partial_b, t < T - 1 ? 1 : 0, status));
         // pass A: dL/dx_t over every pixel
-        k_vmf_adj_tc<false><<<(unsigned)w->pa.grid, kAdjThreads, kAdjSmemBytes, st>>>(
-            w->v_rows, w->ga_rows, w->pk_cols, w->pk_cols, ma, w->partial_a, 0, status);
-        MS_LAUNCH("k_vmf_adj_tc(seeds)");
+        MS_CUDA(launch_after(k_vmf_adj_tc<false>, (unsigned)w->pa.grid, kAdjThreads, kAdjSmemBytes, st, w->v_rows,
+                             w->ga_rows, w->pk_cols, w->pk_cols, ma, w->partial_a, 0, status));
         // dL/dx_t; then gy of step t-1 and its operands, or dL/dx_0
-        k_vmf_adj_link<<<lblocks, 256, 0, st>>>(
-            w->partial_a, ma.chunks, nullptr, iters + (size_t)t * MD, t > 0 ? iters + (size_t)(t - 1) * MD : nullptr,
-            t > 0 ? ynorm + (size_t)(t - 1) * w->M : nullptr, w->M, w->Mp, k2, kappa, status, dX0, (uint16_t*)w->Vk,
-            (uint16_t*)w->Gk, (uint16_t*)w->Gak);
-        MS_LAUNCH("k_vmf_adj_link");
+        MS_CUDA(launch_after(k_vmf_adj_link, lblocks, 256, 0, st, w->partial_a, ma.chunks, nullptr,
+                             iters + (size_t)t * MD, t > 0 ? iters + (size_t)(t - 1) * MD : nullptr,
+                             t > 0 ? ynorm + (size_t)(t - 1) * w->M : nullptr, w->M, w->Mp, k2, kappa, status, dX0,
+                             (uint16_t*)w->Vk, (uint16_t*)w->Gk, (uint16_t*)w->Gak));
     }
     k_vmf_adj_sum<<<(unsigned)((w->N * 16 + 255) / 256), 256, 0, st>>>(w->partial_b, w->N, w->pb.chunks, status, dP,
                                                                        0);
