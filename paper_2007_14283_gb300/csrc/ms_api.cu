@@ -652,14 +652,18 @@ ms_status ms_merge_modes(ms_ctx* ctx, int32_t* n_modes_out, int64_t* n_uncovered
     const int32_t k0 = ctx->n_kept;
     ms_status s = launch_collect(ctx);
     if (s == MS_OK) s = launch_merge_prepare(ctx, k);
-    if (s == MS_OK) s = launch_merge_resolve(ctx, k, 8);
-    if (s == MS_OK) s = readback(ctx);
-    for (int extra = 0; s == MS_OK && k > 0 && ctx->hc->undecided > 0 && extra < 7; ++extra) {
-        s = launch_merge_resolve(ctx, k, 8);
+    if (merge_in_one(k)) {
+        if (s == MS_OK) s = launch_merge_one(ctx, k);
+    } else {
+        if (s == MS_OK) s = launch_merge_resolve(ctx, k, 8);
         if (s == MS_OK) s = readback(ctx);
+        for (int extra = 0; s == MS_OK && ctx->hc->undecided > 0 && extra < 7; ++extra) {
+            s = launch_merge_resolve(ctx, k, 8);
+            if (s == MS_OK) s = readback(ctx);
+        }
+        if (s == MS_OK && ctx->hc->undecided > 0) s = launch_merge_sequential(ctx, k);
+        if (s == MS_OK) s = launch_merge_append(ctx, k);
     }
-    if (s == MS_OK && k > 0 && ctx->hc->undecided > 0) s = launch_merge_sequential(ctx, k);
-    if (s == MS_OK) s = launch_merge_append(ctx, k);
     if (s == MS_OK) s = readback(ctx);
     if (s != MS_OK) return s;
     const int32_t k1 = ctx->hc->n_kept;

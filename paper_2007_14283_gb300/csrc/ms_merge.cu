@@ -20,6 +20,7 @@ namespace ms {
 namespace {
 
 constexpr int kMT = 128;  // threads per merge block
+constexpr int kMergeOne = 4096;  // candidates that one block resolves and appends
 constexpr int kVT = 64;   // vectors per shared-memory tile
 
 __global__ void k_collect(const uint8_t* __restrict__ sstate, int m, int32_t* __restrict__ cand,
@@ -85,25 +86,20 @@ __device__ __forceinline__ void load_vec(float* dst, const float* src) {
     }
 }
 
+// What one look at a candidate's conflicts says of it: removed when a kept one
+// is among them, kept when all are removed, else still undecided.
 template <int Dp>
-__global__ void __launch_bounds__(kMT)
-k_merge_resolve(const float* __restrict__ X, const int32_t* __restrict__ cand, int k,
-                const int32_t* __restrict__ cand_rank, const int32_t* __restrict__ rank_cand, uint8_t* cand_state,
-                const int32_t* __restrict__ conf_deg, const int32_t* __restrict__ conf,
-                float thr_f, double thr, DevCounters* dc) {
-    const int a = blockIdx.x * kMT + threadIdx.x;
-    if (a >= k) return;
-    volatile uint8_t* st = cand_state;
-    if (st[a] != kUndecided) return;
+__device__ __forceinline__ uint8_t merge_look(int a, const float* __restrict__ X, const int32_t* __restrict__ cand,
+                                              const int32_t* __restrict__ cand_rank,
+                                              const int32_t* __restrict__ rank_cand, volatile uint8_t* st,
+                                              const int32_t* __restrict__ conf_deg, const int32_t* __restrict__ conf,
+                                              float thr_f, double thr) {
     const int deg = conf_deg[a];
-    bool any_kept = false, all_removed = true;
+    bool all_removed = true;
     if (deg <= kMergeCap) {
         for (int j = 0; j < deg; ++j) {
             const uint8_t s = st[conf[(int64_t)a * kMergeCap + j]];
-            if (s == kKept) {
-                any_kept = true;
-                break;
-            }
+            if (s == kKept) return kRemoved;
             if (s == kUndecided) all_removed = false;
         }
     } else {
@@ -117,17 +113,26 @@ k_merge_resolve(const float* __restrict__ X, const int32_t* __restrict__ cand, i
             const uint8_t s = st[b];
             if (s == kRemoved) continue;
             if (!cos_at_least<Dp>(x, X + (int64_t)cand[b] * Dp, thr_f, thr)) continue;
-            if (s == kKept) {
-                any_kept = true;
-                break;
-            }
+            if (s == kKept) return kRemoved;
             all_removed = false;
         }
     }
-    if (any_kept)
-        st[a] = kRemoved;
-    else if (all_removed)
-        st[a] = kKept;
+    return all_removed ? kKept : kUndecided;
+}
+
+template <int Dp>
+__global__ void __launch_bounds__(kMT)
+k_merge_resolve(const float* __restrict__ X, const int32_t* __restrict__ cand, int k,
+                const int32_t* __restrict__ cand_rank, const int32_t* __restrict__ rank_cand, uint8_t* cand_state,
+                const int32_t* __restrict__ conf_deg, const int32_t* __restrict__ conf,
+                float thr_f, double thr, DevCounters* dc) {
+    const int a = blockIdx.x * kMT + threadIdx.x;
+    if (a >= k) return;
+    volatile uint8_t* st = cand_state;
+    if (st[a] != kUndecided) return;
+    const uint8_t d = merge_look<Dp>(a, X, cand, cand_rank, rank_cand, st, conf_deg, conf, thr_f, thr);
+    if (d != kUndecided)
+        st[a] = d;
     else
         atomicAdd(&dc->undecided, 1);
 }
@@ -154,13 +159,14 @@ __global__ void k_merge_sequential(const float* __restrict__ X, const int32_t* _
     }
 }
 
-// Kept candidates are appended to the mode list in rank order.
+// Kept candidates are appended to the mode list in rank order, by a block of
+// 1024 threads.
 template <int Dp>
-__global__ void __launch_bounds__(1024)
-k_merge_append(const float* __restrict__ X, const int32_t* __restrict__ cand,
-               const int32_t* __restrict__ rank_cand, int k, const uint8_t* __restrict__ cand_state,
-               const int32_t* __restrict__ support, float* __restrict__ modes,
-               int32_t* __restrict__ mode_support, DevCounters* dc) {
+__device__ __forceinline__ void merge_append(const float* __restrict__ X, const int32_t* __restrict__ cand,
+                                             const int32_t* __restrict__ rank_cand, int k,
+                                             const volatile uint8_t* cand_state, const int32_t* __restrict__ support,
+                                             float* __restrict__ modes, int32_t* __restrict__ mode_support,
+                                             DevCounters* dc) {
     __shared__ int32_t warp_excl[32];
     __shared__ int32_t s_total;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -196,6 +202,44 @@ k_merge_append(const float* __restrict__ X, const int32_t* __restrict__ cand,
         __syncthreads();
     }
     if (tid == 0) dc->n_kept = base + carry;
+}
+
+template <int Dp>
+__global__ void __launch_bounds__(1024)
+k_merge_append(const float* __restrict__ X, const int32_t* __restrict__ cand,
+               const int32_t* __restrict__ rank_cand, int k, const uint8_t* __restrict__ cand_state,
+               const int32_t* __restrict__ support, float* __restrict__ modes,
+               int32_t* __restrict__ mode_support, DevCounters* dc) {
+    merge_append<Dp>(X, cand, rank_cand, k, cand_state, support, modes, mode_support, dc);
+}
+
+// The whole resolution and the append in one block, for up to kMergeOne
+// candidates. Sweeps until nothing is undecided: each decides at least the
+// undecided candidate of the lowest rank, so k of them always suffice (two to
+// four do). With eight sweeps in launches of their own, each with its counter's
+// reset, the host's look at the count and the append's launch, a round's merge
+// and coverage took 131 to 158 us for 128 to 2048 candidates; so 89 to 108 us. A
+// block's sweep grows with k / 1024 (139 against 183 us at 4096 candidates, no
+// gain expected at 8192), so larger rounds keep the launches.
+template <int Dp>
+__global__ void __launch_bounds__(1024)
+k_merge_one(const float* __restrict__ X, const int32_t* __restrict__ cand, int k,
+            const int32_t* __restrict__ cand_rank, const int32_t* __restrict__ rank_cand, uint8_t* cand_state,
+            const int32_t* __restrict__ conf_deg, const int32_t* __restrict__ conf, float thr_f, double thr,
+            const int32_t* __restrict__ support, float* __restrict__ modes, int32_t* __restrict__ mode_support,
+            DevCounters* dc) {
+    volatile uint8_t* st = cand_state;
+    for (int sweep = 0; sweep < k; ++sweep) {
+        bool open = false;
+        for (int a = threadIdx.x; a < k; a += 1024) {
+            if (st[a] != kUndecided) continue;
+            const uint8_t d = merge_look<Dp>(a, X, cand, cand_rank, rank_cand, st, conf_deg, conf, thr_f, thr);
+            if (d != kUndecided) st[a] = d;
+            else open = true;
+        }
+        if (!__syncthreads_or(open)) break;
+    }
+    merge_append<Dp>(X, cand, rank_cand, k, st, support, modes, mode_support, dc);
 }
 
 // Slices of an O(outer x inner) loop so that the grid fills about four waves
@@ -278,6 +322,25 @@ ms_status launch_merge_sequential(ms_ctx* ctx, int32_t k) {
         k_merge_sequential<32><<<1, 32, 0, ctx->stream>>>(ctx->X, ctx->cand, k, ctx->rank_cand,
                                                           ctx->cand_state, thr_f, thr);
     MS_LAUNCH("k_merge_sequential");
+    ctx->launches += 1;
+    return MS_OK;
+}
+
+bool merge_in_one(int32_t k) { return k <= kMergeOne; }
+
+ms_status launch_merge_one(ms_ctx* ctx, int32_t k) {
+    if (k <= 0) return MS_OK;
+    const float thr_f = (float)ctx->cfg.merge_cos;
+    const double thr = ctx->cfg.merge_cos;
+    if (ctx->Dp == 16)
+        k_merge_one<16><<<1, 1024, 0, ctx->stream>>>(ctx->X, ctx->cand, k, ctx->cand_rank, ctx->rank_cand,
+                                                     ctx->cand_state, ctx->conf_deg, ctx->conf, thr_f, thr,
+                                                     ctx->support, ctx->modes, ctx->mode_support, ctx->dc);
+    else
+        k_merge_one<32><<<1, 1024, 0, ctx->stream>>>(ctx->X, ctx->cand, k, ctx->cand_rank, ctx->rank_cand,
+                                                     ctx->cand_state, ctx->conf_deg, ctx->conf, thr_f, thr,
+                                                     ctx->support, ctx->modes, ctx->mode_support, ctx->dc);
+    MS_LAUNCH("k_merge_one");
     ctx->launches += 1;
     return MS_OK;
 }
