@@ -21,8 +21,9 @@
 //          is within 1e-6 of x.p. Whether a warp holds such a pair comes with
 //          the second TMEM load (ld.red min.abs), so the mask costs a byte
 //          permute and a logic op per two pixels and nothing else.
-//   GEMM2  Y += Mask . [Ph | Pm | Pl | 1]    (mask exact in BF16; the ones
-//          column yields the window size), 2 tcgen05 MMAs for each 32-pixel
+//   GEMM2  Y += Mask . [Ph | Pm | Pl | 1]    (mask exact in BF16; a ones
+//          column, 0 in the rows that pad the last tile, yields the window
+//          size), 2 tcgen05 MMAs for each 32-pixel
 //          piece that holds a mask, with the lanes (seeds) of pieces without
 //          one disabled. A skipped product would have added zeros, so the
 //          sums are those of the full product, bit for bit.
@@ -608,7 +609,7 @@ k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
                         uint32_t yc[16];
                         tmem_ld16(ty + 48, yc);
                         tmem_ld_wait();
-                        cntf = __uint_as_float(yc[0]);
+                        cntf = __uint_as_float(yc[kCountCol - 48]);
                         live = slot >= 0 && cntf > 0.f;
                     } else {
                         tmem_ld_wait();
@@ -641,11 +642,12 @@ k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
     if (threadIdx.x == 0 && *abort) atomicOr(status, 2);
 }
 
-// Pixels as BF16 splits for the tensor cores: row i = [Ph | Pm | Pl | 1 1 1 0..0]
+// Pixels as BF16 splits for the tensor cores: row i = [Ph | Pm | Pl | 1 1 1 1 0..0]
 // (64 values, 128 bytes) with p = Ph + Pm + Pl; rows from the foreground count
-// n (read on the device) up to `rows` hold only the ones, so they score
-// S' = -c and never enter a window. For D = 32 a second array of `rows` rows
-// follows, holding dimensions 16..31 the same way without the ones.
+// n (read on the device) up to `rows` hold three ones only, so they score
+// S' = -c and add nothing to a window's sums or size (pack_split_row). For
+// D = 32 a second array of `rows` rows follows, holding dimensions 16..31 the
+// same way without the ones.
 __global__ void k_pack_bf16(const float* __restrict__ P32, const DevCounters* __restrict__ dc, int rows, int D,
                             uint4* __restrict__ Pk) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;

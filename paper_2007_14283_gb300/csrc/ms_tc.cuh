@@ -322,11 +322,14 @@ __device__ __forceinline__ float bf16_round(float x) {
 }
 
 // One 128-byte row of a BF16 split operand for a unit vector v (16 FP32
-// components, or nullptr for a padding row): [vh | vm | vl | 1 1 1 0..0], where
+// components, or nullptr for a padding row): [vh | vm | vl | 1 1 1 v 0..0], where
 // vh = RN(v), vm = RN(v - vh), vl = (v - vh) - vm, so v = vh + vm + vl exactly
-// (|v_k| >= 2^-100 or 0). The ones give a -c column against a split constant
-// and the shift's window size in its second GEMM; ones = false leaves them 0
-// (the second half of a 32-dimensional vector's rows).
+// (|v_k| >= 2^-100 or 0), and the fourth one is there for a vector and 0 for a
+// padding row. Three ones give a -c column against a split constant; the fourth
+// (kCountCol) is the window size in the shift's second GEMM, to which a padding
+// row adds nothing even where its score of -c passes for a window's (c < 0).
+// ones = false leaves them 0 (the second half of a 32-dimensional vector's rows).
+constexpr int kCountCol = 51;
 __device__ __forceinline__ void pack_split_row(const float* v, uint4* row, bool ones = true) {
     uint32_t w[32];
 #pragma unroll
@@ -344,7 +347,7 @@ __device__ __forceinline__ void pack_split_row(const float* v, uint4* row, bool 
     }
     if (ones) {
         w[24] = pack_bf16(1.f, 1.f);
-        w[25] = pack_bf16(1.f, 0.f);
+        w[25] = pack_bf16(1.f, v ? 1.f : 0.f);
     }
 #pragma unroll
     for (int c = 0; c < 8; ++c) row[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
