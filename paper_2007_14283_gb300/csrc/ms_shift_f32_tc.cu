@@ -67,12 +67,11 @@ __device__ __forceinline__ void fma2(unsigned long long& y, unsigned long long m
 template <int kD, class Map>
 __global__ void __launch_bounds__(kFThreads, FDim<kD>::kCtas)
 k_shift_f32_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUtensorMap pmap1,
-               const float* __restrict__ X, unsigned long long* __restrict__ acc, float c_f, Map map, int* status) {
+               const float* X, unsigned long long* __restrict__ acc, float c_f, Map map, int* status) {
     using L = FDim<kD>;
     constexpr int kHalves = L::kHalves, kStages = L::kStages, kStageBytes = L::kStageBytes, kSBufs = L::kSBufs;
     constexpr float kBand = kScoreBand<kD>;
     constexpr uint32_t kCols = 128 * kSBufs;
-    grid_release();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* A1 = smem + L::kOffA1;
@@ -110,6 +109,7 @@ k_shift_f32_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    grid_release();  // TMEM is held
     grid_wait();
     const int items = map.init() ? map.total() : 0;
 

@@ -157,8 +157,7 @@ __device__ __forceinline__ uint32_t sign_halves(uint32_t a, uint32_t b) {
 // and of its FP32 seed tile in shared memory, for seed slot `slot` of X
 // (D components; a padding row, slot < 0: zeros), one half at a time.
 template <int D>
-__device__ __forceinline__ void write_seed_rows(uint8_t* A1, float* Xs, int r, const float* __restrict__ X, int slot,
-                                                float c_f) {
+__device__ __forceinline__ void write_seed_rows(uint8_t* A1, float* Xs, int r, const float* X, int slot, float c_f) {
 #pragma unroll
     for (int hf = 0; hf < D / 16; ++hf) {
         float x[16];
@@ -207,7 +206,7 @@ struct TcSingleMap {
 template <class Shape, int kD, bool kDebug, class Map>
 __global__ void __launch_bounds__(Shape::kThreads, 1)
 k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUtensorMap pmap1,
-           const float* __restrict__ X, unsigned long long* __restrict__ acc, float c_f, Map map, int* status,
+           const float* X, unsigned long long* __restrict__ acc, float c_f, Map map, int* status,
            unsigned long long* band_ctr, float* __restrict__ dbg_S, int64_t dbg_stride) {
     using L = TcDim<kD>;
     constexpr int kHalves = L::kHalves, kStages = L::kStages, kStageBytes = L::kStageBytes;
@@ -215,7 +214,6 @@ k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
     constexpr int kPxPerWarp = Shape::kPxPerWarp, kSub = Shape::kSub;
     constexpr float kBand = kScoreBand<kD>;
     constexpr int kWarpTma = Shape::kWarpTma, kWarpG1 = Shape::kWarpG1, kWarpG2 = Shape::kWarpG2;
-    grid_release();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* A1 = smem + L::kOffA1;               // [item buffer][half] 16 KB tiles
@@ -269,6 +267,7 @@ k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    grid_release();  // TMEM is held
 
     if (warp == kWarpTma) {
         // ------------------------------------------------ TMA producer
