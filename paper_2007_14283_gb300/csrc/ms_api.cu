@@ -652,10 +652,14 @@ ms_status ms_merge_modes(ms_ctx* ctx, int32_t* n_modes_out, int64_t* n_uncovered
     const int32_t k0 = ctx->n_kept;
     ms_status s = launch_collect(ctx);
     if (s == MS_OK) s = launch_merge_prepare(ctx, k);
-    if (merge_in_one(k)) {
-        if (s == MS_OK) s = launch_merge_one(ctx, k);
-    } else {
-        if (s == MS_OK) s = launch_merge_resolve(ctx, k, 8);
+    bool open = k > 0;  // the round is not resolved and appended yet
+    if (s == MS_OK && open && merge_in_one(k)) {
+        s = launch_merge_one(ctx, k);
+        if (s == MS_OK) s = readback(ctx);
+        open = s == MS_OK && ctx->hc->undecided > 0;
+    }
+    if (s == MS_OK && open) {
+        s = launch_merge_resolve(ctx, k, 8);
         if (s == MS_OK) s = readback(ctx);
         for (int extra = 0; s == MS_OK && ctx->hc->undecided > 0 && extra < 7; ++extra) {
             s = launch_merge_resolve(ctx, k, 8);
@@ -663,8 +667,8 @@ ms_status ms_merge_modes(ms_ctx* ctx, int32_t* n_modes_out, int64_t* n_uncovered
         }
         if (s == MS_OK && ctx->hc->undecided > 0) s = launch_merge_sequential(ctx, k);
         if (s == MS_OK) s = launch_merge_append(ctx, k);
+        if (s == MS_OK) s = readback(ctx);
     }
-    if (s == MS_OK) s = readback(ctx);
     if (s != MS_OK) return s;
     const int32_t k1 = ctx->hc->n_kept;
     s = launch_cover(ctx, k0, k1);

@@ -232,7 +232,8 @@ float ceil_to_float(double c);  // smallest float >= c
 ms_status launch_merge_prepare(ms_ctx* ctx, int32_t k);     // ms_merge.cu
 ms_status launch_merge_resolve(ms_ctx* ctx, int32_t k, int sweeps);
 ms_status launch_merge_sequential(ms_ctx* ctx, int32_t k);
-bool merge_in_one(int32_t k);  // up to kMergeOne candidates: launch_merge_one resolves and appends
+bool merge_in_one(int32_t k);  // up to kMergeOne candidates
+// Resolves and appends, or (too many conflicts for one block) leaves dc->undecided = k.
 ms_status launch_merge_one(ms_ctx* ctx, int32_t k);
 ms_status launch_merge_append(ms_ctx* ctx, int32_t k);
 ms_status launch_cover(ms_ctx* ctx, int32_t k0, int32_t k1);

@@ -221,6 +221,10 @@ k_merge_append(const float* __restrict__ X, const int32_t* __restrict__ cand,
 // and coverage took 131 to 158 us for 128 to 2048 candidates; so 89 to 108 us. A
 // block's sweep grows with k / 1024 (139 against 183 us at 4096 candidates, no
 // gain expected at 8192), so larger rounds keep the launches.
+// So do rounds with a candidate of more conflicts than are stored: a look at it
+// tests the candidates ranked above it one by one, and one SM for all of them
+// took 9.9 ms for 4096 candidates of four cells, where the launches take 1.0 ms.
+// The block then leaves all of them undecided (dc->undecided = k).
 template <int Dp>
 __global__ void __launch_bounds__(1024)
 k_merge_one(const float* __restrict__ X, const int32_t* __restrict__ cand, int k,
@@ -229,6 +233,11 @@ k_merge_one(const float* __restrict__ X, const int32_t* __restrict__ cand, int k
             const int32_t* __restrict__ support, float* __restrict__ modes, int32_t* __restrict__ mode_support,
             DevCounters* dc) {
     volatile uint8_t* st = cand_state;
+    bool over = false;
+    for (int a = threadIdx.x; a < k; a += 1024) over |= conf_deg[a] > kMergeCap;
+    over = __syncthreads_or(over);
+    if (threadIdx.x == 0) dc->undecided = over ? k : 0;
+    if (over) return;
     for (int sweep = 0; sweep < k; ++sweep) {
         bool open = false;
         for (int a = threadIdx.x; a < k; a += 1024) {

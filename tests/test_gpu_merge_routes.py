@@ -1,0 +1,45 @@
+"""The merge of rounds in which candidates have up to, and more than, the 32
+stored conflicts: one block resolves the former, launches of their own the
+latter (a look at a candidate of more conflicts tests those ranked above it one
+by one). One tight cluster gives its candidate of rank r exactly r conflicts.
+Modes, supports and labels equal the oracle's on both routes; the launch count
+tells which one ran.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _tight(K, per, seed=3):
+    rng = np.random.default_rng(seed)
+    return np.concatenate([synth.sample_vmf(rng, np.eye(16)[k], 5000.0, per) for k in range(K)]).astype(np.float32)
+
+
+def _run(ms_lib, emb, **kw):
+    import torch
+    r = ms_lib.cluster(torch.from_numpy(emb).cuda(), **kw)
+    ref = oracle.run(emb, **{k: v for k, v in kw.items() if k != "precision"})
+    assert np.array_equal(r.stats["support"], ref.support)
+    assert np.array_equal(r.stats["round_log"], ref.round_log)
+    assert np.array_equal(r.labels.cpu().numpy(), ref.labels)
+    assert (1.0 - (r.modes.cpu().numpy() * ref.modes).sum(1)).max() <= 1e-5
+    return r.stats["launches"]
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_route_follows_the_conflicts(ms_lib, precision):
+    emb = _tight(1, 400)
+    launches = {m: _run(ms_lib, emb, precision=precision, n_initial=m, max_rounds=1) for m in (2, 32, 33, 34, 200)}
+    assert launches[2] == launches[32] == launches[33]
+    assert launches[34] == launches[200] >= launches[33] + 8
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("K,per,kw", [(5, 300, dict(n_initial=600)), (3, 1400, dict(all_seeds=1)),
+                                      (12, 33, dict(all_seeds=1)), (12, 34, dict(all_seeds=1))])
+def test_many_conflicts_equal_the_oracle(ms_lib, K, per, kw, precision):
+    _run(ms_lib, _tight(K, per), precision=precision, **kw)
