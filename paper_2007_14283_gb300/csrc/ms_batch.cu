@@ -732,17 +732,18 @@ __global__ void k_b_rank(const BFrame* __restrict__ frames, const BState* __rest
 template <int Dp>
 __global__ void __launch_bounds__(kMT)
 k_b_merge_resolve(const BFrame* __restrict__ frames, BState* states, int B, const int32_t* __restrict__ off,
-                  const float* __restrict__ X, const int32_t* __restrict__ cand,
-                  const int32_t* __restrict__ cand_rank, const int32_t* __restrict__ rank_cand, uint8_t* cand_state,
+                  const float* __restrict__ Xr, const int32_t* __restrict__ rank_cand, uint8_t* cand_state,
                   const int32_t* __restrict__ conf_deg, const int32_t* __restrict__ conf, float thr_f, double thr,
                   int count_left) {
+    // Threads take candidates by rank (merge_look's reason, ms_merge.cu).
     for (int bb = blockIdx.x; bb < off[B]; bb += gridDim.x) {
         const int f = locate(off, B, bb);
         const int lb = bb - off[f];
         const int64_t base = frames[f].pix0;
         const int k = states[f].dc.n_cand;
-        const int a = lb * kMT + threadIdx.x;
-        if (a >= k) continue;
+        const int r = lb * kMT + threadIdx.x;
+        if (r >= k) continue;
+        const int a = rank_cand[base + r];
         volatile uint8_t* st = cand_state + base;
         if (st[a] != kUndecided) continue;
         const int deg = conf_deg[base + a];
@@ -757,13 +758,11 @@ k_b_merge_resolve(const BFrame* __restrict__ frames, BState* states, int B, cons
             // more conflicts than were stored: test the candidates ranked
             // above this one again, in rank order
             float x[Dp];
-            ldv<Dp>(x, X + (int64_t)cand[base + a] * Dp);
-            const int ra = cand_rank[base + a];
-            for (int rb = 0; rb < ra; ++rb) {
-                const int b2 = rank_cand[base + rb];
-                const uint8_t s = st[b2];
+            ldv<Dp>(x, Xr + (base + r) * Dp);
+            for (int rb = 0; rb < r; ++rb) {
+                const uint8_t s = st[rank_cand[base + rb]];
                 if (s == kRemoved) continue;
-                if (!cos_at_least<Dp>(x, X + (int64_t)cand[base + b2] * Dp, thr_f, thr)) continue;
+                if (!cos_at_least<Dp>(x, Xr + (base + rb) * Dp, thr_f, thr)) continue;
                 if (s == kKept) { any_kept = true; break; }
                 all_removed = false;
             }
@@ -996,9 +995,8 @@ ms_status enqueue_round(ms_batch* b, cudaStream_t s, int64_t* nlaunch) {
     if (st != MS_OK) return st;
     nl += 3;
     for (int sw = 0; sw < 8; ++sw) {
-        k_b_merge_resolve<Dp><<<G, kMT, 0, s>>>(b->frames, b->states, B, b->blk_off, b->X, b->cand, b->cand_rank,
-                                                b->rank_cand, b->cand_state, b->conf_deg, b->conf, mf,
-                                                b->cfg.merge_cos, sw == 7);
+        k_b_merge_resolve<Dp><<<G, kMT, 0, s>>>(b->frames, b->states, B, b->blk_off, b->Xr, b->rank_cand,
+                                                b->cand_state, b->conf_deg, b->conf, mf, b->cfg.merge_cos, sw == 7);
         LAUNCHED("k_b_merge_resolve");
     }
     k_b_merge_sequential<Dp><<<B, 32, 0, s>>>(b->frames, b->states, b->X, b->cand, b->rank_cand, b->cand_state, mf,

@@ -43,3 +43,19 @@ def test_route_follows_the_conflicts(ms_lib, precision):
                                       (12, 33, dict(all_seeds=1)), (12, 34, dict(all_seeds=1))])
 def test_many_conflicts_equal_the_oracle(ms_lib, K, per, kw, precision):
     _run(ms_lib, _tight(K, per), precision=precision, **kw)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("n_initial", [16, 33, 34, 600])
+def test_batches_of_many_conflicts_equal_single_frames(ms_lib, n_initial, precision):
+    import torch
+    embs = [torch.from_numpy(_tight(K, per, K)).cuda() for K, per in ((1, 700), (5, 200), (3, 37))]
+    b = ms_lib.ms_batch_create(ms_lib.ms_config_default(precision=precision, n_initial=n_initial), embs, [None] * 3)
+    try:
+        ms_lib.ms_batch_run(b)
+        for f, e in enumerate(embs):
+            r = ms_lib.cluster(e, precision=precision, n_initial=n_initial, frame_id=f)
+            assert np.array_equal(b.labels[f].cpu().numpy(), r.labels.cpu().numpy())
+            assert np.array_equal(ms_lib.ms_batch_modes(b, f), r.modes.cpu().numpy())
+    finally:
+        b.close()
