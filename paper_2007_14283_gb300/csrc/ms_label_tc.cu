@@ -251,8 +251,11 @@ __device__ __noinline__ int better_mode(const float* p, const float* M, const fl
 // merge_cos decides the pair as the exact test does (kEpsTc bounds the split
 // score, 2e-6 the gap between x.m and the FP64 cosine of near-unit FP32
 // vectors); nearer ones take the exact test itself (cos_at_least). kLbOld:
-// a candidate within merge_cos of an earlier mode is removed. kLbPairs: every candidate ranked above the row
-// that is not removed and within merge_cos joins the row's conflict list.
+// a candidate within merge_cos of an earlier mode is removed. kLbPairs: every
+// candidate ranked above the row that is not removed and within merge_cos joins
+// the row's conflict list. A reader stops once the list has overflowed: that
+// conf_deg is above kMergeCap is all the resolution asks of it then, and the
+// atomics of 8 million conflicts took 0.5 ms (4096 candidates of one cell).
 // The exact tests run in the reader's warp, whose S buffer is free again by
 // then, on the columns in doubt alone. Queued rows that a second kernel tested
 // against every mode took 30 us (coverage) and 49 us (merge) a launch.
@@ -431,6 +434,7 @@ k_label_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
             const bool mrow = kMode != kLbLabel && mi < ii.n &&
                               !(kMode == kLbCover ? out.covered : out.removed_r)[mbase + mi];
             int ma = -1;  // the row's candidate index, read when first needed
+            bool full = false;  // kLbPairs: the row's conflict list is over its capacity
             for (int mt = 0; mt < nmt; ++mt, ++g) {
                 const int b = g % kLSBufs;
                 if (!(ok = lwarp_wait(&s_full[b], (g / kLSBufs) & 1, abort))) break;
@@ -494,7 +498,8 @@ k_label_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
                 }
                 if constexpr (kMode == kLbPairs) {
                     const float lo = out.c_f - kDelta, hi = out.c_f + kDelta;
-                    if (__any_sync(0xffffffffu, mrow && m >= lo) && mrow && m >= lo) {
+                    const bool look = mrow && !full && m >= lo;
+                    if (__any_sync(0xffffffffu, look) && look) {
                         uint32_t near = 0, sure = 0;
 #pragma unroll
                         for (int j = 0; j < 32; ++j) {
@@ -521,7 +526,12 @@ k_label_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
                             if (hit) {
                                 if (ma < 0) ma = out.rank_cand[mbase + mi];
                                 const int slot = atomicAdd(&out.conf_deg[mbase + ma], 1);
-                                if (slot < kMergeCap) out.conf[(mbase + ma) * kMergeCap + slot] = out.rank_cand[mbase + col];
+                                if (slot < kMergeCap) {
+                                    out.conf[(mbase + ma) * kMergeCap + slot] = out.rank_cand[mbase + col];
+                                } else {
+                                    full = true;
+                                    break;
+                                }
                             }
                         }
                     }
