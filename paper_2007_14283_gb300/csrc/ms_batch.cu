@@ -97,6 +97,7 @@ using tc::bf16_round;
 using tc::pack_bf16;
 
 constexpr int kIT = 1024;   // ingest / selection threads
+static_assert(kIT == kFewThreads, "k_b_seed ranks few seeds with its whole block");
 constexpr int kMT = 128;    // merge threads
 constexpr int kVT = 64;     // vectors per shared tile
 constexpr int kPT = 256;    // pixel threads (cover, label)
@@ -309,6 +310,7 @@ k_b_seed(const BFrame* __restrict__ frames, BState* states, const float* __restr
     __shared__ int32_t warp_excl[32];
     __shared__ int32_t s_total, s_cut;
     __shared__ int s_go;
+    __shared__ FewSeeds s_few;
     const int f = blockIdx.x;
     const BFrame& fr = frames[f];
     BState& st = states[f];
@@ -328,6 +330,7 @@ k_b_seed(const BFrame* __restrict__ frames, BState* states, const float* __restr
     int64_t wantl = all_seeds ? (int64_t)n : st.N;
     if (wantl > st.dc.n_uncovered) wantl = st.dc.n_uncovered;
     const int32_t want = (int32_t)wantl;
+    const bool few = want <= kFewSeeds;
     const int64_t base = fr.pix0;
     int32_t cursor = st.dc.cursor;
     const int32_t drawn = st.dc.drawn;
@@ -358,7 +361,8 @@ k_b_seed(const BFrame* __restrict__ frames, BState* states, const float* __restr
         const int32_t r = warp_excl[wid] + __popc(bal & ((1u << lane) - 1u));
         if (flag && taken + r < want) {
             covered[base + p] = kTaken;
-            order_of[base + p] = drawn + taken + r;
+            if (few) s_few.pix[taken + r] = p;
+            else order_of[base + p] = drawn + taken + r;
             if (taken + r == want - 1) s_cut = pos + 1;
         }
         __syncthreads();
@@ -371,29 +375,42 @@ k_b_seed(const BFrame* __restrict__ frames, BState* states, const float* __restr
         }
         __syncthreads();
     }
-    // slots in pixel order (ms_seed.cu); each thread looks at kSlotPx pixels
-    int slots = 0;
-    for (int p0 = 0; p0 < n; p0 += kIT * kSlotPx) {
-        const int q0 = p0 + tid * kSlotPx;
-        unsigned took = 0;
+    // slots in pixel order (ms_seed.cu)
+    auto write = [&](int32_t p, int64_t slot, int32_t order) {
+        covered[base + p] = 1;
+        seed_pix[slot] = p;
+        seed_order[slot] = order;
+        act0[slot] = (int32_t)slot;
+        sstate[slot] = kMoving;
+        const float4* src = reinterpret_cast<const float4*>(P32 + (base + p) * Dp);
+        float4* dst = reinterpret_cast<float4*>(X + slot * Dp);
+        for (int k = 0; k < Dp / 4; ++k) dst[k] = src[k];
+    };
+    if (few) {
+        int rank[2];
+        few_ranks(s_few, taken, n, rank);
 #pragma unroll
-        for (int k = 0; k < kSlotPx; ++k)
-            if (q0 + k < n && covered[base + q0 + k] == kTaken) took |= 1u << k;
-        int tot;
-        int64_t slot = base + slots + block_scan(__popc(took), &tot);
-        for (; took; took &= took - 1) {
-            const int p = q0 + __ffs(took) - 1;
-            covered[base + p] = 1;
-            seed_pix[slot] = p;
-            seed_order[slot] = order_of[base + p];
-            act0[slot] = (int32_t)slot;
-            sstate[slot] = kMoving;
-            const float4* src = reinterpret_cast<const float4*>(P32 + (base + p) * Dp);
-            float4* dst = reinterpret_cast<float4*>(X + slot * Dp);
-            for (int k = 0; k < Dp / 4; ++k) dst[k] = src[k];
-            ++slot;
+        for (int k = 0; k < 2; ++k) {
+            const int t = tid + k * kFewThreads;
+            if (t < taken) write(s_few.pix[t], base + rank[k], drawn + t);
         }
-        slots += tot;
+    } else {
+        // each thread looks at kSlotPx pixels
+        int slots = 0;
+        for (int p0 = 0; p0 < n; p0 += kIT * kSlotPx) {
+            const int q0 = p0 + tid * kSlotPx;
+            unsigned took = 0;
+#pragma unroll
+            for (int k = 0; k < kSlotPx; ++k)
+                if (q0 + k < n && covered[base + q0 + k] == kTaken) took |= 1u << k;
+            int tot;
+            int64_t slot = base + slots + block_scan(__popc(took), &tot);
+            for (; took; took &= took - 1) {
+                const int p = q0 + __ffs(took) - 1;
+                write(p, slot++, order_of[base + p]);
+            }
+            slots += tot;
+        }
     }
     if (tid == 0) {
         DevCounters& dc = st.dc;

@@ -13,6 +13,63 @@ __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.la
 // returns at once in a kernel that was launched the ordinary way.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Few seeds of a selection are put in pixel order by the CTA that took them,
+// instead of by a pass over every pixel of the frame (1 ms for a batched frame of
+// 4 million pixels, 80 us for a single one): counted into kFewThreads ranges of
+// pixels, and ranked among those of their own range.
+constexpr int kFewThreads = 1024;
+constexpr int kFewSeeds = 2 * kFewThreads;
+
+struct FewSeeds {
+    int32_t pix[kFewSeeds];   // in draw order
+    int32_t list[kFewSeeds];  // by range, unordered within one
+    int32_t count[kFewThreads];
+    int32_t first[kFewThreads];
+    int32_t warp[32];
+};
+
+// Ranks in pixel order of the frame's n of the pixels pix[tid] and pix[tid +
+// kFewThreads] among pix[0..m), m <= kFewSeeds, all distinct (where there are such
+// two). Every thread of the CTA calls it, with pix written.
+__device__ __forceinline__ void few_ranks(FewSeeds& s, int m, int n, int rank[2]) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int sh = n > kFewThreads ? 32 - __clz((n - 1) / kFewThreads) : 0;  // (n - 1) >> sh < kFewThreads
+    s.count[tid] = 0;
+    __syncthreads();
+    int32_t p[2], at[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int i = tid + k * kFewThreads;
+        p[k] = i < m ? s.pix[i] : -1;
+        if (p[k] >= 0) at[k] = atomicAdd(&s.count[p[k] >> sh], 1);
+    }
+    __syncthreads();
+    const int c = s.count[tid];
+    int incl = c;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) s.warp[wid] = incl;
+    __syncthreads();
+    int before = lane < wid ? s.warp[lane] : 0;
+    for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    s.first[tid] = before + incl - c;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        if (p[k] >= 0) s.list[s.first[p[k] >> sh] + at[k]] = p[k];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        if (p[k] < 0) continue;
+        const int q0 = s.first[p[k] >> sh], q1 = q0 + s.count[p[k] >> sh];
+        int r = q0;
+        for (int q = q0; q < q1; ++q) r += s.list[q] < p[k];
+        rank[k] = r;
+    }
+}
+
 // Sequential FP32 dot product, k = 0..Dp-1, one fused multiply-add per term.
 template <int Dp>
 __device__ __forceinline__ float dot_seq(const float* a, const float* b) {
