@@ -19,6 +19,11 @@
  *  - Device inputs passed to ms_create are BORROWED: the caller keeps them
  *    alive and unchanged until ms_destroy. Every ms_ctx OWNS its workspace,
  *    allocated in ms_create and freed by ms_destroy.
+ *  - What contexts free, up to 512 MB on a GPU, stays in a memory pool of the
+ *    library for later contexts (and up to 16 pinned buffers of a page each).
+ *    The CUDA driver takes unused pool memory back for any allocation of the
+ *    process that would otherwise be out of memory, and the library does so
+ *    before it reports MS_ERR_OOM.
  *  - Work is enqueued on the stream given to ms_create (NULL = legacy default
  *    stream). Calls that return counts synchronise that stream.
  *  - Errors: every call returns an ms_status; the library never aborts,

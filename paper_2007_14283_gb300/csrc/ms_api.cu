@@ -5,7 +5,6 @@
 // drawn from the foreground only); N doubles while N < L*N_min and shrinks by
 // N_min when N > H*N_min. The GPU does all per-pixel and per-seed work; the
 // host reads back a few counters per call.
-#include <atomic>
 #include <stdint.h>
 #include <math.h>
 #include <stdarg.h>
@@ -15,8 +14,6 @@
 #include <new>
 
 #include "ms_internal.cuh"
-
-#include <mutex>
 
 namespace ms {
 
@@ -28,170 +25,6 @@ ms_status set_error(ms_status code, const char* fmt, ...) {
     vsnprintf(g_err, sizeof(g_err), fmt, ap);
     va_end(ap);
     return code;
-}
-
-static std::atomic<int32_t> g_fail_allocs{0};
-
-bool injected_alloc_failure() {
-    int32_t left = g_fail_allocs.load();
-    while (left > 0 && !g_fail_allocs.compare_exchange_weak(left, left - 1)) {
-    }
-    return left > 0;
-}
-
-cudaError_t workspace_malloc(void** p, size_t bytes) {
-    *p = nullptr;
-    return injected_alloc_failure() ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
-}
-
-// Blocks that destroyed contexts leave for the next one: a program that makes
-// a context per frame paid cudaMalloc, cudaFree and the pinned counters'
-// cudaMallocHost and cudaFreeHost for each: 743 us a frame of 20,000 pixels,
-// 533 us with blocks left by the frame before.
-// A block is kept only once the device is idle (as cudaFree waits for), so it
-// may serve any stream next; lists are under a mutex. Kept at most: kKeepBlocks
-// blocks and kKeepBytes on all devices together; the oldest goes first, a block
-// that 64 later frees did not reuse is given back, and all of a device's are
-// when an allocation there fails.
-namespace {
-
-constexpr size_t kKeepBytes = size_t(512) << 20;
-constexpr int kKeepBlocks = 8, kKeepCounters = 16;
-constexpr uint64_t kKeepFrees = 64;
-
-struct KeptBlock {
-    void* p;
-    size_t bytes;
-    int dev;
-    uint64_t tick;
-};
-std::mutex g_keep_mu;
-KeptBlock g_kept[kKeepBlocks];  // oldest first
-int g_n_kept = 0;
-size_t g_kept_bytes = 0;
-uint64_t g_frees = 0;
-void* g_counters[kKeepCounters];
-int g_n_counters = 0;
-
-void* drop_kept(int i) {
-    void* p = g_kept[i].p;
-    g_kept_bytes -= g_kept[i].bytes;
-    for (--g_n_kept; i < g_n_kept; ++i) g_kept[i] = g_kept[i + 1];
-    return p;
-}
-
-}  // namespace
-
-cudaError_t block_alloc(KeptSize* blk, void** p, size_t bytes) {
-    *p = nullptr;
-    blk->bytes = bytes;
-    cudaError_t e = cudaGetDevice(&blk->dev);
-    if (e != cudaSuccess) return e;
-    {
-        std::lock_guard<std::mutex> lk(g_keep_mu);
-        int pick = -1;
-        for (int i = 0; i < g_n_kept; ++i)
-            if (g_kept[i].dev == blk->dev && g_kept[i].bytes >= bytes && g_kept[i].bytes / 2 <= bytes &&
-                (pick < 0 || g_kept[i].bytes < g_kept[pick].bytes))
-                pick = i;
-        if (pick >= 0) {
-            blk->bytes = g_kept[pick].bytes;
-            *p = drop_kept(pick);
-            return cudaSuccess;
-        }
-    }
-    e = cudaMalloc(p, bytes);
-    if (e != cudaErrorMemoryAllocation) return e;
-    for (;;) {  // give everything of this device back, then try once more
-        void* old = nullptr;
-        {
-            std::lock_guard<std::mutex> lk(g_keep_mu);
-            for (int i = 0; i < g_n_kept && !old; ++i)
-                if (g_kept[i].dev == blk->dev) old = drop_kept(i);
-        }
-        if (!old) break;
-        cudaFree(old);
-    }
-    (void)cudaGetLastError();
-    return cudaMalloc(p, bytes);
-}
-
-void block_free(const KeptSize& blk, void* p) {
-    if (!p) return;
-    int dev = -1;
-    void* out[kKeepBlocks + 1];
-    int n_out = 0;
-    if (blk.bytes > kKeepBytes || cudaGetDevice(&dev) != cudaSuccess || dev != blk.dev ||
-        cudaDeviceSynchronize() != cudaSuccess) {
-        cudaFree(p);
-        return;
-    }
-    {
-        std::lock_guard<std::mutex> lk(g_keep_mu);
-        ++g_frees;
-        while (g_n_kept > 0 && (g_n_kept == kKeepBlocks || g_kept_bytes + blk.bytes > kKeepBytes ||
-                                g_frees - g_kept[0].tick > kKeepFrees))
-            out[n_out++] = drop_kept(0);
-        g_kept[g_n_kept++] = KeptBlock{p, blk.bytes, blk.dev, g_frees};
-        g_kept_bytes += blk.bytes;
-    }
-    for (int i = 0; i < n_out; ++i) cudaFree(out[i]);
-}
-
-// Pinned DevCounters for one context.
-cudaError_t counters_alloc(DevCounters** p) {
-    {
-        std::lock_guard<std::mutex> lk(g_keep_mu);
-        if (g_n_counters > 0) {
-            *p = (DevCounters*)g_counters[--g_n_counters];
-            return cudaSuccess;
-        }
-    }
-    return cudaMallocHost((void**)p, sizeof(DevCounters));
-}
-
-// After the context's last copy into them (block_free's wait).
-void counters_free(DevCounters* p) {
-    if (!p) return;
-    {
-        std::lock_guard<std::mutex> lk(g_keep_mu);
-        if (g_n_counters < kKeepCounters) {
-            g_counters[g_n_counters++] = p;
-            return;
-        }
-    }
-    cudaFreeHost(p);
-}
-
-// The library's own stream-ordered pool on each device. It keeps freed memory
-// mapped (release threshold: never), so calls that allocate a workspace per
-// call and synchronise do not re-map it each time; the process's default
-// pool is left as the caller configured it.
-cudaError_t scratch_malloc_async(void** p, size_t bytes, cudaStream_t st) {
-    static std::mutex mu;
-    static cudaMemPool_t pools[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaMallocAsync(p, bytes, st);
-    cudaMemPool_t pool;
-    {
-        std::lock_guard<std::mutex> lk(mu);
-        if (!pools[dev]) {
-            cudaMemPoolProps props = {};
-            props.allocType = cudaMemAllocationTypePinned;
-            props.location.type = cudaMemLocationTypeDevice;
-            props.location.id = dev;
-            if ((e = cudaMemPoolCreate(&pools[dev], &props)) != cudaSuccess) {
-                pools[dev] = nullptr;
-                return e;
-            }
-            uint64_t keep = UINT64_MAX;
-            cudaMemPoolSetAttribute(pools[dev], cudaMemPoolAttrReleaseThreshold, &keep);
-        }
-        pool = pools[dev];
-    }
-    return cudaMallocFromPoolAsync(p, bytes, pool, st);
 }
 
 ms_status cuda_check(cudaError_t e, const char* what) {
@@ -357,7 +190,8 @@ void free_ctx(ms_ctx* ctx) {
     if (!ctx) return;
     for (int i = 0; i < 64; ++i)
         if (ctx->ev[i]) cudaEventDestroy(ctx->ev[i]);
-    block_free(ctx->ws_block, ctx->ws);
+    cudaStreamSynchronize(ctx->stream);
+    block_free(ctx->ws);
     counters_free(ctx->hc);
     delete[] ctx->round_log;
     delete ctx;
@@ -367,8 +201,6 @@ void free_ctx(ms_ctx* ctx) {
 }  // namespace ms
 
 using namespace ms;
-
-extern "C" void ms_inject_alloc_failure(int32_t count) { g_fail_allocs.store(count > 0 ? count : 0); }
 
 extern "C" {
 
@@ -426,13 +258,12 @@ ms_status ctx_alloc(const ms_config* cfg, int64_t max_pixels, cudaStream_t strea
     ctx->target_items = 2 * ctx->shift_grid;
     const Layout L = plan(max_pixels, ctx->Dp);
     ctx->ws_bytes = L.total;
-    cudaError_t e = injected_alloc_failure() ? cudaErrorMemoryAllocation
-                                             : block_alloc(&ctx->ws_block, &ctx->ws, L.total);
+    cudaError_t e = injected_alloc_failure() ? cudaErrorMemoryAllocation : block_alloc(&ctx->ws, L.total, stream);
     if (e != cudaSuccess) {
         free_ctx(ctx);
         return cuda_check(e, "cudaMalloc(workspace)");
     }
-    e = counters_alloc(&ctx->hc);
+    e = counters_alloc(&ctx->hc, sizeof(DevCounters));
     if (e != cudaSuccess) {
         free_ctx(ctx);
         return cuda_check(e, "cudaMallocHost(counters)");
@@ -714,8 +545,6 @@ ms_status ms_label(ms_ctx* ctx, int32_t* d_labels_out, float* d_modes_out, int32
 }
 
 void ms_destroy(ms_ctx* ctx) {
-    if (!ctx) return;
-    cudaStreamSynchronize(ctx->stream);
     free_ctx(ctx);
 }
 
@@ -769,8 +598,7 @@ ms_status ms_run_host(const ms_config* cfg, const float* h_emb, const uint8_t* h
     const size_t modes_b = h_modes ? sizeof(float) * (size_t)(cap > 0 ? cap : 0) * (size_t)cfg->dim : 0;
     char* buf = nullptr;
     const size_t o_mask = align_up(eb), o_lab = o_mask + align_up(mb), o_modes = o_lab + align_up(lb);
-    KeptSize buf_block;
-    MS_CUDA(block_alloc(&buf_block, (void**)&buf, o_modes + align_up(modes_b) + kAlign));
+    MS_CUDA(block_alloc((void**)&buf, o_modes + align_up(modes_b) + kAlign, st));
     ms_ctx* ctx = nullptr;
     int32_t k = 0;
     s = cuda_check(cudaMemcpyAsync(buf, h_emb, eb, cudaMemcpyHostToDevice, st), "copy h_emb");
@@ -785,7 +613,8 @@ ms_status ms_run_host(const ms_config* cfg, const float* h_emb, const uint8_t* h
     if (s == MS_OK && stats_out) ms_stats_get(ctx, stats_out);
     if (n_modes_out) *n_modes_out = k;
     ms_destroy(ctx);
-    block_free(buf_block, buf);
+    cudaStreamSynchronize(st);
+    block_free(buf);
     return s;
 }
 
@@ -881,7 +710,7 @@ extern "C" ms_status ms_tc_selftest(const float* d_X, const float* d_P, int32_t 
     memset(&dc0, 0, sizeof(dc0));
     dc0.n_active = 128;
     dc0.m_round = 128;
-    s = cuda_check(cudaMalloc(&dbg, sizeof(float) * 128 * n_pad), "cudaMalloc");
+    s = cuda_check(device_malloc((void**)&dbg, sizeof(float) * 128 * n_pad), "cudaMalloc");
     if (s == MS_OK) s = cuda_check(cudaMemset(dbg, 0, sizeof(float) * 128 * n_pad), "cudaMemset");
     if (s == MS_OK) s = cuda_check(cudaMemcpy(ctx->X, d_X, sizeof(float) * 128 * 16, cudaMemcpyDeviceToDevice), "copy X");
     if (s == MS_OK) s = cuda_check(cudaMemcpy(ctx->active[0], iota, sizeof(iota), cudaMemcpyHostToDevice), "copy active");

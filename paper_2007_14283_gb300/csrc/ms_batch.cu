@@ -1303,7 +1303,7 @@ extern "C" ms_status ms_batch_create(const ms_config* cfg, int32_t B, const floa
         offs[i] = tot;
         tot += (sizes[i] + 255) / 256 * 256;
     }
-    cudaError_t e = workspace_malloc(&b->ws, tot);
+    const cudaError_t e = injected_alloc_failure() ? cudaErrorMemoryAllocation : device_malloc(&b->ws, tot);
     if (e != cudaSuccess) {
         free_batch(b);
         return cuda_check(e, "cudaMalloc(batch workspace)");

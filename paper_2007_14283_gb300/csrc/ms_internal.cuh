@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "../../include/ms.h"
+#include "ms_blocks.cuh"
 
 namespace ms {
 
@@ -62,12 +63,6 @@ struct DevCounters {
     int64_t band_pairs;  // BF16 form: pairs rechecked in FP32
 };
 
-// A workspace block's size (at least what was asked for) and device.
-struct KeptSize {
-    size_t bytes;
-    int dev;
-};
-
 // Active seeds per finalize block, four lanes each: one warp for each of an
 // SM's FP64 pipes, so that few seeds spread over many SMs. (256 seeds a block
 // took 6 us for 256 seeds.)
@@ -112,7 +107,6 @@ struct ms_ctx {
     int shift_grid;     // persistent grid of the shift kernel
     int target_items;   // work items per shift iteration
     // workspace (one allocation)
-    ms::KeptSize ws_block;   // the workspace block's size and device
     void* ws;
     size_t ws_bytes;
     float* P32;          // [n_pixels, Dp] normalised foreground
@@ -173,17 +167,6 @@ namespace ms {
 // Error plumbing (ms_api.cu).
 ms_status set_error(ms_status code, const char* fmt, ...);
 ms_status cuda_check(cudaError_t e, const char* what);
-// cudaMalloc of a context's or batch's workspace, failing first when a test
-// asked for it through ms_inject_alloc_failure (ms_api.cu).
-cudaError_t workspace_malloc(void** p, size_t bytes);
-// True when a test asked for the next workspace allocation to fail.
-bool injected_alloc_failure();
-// Device memory from the blocks that freed contexts left, else cudaMalloc, and
-// its return: to that list once the device is idle, else cudaFree.
-cudaError_t block_alloc(KeptSize* blk, void** p, size_t bytes);
-void block_free(const KeptSize& blk, void* p);
-// Stream-ordered scratch from the library's own pool (kept mapped between calls); free with cudaFreeAsync.
-cudaError_t scratch_malloc_async(void** p, size_t bytes, cudaStream_t st);
 #define MS_CUDA(call)                                                 \
     do {                                                              \
         ms_status _s = ::ms::cuda_check((call), #call);               \

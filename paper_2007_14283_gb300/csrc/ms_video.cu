@@ -62,7 +62,9 @@ extern "C" ms_status ms_video_create(const ms_config* cfg, int64_t max_pixels, v
     s = cuda_check(cudaStreamCreateWithFlags(&v->side, cudaStreamNonBlocking), "cudaStreamCreate");
     for (int i = 0; i < 2 && s == MS_OK; ++i) {
         s = cuda_check(cudaEventCreateWithFlags(&v->freed[i], cudaEventDisableTiming), "cudaEventCreate");
-        if (s == MS_OK) s = ctx_alloc(cfg, max_pixels, v->stream, &v->ctx[i]);
+        // allocated on the stream of its first use, a bind; later work waits for binds
+        if (s == MS_OK) s = ctx_alloc(cfg, max_pixels, v->side, &v->ctx[i]);
+        if (s == MS_OK) v->ctx[i]->stream = v->stream;
     }
     if (s != MS_OK) {
         video_free(v);
