@@ -181,19 +181,15 @@ k_shift_f32_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__
             const TcItem ni = map.item(item);
             const int pos = ni.seed0 + r;
             slot_n = pos < ni.n_active ? ni.active[pos] : -1;
+            float x[kD];
+            load_seed_row<kD>(X, slot_n, x);
 #pragma unroll
-            for (int hf = 0; hf < kHalves; ++hf) {
-                float x[16];
+            for (int k = 0; k < kD; k += 4)
+                *reinterpret_cast<float4*>(Xs + (n & 1) * 128 * kD + k) =
+                    make_float4(x[k], x[k + 1], x[k + 2], x[k + 3]);
 #pragma unroll
-                for (int k = 0; k < 16; k += 4) {
-                    const float4 v = slot_n >= 0
-                                         ? *reinterpret_cast<const float4*>(X + (int64_t)slot_n * kD + 16 * hf + k)
-                                         : make_float4(0.f, 0.f, 0.f, 0.f);
-                    x[k] = v.x; x[k + 1] = v.y; x[k + 2] = v.z; x[k + 3] = v.w;
-                    *reinterpret_cast<float4*>(Xs + (n & 1) * 128 * kD + 16 * hf + k) = v;
-                }
-                write_a1_half(A1 + ((n & 1) * kHalves + hf) * kTileBytes, r, x, c_f, hf == 0);
-            }
+            for (int hf = 0; hf < kHalves; ++hf)
+                write_a1_half(A1 + ((n & 1) * kHalves + hf) * kTileBytes, r, x + 16 * hf, c_f, hf == 0);
             fence_proxy_async();
             __syncwarp();
             if (lane == 0) {

@@ -155,21 +155,16 @@ __device__ __forceinline__ uint32_t sign_halves(uint32_t a, uint32_t b) {
 
 // Row r of an item's seed operand (one 16 KB tile per 16-dimensional half)
 // and of its FP32 seed tile in shared memory, for seed slot `slot` of X
-// (D components; a padding row, slot < 0: zeros), one half at a time.
+// (D components; a padding row, slot < 0: zeros).
 template <int D>
 __device__ __forceinline__ void write_seed_rows(uint8_t* A1, float* Xs, int r, const float* X, int slot, float c_f) {
+    float x[D];
+    load_seed_row<D>(X, slot, x);
 #pragma unroll
-    for (int hf = 0; hf < D / 16; ++hf) {
-        float x[16];
+    for (int k = 0; k < D; k += 4)
+        *reinterpret_cast<float4*>(Xs + r * D + k) = make_float4(x[k], x[k + 1], x[k + 2], x[k + 3]);
 #pragma unroll
-        for (int k = 0; k < 16; k += 4) {
-            const float4 v = slot >= 0 ? *reinterpret_cast<const float4*>(X + (int64_t)slot * D + 16 * hf + k)
-                                       : make_float4(0.f, 0.f, 0.f, 0.f);
-            x[k] = v.x; x[k + 1] = v.y; x[k + 2] = v.z; x[k + 3] = v.w;
-            *reinterpret_cast<float4*>(Xs + r * D + 16 * hf + k) = v;
-        }
-        write_a1_half(A1 + hf * kTileBytes, r, x, c_f, hf == 0);
-    }
+    for (int hf = 0; hf < D / 16; ++hf) write_a1_half(A1 + hf * kTileBytes, r, x + 16 * hf, c_f, hf == 0);
 }
 
 // Work items of one frame: seed tiles of 128 x chunks of 128-pixel tiles.

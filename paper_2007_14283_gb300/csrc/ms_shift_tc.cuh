@@ -27,6 +27,19 @@ __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
         if (clock64() - t0 > kWaitCycles) return;
 }
 
+// Seed `slot` of X (D components; slot < 0: zeros). X is written by the kernel
+// ahead, so its pointer promises nothing: all loads come before whatever the caller
+// stores, or each would wait for the one before it (1.2 us a launch).
+template <int D>
+__device__ __forceinline__ void load_seed_row(const float* X, int slot, float (&x)[D]) {
+#pragma unroll
+    for (int k = 0; k < D; k += 4) {
+        const float4 v = slot >= 0 ? *reinterpret_cast<const float4*>(X + (int64_t)slot * D + k)
+                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+        x[k] = v.x; x[k + 1] = v.y; x[k + 2] = v.z; x[k + 3] = v.w;
+    }
+}
+
 // Row r of one 16-dimensional half of a seed operand tile:
 // [Xh | Xl | -c split, 0 | unused] for the first half, [Xh | Xl | unused] for
 // the second (the -c column is added once), 128-byte swizzle.
