@@ -123,9 +123,8 @@ ms_status validate(const ms_config* c) {
 constexpr size_t kAlign = 256;
 
 struct Layout {
-    size_t off[29];
+    size_t off[24];
     size_t total;
-
 };
 
 size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
@@ -133,39 +132,39 @@ size_t align_up(size_t v) { return (v + kAlign - 1) / kAlign * kAlign; }
 Layout plan(int64_t np, int Dp) {
     Layout L;
     const size_t n = (size_t)(np > 0 ? np : 1);
+    const size_t split = (n + 127) / 128 * 128 * 128 * (Dp / 16);  // BF16 split rows, one array per 16 dimensions
+    const size_t acc = n * (Dp + 1) * sizeof(unsigned long long);
     const size_t sizes[] = {
         n * Dp * sizeof(float),           // 0 P32
         n * sizeof(int32_t),              // 1 pix
         n,                                // 2 covered
-        n * Dp * sizeof(float),           // 3 X
-        n * sizeof(int32_t),              // 4 seed_pix
-        n * sizeof(int32_t),              // 5 seed_order
-        n,                                // 6 sstate
-        n * sizeof(int32_t),              // 7 support
-        n * sizeof(int32_t),              // 8 active0
-        n * sizeof(int32_t),              // 9 active1
-        n * sizeof(int32_t),              // 10 seed_log
-        n * (Dp + 1) * sizeof(unsigned long long),  // 11 acc
-        n * Dp * sizeof(float),           // 12 modes
-        n * sizeof(int32_t),              // 13 mode_support
-        n * sizeof(int32_t),              // 14 cand
-        n * sizeof(int32_t),              // 15 cand_rank
-        n * sizeof(int32_t),              // 16 rank_cand
-        n,                                // 17 cand_state
-        n * sizeof(int32_t),              // 18 conf_deg
-        n * kMergeCap * sizeof(int32_t),  // 19 conf
-        ((n + 1023) / 1024 + 1) * sizeof(int32_t),  // 20 block_tmp
-        sizeof(DevCounters),              // 21 dc
-        (n + 127) / 128 * 128 * 128 * (Dp / 16),  // 22 Pk (one array per 16 dimensions)
-        (n + 127) / 128 * 128 * 128 * (Dp / 16),  // 23 Mk (labelling on the tensor cores)
-        n * sizeof(int2) + 16,                     // 24 label_fix + count
-        n * Dp * sizeof(float),                    // 25 Xr (merge candidates in rank order)
-        n,                                         // 26 removed_r
-        (n + 127) / 128 * 128 * 128 * (Dp / 16),  // 27 Ck (their BF16 split rows)
-        (n + kFinSeeds - 1) / kFinSeeds * sizeof(uint32_t),  // 28 moving
+        n * Dp * sizeof(float),           // 3 X | label_fix + count
+        n * sizeof(int32_t),              // 4 seed_order
+        n,                                // 5 sstate
+        n * sizeof(int32_t),              // 6 support
+        n * sizeof(int32_t),              // 7 active0
+        n * sizeof(int32_t),              // 8 active1
+        n * sizeof(int32_t),              // 9 seed_log
+        acc > split ? acc : split,        // 10 acc | Ck | Mk
+        n * Dp * sizeof(float),           // 11 modes | Xr
+        n * sizeof(int32_t),              // 12 mode_support
+        n * sizeof(int32_t),              // 13 cand
+        n * sizeof(int32_t),              // 14 cand_rank
+        n * sizeof(int32_t),              // 15 rank_cand
+        n,                                // 16 cand_state
+        n * sizeof(int32_t),              // 17 conf_deg
+        split,                            // 18 Pk | modes of earlier rounds | conf
+        ((n + 1023) / 1024 + 1) * sizeof(int32_t),  // 19 block_tmp
+        sizeof(DevCounters),              // 20 dc
+        n,                                // 21 removed_r
+        (n + kFinSeeds - 1) / kFinSeeds * sizeof(uint32_t),  // 22 moving
     };
+    static_assert(kMergeCap * sizeof(int32_t) == 128, "a conflict list takes a row of Pk");
+    static_assert(16 * sizeof(float) >= sizeof(int2) + 16, "X holds the near-tie queue and its count");
+    constexpr int kArrays = sizeof(sizes) / sizeof(sizes[0]);
+    static_assert(kArrays <= sizeof(L.off) / sizeof(L.off[0]), "offsets");
     size_t t = 0;
-    for (int i = 0; i < 29; ++i) {
+    for (int i = 0; i < kArrays; ++i) {
         L.off[i] = t;
         t += align_up(sizes[i]);
     }
@@ -273,31 +272,29 @@ ms_status ctx_alloc(const ms_config* cfg, int64_t max_pixels, cudaStream_t strea
     ctx->pix = (int32_t*)(b + L.off[1]);
     ctx->covered = (uint8_t*)(b + L.off[2]);
     ctx->X = (float*)(b + L.off[3]);
-    ctx->seed_pix = (int32_t*)(b + L.off[4]);
-    ctx->seed_order = (int32_t*)(b + L.off[5]);
-    ctx->sstate = (uint8_t*)(b + L.off[6]);
-    ctx->support = (int32_t*)(b + L.off[7]);
-    ctx->active[0] = (int32_t*)(b + L.off[8]);
-    ctx->active[1] = (int32_t*)(b + L.off[9]);
-    ctx->seed_log = (int32_t*)(b + L.off[10]);
-    ctx->acc = (unsigned long long*)(b + L.off[11]);
-    ctx->modes = (float*)(b + L.off[12]);
-    ctx->mode_support = (int32_t*)(b + L.off[13]);
-    ctx->cand = (int32_t*)(b + L.off[14]);
-    ctx->cand_rank = (int32_t*)(b + L.off[15]);
-    ctx->rank_cand = (int32_t*)(b + L.off[16]);
-    ctx->cand_state = (uint8_t*)(b + L.off[17]);
-    ctx->conf_deg = (int32_t*)(b + L.off[18]);
-    ctx->conf = (int32_t*)(b + L.off[19]);
-    ctx->block_tmp = (int32_t*)(b + L.off[20]);
-    ctx->dc = (DevCounters*)(b + L.off[21]);
-    ctx->Pk = (void*)(b + L.off[22]);
-    ctx->Mk = (void*)(b + L.off[23]);
-    ctx->label_fix = (int2*)(b + L.off[24]);
-    ctx->Xr = (float*)(b + L.off[25]);
-    ctx->removed_r = (uint8_t*)(b + L.off[26]);
-    ctx->Ck = (void*)(b + L.off[27]);
-    ctx->moving = (uint32_t*)(b + L.off[28]);
+    ctx->label_fix = (int2*)(b + L.off[3]);
+    ctx->seed_order = (int32_t*)(b + L.off[4]);
+    ctx->sstate = (uint8_t*)(b + L.off[5]);
+    ctx->support = (int32_t*)(b + L.off[6]);
+    ctx->active[0] = (int32_t*)(b + L.off[7]);
+    ctx->active[1] = (int32_t*)(b + L.off[8]);
+    ctx->seed_log = (int32_t*)(b + L.off[9]);
+    ctx->acc = (unsigned long long*)(b + L.off[10]);
+    ctx->Ck = (void*)(b + L.off[10]);
+    ctx->Mk = (void*)(b + L.off[10]);
+    ctx->modes = (float*)(b + L.off[11]);
+    ctx->mode_support = (int32_t*)(b + L.off[12]);
+    ctx->cand = (int32_t*)(b + L.off[13]);
+    ctx->cand_rank = (int32_t*)(b + L.off[14]);
+    ctx->rank_cand = (int32_t*)(b + L.off[15]);
+    ctx->cand_state = (uint8_t*)(b + L.off[16]);
+    ctx->conf_deg = (int32_t*)(b + L.off[17]);
+    ctx->Pk = (void*)(b + L.off[18]);
+    ctx->conf = (int32_t*)(b + L.off[18]);
+    ctx->block_tmp = (int32_t*)(b + L.off[19]);
+    ctx->dc = (DevCounters*)(b + L.off[20]);
+    ctx->removed_r = (uint8_t*)(b + L.off[21]);
+    ctx->moving = (uint32_t*)(b + L.off[22]);
     ctx->round_log_cap = 64;
     ctx->round_log = new (std::nothrow) int64_t[ctx->round_log_cap * 4];
     if (!ctx->round_log) {
@@ -319,7 +316,6 @@ ms_status ctx_bind_async(ms_ctx* ctx, const float* d_emb, const uint8_t* d_mask,
     const size_t nn = (size_t)(n_pixels > 0 ? n_pixels : 1);
     MS_CUDA(cudaMemsetAsync(ctx->covered, 0, nn, st));
     MS_CUDA(cudaMemsetAsync(ctx->dc, 0, sizeof(DevCounters), st));
-    MS_CUDA(cudaMemsetAsync(ctx->acc, 0, sizeof(unsigned long long) * (size_t)(ctx->Dp + 1) * nn, st));
     const cudaStream_t keep = ctx->stream;
     ctx->stream = st;
     ms_status s = launch_ingest(ctx);
@@ -502,7 +498,7 @@ ms_status ms_merge_modes(ms_ctx* ctx, int32_t* n_modes_out, int64_t* n_uncovered
     }
     if (s != MS_OK) return s;
     const int32_t k1 = ctx->hc->n_kept;
-    s = launch_cover(ctx, k0, k1);
+    s = launch_cover(ctx, k, k0, k1);
     if (s == MS_OK) s = readback(ctx);
     if (s != MS_OK) return s;
     ctx->n_kept = k1;
@@ -699,9 +695,15 @@ extern "C" ms_status ms_tc_selftest(const float* d_X, const float* d_P, int32_t 
     ms_config_default(&cfg);
     cfg.precision = MS_BF16;
     cfg.bandwidth_cos = c;
-    ms_ctx* ctx = nullptr;
-    ms_status s = ms_create(&cfg, d_P, nullptr, n_pix, nullptr, &ctx);
-    if (s != MS_OK) return s;
+    ms_status s = validate(&cfg);
+    ms_ctx* ctx = nullptr;  // room for the 128 seeds, however few the pixels
+    if (s == MS_OK) s = ctx_alloc(&cfg, n_pix < 128 ? 128 : n_pix, nullptr, &ctx);
+    if (s == MS_OK) s = ctx_bind_async(ctx, d_P, nullptr, n_pix, nullptr);
+    if (s == MS_OK) s = ctx_bind_finish(ctx, nullptr, cfg.frame_id, cfg.n_initial);
+    if (s != MS_OK) {
+        free_ctx(ctx);
+        return s;
+    }
     float* dbg = nullptr;
     const size_t n_pad = (size_t)ctx->n_pad;
     int32_t iota[128];
@@ -715,6 +717,7 @@ extern "C" ms_status ms_tc_selftest(const float* d_X, const float* d_P, int32_t 
     if (s == MS_OK) s = cuda_check(cudaMemcpy(ctx->X, d_X, sizeof(float) * 128 * 16, cudaMemcpyDeviceToDevice), "copy X");
     if (s == MS_OK) s = cuda_check(cudaMemcpy(ctx->active[0], iota, sizeof(iota), cudaMemcpyHostToDevice), "copy active");
     if (s == MS_OK) s = cuda_check(cudaMemcpy(ctx->dc, &dc0, sizeof(dc0), cudaMemcpyHostToDevice), "copy counters");
+    if (s == MS_OK) s = cuda_check(cudaMemset(ctx->acc, 0, sizeof(int64_t) * 128 * 17), "clear acc");
     if (s == MS_OK) s = launch_shift_tc(ctx, ctx->active[0], 1, 1, dbg);
     if (s == MS_OK) s = cuda_check(cudaDeviceSynchronize(), "self-test kernel");
     if (s == MS_OK) s = readback(ctx);

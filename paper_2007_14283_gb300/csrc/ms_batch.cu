@@ -49,7 +49,6 @@ struct ms_batch {
     int32_t* pix;
     uint8_t* covered;
     float* X;
-    int32_t* seed_pix;
     int32_t* seed_order;
     uint8_t* sstate;
     int32_t* support;
@@ -59,21 +58,16 @@ struct ms_batch {
     int32_t* cand;
     int32_t* cand_rank;
     int32_t* rank_cand;
-    float* Xr;                // candidates' seed positions in rank order (merge)
     uint8_t* removed_r;       // candidates removed by a mode of an earlier round, in rank order
     uint8_t* cand_state;
     int32_t* conf_deg;
     int32_t* conf;
     int32_t* block_tmp;       // [B, nblk_max]
     void* Pk;
-    void* Mk;                 // kept modes as BF16 split rows at the frames' Pk offsets (labelling)
-    void* Ck;                 // merge candidates (rank order) as BF16 split rows at the frames' Pk offsets
     int32_t** label_ptrs;     // device array of B label buffers
     CUtensorMap pmap;
     CUtensorMap pmap1;        // d = 32: dimensions 16..31 (the second Pk array)
-    CUtensorMap mmap;
-    CUtensorMap mmap1;        // d = 32: the modes' dimensions 16..31 (the second Mk array)
-    CUtensorMap cmap, cmap1;  // Ck, and its second array (d = 32)
+    CUtensorMap amap;         // acc as split rows (candidates, modes)
     ms::LabelTcScratch lsc;
     cudaGraph_t graph;
     cudaGraphExec_t exec;
@@ -304,7 +298,7 @@ __global__ void k_b_labels_clear(const BFrame* __restrict__ frames, int32_t* con
 // ------------------------------------------------------------ seeds
 __global__ void __launch_bounds__(kIT)
 k_b_seed(const BFrame* __restrict__ frames, BState* states, const float* __restrict__ P32, int Dp,
-         uint8_t* __restrict__ covered, float* __restrict__ X, int32_t* __restrict__ seed_pix,
+         uint8_t* __restrict__ covered, float* __restrict__ X, unsigned long long* __restrict__ acc,
          int32_t* __restrict__ seed_order, int32_t* __restrict__ act0, uint8_t* __restrict__ sstate,
          int32_t* __restrict__ order_of, int max_rounds, int all_seeds) {
     __shared__ int32_t warp_excl[32];
@@ -378,7 +372,6 @@ k_b_seed(const BFrame* __restrict__ frames, BState* states, const float* __restr
     // slots in pixel order (ms_seed.cu)
     auto write = [&](int32_t p, int64_t slot, int32_t order) {
         covered[base + p] = 1;
-        seed_pix[slot] = p;
         seed_order[slot] = order;
         act0[slot] = (int32_t)slot;
         sstate[slot] = kMoving;
@@ -386,6 +379,8 @@ k_b_seed(const BFrame* __restrict__ frames, BState* states, const float* __restr
         float4* dst = reinterpret_cast<float4*>(X + slot * Dp);
         for (int k = 0; k < Dp / 4; ++k) dst[k] = src[k];
     };
+    unsigned long long* sums = acc + (int64_t)fr.pk_row0 * (Dp + 1);
+    for (int64_t i = tid; i < (int64_t)taken * (Dp + 1); i += kIT) sums[i] = 0ull;
     if (few) {
         int rank[2];
         few_ranks(s_few, taken, n, rank);
@@ -524,8 +519,10 @@ k_b_finalize(const BFrame* __restrict__ frames, BState* states, int B, BPlan pla
         const int pos = (blk - plan.seed_off[f]) * kFinSeeds + wid * 8 + (lane & 7);
         DevCounters& dc = states[f].dc;
         const bool live = pos < dc.n_active;
-        const int64_t slot = live ? ((dc.iters & 1) ? act1 : act0)[frames[f].pix0 + pos] : 0;
-        const SeedEnd e = finalize_seed<Dp>(live, acc + slot * (Dp + 1), X + slot * Dp, sstate + slot, support + slot,
+        const BFrame& fr = frames[f];
+        const int64_t slot = live ? ((dc.iters & 1) ? act1 : act0)[fr.pix0 + pos] : fr.pix0;
+        const SeedEnd e = finalize_seed<Dp>(live, acc + (slot - fr.pix0 + fr.pk_row0) * (Dp + 1), X + slot * Dp,
+                                            sstate + slot, support + slot,
                                             tol, band);
         const bool first = lane < 8;  // one lane per seed
         const uint32_t mv = __ballot_sync(0xffffffffu, first && e.move);
@@ -671,12 +668,13 @@ __global__ void k_b_merge_zero(const BFrame* __restrict__ frames, const BState* 
 }
 
 // rank_cand inverts cand_rank; each candidate's seed position is copied to
-// its rank's row of Xr, so the conflict search reads contiguous rows.
+// its rank's row of Xr, so the conflict search reads contiguous rows. Xr is the
+// modes' rows from n_kept on.
 template <int Dp>
 __global__ void k_b_rank_invert(const BFrame* __restrict__ frames, const BState* __restrict__ states, int B,
                                 const int32_t* __restrict__ off, const int32_t* __restrict__ cand_rank,
                                 const int32_t* __restrict__ cand, const float* __restrict__ X,
-                                int32_t* __restrict__ rank_cand, float* __restrict__ Xr) {
+                                int32_t* __restrict__ rank_cand, float* __restrict__ modes) {
     for (int bb = blockIdx.x; bb < off[B]; bb += gridDim.x) {
         const int f = locate(off, B, bb);
         const int a = (bb - off[f]) * kMT + threadIdx.x;
@@ -685,7 +683,7 @@ __global__ void k_b_rank_invert(const BFrame* __restrict__ frames, const BState*
             const int r = cand_rank[base + a];
             rank_cand[base + r] = a;
             const float4* src = reinterpret_cast<const float4*>(X + (int64_t)cand[base + a] * Dp);
-            float4* dst = reinterpret_cast<float4*>(Xr + (base + r) * Dp);
+            float4* dst = reinterpret_cast<float4*>(modes + (base + states[f].dc.n_kept + r) * Dp);
 #pragma unroll
             for (int q = 0; q < Dp / 4; ++q) dst[q] = src[q];
         }
@@ -749,10 +747,10 @@ __global__ void k_b_rank(const BFrame* __restrict__ frames, const BState* __rest
 template <int Dp>
 __global__ void __launch_bounds__(kMT)
 k_b_merge_resolve(const BFrame* __restrict__ frames, BState* states, int B, const int32_t* __restrict__ off,
-                  const float* __restrict__ Xr, const int32_t* __restrict__ rank_cand, uint8_t* cand_state,
+                  const float* __restrict__ modes, const int32_t* __restrict__ rank_cand, uint8_t* cand_state,
                   const int32_t* __restrict__ conf_deg, const int32_t* __restrict__ conf, float thr_f, double thr,
                   int count_left) {
-    // Threads take candidates by rank (merge_look's reason, ms_merge.cu).
+    // Threads take candidates by rank (merge_look_all's reason, ms_merge.cu).
     for (int bb = blockIdx.x; bb < off[B]; bb += gridDim.x) {
         const int f = locate(off, B, bb);
         const int lb = bb - off[f];
@@ -767,7 +765,7 @@ k_b_merge_resolve(const BFrame* __restrict__ frames, BState* states, int B, cons
         bool any_kept = false, all_removed = true;
         if (deg <= kMergeCap) {
             for (int j = 0; j < deg; ++j) {
-                const uint8_t s = st[conf[(base + a) * kMergeCap + j]];
+                const uint8_t s = st[conf[((int64_t)frames[f].pk_row0 + a) * kMergeCap + j]];
                 if (s == kKept) { any_kept = true; break; }
                 if (s == kUndecided) all_removed = false;
             }
@@ -775,11 +773,12 @@ k_b_merge_resolve(const BFrame* __restrict__ frames, BState* states, int B, cons
             // more conflicts than were stored: test the candidates ranked
             // above this one again, in rank order
             float x[Dp];
-            ldv<Dp>(x, Xr + (base + r) * Dp);
+            const float* Xr = modes + (base + states[f].dc.n_kept) * Dp;
+            ldv<Dp>(x, Xr + (int64_t)r * Dp);
             for (int rb = 0; rb < r; ++rb) {
                 const uint8_t s = st[rank_cand[base + rb]];
                 if (s == kRemoved) continue;
-                if (!cos_at_least<Dp>(x, Xr + (base + rb) * Dp, thr_f, thr)) continue;
+                if (!cos_at_least<Dp>(x, Xr + (int64_t)rb * Dp, thr_f, thr)) continue;
                 if (s == kKept) { any_kept = true; break; }
                 all_removed = false;
             }
@@ -910,7 +909,7 @@ float ceil_f(double c) { return ceil_to_float(c); }
 
 template <int Dp>
 ms_status enqueue_seed(ms_batch* b, cudaStream_t s) {
-    k_b_seed<<<b->B, kIT, 0, s>>>(b->frames, b->states, b->P32, Dp, b->covered, b->X, b->seed_pix, b->seed_order,
+    k_b_seed<<<b->B, kIT, 0, s>>>(b->frames, b->states, b->P32, Dp, b->covered, b->X, b->acc, b->seed_order,
                                   b->act[0], b->sstate, b->cand_rank, b->cfg.max_rounds, b->cfg.all_seeds);
     MS_LAUNCH("k_b_seed");
     return MS_OK;
@@ -1004,15 +1003,15 @@ ms_status enqueue_round(ms_batch* b, cudaStream_t s, int64_t* nlaunch) {
                                b->cand_rank);
     LAUNCHED("k_b_rank");
     k_b_rank_invert<Dp><<<G, kMT, 0, s>>>(b->frames, b->states, B, b->blk_off, b->cand_rank, b->cand, b->X,
-                                          b->rank_cand, b->Xr);
+                                          b->rank_cand, b->modes);
     LAUNCHED("k_b_rank_invert");
-    st = launch_merge_tc_batch(b->cmap, b->cmap1, b->mmap, b->mmap1, b->Ck, b->total_pk_rows, Dp, b->frames, b->states,
-                               B, (int)b->max_pk_rows, b->Xr, b->modes, b->rank_cand, b->cand_state, b->removed_r,
-                               b->conf_deg, b->conf, mf, b->cfg.merge_cos, b->blk_off, b->num_sms, b->misc + 1, s);
+    st = launch_merge_tc_batch(b->pmap, b->pmap1, b->amap, b->Pk, b->total_pk_rows, b->acc, Dp, b->frames, b->states, B,
+                               (int)b->max_pk_rows, b->modes, b->rank_cand, b->cand_state, b->removed_r, b->conf_deg,
+                               b->conf, mf, b->cfg.merge_cos, b->blk_off, b->num_sms, b->misc + 1, s);
     if (st != MS_OK) return st;
     nl += 3;
     for (int sw = 0; sw < 8; ++sw) {
-        k_b_merge_resolve<Dp><<<G, kMT, 0, s>>>(b->frames, b->states, B, b->blk_off, b->Xr, b->rank_cand,
+        k_b_merge_resolve<Dp><<<G, kMT, 0, s>>>(b->frames, b->states, B, b->blk_off, b->modes, b->rank_cand,
                                                 b->cand_state, b->conf_deg, b->conf, mf, b->cfg.merge_cos, sw == 7);
         LAUNCHED("k_b_merge_resolve");
     }
@@ -1028,9 +1027,9 @@ ms_status enqueue_round(ms_batch* b, cudaStream_t s, int64_t* nlaunch) {
     }
     k_b_blocks<<<1, 32, 0, s>>>(b->frames, b->states, B, kSelDonePixels, 128, b->blk_off, nullptr, 0);
     LAUNCHED("k_b_blocks");
-    st = launch_cover_tc_batch(b->pmap, b->mmap, b->pmap1, b->mmap1, b->Mk, b->total_pk_rows, Dp, b->frames, b->states,
-                               B, (int)b->max_pk_rows, b->modes, b->P32, b->pix, b->d, b->cfg.bandwidth_cos,
-                               b->covered, b->blk_off, b->num_sms, b->misc + 1, s);
+    st = launch_cover_tc_batch(b->pmap, b->pmap1, b->amap, b->Pk, b->total_pk_rows, b->acc, Dp, b->frames, b->states, B,
+                               (int)b->max_pk_rows, b->modes, b->P32, b->pix, b->d, b->cfg.bandwidth_cos, b->covered,
+                               b->blk_off, b->num_sms, b->misc + 1, s);
     if (st != MS_OK) return st;
     nl += 2;
     if (b->prof_phases) {
@@ -1073,7 +1072,6 @@ template <int Dp>
 ms_status enqueue_setup(ms_batch* b, cudaStream_t s) {
     const int B = b->B;
     MS_CUDA(cudaMemsetAsync(b->covered, 0, (size_t)b->total_px, s));
-    MS_CUDA(cudaMemsetAsync(b->acc, 0, sizeof(unsigned long long) * (size_t)b->total_px * (Dp + 1), s));
     MS_CUDA(cudaMemsetAsync(b->misc, 0, sizeof(b->h_misc), s));
     if (b->prof_phases) {
         k_b_phase<<<1, 1, 0, s>>>(b->misc, -1);
@@ -1111,9 +1109,9 @@ ms_status enqueue_label_tick(ms_batch* b, cudaStream_t s) {
 
 template <int Dp>
 ms_status enqueue_label(ms_batch* b, cudaStream_t s) {
-    return launch_label_tc_batch(b->pmap, b->mmap, b->pmap1, b->mmap1, b->Mk, b->total_pk_rows, Dp, b->frames,
-                                 b->states, b->B, (int)b->max_pk_rows, b->modes, b->P32, b->pix, b->d, b->label_ptrs,
-                                 b->lsc, b->num_sms, b->misc + 1, s);
+    return launch_label_tc_batch(b->pmap, b->pmap1, b->amap, b->acc, Dp, b->frames, b->states, b->B,
+                                 (int)b->max_pk_rows, b->modes, b->P32, b->pix, b->d, b->label_ptrs, b->lsc,
+                                 b->num_sms, b->misc + 1, s);
 }
 
 // The nodes that the next one captured on s would depend on.
@@ -1289,14 +1287,34 @@ extern "C" ms_status ms_batch_create(const ms_config* cfg, int32_t B, const floa
     b->nblk_max = (b->max_np + kIT - 1) / kIT;
     const int Dp = b->Dp;
     const size_t n = (size_t)b->total_px;
+    const size_t rows_pk = (size_t)b->total_pk_rows;
     const size_t sizes[] = {
-        sizeof(BFrame) * B, sizeof(BState) * B, sizeof(int32_t) * ((B + 1) * 4 + (B + 2) * 2), sizeof(b->h_misc),
-        n * Dp * 4, n * 4, n, n * Dp * 4, n * 4, n * 4, n, n * 4, n * 4, n * 4,
-        n * (Dp + 1) * 8, n * Dp * 4, n * 4, n * 4, n * 4, n, n * 4, n * kMergeCap * 4,
-        (size_t)B * b->nblk_max * 4 + 4, (size_t)b->total_pk_rows * 128 * (Dp / 16), sizeof(int32_t*) * B,
-        (size_t)b->total_pk_rows * 128 * (Dp / 16), n * sizeof(int2), sizeof(int32_t) * (B + 1) + 16,
-        n * Dp * 4, n, (size_t)b->total_pk_rows * 128 * (Dp / 16),
-        (n / kFinSeeds + B) * sizeof(uint32_t)};
+        sizeof(BFrame) * B,                        // 0 frames
+        sizeof(BState) * B,                        // 1 states
+        sizeof(int32_t) * ((B + 1) * 4 + (B + 2) * 2),  // 2 plan, work lists
+        sizeof(b->h_misc),                         // 3 misc
+        n * Dp * 4,                                // 4 P32
+        n * 4,                                     // 5 pix
+        n,                                         // 6 covered
+        n * Dp * 4,                                // 7 X | near-tie queue
+        n * 4,                                     // 8 seed_order
+        n,                                         // 9 sstate
+        n * 4,                                     // 10 support
+        n * 4,                                     // 11 act[0]
+        n * 4,                                     // 12 act[1]
+        rows_pk * (Dp + 1) * 8,                    // 13 acc | split rows of candidates, of modes
+        n * Dp * 4,                                // 14 modes | Xr
+        n * 4,                                     // 15 cand
+        n * 4,                                     // 16 cand_rank
+        n * 4,                                     // 17 rank_cand
+        n,                                         // 18 cand_state
+        n * 4,                                     // 19 conf_deg
+        rows_pk * 128 * (Dp / 16),                 // 20 Pk | split rows of earlier modes | conf
+        (size_t)B * b->nblk_max * 4 + 4,           // 21 block_tmp
+        sizeof(int32_t*) * B,                      // 22 label_ptrs
+        sizeof(int32_t) * (B + 1) + 16,            // 23 label items, near-tie count
+        n,                                         // 24 removed_r
+        (n / kFinSeeds + B) * sizeof(uint32_t)};   // 25 moving
     const int NS = (int)(sizeof(sizes) / sizeof(sizes[0]));
     size_t offs[32], tot = 0;
     for (int i = 0; i < NS; ++i) {
@@ -1324,31 +1342,27 @@ extern "C" ms_status ms_batch_create(const ms_config* cfg, int32_t B, const floa
     b->pix = (int32_t*)(w + offs[5]);
     b->covered = (uint8_t*)(w + offs[6]);
     b->X = (float*)(w + offs[7]);
-    b->seed_pix = (int32_t*)(w + offs[8]);
-    b->seed_order = (int32_t*)(w + offs[9]);
-    b->sstate = (uint8_t*)(w + offs[10]);
-    b->support = (int32_t*)(w + offs[11]);
-    b->act[0] = (int32_t*)(w + offs[12]);
-    b->act[1] = (int32_t*)(w + offs[13]);
-    b->acc = (unsigned long long*)(w + offs[14]);
-    b->modes = (float*)(w + offs[15]);
-    b->cand = (int32_t*)(w + offs[16]);
-    b->cand_rank = (int32_t*)(w + offs[17]);
-    b->rank_cand = (int32_t*)(w + offs[18]);
-    b->cand_state = (uint8_t*)(w + offs[19]);
-    b->conf_deg = (int32_t*)(w + offs[20]);
-    b->conf = (int32_t*)(w + offs[21]);
-    b->block_tmp = (int32_t*)(w + offs[22]);
-    b->Pk = (void*)(w + offs[23]);
-    b->label_ptrs = (int32_t**)(w + offs[24]);
-    b->Mk = (void*)(w + offs[25]);
-    b->lsc.fix = (int2*)(w + offs[26]);
-    b->lsc.off = (int32_t*)(w + offs[27]);
+    b->lsc.fix = (int2*)(w + offs[7]);
+    b->seed_order = (int32_t*)(w + offs[8]);
+    b->sstate = (uint8_t*)(w + offs[9]);
+    b->support = (int32_t*)(w + offs[10]);
+    b->act[0] = (int32_t*)(w + offs[11]);
+    b->act[1] = (int32_t*)(w + offs[12]);
+    b->acc = (unsigned long long*)(w + offs[13]);
+    b->modes = (float*)(w + offs[14]);
+    b->cand = (int32_t*)(w + offs[15]);
+    b->cand_rank = (int32_t*)(w + offs[16]);
+    b->rank_cand = (int32_t*)(w + offs[17]);
+    b->cand_state = (uint8_t*)(w + offs[18]);
+    b->conf_deg = (int32_t*)(w + offs[19]);
+    b->Pk = (void*)(w + offs[20]);
+    b->conf = (int32_t*)(w + offs[20]);
+    b->block_tmp = (int32_t*)(w + offs[21]);
+    b->label_ptrs = (int32_t**)(w + offs[22]);
+    b->lsc.off = (int32_t*)(w + offs[23]);
     b->lsc.fix_count = b->lsc.off + (B + 1);
-    b->Xr = (float*)(w + offs[28]);
-    b->removed_r = (uint8_t*)(w + offs[29]);
-    b->Ck = (void*)(w + offs[30]);
-    b->moving = (uint32_t*)(w + offs[31]);
+    b->removed_r = (uint8_t*)(w + offs[24]);
+    b->moving = (uint32_t*)(w + offs[25]);
     ms_status s = cuda_check(cudaMallocHost((void**)&b->h_states, sizeof(BState) * B), "cudaMallocHost");
     if (s == MS_OK) s = cuda_check(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking), "cudaStreamCreate");
     if (s == MS_OK)
@@ -1364,14 +1378,7 @@ extern "C" ms_status ms_batch_create(const ms_config* cfg, int32_t B, const floa
     if (s == MS_OK)
         s = encode_pk_map(Dp == 32 ? (uint8_t*)b->Pk + (size_t)b->total_pk_rows * 128 : b->Pk, (int)b->total_pk_rows,
                           &b->pmap1);
-    if (s == MS_OK) s = encode_pk_map(b->Mk, (int)b->total_pk_rows, &b->mmap);
-    if (s == MS_OK) b->mmap1 = b->mmap;
-    if (s == MS_OK && Dp == 32)
-        s = encode_pk_map((uint8_t*)b->Mk + (size_t)b->total_pk_rows * 128, (int)b->total_pk_rows, &b->mmap1);
-    if (s == MS_OK) s = encode_pk_map(b->Ck, (int)b->total_pk_rows, &b->cmap);
-    if (s == MS_OK) b->cmap1 = b->cmap;
-    if (s == MS_OK && Dp == 32)
-        s = encode_pk_map((uint8_t*)b->Ck + (size_t)b->total_pk_rows * 128, (int)b->total_pk_rows, &b->cmap1);
+    if (s == MS_OK) s = encode_pk_map(b->acc, (int)(b->total_pk_rows / 16 * (Dp + 1)), &b->amap);
     if (s == MS_OK) s = label_tc_setup();
     if (s == MS_OK) s = rebuild_graph(b);
     if (s != MS_OK) {

@@ -12,10 +12,12 @@ enum BPhase : int32_t { kNeedSeed = 0, kIterating = 1, kRoundDone = 2, kFinished
 
 // Per-frame constants, fixed after set-up. Frame f owns the rows
 // [pix0, pix0 + n) of every per-pixel, per-seed, per-candidate and per-mode
-// array, and the Pk rows [pk_row0, pk_row0 + n_ptiles * 128).
+// array, and the rows [pk_row0, pk_row0 + pk_rows) of Pk and of acc. As in a
+// context (ms_ctx), Pk shares its memory with the earlier modes' split rows and
+// the conflict lists (candidate a's at row pk_row0 + a), acc with the split rows of
+// candidates and of modes (split_row0), and the modes with Xr.
 struct BFrame {
     int64_t pix0;
-    int64_t in0;        // offset of the frame's input pixels (labels, masks)
     int64_t n_pixels;   // input pixels
     int32_t n;          // foreground pixels
     int32_t n_ptiles;   // ceil(n / 128)
@@ -25,6 +27,14 @@ struct BFrame {
     const float* emb;   // borrowed input [n_pixels, d]
     const uint8_t* mask;
 };
+
+// The frame's padded rows.
+__host__ __device__ inline int pk_rows(const BFrame& fr) { return (int)((fr.n_pixels + 127) / 128 * 128); }
+
+// The frame's first 128-byte row in acc, read as split rows: its first acc row lies
+// pk_row0 * (Dp + 1) * 8 bytes in, a whole number of them as pk_row0 is a multiple
+// of 128. Its share holds Dp / 16 arrays of pk_rows split rows.
+__host__ __device__ inline int split_row0(const BFrame& fr, int Dp) { return fr.pk_row0 / 16 * (Dp + 1); }
 
 // Per-frame state, advanced only by device code.
 struct BState {
@@ -87,41 +97,42 @@ ms_status launch_label_tc_single(const CUtensorMap& pmap, const CUtensorMap& pma
                                  const float* modes, int K, int n, const float* P32, const int32_t* pix,
                                  const float* emb, int d, int32_t* labels, LabelTcScratch sc, int grid, int* status,
                                  cudaStream_t st);
-// Coverage against one frame's new modes [k0, k1) on the tensor cores (BF16
-// form): exact decisions, the near-threshold pixels re-decided as the FP32
-// form decides them.
-ms_status launch_cover_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, void* Mk, int64_t n_pad, int Dp,
-                                 const float* modes, int k0, int k1, int n, const float* P32, const int32_t* pix,
-                                 const float* emb, int d, double c, uint8_t* covered, int* n_uncovered,
-                                 int grid, int* status, cudaStream_t st);
+// Coverage against one frame's new modes [k0, k1) on the tensor cores, after the
+// first `taken` rows of Pk (second array pk_half rows on) are the pixels' again:
+// exact decisions.
+ms_status launch_cover_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, void* Pk, int64_t pk_half,
+                                 int taken, void* Mk, int64_t n_pad, int Dp, const float* modes, int k0, int k1, int n,
+                                 const float* P32, const int32_t* pix, const float* emb, int d, double c,
+                                 uint8_t* covered, int* n_uncovered, int grid, int* status, cudaStream_t st);
 // The same for the frames of a batch whose round ended (tile_off: their pixel
-// tiles, from k_b_blocks with 128 pixels per block).
-ms_status launch_cover_tc_batch(const CUtensorMap& pmap, const CUtensorMap& mmap, const CUtensorMap& pmap1,
-                                const CUtensorMap& mmap1, void* Mk, int64_t mk_rows, int Dp, const BFrame* frames,
-                                BState* states, int B, int max_pk_rows, const float* modes, const float* P32,
-                                const int32_t* pix, int d, double c, uint8_t* covered, const int32_t* tile_off,
-                                int grid, int* status, cudaStream_t st);
+// tiles, from k_b_blocks with 128 pixels per block). amap: the split rows in acc.
+ms_status launch_cover_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, const CUtensorMap& amap, void* Pk,
+                                int64_t pk_half, void* Mk, int Dp, const BFrame* frames, BState* states, int B,
+                                int max_pk_rows, const float* modes, const float* P32, const int32_t* pix, int d,
+                                double c, uint8_t* covered, const int32_t* tile_off, int grid, int* status,
+                                cudaStream_t st);
 // The merge's two contractions on the tensor cores for the frames whose round
 // ended (tile_off: their candidates in blocks of 128): the candidates in rank
-// order (Xr, packed into Ck) against their earlier modes (Mk), then against
-// one another; exact decisions (merge_cos), the near-threshold pairs decided
-// by the FP32-then-FP64 test. Sets removed_r / cand_state and fills the
-// conflict lists as k_b_merge_old and k_b_merge_pairs do.
-ms_status launch_merge_tc_batch(const CUtensorMap& cmap, const CUtensorMap& cmap1, const CUtensorMap& mmap,
-                                const CUtensorMap& mmap1, void* Ck, int64_t rows, int Dp, const BFrame* frames,
-                                BState* states, int B, int max_pk_rows, const float* Xr, const float* modes,
-                                const int32_t* rank_cand, uint8_t* cand_state, uint8_t* removed_r, int32_t* conf_deg,
-                                int32_t* conf, float thr_f, double thr, const int32_t* tile_off, int grid, int* status, cudaStream_t st);
-// The same for one frame: k candidates (Xr, packed into Ck) against its K_old
-// earlier modes (Mk), then against one another.
-ms_status launch_merge_tc_single(void* Ck, void* Mk, int64_t n_pad, int Dp, int k, int K_old, const float* Xr,
+// order (Xr, packed into Ck) against their earlier modes (packed into Pk), then
+// against one another; exact decisions (merge_cos), the near-threshold pairs decided
+// by the FP32-then-FP64 test. Sets removed_r and cand_state and fills the conflict
+// lists.
+ms_status launch_merge_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, const CUtensorMap& amap, void* Pk,
+                                int64_t pk_half, void* Ck, int Dp, const BFrame* frames, BState* states, int B,
+                                int max_pk_rows, const float* modes, const int32_t* rank_cand, uint8_t* cand_state,
+                                uint8_t* removed_r, int32_t* conf_deg, int32_t* conf, float thr_f, double thr,
+                                const int32_t* tile_off, int grid, int* status, cudaStream_t st);
+// The same for one frame: k candidates (Xr) against its K_old earlier modes, then
+// against one another.
+ms_status launch_merge_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, void* Pk, int64_t pk_half,
+                                 void* Ck, int64_t n_pad, int Dp, int k, int K_old, const float* Xr,
                                  const float* modes, const int32_t* rank_cand, uint8_t* cand_state, uint8_t* removed_r,
-                                 int32_t* conf_deg, int32_t* conf, float thr_f, double thr, int grid, int* status, cudaStream_t st);
-ms_status launch_label_tc_batch(const CUtensorMap& pmap, const CUtensorMap& mmap, const CUtensorMap& pmap1,
-                                const CUtensorMap& mmap1, void* Mk, int64_t mk_rows, int Dp, const BFrame* frames,
-                                const BState* states, int B, int max_pk_rows, const float* modes, const float* P32,
-                                const int32_t* pix, int d, int32_t* const* labels, LabelTcScratch sc, int grid,
-                                int* status, cudaStream_t st);
+                                 int32_t* conf_deg, int32_t* conf, float thr_f, double thr, int grid, int* status,
+                                 cudaStream_t st);
+ms_status launch_label_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, const CUtensorMap& amap, void* Mk,
+                                int Dp, const BFrame* frames, const BState* states, int B, int max_pk_rows,
+                                const float* modes, const float* P32, const int32_t* pix, int d,
+                                int32_t* const* labels, LabelTcScratch sc, int grid, int* status, cudaStream_t st);
 
 // Pixel tiles per chunk when a frame's seed tiles (128 seeds each) are cut
 // into tiles x chunks work items for the tensor-core shift. The plain rule

@@ -106,14 +106,19 @@ struct ms_ctx {
     int num_sms;
     int shift_grid;     // persistent grid of the shift kernel
     int target_items;   // work items per shift iteration
-    // workspace (one allocation)
+    // Workspace (one allocation). What is not live at the same time shares memory:
+    //  - acc (a round's iterations) with Ck (its merge) with Mk (coverage, labelling);
+    //    the selection of a round clears its seeds' rows of acc;
+    //  - Pk with Mk_old and conf (the merge); coverage first restores the rows of Pk
+    //    that those took;
+    //  - the modes' rows from n_kept on with Xr (the merge, until it appends there);
+    //  - X with label_fix (labelling, between rounds).
     void* ws;
     size_t ws_bytes;
     float* P32;          // [n_pixels, Dp] normalised foreground
     int32_t* pix;        // [n_pixels] foreground index -> pixel index
     uint8_t* covered;    // [n_pixels]
     float* X;            // [n_pixels, Dp] seed positions by slot
-    int32_t* seed_pix;   // [n_pixels]
     int32_t* seed_order; // [n_pixels]
     uint8_t* sstate;     // [n_pixels]
     int32_t* support;    // [n_pixels]
@@ -127,7 +132,7 @@ struct ms_ctx {
     int32_t* rank_cand;  // [n_pixels] inverse of cand_rank
     uint8_t* cand_state; // [n_pixels]
     int32_t* conf_deg;   // [n_pixels]
-    int32_t* conf;       // [n_pixels * kMergeCap]
+    int32_t* conf;       // [n_pixels, kMergeCap]: a candidate's list is as long as a row of Pk
     int32_t* block_tmp;  // ingest and seed-selection scan scratch
     uint32_t* moving;    // per kFinSeeds (32) active seeds: the mask of those still moving
     ms::DevCounters* dc;
@@ -151,11 +156,11 @@ struct ms_ctx {
     CUtensorMap pmap;    // TMA map of Pk: boxes of 128 rows x 128 bytes, 128-byte swizzle
     CUtensorMap pmap1;   // d = 32: the same for dimensions 16..31 (the second Pk array)
     int tc_grid;         // persistent grid of the tensor-core shift kernel
-    void* Mk;            // [n_pad, 64] bf16 split rows of the kept modes (labelling)
+    void* Mk;            // [n_pad, 64] bf16 split rows of the kept modes
     int2* label_fix;     // [n] near-tie queue of the tensor-core labelling, then its count
-    float* Xr;           // [n, Dp] merge candidates' positions in rank order
     uint8_t* removed_r;  // [n] candidates removed by an earlier mode, by rank
-    void* Ck;            // [n_pad, 64] bf16 split rows of Xr (a second array for Dp = 32)
+    void* Ck;            // [n_pad, 64] bf16 split rows of the merge candidates in rank order (a
+                         // second array for Dp = 32, as for Mk)
     // measurement
     bool prof;
     cudaEvent_t ev[64];  // start/end pairs around shift launches of one batch
@@ -207,6 +212,9 @@ cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned threads, size
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// Rows from Pk's first array to its second (Dp = 32).
+inline int64_t pk_half_rows(const ms_ctx* ctx) { return (ctx->n_pixels + 127) / 128 * 128; }
+
 // Kernel launchers. Each enqueues on ctx->stream and returns MS_OK or MS_ERR_CUDA.
 ms_status launch_ingest(ms_ctx* ctx);                       // ms_ingest.cu
 ms_status launch_seed_select(ms_ctx* ctx, int32_t want);    // ms_seed.cu
@@ -219,7 +227,8 @@ bool merge_in_one(int32_t k);  // up to kMergeOne candidates
 // Resolves and appends, or (too many conflicts for one block) leaves dc->undecided = k.
 ms_status launch_merge_one(ms_ctx* ctx, int32_t k);
 ms_status launch_merge_append(ms_ctx* ctx, int32_t k);
-ms_status launch_cover(ms_ctx* ctx, int32_t k0, int32_t k1);
+// Coverage by the modes [k0, k1) of a merge of k candidates, whose rows of Pk it restores.
+ms_status launch_cover(ms_ctx* ctx, int32_t k, int32_t k0, int32_t k1);
 ms_status launch_label(ms_ctx* ctx, int32_t* d_labels);     // ms_label_tc.cu
 ms_status launch_collect(ms_ctx* ctx);                      // ms_merge.cu
 int shift_blocks_per_sm();                                  // ms_shift_fp32.cu

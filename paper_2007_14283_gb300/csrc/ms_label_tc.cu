@@ -68,11 +68,14 @@ struct LbDim {
 // What an item covers.
 struct LbItem {
     int frame;
-    int pk_row0;   // Pk / Mk row of the frame's pixel 0 and mode 0 (multiple of 128)
-    int pt;        // pixel tile
-    int n;         // the frame's foreground count
-    int K;         // the frame's kept modes (the end of the scored mode range)
-    int k0;        // the first scored mode (0 for labelling; coverage scores a round's new modes)
+    int r0, r1;    // first row of the row operand (tile 0) in pmap, and in pmap1 (dimensions 16-31)
+    int c0, c1;    // the same of the column operand, in mmap and mmap1
+    int pt;        // row tile
+    int n;         // rows of the operand (the frame's foreground or candidate count)
+    int K;         // end of the scored columns (modes or candidates)
+    int k0;        // the first scored column (0 for labelling; coverage scores a round's new modes)
+    int x0;        // merge: Xr row of the candidate of rank 0
+    int conf0;     // merge: conflict list of candidate 0
 };
 
 struct LbSingle {
@@ -80,35 +83,19 @@ struct LbSingle {
     __device__ __forceinline__ bool init() { return n > 0; }
     __device__ __forceinline__ int total() const { return (n + 127) / 128; }
     int k0 = 0;
-    __device__ __forceinline__ LbItem item(int i) const { return LbItem{0, 0, i, n, K, k0}; }
+    __device__ __forceinline__ LbItem item(int i) const { return LbItem{0, 0, 0, 0, 0, i, n, K, k0, 0, 0}; }
 };
 
-struct LbBatch {
-    const BFrame* frames;
-    const BState* states;
-    const int32_t* off;   // pixel-tile offsets over frames (B + 1)
-    int B;
-    int total_;
-    __device__ __forceinline__ bool init() {
-        total_ = off[B];
-        return total_ > 0;
-    }
-    __device__ __forceinline__ int total() const { return total_; }
-    __device__ __forceinline__ LbItem item(int i) const {
-        const int f = locate(off, B, i);
-        const BFrame& fr = frames[f];
-        return LbItem{f, fr.pk_row0, i - off[f], fr.n, states[f].dc.n_kept, 0};
-    }
-};
-
-// Coverage in the batch: the pixel tiles of the frames whose round ended
-// (off from k_b_blocks with 128 pixels per block), each against its frame's
-// new modes [k0, n_kept).
-struct LbBatchCover {
+// Coverage and labelling in the batch: the pixel tiles of the frames of a work
+// list (off: their offsets, B + 1), each against its frame's modes: all of them, or
+// for coverage those of the round that ended. The modes' split rows lie in the
+// frame's share of acc (split_row0).
+template <bool kNew>
+struct LbBatchPixels {
     const BFrame* frames;
     const BState* states;
     const int32_t* off;
-    int B;
+    int B, Dp;
     int total_;
     __device__ __forceinline__ bool init() {
         total_ = off[B];
@@ -118,19 +105,24 @@ struct LbBatchCover {
     __device__ __forceinline__ LbItem item(int i) const {
         const int f = locate(off, B, i);
         const BFrame& fr = frames[f];
-        return LbItem{f, fr.pk_row0, i - off[f], fr.n, states[f].dc.n_kept, states[f].k0};
+        const int s0 = split_row0(fr, Dp);
+        return LbItem{f,    fr.pk_row0, fr.pk_row0,           s0, s0 + pk_rows(fr), i - off[f],
+                      fr.n, states[f].dc.n_kept, kNew ? states[f].k0 : 0, 0,  0};
     }
 };
+using LbBatch = LbBatchPixels<false>;
+using LbBatchCover = LbBatchPixels<true>;
 
 // The merge of the frames whose round ended (off from k_b_blocks with 128
 // candidates per block): row tile t of a frame's k candidates, in rank order
-// (Ck rows), against its modes kept in earlier rounds (Mk, LbBatchOld) or
-// against the candidates ranked up to the tile's end (Ck, LbBatchPairs).
+// (their split rows in the frame's share of acc), against its modes kept in earlier
+// rounds (at its rows of Pk, LbBatchOld) or against the candidates ranked up to the
+// tile's end (LbBatchPairs).
 struct LbBatchOld {
     const BFrame* frames;
     const BState* states;
     const int32_t* off;
-    int B;
+    int B, Dp;
     int total_;
     __device__ __forceinline__ bool init() {
         total_ = off[B];
@@ -139,14 +131,17 @@ struct LbBatchOld {
     __device__ __forceinline__ int total() const { return total_; }
     __device__ __forceinline__ LbItem item(int i) const {
         const int f = locate(off, B, i);
-        return LbItem{f, frames[f].pk_row0, i - off[f], states[f].dc.n_cand, states[f].dc.n_kept, 0};
+        const BFrame& fr = frames[f];
+        const int s0 = split_row0(fr, Dp), K = states[f].dc.n_kept;
+        return LbItem{f, s0, s0 + pk_rows(fr), fr.pk_row0, fr.pk_row0, i - off[f], states[f].dc.n_cand, K, 0, K,
+                      fr.pk_row0};
     }
 };
 struct LbBatchPairs {
     const BFrame* frames;
     const BState* states;
     const int32_t* off;
-    int B;
+    int B, Dp;
     int total_;
     __device__ __forceinline__ bool init() {
         total_ = off[B];
@@ -155,8 +150,10 @@ struct LbBatchPairs {
     __device__ __forceinline__ int total() const { return total_; }
     __device__ __forceinline__ LbItem item(int i) const {
         const int f = locate(off, B, i);
+        const BFrame& fr = frames[f];
+        const int s0 = split_row0(fr, Dp), s1 = s0 + pk_rows(fr);
         const int t = i - off[f], k = states[f].dc.n_cand;
-        return LbItem{f, frames[f].pk_row0, t, k, min(k, (t + 1) * 128), 0};
+        return LbItem{f, s0, s1, s0, s1, t, k, min(k, (t + 1) * 128), 0, states[f].dc.n_kept, fr.pk_row0};
     }
 };
 
@@ -167,7 +164,7 @@ struct LbSingleMerge {
     __device__ __forceinline__ bool init() { return k > 0; }
     __device__ __forceinline__ int total() const { return (k + 127) / 128; }
     __device__ __forceinline__ LbItem item(int i) const {
-        return LbItem{0, 0, i, k, pairs ? min(k, (i + 1) * 128) : K, 0};
+        return LbItem{0, 0, 0, 0, 0, i, k, pairs ? min(k, (i + 1) * 128) : K, 0, 0, 0};
     }
 };
 
@@ -340,9 +337,9 @@ k_label_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
             if (ia >= 2 && !(ok = lwarp_wait(&a_empty[ab], ((ia >> 1) - 1) & 1, abort))) break;
             if (lane == 0) {
                 mbar_arrive_expect_tx(&a_full[ab], kHalves * kLTile);
-                tma_load_2d(Ab + ab * kHalves * kLTile, &pmap, 0, ii.pk_row0 + ii.pt * 128, &a_full[ab]);
+                tma_load_2d(Ab + ab * kHalves * kLTile, &pmap, 0, ii.r0 + ii.pt * 128, &a_full[ab]);
                 if (kHalves > 1)
-                    tma_load_2d(Ab + (ab * kHalves + 1) * kLTile, &pmap1, 0, ii.pk_row0 + ii.pt * 128, &a_full[ab]);
+                    tma_load_2d(Ab + (ab * kHalves + 1) * kLTile, &pmap1, 0, ii.r1 + ii.pt * 128, &a_full[ab]);
             }
             __syncwarp();
             ++ia;
@@ -351,9 +348,9 @@ k_label_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
                 if (g >= kLStages && !(ok = lwarp_wait(&b_empty[s], ((g / kLStages) - 1) & 1, abort))) break;
                 if (lane == 0) {
                     mbar_arrive_expect_tx(&b_full[s], kHalves * kLTile);
-                    tma_load_2d(Bst + s * kHalves * kLTile, &mmap, 0, ii.pk_row0 + ii.k0 + mt * 128, &b_full[s]);
+                    tma_load_2d(Bst + s * kHalves * kLTile, &mmap, 0, ii.c0 + ii.k0 + mt * 128, &b_full[s]);
                     if (kHalves > 1)
-                        tma_load_2d(Bst + (s * kHalves + 1) * kLTile, &mmap1, 0, ii.pk_row0 + ii.k0 + mt * 128,
+                        tma_load_2d(Bst + (s * kHalves + 1) * kLTile, &mmap1, 0, ii.c1 + ii.k0 + mt * 128,
                                     &b_full[s]);
                 }
                 __syncwarp();
@@ -473,7 +470,7 @@ k_label_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
 #pragma unroll
                         for (int j = 0; j < 32; ++j) near |= (uint32_t)(__uint_as_float(v[j]) >= lo) << j;
                         float xr[kD];
-                        const float* row = (kMode == kLbCover ? out.P32 : out.Xr) + (mbase + mi) * kD;
+                        const float* row = kMode == kLbCover ? out.P32 + (mbase + mi) * kD : out.Xr + (mbase + ii.x0 + mi) * kD;
 #pragma unroll
                         for (int k = 0; k < kD; ++k) xr[k] = row[k];
                         for (; near; near &= near - 1) {
@@ -518,16 +515,16 @@ k_label_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
                             if (!hit) {
                                 if (!have_x) {
 #pragma unroll
-                                    for (int k = 0; k < kD; ++k) xr[k] = out.Xr[(mbase + mi) * kD + k];
+                                    for (int k = 0; k < kD; ++k) xr[k] = out.Xr[(mbase + ii.x0 + mi) * kD + k];
                                     have_x = true;
                                 }
-                                hit = cos_at_least<kD>(xr, out.Xr + (mbase + col) * kD, out.c_f, out.thr);
+                                hit = cos_at_least<kD>(xr, out.Xr + (mbase + ii.x0 + col) * kD, out.c_f, out.thr);
                             }
                             if (hit) {
                                 if (ma < 0) ma = out.rank_cand[mbase + mi];
                                 const int slot = atomicAdd(&out.conf_deg[mbase + ma], 1);
                                 if (slot < kMergeCap) {
-                                    out.conf[(mbase + ma) * kMergeCap + slot] = out.rank_cand[mbase + col];
+                                    out.conf[((int64_t)ii.conf0 + ma) * kMergeCap + slot] = out.rank_cand[mbase + col];
                                 } else {
                                     full = true;
                                     break;
@@ -846,8 +843,8 @@ __device__ __forceinline__ void pack_mode(const float* mode, uint4* Mk, int64_t 
     if (Dp == 32) pack_split_row(mode ? mode + 16 : nullptr, Mk + (half_rows + r) * 8, false);
 }
 
-// Modes as BF16 split rows at the frame's Pk row offsets (padding rows hold
-// the ones only; their columns are masked out by the score readers).
+// One frame's modes [0, K) as BF16 split rows [0, K_pad) (padding rows hold the
+// ones only; their columns are masked out by the score readers).
 template <int Dp>
 __global__ void k_pack_modes_single(const float* __restrict__ modes, int K, int K_pad, uint4* __restrict__ Mk,
                                     int64_t half_rows) {
@@ -856,59 +853,73 @@ __global__ void k_pack_modes_single(const float* __restrict__ modes, int K, int 
     pack_mode<Dp>(r < K ? modes + (int64_t)r * Dp : nullptr, Mk, r, half_rows);
 }
 
+// The same for every frame of a batch, in the frames' shares of acc.
 template <int Dp>
 __global__ void k_pack_modes_batch(const BFrame* __restrict__ frames, const BState* __restrict__ states,
-                                   const float* __restrict__ modes, uint4* __restrict__ Mk, int64_t half_rows) {
+                                   const float* __restrict__ modes, uint4* __restrict__ Mk) {
     const BFrame& fr = frames[blockIdx.y];
     const int K = states[blockIdx.y].dc.n_kept;
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= (K + 127) / 128 * 128) return;
-    pack_mode<Dp>(r < K ? modes + (fr.pix0 + r) * Dp : nullptr, Mk, fr.pk_row0 + r, half_rows);
+    pack_mode<Dp>(r < K ? modes + (fr.pix0 + r) * Dp : nullptr, Mk, split_row0(fr, Dp) + r, pk_rows(fr));
 }
 
-// Modes [k0, k1) of one frame as BF16 split rows at their Mk rows.
+// What coverage needs after one frame's merge: the modes [k0, k1) at their rows of
+// Mk, and the pixels' first `taken` rows of Pk, which held the earlier modes and the
+// conflict lists.
 template <int Dp>
-__global__ void k_pack_modes_range(const float* __restrict__ modes, int k0, int k1, uint4* __restrict__ Mk,
-                                   int64_t half_rows) {
-    const int r = k0 + blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= k1) return;
-    pack_mode<Dp>(modes + (int64_t)r * Dp, Mk, r, half_rows);
+__global__ void k_pack_cover_single(const float* __restrict__ P32, int taken, uint4* __restrict__ Pk,
+                                    int64_t pk_half_rows, const float* __restrict__ modes, int k0, int k1,
+                                    uint4* __restrict__ Mk, int64_t half_rows) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x, m = k0 + r - taken;
+    if (r < taken)
+        pack_mode<Dp>(P32 + (int64_t)r * Dp, Pk, r, pk_half_rows);
+    else if (m < k1)
+        pack_mode<Dp>(modes + (int64_t)m * Dp, Mk, m, half_rows);
 }
 
-// The batch form of k_pack_modes_range: every frame whose round ended packs
-// its new modes [k0, n_kept) at its Mk rows.
+// The same for every frame of a batch whose round ended (blockIdx.z: 0 the pixels,
+// 1 the modes).
 template <int Dp>
-__global__ void k_pack_modes_new_batch(const BFrame* __restrict__ frames, const BState* __restrict__ states,
-                                       const float* __restrict__ modes, uint4* __restrict__ Mk, int64_t half_rows) {
+__global__ void k_pack_cover_batch(const BFrame* __restrict__ frames, const BState* __restrict__ states,
+                                   const float* __restrict__ P32, uint4* __restrict__ Pk, int64_t pk_half_rows,
+                                   const float* __restrict__ modes, uint4* __restrict__ Mk) {
     const BFrame& fr = frames[blockIdx.y];
     const BState& st = states[blockIdx.y];
-    if (st.phase != kRoundDone) return;
-    const int r = st.k0 + blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= st.dc.n_kept) return;
-    pack_mode<Dp>(modes + (fr.pix0 + r) * Dp, Mk, fr.pk_row0 + r, half_rows);
+    if (st.phase != kRoundDone || st.dc.n_cand == 0) return;
+    const int r = blockIdx.x * blockDim.x + threadIdx.x, m = st.k0 + r;
+    if (blockIdx.z == 0 && r < max(st.dc.n_cand, st.k0))
+        pack_mode<Dp>(P32 + (fr.pix0 + r) * Dp, Pk, fr.pk_row0 + r, pk_half_rows);
+    if (blockIdx.z == 1 && m < st.dc.n_kept)
+        pack_mode<Dp>(modes + (fr.pix0 + m) * Dp, Mk, split_row0(fr, Dp) + m, pk_rows(fr));
 }
 
-// The candidates of every frame whose round ended, in rank order (Xr), as
-// BF16 split rows at the frame's Pk row offsets.
+// What one frame's merge needs: its k candidates (rank order, Xr) as split rows
+// [0, kp) of Ck, and its K_old earlier modes as rows of Pk.
 template <int Dp>
-__global__ void k_pack_cands_batch(const BFrame* __restrict__ frames, const BState* __restrict__ states,
-                                   const float* __restrict__ Xr, uint4* __restrict__ Ck, int64_t half_rows) {
+__global__ void k_pack_merge_single(const float* Xr, int k, int kp, uint4* __restrict__ Ck, int64_t half_rows,
+                                    const float* modes, int K_old, uint4* __restrict__ Pk, int64_t pk_half_rows) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r < kp)
+        pack_mode<Dp>(r < k ? Xr + (int64_t)r * Dp : nullptr, Ck, r, half_rows);
+    else if (r - kp < K_old)
+        pack_mode<Dp>(modes + (int64_t)(r - kp) * Dp, Pk, r - kp, pk_half_rows);
+}
+
+// The same for every frame of a batch whose round ended (Xr: the modes' rows from
+// n_kept on; blockIdx.z: 0 the candidates, 1 the earlier modes).
+template <int Dp>
+__global__ void k_pack_merge_batch(const BFrame* __restrict__ frames, const BState* __restrict__ states,
+                                   const float* __restrict__ modes, uint4* __restrict__ Ck, uint4* __restrict__ Pk,
+                                   int64_t pk_half_rows) {
     const BFrame& fr = frames[blockIdx.y];
     const BState& st = states[blockIdx.y];
-    if (st.phase != kRoundDone) return;
-    const int k = st.dc.n_cand;
+    const int k = st.dc.n_cand, K = st.dc.n_kept;
+    if (st.phase != kRoundDone || k == 0) return;
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= (k + 127) / 128 * 128) return;
-    pack_mode<Dp>(r < k ? Xr + (fr.pix0 + r) * Dp : nullptr, Ck, fr.pk_row0 + r, half_rows);
-}
-
-// One frame's k candidates (rank order, Xr) as BF16 split rows [0, kp).
-template <int Dp>
-__global__ void k_pack_cands_single(const float* __restrict__ Xr, int k, int kp, uint4* __restrict__ Ck,
-                                    int64_t half_rows) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= kp) return;
-    pack_mode<Dp>(r < k ? Xr + (int64_t)r * Dp : nullptr, Ck, r, half_rows);
+    if (blockIdx.z == 0 && r < (k + 127) / 128 * 128)
+        pack_mode<Dp>(r < k ? modes + (fr.pix0 + K + r) * Dp : nullptr, Ck, split_row0(fr, Dp) + r, pk_rows(fr));
+    if (blockIdx.z == 1 && r < K) pack_mode<Dp>(modes + (fr.pix0 + r) * Dp, Pk, fr.pk_row0 + r, pk_half_rows);
 }
 
 // Per-frame offsets of the label items (128-pixel tiles); clears the queue.
@@ -943,22 +954,26 @@ ms_status label_tc_setup_dim() {
     return MS_OK;
 }
 
+// The TMA maps of one frame's split rows at `rows`, its second array n_pad rows on.
 template <int Dp>
-ms_status merge_tc_single(void* Ck, void* Mk, int64_t n_pad, int k, int K_old, const float* Xr, const float* modes,
-                          const int32_t* rank_cand, uint8_t* cand_state, uint8_t* removed_r, int32_t* conf_deg,
-                          int32_t* conf, float thr_f, double thr, int grid, int* status,
-                          cudaStream_t st) {
-    const int kp = (k + 127) / 128 * 128;
-    k_pack_cands_single<Dp><<<(kp + 255) / 256, 256, 0, st>>>(Xr, k, kp, (uint4*)Ck, n_pad);
-    MS_LAUNCH("k_pack_cands_single");
-    CUtensorMap cmap, cmap1, mmap, mmap1;
-    ms_status s = encode_pk_map(Ck, (int)n_pad, &cmap);
-    if (s == MS_OK) s = encode_pk_map(Mk, (int)n_pad, &mmap);
+ms_status split_maps(void* rows, int64_t n_pad, CUtensorMap* m0, CUtensorMap* m1) {
+    ms_status s = encode_pk_map(rows, (int)n_pad, m0);
     if (s != MS_OK) return s;
-    cmap1 = cmap;
-    mmap1 = mmap;
-    if (Dp == 32 && (s = encode_pk_map((uint8_t*)Ck + n_pad * 128, (int)n_pad, &cmap1)) != MS_OK) return s;
-    if (Dp == 32 && (s = encode_pk_map((uint8_t*)Mk + n_pad * 128, (int)n_pad, &mmap1)) != MS_OK) return s;
+    *m1 = *m0;
+    return Dp == 32 ? encode_pk_map((uint8_t*)rows + n_pad * 128, (int)n_pad, m1) : s;
+}
+
+template <int Dp>
+ms_status merge_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, void* Pk, int64_t pk_half, void* Ck,
+                          int64_t n_pad, int k, int K_old, const float* Xr, const float* modes,
+                          const int32_t* rank_cand, uint8_t* cand_state, uint8_t* removed_r, int32_t* conf_deg,
+                          int32_t* conf, float thr_f, double thr, int grid, int* status, cudaStream_t st) {
+    const int kp = (k + 127) / 128 * 128, rows = kp + K_old;
+    k_pack_merge_single<Dp><<<(rows + 255) / 256, 256, 0, st>>>(Xr, k, kp, (uint4*)Ck, n_pad, modes, K_old, (uint4*)Pk,
+                                                                pk_half);
+    MS_LAUNCH("k_pack_merge_single");
+    CUtensorMap cmap, cmap1;
+    if (ms_status s = split_maps<Dp>(Ck, n_pad, &cmap, &cmap1); s != MS_OK) return s;
     LbOut out{};
     out.c_f = thr_f;
     out.modes = modes;
@@ -971,7 +986,7 @@ ms_status merge_tc_single(void* Ck, void* Mk, int64_t n_pad, int k, int K_old, c
     out.thr = thr;
     if (K_old > 0) {
         LbSingleMerge om{k, K_old, 0};
-        k_label_tc<LbSingleMerge, kLbOld, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(cmap, mmap, cmap1, mmap1,
+        k_label_tc<LbSingleMerge, kLbOld, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(cmap, pmap, cmap1, pmap1,
                                                                                             om, out, status);
         MS_LAUNCH("k_label_tc(merge, earlier modes)");
     }
@@ -983,48 +998,46 @@ ms_status merge_tc_single(void* Ck, void* Mk, int64_t n_pad, int k, int K_old, c
 }
 
 template <int Dp>
-ms_status merge_tc_batch(const CUtensorMap& cmap, const CUtensorMap& cmap1, const CUtensorMap& mmap,
-                         const CUtensorMap& mmap1, void* Ck, int64_t rows, const BFrame* frames, BState* states, int B,
-                         int max_pk_rows, const float* Xr, const float* modes, const int32_t* rank_cand,
-                         uint8_t* cand_state, uint8_t* removed_r, int32_t* conf_deg, int32_t* conf, float thr_f,
-                         double thr, const int32_t* tile_off, int grid, int* status,
-                         cudaStream_t st) {
-    const dim3 gp((unsigned)((max_pk_rows + 255) / 256), (unsigned)B);
-    k_pack_cands_batch<Dp><<<gp, 256, 0, st>>>(frames, states, Xr, (uint4*)Ck, rows);
-    MS_LAUNCH("k_pack_cands_batch");
+ms_status merge_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, const CUtensorMap& amap, void* Pk,
+                         int64_t pk_half, void* Ck, const BFrame* frames, BState* states, int B, int max_pk_rows,
+                         const float* modes, const int32_t* rank_cand, uint8_t* cand_state, uint8_t* removed_r,
+                         int32_t* conf_deg, int32_t* conf, float thr_f, double thr, const int32_t* tile_off, int grid,
+                         int* status, cudaStream_t st) {
+    const dim3 gp((unsigned)((max_pk_rows + 255) / 256), (unsigned)B, 2);
+    k_pack_merge_batch<Dp><<<gp, 256, 0, st>>>(frames, states, modes, (uint4*)Ck, (uint4*)Pk, pk_half);
+    MS_LAUNCH("k_pack_merge_batch");
     LbOut out{};
     out.frames = frames;
     out.c_f = thr_f;
     out.modes = modes;
-    out.Xr = Xr;
+    out.Xr = modes;
     out.removed_r = removed_r;
     out.rank_cand = rank_cand;
     out.cand_state = cand_state;
     out.conf_deg = conf_deg;
     out.conf = conf;
     out.thr = thr;
-    LbBatchOld om{frames, states, tile_off, B, 0};
-    k_label_tc<LbBatchOld, kLbOld, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(cmap, mmap, cmap1, mmap1, om,
+    LbBatchOld om{frames, states, tile_off, B, Dp, 0};
+    k_label_tc<LbBatchOld, kLbOld, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(amap, pmap, amap, pmap1, om,
                                                                                      out, status);
     MS_LAUNCH("k_label_tc(merge, earlier modes)");
-    LbBatchPairs pm{frames, states, tile_off, B, 0};
-    k_label_tc<LbBatchPairs, kLbPairs, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(cmap, cmap, cmap1, cmap1,
-                                                                                         pm, out, status);
+    LbBatchPairs pm{frames, states, tile_off, B, Dp, 0};
+    k_label_tc<LbBatchPairs, kLbPairs, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(amap, amap, amap, amap, pm,
+                                                                                         out, status);
     MS_LAUNCH("k_label_tc(merge, conflicts)");
     return MS_OK;
 }
 
 template <int Dp>
-ms_status cover_tc_batch(const CUtensorMap& pmap, const CUtensorMap& mmap, const CUtensorMap& pmap1,
-                         const CUtensorMap& mmap1, void* Mk, int64_t mk_rows, const BFrame* frames, BState* states,
-                         int B, int max_pk_rows, const float* modes, const float* P32, const int32_t* pix, int d,
-                         double c, uint8_t* covered, const int32_t* tile_off, int grid, int* status,
-                         cudaStream_t st) {
-    const dim3 gp((unsigned)((max_pk_rows + 255) / 256), (unsigned)B);
-    k_pack_modes_new_batch<Dp><<<gp, 256, 0, st>>>(frames, states, modes, (uint4*)Mk, mk_rows);
-    MS_LAUNCH("k_pack_modes_new_batch");
+ms_status cover_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, const CUtensorMap& amap, void* Pk,
+                         int64_t pk_half, void* Mk, const BFrame* frames, BState* states, int B, int max_pk_rows,
+                         const float* modes, const float* P32, const int32_t* pix, int d, double c, uint8_t* covered,
+                         const int32_t* tile_off, int grid, int* status, cudaStream_t st) {
+    const dim3 gp((unsigned)((max_pk_rows + 255) / 256), (unsigned)B, 2);
+    k_pack_cover_batch<Dp><<<gp, 256, 0, st>>>(frames, states, P32, (uint4*)Pk, pk_half, modes, (uint4*)Mk);
+    MS_LAUNCH("k_pack_cover_batch");
     const float c_f = (float)c;
-    LbBatchCover map{frames, states, tile_off, B, 0};
+    LbBatchCover map{frames, states, tile_off, B, Dp, 0};
     LbOut out{};
     out.frames = frames;
     out.pix = pix;
@@ -1035,23 +1048,24 @@ ms_status cover_tc_batch(const CUtensorMap& pmap, const CUtensorMap& mmap, const
     out.P32 = P32;
     out.modes = modes;
     out.d = d;
-    k_label_tc<LbBatchCover, kLbCover, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(pmap, mmap, pmap1, mmap1, map,
+    k_label_tc<LbBatchCover, kLbCover, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(pmap, amap, pmap1, amap, map,
                                                                                        out, status);
     MS_LAUNCH("k_label_tc(cover, batch)");
     return MS_OK;
 }
 
 template <int Dp>
-ms_status cover_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, void* Mk, int64_t n_pad,
-                          const float* modes, int k0, int k1, int n, const float* P32, const int32_t* pix,
-                          const float* emb, int d, double c, uint8_t* covered, int* n_uncovered, int grid, int* status, cudaStream_t st) {
-    k_pack_modes_range<Dp><<<(k1 - k0 + 255) / 256, 256, 0, st>>>(modes, k0, k1, (uint4*)Mk, n_pad);
-    MS_LAUNCH("k_pack_modes_range");
+ms_status cover_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, void* Pk, int64_t pk_half, int taken,
+                          void* Mk, int64_t n_pad, const float* modes, int k0, int k1, int n, const float* P32,
+                          const int32_t* pix, const float* emb, int d, double c, uint8_t* covered, int* n_uncovered,
+                          int grid, int* status, cudaStream_t st) {
+    const int rows = taken + k1 - k0;
+    k_pack_cover_single<Dp><<<(rows + 255) / 256, 256, 0, st>>>(P32, taken, (uint4*)Pk, pk_half, modes, k0, k1,
+                                                                (uint4*)Mk, n_pad);
+    MS_LAUNCH("k_pack_cover_single");
+    if (k1 <= k0) return MS_OK;
     CUtensorMap mmap, mmap1;
-    ms_status s = encode_pk_map(Mk, (int)n_pad, &mmap);
-    if (s != MS_OK) return s;
-    mmap1 = mmap;
-    if (Dp == 32 && (s = encode_pk_map((uint8_t*)Mk + n_pad * 128, (int)n_pad, &mmap1)) != MS_OK) return s;
+    if (ms_status s = split_maps<Dp>(Mk, n_pad, &mmap, &mmap1); s != MS_OK) return s;
     LbSingle map{n, k1};
     map.k0 = k0;
     const float c_f = (float)c;
@@ -1082,10 +1096,7 @@ ms_status label_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, voi
         MS_LAUNCH("k_pack_modes_single");
     }
     CUtensorMap mmap, mmap1;
-    ms_status s = encode_pk_map(Mk, (int)n_pad, &mmap);
-    if (s != MS_OK) return s;
-    mmap1 = mmap;
-    if (Dp == 32 && (s = encode_pk_map((uint8_t*)Mk + n_pad * 128, (int)n_pad, &mmap1)) != MS_OK) return s;
+    if (ms_status s = split_maps<Dp>(Mk, n_pad, &mmap, &mmap1); s != MS_OK) return s;
     LbSingle map{n, K};
     LbOut out{};
     out.labels1 = labels;
@@ -1108,17 +1119,16 @@ ms_status label_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, voi
 }
 
 template <int Dp>
-ms_status label_tc_batch(const CUtensorMap& pmap, const CUtensorMap& mmap, const CUtensorMap& pmap1,
-                         const CUtensorMap& mmap1, void* Mk, int64_t mk_rows, const BFrame* frames,
-                         const BState* states, int B, int max_pk_rows, const float* modes, const float* P32,
-                         const int32_t* pix, int d, int32_t* const* labels, LabelTcScratch sc, int grid, int* status,
-                         cudaStream_t st) {
+ms_status label_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, const CUtensorMap& amap, void* Mk,
+                         const BFrame* frames, const BState* states, int B, int max_pk_rows, const float* modes,
+                         const float* P32, const int32_t* pix, int d, int32_t* const* labels, LabelTcScratch sc,
+                         int grid, int* status, cudaStream_t st) {
     const dim3 gp((unsigned)((max_pk_rows + 255) / 256), (unsigned)B);
-    k_pack_modes_batch<Dp><<<gp, 256, 0, st>>>(frames, states, modes, (uint4*)Mk, mk_rows);
+    k_pack_modes_batch<Dp><<<gp, 256, 0, st>>>(frames, states, modes, (uint4*)Mk);
     MS_LAUNCH("k_pack_modes_batch");
     k_label_items<<<1, 32, 0, st>>>(frames, B, sc.off, sc.fix_count);
     MS_LAUNCH("k_label_items");
-    LbBatch map{frames, states, sc.off, B, 0};
+    LbBatch map{frames, states, sc.off, B, Dp, 0};
     LbOut out{};
     out.labels = labels;
     out.frames = frames;
@@ -1128,7 +1138,7 @@ ms_status label_tc_batch(const CUtensorMap& pmap, const CUtensorMap& mmap, const
     out.P32 = P32;
     out.modes = modes;
     out.d = d;
-    k_label_tc<LbBatch, kLbLabel, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(pmap, mmap, pmap1, mmap1, map,
+    k_label_tc<LbBatch, kLbLabel, Dp><<<grid, kLThreads, LbDim<Dp>::kSmemBytes, st>>>(pmap, amap, pmap1, amap, map,
                                                                                    out, status);
     MS_LAUNCH("k_label_tc(batch)");
     k_label_fix<Dp><<<grid, 256, 0, st>>>(sc.fix, sc.fix_count, P32, modes, frames, states, pix, nullptr, 0, d, labels,
@@ -1144,49 +1154,44 @@ ms_status label_tc_setup() {
     return s == MS_OK ? label_tc_setup_dim<32>() : s;
 }
 
-ms_status launch_merge_tc_batch(const CUtensorMap& cmap, const CUtensorMap& cmap1, const CUtensorMap& mmap,
-                                const CUtensorMap& mmap1, void* Ck, int64_t rows, int Dp, const BFrame* frames,
-                                BState* states, int B, int max_pk_rows, const float* Xr, const float* modes,
-                                const int32_t* rank_cand, uint8_t* cand_state, uint8_t* removed_r, int32_t* conf_deg,
-                                int32_t* conf, float thr_f, double thr, const int32_t* tile_off, int grid, int* status, cudaStream_t st) {
-    return Dp == 32 ? merge_tc_batch<32>(cmap, cmap1, mmap, mmap1, Ck, rows, frames, states, B, max_pk_rows, Xr, modes,
-                                         rank_cand, cand_state, removed_r, conf_deg, conf, thr_f, thr, tile_off,
-                                         grid, status, st)
-                    : merge_tc_batch<16>(cmap, cmap1, mmap, mmap1, Ck, rows, frames, states, B, max_pk_rows, Xr, modes,
-                                         rank_cand, cand_state, removed_r, conf_deg, conf, thr_f, thr, tile_off,
-                                         grid, status, st);
+ms_status launch_merge_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, const CUtensorMap& amap, void* Pk,
+                                int64_t pk_half, void* Ck, int Dp, const BFrame* frames, BState* states, int B,
+                                int max_pk_rows, const float* modes, const int32_t* rank_cand, uint8_t* cand_state,
+                                uint8_t* removed_r, int32_t* conf_deg, int32_t* conf, float thr_f, double thr,
+                                const int32_t* tile_off, int grid, int* status, cudaStream_t st) {
+    auto* run = Dp == 32 ? merge_tc_batch<32> : merge_tc_batch<16>;
+    return run(pmap, pmap1, amap, Pk, pk_half, Ck, frames, states, B, max_pk_rows, modes, rank_cand, cand_state,
+               removed_r, conf_deg, conf, thr_f, thr, tile_off, grid, status, st);
 }
 
-ms_status launch_merge_tc_single(void* Ck, void* Mk, int64_t n_pad, int Dp, int k, int K_old, const float* Xr,
+ms_status launch_merge_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, void* Pk, int64_t pk_half,
+                                 void* Ck, int64_t n_pad, int Dp, int k, int K_old, const float* Xr,
                                  const float* modes, const int32_t* rank_cand, uint8_t* cand_state, uint8_t* removed_r,
-                                 int32_t* conf_deg, int32_t* conf, float thr_f, double thr, int grid, int* status, cudaStream_t st) {
+                                 int32_t* conf_deg, int32_t* conf, float thr_f, double thr, int grid, int* status,
+                                 cudaStream_t st) {
     if (k <= 0) return MS_OK;
-    return Dp == 32 ? merge_tc_single<32>(Ck, Mk, n_pad, k, K_old, Xr, modes, rank_cand, cand_state, removed_r,
-                                          conf_deg, conf, thr_f, thr,  grid, status, st)
-                    : merge_tc_single<16>(Ck, Mk, n_pad, k, K_old, Xr, modes, rank_cand, cand_state, removed_r,
-                                          conf_deg, conf, thr_f, thr,  grid, status, st);
+    auto* run = Dp == 32 ? merge_tc_single<32> : merge_tc_single<16>;
+    return run(pmap, pmap1, Pk, pk_half, Ck, n_pad, k, K_old, Xr, modes, rank_cand, cand_state, removed_r, conf_deg,
+               conf, thr_f, thr, grid, status, st);
 }
 
-ms_status launch_cover_tc_batch(const CUtensorMap& pmap, const CUtensorMap& mmap, const CUtensorMap& pmap1,
-                                const CUtensorMap& mmap1, void* Mk, int64_t mk_rows, int Dp, const BFrame* frames,
-                                BState* states, int B, int max_pk_rows, const float* modes, const float* P32,
-                                const int32_t* pix, int d, double c, uint8_t* covered, const int32_t* tile_off,
-                                int grid, int* status, cudaStream_t st) {
-    return Dp == 32 ? cover_tc_batch<32>(pmap, mmap, pmap1, mmap1, Mk, mk_rows, frames, states, B, max_pk_rows, modes,
-                                         P32, pix, d, c, covered, tile_off,  grid, status, st)
-                    : cover_tc_batch<16>(pmap, mmap, pmap1, mmap1, Mk, mk_rows, frames, states, B, max_pk_rows, modes,
-                                         P32, pix, d, c, covered, tile_off,  grid, status, st);
+ms_status launch_cover_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, const CUtensorMap& amap, void* Pk,
+                                int64_t pk_half, void* Mk, int Dp, const BFrame* frames, BState* states, int B,
+                                int max_pk_rows, const float* modes, const float* P32, const int32_t* pix, int d,
+                                double c, uint8_t* covered, const int32_t* tile_off, int grid, int* status,
+                                cudaStream_t st) {
+    auto* run = Dp == 32 ? cover_tc_batch<32> : cover_tc_batch<16>;
+    return run(pmap, pmap1, amap, Pk, pk_half, Mk, frames, states, B, max_pk_rows, modes, P32, pix, d, c, covered,
+               tile_off, grid, status, st);
 }
 
-ms_status launch_cover_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, void* Mk, int64_t n_pad, int Dp,
-                                 const float* modes, int k0, int k1, int n, const float* P32, const int32_t* pix,
-                                 const float* emb, int d, double c, uint8_t* covered, int* n_uncovered,
-                                 int grid, int* status, cudaStream_t st) {
-    if (n == 0 || k1 <= k0) return MS_OK;
-    return Dp == 32 ? cover_tc_single<32>(pmap, pmap1, Mk, n_pad, modes, k0, k1, n, P32, pix, emb, d, c, covered,
-                                          n_uncovered,  grid, status, st)
-                    : cover_tc_single<16>(pmap, pmap1, Mk, n_pad, modes, k0, k1, n, P32, pix, emb, d, c, covered,
-                                          n_uncovered,  grid, status, st);
+ms_status launch_cover_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, void* Pk, int64_t pk_half,
+                                 int taken, void* Mk, int64_t n_pad, int Dp, const float* modes, int k0, int k1, int n,
+                                 const float* P32, const int32_t* pix, const float* emb, int d, double c,
+                                 uint8_t* covered, int* n_uncovered, int grid, int* status, cudaStream_t st) {
+    auto* run = Dp == 32 ? cover_tc_single<32> : cover_tc_single<16>;
+    return run(pmap, pmap1, Pk, pk_half, taken, Mk, n_pad, modes, k0, k1, n, P32, pix, emb, d, c, covered, n_uncovered,
+               grid, status, st);
 }
 
 ms_status launch_label_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, void* Mk, int64_t n_pad, int Dp,
@@ -1200,15 +1205,13 @@ ms_status launch_label_tc_single(const CUtensorMap& pmap, const CUtensorMap& pma
                                           status, st);
 }
 
-ms_status launch_label_tc_batch(const CUtensorMap& pmap, const CUtensorMap& mmap, const CUtensorMap& pmap1,
-                                const CUtensorMap& mmap1, void* Mk, int64_t mk_rows, int Dp, const BFrame* frames,
-                                const BState* states, int B, int max_pk_rows, const float* modes, const float* P32,
-                                const int32_t* pix, int d, int32_t* const* labels, LabelTcScratch sc, int grid,
-                                int* status, cudaStream_t st) {
-    return Dp == 32 ? label_tc_batch<32>(pmap, mmap, pmap1, mmap1, Mk, mk_rows, frames, states, B, max_pk_rows, modes,
-                                         P32, pix, d, labels, sc, grid, status, st)
-                    : label_tc_batch<16>(pmap, mmap, pmap1, mmap1, Mk, mk_rows, frames, states, B, max_pk_rows, modes,
-                                         P32, pix, d, labels, sc, grid, status, st);
+ms_status launch_label_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, const CUtensorMap& amap, void* Mk,
+                                int Dp, const BFrame* frames, const BState* states, int B, int max_pk_rows,
+                                const float* modes, const float* P32, const int32_t* pix, int d,
+                                int32_t* const* labels, LabelTcScratch sc, int grid, int* status, cudaStream_t st) {
+    auto* run = Dp == 32 ? label_tc_batch<32> : label_tc_batch<16>;
+    return run(pmap, pmap1, amap, Mk, frames, states, B, max_pk_rows, modes, P32, pix, d, labels, sc, grid, status,
+               st);
 }
 
 ms_status launch_label(ms_ctx* ctx, int32_t* d_labels) {

@@ -86,37 +86,36 @@ __device__ __forceinline__ void load_vec(float* dst, const float* src) {
     }
 }
 
-// What one look at the conflicts of the candidate of rank r says of it: removed
-// when a kept one is among them, kept when all are removed, else still undecided.
-// Threads take candidates by rank: of those with more conflicts than were stored,
-// a warp's then read the same few higher ranks, whose positions lie in a row in Xr
-// (by candidate, in pixel order, that look took four times as long: 2.8 ms for
-// 4096 candidates of one cell).
-template <int Dp>
-__device__ __forceinline__ uint8_t merge_look(int r, int a, const float* __restrict__ Xr,
-                                              const int32_t* __restrict__ rank_cand, volatile uint8_t* st,
-                                              const int32_t* __restrict__ conf_deg, const int32_t* __restrict__ conf,
-                                              float thr_f, double thr) {
-    const int deg = conf_deg[a];
+// What a look at a candidate's stored conflicts says of it: removed when a kept
+// one is among them, kept when all are removed, else still undecided.
+__device__ __forceinline__ uint8_t merge_look(const int32_t* conf, int deg, const volatile uint8_t* st) {
     bool all_removed = true;
-    if (deg <= kMergeCap) {
-        for (int j = 0; j < deg; ++j) {
-            const uint8_t s = st[conf[(int64_t)a * kMergeCap + j]];
-            if (s == kKept) return kRemoved;
-            if (s == kUndecided) all_removed = false;
-        }
-    } else {
-        // more conflicts than were stored: test the candidates ranked above
-        // this one again, in rank order
-        float x[Dp];
-        load_vec<Dp>(x, Xr + (int64_t)r * Dp);
-        for (int rb = 0; rb < r; ++rb) {
-            const uint8_t s = st[rank_cand[rb]];
-            if (s == kRemoved) continue;
-            if (!cos_at_least<Dp>(x, Xr + (int64_t)rb * Dp, thr_f, thr)) continue;
-            if (s == kKept) return kRemoved;
-            all_removed = false;
-        }
+    for (int j = 0; j < deg; ++j) {
+        const uint8_t s = st[conf[j]];
+        if (s == kKept) return kRemoved;
+        if (s == kUndecided) all_removed = false;
+    }
+    return all_removed ? kKept : kUndecided;
+}
+
+// The same for a candidate, of rank r, with more conflicts than were stored: the
+// candidates ranked above it are tested again, in rank order. Threads take
+// candidates by rank: a warp's then read the same few higher ranks, whose positions
+// lie in a row in Xr (by candidate, in pixel order, that look took four times as
+// long: 2.8 ms for 4096 candidates of one cell).
+template <int Dp>
+__device__ __forceinline__ uint8_t merge_look_all(int r, const float* __restrict__ Xr,
+                                                  const int32_t* __restrict__ rank_cand, const volatile uint8_t* st,
+                                                  float thr_f, double thr) {
+    bool all_removed = true;
+    float x[Dp];
+    load_vec<Dp>(x, Xr + (int64_t)r * Dp);
+    for (int rb = 0; rb < r; ++rb) {
+        const uint8_t s = st[rank_cand[rb]];
+        if (s == kRemoved) continue;
+        if (!cos_at_least<Dp>(x, Xr + (int64_t)rb * Dp, thr_f, thr)) continue;
+        if (s == kKept) return kRemoved;
+        all_removed = false;
     }
     return all_removed ? kKept : kUndecided;
 }
@@ -131,7 +130,9 @@ k_merge_resolve(const float* __restrict__ Xr, int k, const int32_t* __restrict__
     const int a = rank_cand[r];
     volatile uint8_t* st = cand_state;
     if (st[a] != kUndecided) return;
-    const uint8_t d = merge_look<Dp>(r, a, Xr, rank_cand, st, conf_deg, conf, thr_f, thr);
+    const int deg = conf_deg[a];
+    const uint8_t d = deg <= kMergeCap ? merge_look(conf + (int64_t)a * kMergeCap, deg, st)
+                                       : merge_look_all<Dp>(r, Xr, rank_cand, st, thr_f, thr);
     if (d != kUndecided)
         st[a] = d;
     else
@@ -228,11 +229,10 @@ k_merge_append(const float* __restrict__ X, const int32_t* __restrict__ cand,
 // The block then leaves all of them undecided (dc->undecided = k).
 template <int Dp>
 __global__ void __launch_bounds__(1024)
-k_merge_one(const float* __restrict__ X, const float* __restrict__ Xr, const int32_t* __restrict__ cand, int k,
-            const int32_t* __restrict__ rank_cand, uint8_t* cand_state,
-            const int32_t* __restrict__ conf_deg, const int32_t* __restrict__ conf, float thr_f, double thr,
-            const int32_t* __restrict__ support, float* __restrict__ modes, int32_t* __restrict__ mode_support,
-            DevCounters* dc) {
+k_merge_one(const float* __restrict__ X, const int32_t* __restrict__ cand, int k,
+            const int32_t* __restrict__ rank_cand, uint8_t* cand_state, const int32_t* __restrict__ conf_deg,
+            const int32_t* __restrict__ conf, const int32_t* __restrict__ support, float* __restrict__ modes,
+            int32_t* __restrict__ mode_support, DevCounters* dc) {
     volatile uint8_t* st = cand_state;
     bool over = false;
     for (int a = threadIdx.x; a < k; a += 1024) over |= conf_deg[a] > kMergeCap;
@@ -241,10 +241,9 @@ k_merge_one(const float* __restrict__ X, const float* __restrict__ Xr, const int
     if (over) return;
     for (int sweep = 0; sweep < k; ++sweep) {
         bool open = false;
-        for (int r = threadIdx.x; r < k; r += 1024) {
-            const int a = rank_cand[r];
+        for (int a = threadIdx.x; a < k; a += 1024) {
             if (st[a] != kUndecided) continue;
-            const uint8_t d = merge_look<Dp>(r, a, Xr, rank_cand, st, conf_deg, conf, thr_f, thr);
+            const uint8_t d = merge_look(conf + (int64_t)a * kMergeCap, conf_deg[a], st);
             if (d != kUndecided) st[a] = d;
             else open = true;
         }
@@ -263,6 +262,9 @@ unsigned inner_slices(int outer_blocks, int inner, int num_sms) {
     return (unsigned)(sl < 1 ? 1 : sl);
 }
 
+// The candidates' positions in rank order: in the modes' rows that are still free.
+float* merge_xr(const ms_ctx* ctx) { return ctx->modes + (int64_t)ctx->n_kept * ctx->Dp; }
+
 template <int Dp>
 ms_status merge_prepare_t(ms_ctx* ctx, int32_t k) {
     const float thr_f = (float)ctx->cfg.merge_cos;
@@ -275,11 +277,13 @@ ms_status merge_prepare_t(ms_ctx* ctx, int32_t k) {
         ctx->cand, k, ctx->support, ctx->seed_order, ctx->cand_rank);
     MS_LAUNCH("k_rank");
     MS_CUDA(cudaMemsetAsync(ctx->removed_r, 0, (size_t)k, ctx->stream));
-    k_rank_invert_xr<Dp><<<g256, 256, 0, ctx->stream>>>(ctx->cand_rank, k, ctx->cand, ctx->X, ctx->rank_cand, ctx->Xr);
+    float* Xr = merge_xr(ctx);
+    k_rank_invert_xr<Dp><<<g256, 256, 0, ctx->stream>>>(ctx->cand_rank, k, ctx->cand, ctx->X, ctx->rank_cand, Xr);
     MS_LAUNCH("k_rank_invert_xr");
-    const ms_status s = launch_merge_tc_single(ctx->Ck, ctx->Mk, ctx->n_pad, Dp, k, ctx->n_kept, ctx->Xr, ctx->modes,
-                                               ctx->rank_cand, ctx->cand_state, ctx->removed_r, ctx->conf_deg,
-                                               ctx->conf, thr_f, thr, ctx->num_sms, &ctx->dc->status, ctx->stream);
+    const ms_status s = launch_merge_tc_single(ctx->pmap, ctx->pmap1, ctx->Pk, pk_half_rows(ctx), ctx->Ck, ctx->n_pad,
+                                               Dp, k, ctx->n_kept, Xr, ctx->modes, ctx->rank_cand, ctx->cand_state,
+                                               ctx->removed_r, ctx->conf_deg, ctx->conf, thr_f, thr, ctx->num_sms,
+                                               &ctx->dc->status, ctx->stream);
     ctx->launches += 4 + (ctx->n_kept > 0 ? 1 : 0);
     return s;
 }
@@ -309,10 +313,10 @@ ms_status launch_merge_resolve(ms_ctx* ctx, int32_t k, int sweeps) {
     for (int s = 0; s < sweeps; ++s) {
         MS_CUDA(cudaMemsetAsync(&ctx->dc->undecided, 0, sizeof(int32_t), ctx->stream));
         if (ctx->Dp == 16)
-            k_merge_resolve<16><<<gm, kMT, 0, ctx->stream>>>(ctx->Xr, k, ctx->rank_cand, ctx->cand_state,
+            k_merge_resolve<16><<<gm, kMT, 0, ctx->stream>>>(merge_xr(ctx), k, ctx->rank_cand, ctx->cand_state,
                                                              ctx->conf_deg, ctx->conf, thr_f, thr, ctx->dc);
         else
-            k_merge_resolve<32><<<gm, kMT, 0, ctx->stream>>>(ctx->Xr, k, ctx->rank_cand, ctx->cand_state,
+            k_merge_resolve<32><<<gm, kMT, 0, ctx->stream>>>(merge_xr(ctx), k, ctx->rank_cand, ctx->cand_state,
                                                              ctx->conf_deg, ctx->conf, thr_f, thr, ctx->dc);
         MS_LAUNCH("k_merge_resolve");
         ctx->launches += 1;
@@ -339,16 +343,14 @@ bool merge_in_one(int32_t k) { return k <= kMergeOne; }
 
 ms_status launch_merge_one(ms_ctx* ctx, int32_t k) {
     if (k <= 0) return MS_OK;
-    const float thr_f = (float)ctx->cfg.merge_cos;
-    const double thr = ctx->cfg.merge_cos;
     if (ctx->Dp == 16)
-        k_merge_one<16><<<1, 1024, 0, ctx->stream>>>(ctx->X, ctx->Xr, ctx->cand, k, ctx->rank_cand,
-                                                     ctx->cand_state, ctx->conf_deg, ctx->conf, thr_f, thr,
-                                                     ctx->support, ctx->modes, ctx->mode_support, ctx->dc);
+        k_merge_one<16><<<1, 1024, 0, ctx->stream>>>(ctx->X, ctx->cand, k, ctx->rank_cand, ctx->cand_state,
+                                                     ctx->conf_deg, ctx->conf, ctx->support, ctx->modes,
+                                                     ctx->mode_support, ctx->dc);
     else
-        k_merge_one<32><<<1, 1024, 0, ctx->stream>>>(ctx->X, ctx->Xr, ctx->cand, k, ctx->rank_cand,
-                                                     ctx->cand_state, ctx->conf_deg, ctx->conf, thr_f, thr,
-                                                     ctx->support, ctx->modes, ctx->mode_support, ctx->dc);
+        k_merge_one<32><<<1, 1024, 0, ctx->stream>>>(ctx->X, ctx->cand, k, ctx->rank_cand, ctx->cand_state,
+                                                     ctx->conf_deg, ctx->conf, ctx->support, ctx->modes,
+                                                     ctx->mode_support, ctx->dc);
     MS_LAUNCH("k_merge_one");
     ctx->launches += 1;
     return MS_OK;
@@ -369,13 +371,13 @@ ms_status launch_merge_append(ms_ctx* ctx, int32_t k) {
     return MS_OK;
 }
 
-ms_status launch_cover(ms_ctx* ctx, int32_t k0, int32_t k1) {
-    if (k1 <= k0 || ctx->n == 0) return MS_OK;
-    const ms_status s = launch_cover_tc_single(ctx->pmap, ctx->pmap1, ctx->Mk, ctx->n_pad, ctx->Dp, ctx->modes, k0, k1,
-                                               (int)ctx->n, ctx->P32, ctx->pix, ctx->emb, ctx->d,
-                                               ctx->cfg.bandwidth_cos, ctx->covered, &ctx->dc->n_uncovered,
-                                               ctx->num_sms, &ctx->dc->status, ctx->stream);
-    ctx->launches += 2;
+ms_status launch_cover(ms_ctx* ctx, int32_t k, int32_t k0, int32_t k1) {
+    if (k <= 0 || ctx->n == 0) return MS_OK;
+    const ms_status s = launch_cover_tc_single(ctx->pmap, ctx->pmap1, ctx->Pk, pk_half_rows(ctx), k > k0 ? k : k0,
+                                               ctx->Mk, ctx->n_pad, ctx->Dp, ctx->modes, k0, k1, (int)ctx->n, ctx->P32,
+                                               ctx->pix, ctx->emb, ctx->d, ctx->cfg.bandwidth_cos, ctx->covered,
+                                               &ctx->dc->n_uncovered, ctx->num_sms, &ctx->dc->status, ctx->stream);
+    ctx->launches += k1 > k0 ? 2 : 1;
     return s;
 }
 

@@ -23,6 +23,7 @@ namespace {
 constexpr int kSelThreads = 1024;
 constexpr int kSelOne = 4096;       // pixels of a frame that one CTA selects
 constexpr uint8_t kTaken = 2;       // covered[]: drawn by the running selection
+static_assert(kSelThreads == kFewThreads, "blocks of one size");
 
 // Exclusive prefix of `flag` over the block's threads; *total: the block's count.
 __device__ __forceinline__ int block_rank(bool flag, int* total) {
@@ -66,7 +67,7 @@ struct SelArgs {
     int32_t* order_of;   // [n] draw number of a taken pixel (scratch)
     int32_t* counts;     // per block of 1024 (scratch)
     float* X;
-    int32_t* seed_pix;
+    unsigned long long* acc;
     int32_t* seed_order;
     int32_t* active0;
     uint8_t* sstate;
@@ -88,13 +89,18 @@ __device__ __forceinline__ void sel_take(const SelArgs& s, int32_t p, int32_t po
 
 __device__ __forceinline__ void sel_write(const SelArgs& s, int32_t p, int32_t slot, int32_t order) {
     s.covered[p] = 1;
-    s.seed_pix[slot] = p;
     s.seed_order[slot] = order;
     s.active0[slot] = slot;
     s.sstate[slot] = kMoving;
     const float4* src = reinterpret_cast<const float4*>(s.P32 + (int64_t)p * s.Dp);
     float4* dst = reinterpret_cast<float4*>(s.X + (int64_t)slot * s.Dp);
     for (int k = 0; k < s.Dp / 4; ++k) dst[k] = src[k];
+}
+
+// The block clears the window sums of slots [first, first + count).
+__device__ __forceinline__ void sel_clear(const SelArgs& s, int32_t first, int32_t count) {
+    unsigned long long* a = s.acc + (int64_t)first * (s.Dp + 1);
+    for (int64_t i = threadIdx.x; i < (int64_t)count * (s.Dp + 1); i += kSelThreads) a[i] = 0ull;
 }
 
 __device__ __forceinline__ void sel_finish(const SelArgs& s, int32_t taken) {
@@ -148,6 +154,7 @@ __global__ void __launch_bounds__(kSelThreads) k_slot_write(SelArgs s) {
     int total;
     const int r = before + block_rank(flag, &total);
     if (flag) sel_write(s, p, r, s.order_of[p]);
+    sel_clear(s, before, total);
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) sel_finish(s, before + total);
 }
 
@@ -178,6 +185,7 @@ __global__ void __launch_bounds__(kSelThreads) k_seed_select(SelArgs s) {
         if (flag) sel_write(s, p, r, s.order_of[p]);
         slots += total;
     }
+    sel_clear(s, 0, taken);
     if (threadIdx.x == 0) sel_finish(s, taken);
 }
 
@@ -212,6 +220,7 @@ __global__ void __launch_bounds__(kFewThreads) k_seed_few(SelArgs s) {
         const int t = threadIdx.x + k * kFewThreads;
         if (t < taken) sel_write(s, few.pix[t], rank[k], drawn + t);
     }
+    sel_clear(s, 0, taken);
     if (threadIdx.x == 0) sel_finish(s, taken);
 }
 
@@ -231,7 +240,7 @@ bool few_seeds(const ms_ctx* ctx, int32_t want) {
 
 ms_status launch_seed_select(ms_ctx* ctx, int32_t want) {
     const SelArgs s{(int32_t)ctx->n, (uint64_t)ctx->perm_a, (uint64_t)ctx->perm_b, want, ctx->Dp, ctx->P32,
-                    ctx->covered, ctx->cand_rank, ctx->block_tmp, ctx->X, ctx->seed_pix, ctx->seed_order,
+                    ctx->covered, ctx->cand_rank, ctx->block_tmp, ctx->X, ctx->acc, ctx->seed_order,
                     ctx->active[0], ctx->sstate, ctx->seed_log, ctx->dc};
     if (ctx->n <= kSelOne) {
         k_seed_select<<<1, kSelThreads, 0, ctx->stream>>>(s);

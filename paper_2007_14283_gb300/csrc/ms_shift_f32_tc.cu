@@ -304,7 +304,7 @@ k_shift_f32_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__
             }
             if (!ok) break;
             if (slot >= 0 && cnt > 0.f) {
-                unsigned long long* a = acc + (int64_t)slot * (kD + 1);
+                unsigned long long* a = acc + (slot - ii.pix0 + ii.pk_row0) * (kD + 1);
 #pragma unroll
                 for (int k = 0; k < kD; ++k) {
                     const float yk = __uint_as_float((uint32_t)(y[k / 2] >> (32 * (k & 1))));

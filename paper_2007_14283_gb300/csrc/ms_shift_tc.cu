@@ -616,7 +616,7 @@ k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
                         mbar_arrive(d_empty);
                     }
                     if (live) {
-                        unsigned long long* a = acc + (int64_t)slot * (kD + 1);
+                        unsigned long long* a = acc + (slot - ii.pix0 + ii.pk_row0) * (kD + 1);
 #pragma unroll
                         for (int k = 0; k < 16; ++k) {
                             const float y = __uint_as_float(yh[k]) + __uint_as_float(ym[k]) + __uint_as_float(yl[k]);

@@ -130,8 +130,8 @@ struct TcItem {
     int n_active;           // length of that list
     int seed0;              // list position of the item's first seed
     int pt0, pt1;           // the frame's 128-pixel tiles [pt0, pt1)
-    int pk_row0;            // Pk row of the frame's pixel 0 (multiple of 128)
-    int64_t pix0;           // P32 row of the frame's pixel 0
+    int pk_row0;            // Pk row of the frame's pixel 0 and acc row of its slot 0 (multiple of 128)
+    int64_t pix0;           // the frame's slot 0
     int n;                  // the frame's pixel count
 };
 
