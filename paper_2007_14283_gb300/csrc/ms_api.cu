@@ -34,6 +34,13 @@ ms_status cuda_check(cudaError_t e, const char* what) {
     return set_error(MS_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+int device_sms() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
+    return sms > 0 ? sms : 1;
+}
+
 namespace {
 
 // SplitMix64 (Steele, Lea and Flood, OOPSLA 2014).
@@ -170,13 +177,6 @@ Layout plan(int64_t np, int Dp) {
     }
     L.total = t;
     return L;
-}
-
-int device_sms() {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
-    return sms > 0 ? sms : 1;
 }
 
 ms_status readback(ms_ctx* ctx) {

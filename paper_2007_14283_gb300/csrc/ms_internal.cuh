@@ -172,6 +172,7 @@ namespace ms {
 // Error plumbing (ms_api.cu).
 ms_status set_error(ms_status code, const char* fmt, ...);
 ms_status cuda_check(cudaError_t e, const char* what);
+int device_sms();  // SMs of the current device (1 if that cannot be told)
 #define MS_CUDA(call)                                                 \
     do {                                                              \
         ms_status _s = ::ms::cuda_check((call), #call);               \

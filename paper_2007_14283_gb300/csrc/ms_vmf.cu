@@ -238,7 +238,7 @@ __global__ void k_vmf_bwd_reduce(const float* __restrict__ partial, VSplit sp, i
 // from shared memory; each seed's x and gy are read once for both.
 // Bound by FMA issue (64 a pixel and seed). 65536 pixels are 256 such blocks,
 // 1.7 per SM; blockIdx.y splits the seeds into chunks of `len` (a multiple of
-// 64) until the blocks fill the GPU about twice (vmf_alloc), and chunk c > 0
+// 64) where that evens out the SMs (vmf_seed_chunks), and chunk c > 0
 // sums into its own copy of dP, `extra`, which k_vmf_bwd_join adds after the
 // last step. The 10-step adjoint of 65536 pixels and 1024 seeds, forward steps
 // included: 4.91 ms in one chunk, 4.63 in four.
@@ -353,17 +353,35 @@ ms_status vmf_validate(const float* P, int64_t N, const float* X0, int32_t M, in
     return MS_OK;
 }
 
+// Pass B's seed chunks: as many, up to four of at least 128 seeds, as save the most
+// time by the model below, and no more than fill the GPU's slots twice (the copies
+// of dP then take 60 MB at most). A block's 256 pixels take 0.125 us per seed, an SM
+// does a block's worth at a time, so pass B takes as long as the SM with the most
+// blocks; each chunk beyond the first is a copy of dP that is cleared, added to in
+// every step and joined, at 4 TB/s. (One step, 512 seeds: 155,000 pixels, where a
+// split shortens nothing, 564 us in one chunk and 579 in three; 160,000, where two
+// chunks take 4.5 blocks' time instead of 5, 622 and 608; 300,000, again nothing,
+// 1000 and 1021.)
+int64_t vmf_seed_chunks(int64_t N, int32_t M, int32_t T, int slots, int sms) {
+    const int64_t blocks = (N + kBT * kBP - 1) / (kBT * kBP);
+    auto waves = [&](int64_t c) { return (double)((blocks * c + sms - 1) / sms) / (double)c; };
+    int64_t best = 1;
+    double best_us = 0.0;
+    for (int64_t c = 2; c <= 4 && c <= M / 128 && (c - 1) * blocks < 2 * (int64_t)slots; ++c) {
+        const double us = (waves(1) - waves(c)) * 0.125 * M * T - 4.0 - (double)(c - 1) * N * 64.0 * (3 + 2 * T) / 4e6;
+        if (us > best_us) {
+            best_us = us;
+            best = c;
+        }
+    }
+    return best;
+}
+
 ms_status vmf_alloc(VmfWork* w, int64_t N, int32_t M, int32_t T, bool tc, bool adjoint, cudaStream_t st) {
     w->tc = tc;
     w->sp = vsplit(M, N, vmf_slots(k_vmf_fwd_partial, kFT), kFSeeds);
     w->spa = vsplit(M, N, vmf_slots(k_vmf_bwd_seeds, kAT), kASeeds);
-    // Pass B's seed chunks: blocks for two full waves, at least 128 seeds each,
-    // at most four (a copy of dP each beyond the first, together at most 60 MB).
-    const int64_t pblocks = (N + kBT * kBP - 1) / (kBT * kBP);
-    int64_t bc = adjoint && !tc ? (2 * (int64_t)vmf_slots(k_vmf_bwd_pixels, kBT) + pblocks - 1) / pblocks : 1;
-    bc = bc > 4 ? 4 : bc;
-    bc = bc > M / 128 ? M / 128 : bc;
-    bc = bc < 1 ? 1 : bc;
+    const int64_t bc = adjoint && !tc ? vmf_seed_chunks(N, M, T, vmf_slots(k_vmf_bwd_pixels, kBT), device_sms()) : 1;
     w->b_len = (int)((M + bc * 64 - 1) / (bc * 64) * 64);
     w->b_chunks = (M + w->b_len - 1) / w->b_len;
     const size_t extra_b = (size_t)(w->b_chunks - 1) * (size_t)N * kVD * sizeof(float);
