@@ -62,10 +62,14 @@ typedef int32_t ms_status;
 #define MS_FLAT 0 /* flat kernel, Eq. 11 */
 #define MS_VMF 1  /* smooth kernel exp(kappa * cos): only the ms_vmf_* calls */
 
-#define MS_FP32 0 /* plain FP32 SIMT similarity and sums */
-#define MS_BF16 1 /* BF16 tensor-core GEMMs with FP32 accumulation and an FP32 recheck band (the
-                     shift, coverage, labelling and, in batches and single frames, the merge's
-                     two contractions; every decision equal to the FP32 form's) */
+#define MS_FP32 0 /* window decisions and window sums of the FP32 dot product and FP32 additions. Both
+                     forms find the pairs that may matter with BF16-split tensor-core scores
+                     (FP32 accumulation), here and in coverage, labelling and the merge; a pair
+                     within the scores' error bound of a threshold is decided by the FP32 dot
+                     product (windows) or by FP32, then FP64 (the others), so that every decision
+                     is the one those give for all pairs */
+#define MS_BF16 1 /* the same decisions; the window sums are tensor-core GEMMs too (the pixels' exact
+                     BF16 splits, FP32 accumulation), whose additions round in another order */
 
 #define MS_MAX_DIM 32
 
@@ -75,7 +79,9 @@ typedef struct ms_config {
     int32_t kernel;       /* MS_FLAT (MS_VMF is only for ms_vmf_*) */
     double bandwidth_cos; /* c = 1 - h; default 0.9 (h = 0.1, Sec. 4.2/4.3) */
     double kappa;         /* vMF concentration for MS_VMF */
-    double tol;           /* convergence ||x' - x||_2 < tol, evaluated in FP64; default 1e-6 */
+    double tol;           /* convergence ||x' - x||_2 < tol as FP64 decides it (an FP32 norm whose
+                             square is farther than 1e-5 tol^2 from tol^2 settles it first);
+                             default 1e-6 */
     int32_t max_iter;     /* iterations per round before the round is cut; default 300 */
     int32_t n_initial;    /* N_initial = 128 (Sec. 3.2.4) */
     double gamma;         /* early stop when #converged > gamma * N; 0.9 (Sec. 3.2.3) */
@@ -88,8 +94,9 @@ typedef struct ms_config {
     uint64_t frame_id;
     int32_t precision;    /* MS_FP32 or MS_BF16 */
     int32_t max_rounds;   /* guard on OSOP rounds; default 1000000 */
-    double eps_band;      /* reserved, 0: the BF16 recheck band is the library's derived bound
-                             (2^-14 around c; other values are ignored) */
+    double eps_band;      /* reserved, 0: the recheck band of the scores is the library's derived
+                             bound (2^-14 around c for dim <= 16, 7.5e-5 above; other values are
+                             ignored) */
     int32_t all_seeds;    /* 1 = Algorithm 1: every pixel seeds a single round, gamma = 1 */
     int32_t batch_split;  /* ms_batch_* only: 0 = each frame split into work items as on its own
                              (results bit-identical to ms_run on that frame); 1 = the batch's
@@ -100,11 +107,13 @@ typedef struct ms_config {
     int32_t video_restart; /* ms_video_* only: 1 = every frame starts from n_initial instead of the
                               seed count carried from the previous frame */
     int32_t tc_shape;     /* BF16 form: warp arrangement of the shift kernel, the same arithmetic in
-                             each (results bit-identical). Mask warps in
-                             groups that take the pixel tiles in turn, and S buffers: 0 = 8 in two
-                             groups, three (default); 1 = 16 in one, three; 2 = 4 in one, three;
-                             3 = 8 in one, three; 4 = 16 in two, three; 5 = 12 in three, three;
-                             6 = 16 in two, two; 7 = 8 in two, two */
+                             each (results bit-identical). Mask warps in groups that take the pixel
+                             tiles in turn, and S buffers: 0 = 8 in two groups, three (default);
+                             1 = 16 in one, three; 2 = 4 in one, three; 3 = 8 in one, three; 4 = 16
+                             in two, three; 5 = 12 in three, three; 6 = 16 in two, two; 7 = 8 in
+                             two, two. A speed setting only, tuned for one build of the library:
+                             the arrangements behind the numbers change with the kernel, so a
+                             stored choice is timed again (ms_batch_autotune) after an update */
     int32_t reserved[3];  /* zero */
 } ms_config;
 
@@ -381,7 +390,7 @@ MS_API ms_status ms_window_sums_static(const float* d_X, int32_t m, const float*
  * uint8 [n_pixels[t]], d_labels[t] device int32 [n_pixels[t]] receives the
  * labels (-1 background). All borrowed for the duration of the call; the host
  * arrays are read during the call only. While frame t runs its rounds on
- * `stream`, frame t+1 is compacted, normalised and (MS_BF16) split on the
+ * `stream`, frame t+1 is compacted, normalised and split on the
  * internal stream into the other workspace. h_n_start (nullable, host int64
  * [T]) receives the N each frame started from, h_n_modes (nullable, host int32
  * [T]) its mode count. Returns after the last frame's rounds; its labels are
@@ -410,8 +419,9 @@ MS_API void ms_video_destroy(ms_video* v);
  * in different rounds at the same time.
  *
  * ms_batch_create binds the frames and builds the graph (a set-up stage, a
- * conditional WHILE node whose body advances every frame by one iteration,
- * then labelling); it allocates the workspace (one cudaMalloc) and
+ * conditional WHILE node whose body advances every frame by one iteration and,
+ * in a conditional node of its own, ends the rounds that are done, then
+ * labelling); it allocates the workspace (one cudaMalloc) and
  * synchronises `stream`. Arguments:
  *  cfg       as for ms_create (MS_FLAT).
  *  B         1..4096 frames.
