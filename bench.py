@@ -426,6 +426,7 @@ def roofline_of(form, tot, step_ms, clk, n_sm):
         peaks = load_peaks()
         peak = peaks.get("bf16_tflops_sustained") or 1700.0
         bound, kernel = "tensor", "k_shift_tc"
+        frac_note = None
         peak_source = ("of measured: cuBLAS bf16 dense, sustained (MEASURED_PEAKS.json)"
                        if peaks.get("bf16_tflops_sustained") else "of fallback: 1.7 PFLOP/s sustained")
     else:
@@ -433,11 +434,17 @@ def roofline_of(form, tot, step_ms, clk, n_sm):
         bound, kernel = "alu", "k_shift_fp32"
         peak_source = (f"FP32 FMA peak = {n_sm} SMs x {FP32_LANES_PER_SM} lanes x 2 flop x {sm_mhz:.0f} MHz "
                        "(median SM clock sampled under load)")
+        # The form finds windows on the tensor cores and adds only their pixels: most of
+        # the algorithmic flops (every pair's dot product and masked sum) are not FP32
+        # FMAs, so their rate over the FMA peak is no fraction of a roofline.
+        frac_note = ("none: k_shift_f32_tc runs, which finds windows with tensor-core scores; the FMA peak bounds "
+                     "only a scan of all pairs (k_shift_fp32)")
     tpu = shift_traffic_per_unit(kernel)
     per_launch_si = tot["seed_iters"] / max(1, tot["shift_launches"])
     per_launch_fi = tot.get("frame_iters", 0) / max(1, tot["shift_launches"])
     return {"bound": bound, "kernel": kernel, "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-            "frac": (achieved / peak) if achieved else None,
+            "frac": (achieved / peak) if achieved and not frac_note else None, "frac_note": frac_note,
+            "runs": kernel if not frac_note else "k_shift_f32_tc",
             "traffic": (tpu * per_launch_fi) if (tpu and per_launch_fi) else None,
             "traffic_basis": "ncu dram bytes of one frame-iteration (profiles/ncu_traffic.txt) x "
                              f"{per_launch_fi:.2f} frame-iterations per launch",
