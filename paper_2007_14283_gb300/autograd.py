@@ -34,5 +34,5 @@ class VMFMeanShift(torch.autograd.Function):
 def vmf_mean_shift(P: torch.Tensor, X0: torch.Tensor, kappa: float = 20.0, T: int = 10,
                    precision: int = MS_FP32) -> torch.Tensor:
     """precision MS_BF16 runs the forward steps (and the backward's recomputed
-    iterates) on the tensor cores; the adjoint passes are FP32."""
+    iterates) and the adjoint passes on the tensor cores."""
     return VMFMeanShift.apply(P, X0, kappa, T, precision)

@@ -431,7 +431,7 @@ ms_status ms_iterate(ms_ctx* ctx, int32_t max_iter, int32_t* n_converged_out, in
     const int64_t seed_iters0 = ctx->hc->seed_iters;
     // Iterations queued before the first look at the counters: as many as the
     // last round took (rounds of a frame mostly take the same number; queued
-    // iterations after the stop return at once, but each is three launches).
+    // iterations after the stop return at once, but each is two launches).
     int t = 0, batch = ctx->last_iters > 0 ? ctx->last_iters : 4;
     batch = batch < 32 ? batch : 32;
     for (;;) {

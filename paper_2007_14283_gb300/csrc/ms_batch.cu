@@ -87,19 +87,14 @@ struct ms_batch {
 namespace ms {
 namespace {
 
-using tc::bf16_round;
-using tc::pack_bf16;
-
 constexpr int kIT = 1024;   // ingest / selection threads
 static_assert(kIT == kFewThreads, "k_b_seed ranks few seeds with its whole block");
 constexpr int kMT = 128;    // merge threads
-constexpr int kVT = 64;     // vectors per shared tile
-constexpr int kPT = 256;    // pixel threads (cover, label)
 constexpr int kSlotPx = 8;  // pixels a selection thread looks at when giving out slots
 constexpr uint8_t kTaken = 2;  // covered[]: drawn by the running selection
 constexpr int kDefaultMaxPasses = 200000;  // loop guard: far above any real run (rounds x iterations)
 
-enum BlockSel { kSelDoneSeeds = 0, kSelDoneCands = 1, kSelDonePixels = 2, kSelAllPixels = 3 };
+enum BlockSel { kSelDoneSeeds = 0, kSelDoneCands = 1, kSelDonePixels = 2 };
 // Phase sums of profiling level 2 (ms_batch_phase_ms): set-up; per pass the
 // loop's relaunch gap with seed selection and the work plan, the shift, its
 // finalisation and early-stop check, the merge chain, coverage, the schedule
@@ -618,8 +613,7 @@ __global__ void k_b_blocks(const BFrame* __restrict__ frames, const BState* __re
         int cnt = 0;
         if (f < B) {
             const BState& st = states[f];
-            if (sel == kSelAllPixels) cnt = frames[f].n;
-            else if (st.phase == kRoundDone) cnt = sel == kSelDoneSeeds ? st.dc.m_round
+            if (st.phase == kRoundDone) cnt = sel == kSelDoneSeeds ? st.dc.m_round
                                                  : sel == kSelDoneCands ? st.dc.n_cand : frames[f].n;
         }
         const int nb = (cnt + per_block - 1) / per_block;

@@ -89,8 +89,8 @@ struct LabelTcScratch {
 };
 
 ms_status label_tc_setup();
-// Labelling on the tensor cores (BF16 form, Dp = 16 or 32): exact FP64-argmax
-// labels, near-ties re-decided as the FP32 form decides them. pmap1: the
+// Labelling on the tensor cores (Dp = 16 or 32): exact FP64-argmax labels,
+// near-ties decided by FP32 scores, then FP64. pmap1: the
 // pixels' dimensions 16-31 (Dp = 32); Mk holds the modes' split rows, for
 // Dp = 32 followed by a second array of n_pad (mk_rows) rows.
 ms_status launch_label_tc_single(const CUtensorMap& pmap, const CUtensorMap& pmap1, void* Mk, int64_t n_pad, int Dp,

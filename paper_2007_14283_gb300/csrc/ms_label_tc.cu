@@ -1,4 +1,4 @@
-// Labelling, BF16 tensor-core form (the labelling step of Algorithm 2): every
+// Labelling on the tensor cores (the labelling step of Algorithm 2): every
 // foreground vector takes the mode of highest cosine, lowest index on ties.
 //
 // The pixel-by-mode score matrix is a GEMM with K = d = 16 (or 32, as two
@@ -650,8 +650,7 @@ k_label_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
     if (threadIdx.x == 0 && *abort) atomicOr(status, 2);
 }
 
-// Near-ties: one warp per queued pixel re-decides its label as the FP32 form
-// does. FP32 scores over all modes (lanes stride the modes), the best of
+// Near-ties: one warp per queued pixel decides its label. FP32 scores over all modes (lanes stride the modes), the best of
 // them, then the FP64 cosine of the raw embedding for every mode within
 // 2 * kEpsF32 of that best; the largest wins, the lowest index on ties.
 template <int Dp>

@@ -5,7 +5,7 @@
 //
 // Two workspaces alternate. While frame t runs its OSOP rounds on the video's
 // stream, frame t+1 is bound to the other workspace on a second stream:
-// foreground compaction, normalisation and (BF16 form) the split rows for the
+// foreground compaction, normalisation and the split rows for the
 // tensor cores. An event recorded after frame t-1's labelling keeps that bind
 // from touching the workspace before frame t-1's last kernel has read it.
 // Each frame's results are those of ms_create + ms_set_state(carried N) +
