@@ -10,10 +10,9 @@
 //
 // Four passes, each over blocks of 1024 positions or pixels: count the
 // uncovered positions, take them (block prefix from the counts), count the
-// taken pixels, write their slots. A frame of up to kSelOne pixels runs them
-// in one CTA (one launch instead of four), and so does a batch of up to
-// kFewSeeds seeds that are found within few positions: it needs no pass over
-// the pixels, as its seeds are ranked among themselves.
+// taken pixels, write their slots. Up to kFewSeeds seeds that are found within
+// few positions are one CTA's work: it needs no pass over the pixels, as its
+// seeds are ranked among themselves.
 #include "ms_device.cuh"
 #include "ms_internal.cuh"
 
@@ -21,7 +20,6 @@ namespace ms {
 namespace {
 
 constexpr int kSelThreads = 1024;
-constexpr int kSelOne = 4096;       // pixels of a frame that one CTA selects
 constexpr uint8_t kTaken = 2;       // covered[]: drawn by the running selection
 static_assert(kSelThreads == kFewThreads, "blocks of one size");
 
@@ -158,37 +156,6 @@ __global__ void __launch_bounds__(kSelThreads) k_slot_write(SelArgs s) {
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) sel_finish(s, before + total);
 }
 
-// The four passes in one CTA.
-__global__ void __launch_bounds__(kSelThreads) k_seed_select(SelArgs s) {
-    const int32_t cursor = s.dc->cursor, drawn = s.dc->drawn;
-    int32_t taken = 0;
-    for (int32_t base = cursor; base < s.n && taken < s.want; base += kSelThreads) {
-        const int32_t pos = base + threadIdx.x;
-        int32_t p = -1;
-        bool flag = false;
-        if (pos < s.n) {
-            p = sel_pixel(s, pos);
-            flag = s.covered[p] == 0;
-        }
-        int total;
-        const int r = taken + block_rank(flag, &total);
-        if (flag && r < s.want) sel_take(s, p, pos, r, drawn);
-        taken = min(taken + total, s.want);
-    }
-    __syncthreads();
-    int32_t slots = 0;
-    for (int32_t base = 0; base < s.n; base += kSelThreads) {
-        const int32_t p = base + threadIdx.x;
-        const bool flag = p < s.n && s.covered[p] == kTaken;
-        int total;
-        const int r = slots + block_rank(flag, &total);
-        if (flag) sel_write(s, p, r, s.order_of[p]);
-        slots += total;
-    }
-    sel_clear(s, 0, taken);
-    if (threadIdx.x == 0) sel_finish(s, taken);
-}
-
 // Up to kFewSeeds seeds: one CTA takes the positions 1024 at a time and ranks
 // what it took.
 __global__ void __launch_bounds__(kFewThreads) k_seed_few(SelArgs s) {
@@ -242,12 +209,6 @@ ms_status launch_seed_select(ms_ctx* ctx, int32_t want) {
     const SelArgs s{(int32_t)ctx->n, (uint64_t)ctx->perm_a, (uint64_t)ctx->perm_b, want, ctx->Dp, ctx->P32,
                     ctx->covered, ctx->cand_rank, ctx->block_tmp, ctx->X, ctx->acc, ctx->seed_order,
                     ctx->active[0], ctx->sstate, ctx->seed_log, ctx->dc};
-    if (ctx->n <= kSelOne) {
-        k_seed_select<<<1, kSelThreads, 0, ctx->stream>>>(s);
-        MS_LAUNCH("k_seed_select");
-        ctx->launches += 1;
-        return MS_OK;
-    }
     if (few_seeds(ctx, want)) {
         k_seed_few<<<1, kFewThreads, 0, ctx->stream>>>(s);
         MS_LAUNCH("k_seed_few");
