@@ -381,7 +381,8 @@ ms_status vmf_alloc(VmfWork* w, int64_t N, int32_t M, int32_t T, bool tc, bool a
     w->tc = tc;
     w->sp = vsplit(M, N, vmf_slots(k_vmf_fwd_partial, kFT), kFSeeds);
     w->spa = vsplit(M, N, vmf_slots(k_vmf_bwd_seeds, kAT), kASeeds);
-    const int64_t bc = adjoint && !tc ? vmf_seed_chunks(N, M, T, vmf_slots(k_vmf_bwd_pixels, kBT), device_sms()) : 1;
+    const bool split_b = adjoint && !tc && M >= 256;  // two chunks of 128 seeds at least
+    const int64_t bc = split_b ? vmf_seed_chunks(N, M, T, vmf_slots(k_vmf_bwd_pixels, kBT), device_sms()) : 1;
     w->b_len = (int)((M + bc * 64 - 1) / (bc * 64) * 64);
     w->b_chunks = (M + w->b_len - 1) / w->b_len;
     const size_t extra_b = (size_t)(w->b_chunks - 1) * (size_t)N * kVD * sizeof(float);
