@@ -858,9 +858,8 @@ __global__ void k_pack_modes_batch(const BFrame* __restrict__ frames, const BSta
                                    const float* __restrict__ modes, uint4* __restrict__ Mk) {
     const BFrame& fr = frames[blockIdx.y];
     const int K = states[blockIdx.y].dc.n_kept;
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= (K + 127) / 128 * 128) return;
-    pack_mode<Dp>(r < K ? modes + (fr.pix0 + r) * Dp : nullptr, Mk, split_row0(fr, Dp) + r, pk_rows(fr));
+    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < (K + 127) / 128 * 128; r += gridDim.x * blockDim.x)
+        pack_mode<Dp>(r < K ? modes + (fr.pix0 + r) * Dp : nullptr, Mk, split_row0(fr, Dp) + r, pk_rows(fr));
 }
 
 // What coverage needs after one frame's merge: the modes [k0, k1) at their rows of
@@ -886,11 +885,15 @@ __global__ void k_pack_cover_batch(const BFrame* __restrict__ frames, const BSta
     const BFrame& fr = frames[blockIdx.y];
     const BState& st = states[blockIdx.y];
     if (st.phase != kRoundDone || st.dc.n_cand == 0) return;
-    const int r = blockIdx.x * blockDim.x + threadIdx.x, m = st.k0 + r;
-    if (blockIdx.z == 0 && r < max(st.dc.n_cand, st.k0))
-        pack_mode<Dp>(P32 + (fr.pix0 + r) * Dp, Pk, fr.pk_row0 + r, pk_half_rows);
-    if (blockIdx.z == 1 && m < st.dc.n_kept)
-        pack_mode<Dp>(modes + (fr.pix0 + m) * Dp, Mk, split_row0(fr, Dp) + m, pk_rows(fr));
+    const int r0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+    if (blockIdx.z == 0) {
+        const int taken = max(st.dc.n_cand, st.k0);
+        for (int r = r0; r < taken; r += step)
+            pack_mode<Dp>(P32 + (fr.pix0 + r) * Dp, Pk, fr.pk_row0 + r, pk_half_rows);
+    } else {
+        for (int m = st.k0 + r0; m < st.dc.n_kept; m += step)
+            pack_mode<Dp>(modes + (fr.pix0 + m) * Dp, Mk, split_row0(fr, Dp) + m, pk_rows(fr));
+    }
 }
 
 // What one frame's merge needs: its k candidates (rank order, Xr) as split rows
@@ -915,10 +918,21 @@ __global__ void k_pack_merge_batch(const BFrame* __restrict__ frames, const BSta
     const BState& st = states[blockIdx.y];
     const int k = st.dc.n_cand, K = st.dc.n_kept;
     if (st.phase != kRoundDone || k == 0) return;
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (blockIdx.z == 0 && r < (k + 127) / 128 * 128)
-        pack_mode<Dp>(r < k ? modes + (fr.pix0 + K + r) * Dp : nullptr, Ck, split_row0(fr, Dp) + r, pk_rows(fr));
-    if (blockIdx.z == 1 && r < K) pack_mode<Dp>(modes + (fr.pix0 + r) * Dp, Pk, fr.pk_row0 + r, pk_half_rows);
+    const int r0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+    if (blockIdx.z == 0) {
+        for (int r = r0; r < (k + 127) / 128 * 128; r += step)
+            pack_mode<Dp>(r < k ? modes + (fr.pix0 + K + r) * Dp : nullptr, Ck, split_row0(fr, Dp) + r, pk_rows(fr));
+    } else {
+        for (int r = r0; r < K; r += step) pack_mode<Dp>(modes + (fr.pix0 + r) * Dp, Pk, fr.pk_row0 + r, pk_half_rows);
+    }
+}
+
+// Grid of a packing kernel of the batch: about eight blocks an SM over all frames.
+// (A block for every 256 rows that a frame could have was 37,000 of them for 24
+// frames of up to 200,000 pixels, most with nothing to do, 14 us a launch.)
+dim3 pack_grid(int max_pk_rows, int B, int sms, unsigned jobs) {
+    const int rows = (max_pk_rows + 255) / 256, want = (8 * sms + B - 1) / B;
+    return dim3((unsigned)(rows < 1 ? 1 : (rows < want ? rows : want)), (unsigned)B, jobs);
 }
 
 // Per-frame offsets of the label items (128-pixel tiles); clears the queue.
@@ -1002,7 +1016,7 @@ ms_status merge_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, cons
                          const float* modes, const int32_t* rank_cand, uint8_t* cand_state, uint8_t* removed_r,
                          int32_t* conf_deg, int32_t* conf, float thr_f, double thr, const int32_t* tile_off, int grid,
                          int* status, cudaStream_t st) {
-    const dim3 gp((unsigned)((max_pk_rows + 255) / 256), (unsigned)B, 2);
+    const dim3 gp = pack_grid(max_pk_rows, B, grid, 2);
     k_pack_merge_batch<Dp><<<gp, 256, 0, st>>>(frames, states, modes, (uint4*)Ck, (uint4*)Pk, pk_half);
     MS_LAUNCH("k_pack_merge_batch");
     LbOut out{};
@@ -1032,7 +1046,7 @@ ms_status cover_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, cons
                          int64_t pk_half, void* Mk, const BFrame* frames, BState* states, int B, int max_pk_rows,
                          const float* modes, const float* P32, const int32_t* pix, int d, double c, uint8_t* covered,
                          const int32_t* tile_off, int grid, int* status, cudaStream_t st) {
-    const dim3 gp((unsigned)((max_pk_rows + 255) / 256), (unsigned)B, 2);
+    const dim3 gp = pack_grid(max_pk_rows, B, grid, 2);
     k_pack_cover_batch<Dp><<<gp, 256, 0, st>>>(frames, states, P32, (uint4*)Pk, pk_half, modes, (uint4*)Mk);
     MS_LAUNCH("k_pack_cover_batch");
     const float c_f = (float)c;
@@ -1122,7 +1136,7 @@ ms_status label_tc_batch(const CUtensorMap& pmap, const CUtensorMap& pmap1, cons
                          const BFrame* frames, const BState* states, int B, int max_pk_rows, const float* modes,
                          const float* P32, const int32_t* pix, int d, int32_t* const* labels, LabelTcScratch sc,
                          int grid, int* status, cudaStream_t st) {
-    const dim3 gp((unsigned)((max_pk_rows + 255) / 256), (unsigned)B);
+    const dim3 gp = pack_grid(max_pk_rows, B, grid, 1);
     k_pack_modes_batch<Dp><<<gp, 256, 0, st>>>(frames, states, modes, (uint4*)Mk);
     MS_LAUNCH("k_pack_modes_batch");
     k_label_items<<<1, 32, 0, st>>>(frames, B, sc.off, sc.fix_count);
