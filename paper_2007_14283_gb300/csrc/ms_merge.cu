@@ -21,6 +21,7 @@ namespace {
 
 constexpr int kMT = 128;  // threads per merge block
 constexpr int kMergeOne = 4096;  // candidates that one block resolves and appends
+constexpr int kMergeScan = 1024; // the same with more conflicts than are stored
 constexpr int kVT = 64;   // vectors per shared-memory tile
 
 __global__ void k_collect(const uint8_t* __restrict__ sstate, int m, int32_t* __restrict__ cand,
@@ -104,9 +105,8 @@ __device__ __forceinline__ uint8_t merge_look(const int32_t* conf, int deg, cons
 // lie in a row in Xr (by candidate, in pixel order, that look took four times as
 // long: 2.8 ms for 4096 candidates of one cell).
 template <int Dp>
-__device__ __forceinline__ uint8_t merge_look_all(int r, const float* __restrict__ Xr,
-                                                  const int32_t* __restrict__ rank_cand, const volatile uint8_t* st,
-                                                  float thr_f, double thr) {
+__device__ __forceinline__ uint8_t merge_look_all(int r, const float* Xr, const int32_t* __restrict__ rank_cand,
+                                                  const volatile uint8_t* st, float thr_f, double thr) {
     bool all_removed = true;
     float x[Dp];
     load_vec<Dp>(x, Xr + (int64_t)r * Dp);
@@ -167,8 +167,7 @@ template <int Dp>
 __device__ __forceinline__ void merge_append(const float* __restrict__ X, const int32_t* __restrict__ cand,
                                              const int32_t* __restrict__ rank_cand, int k,
                                              const volatile uint8_t* cand_state, const int32_t* __restrict__ support,
-                                             float* __restrict__ modes, int32_t* __restrict__ mode_support,
-                                             DevCounters* dc) {
+                                             float* modes, int32_t* __restrict__ mode_support, DevCounters* dc) {
     __shared__ int32_t warp_excl[32];
     __shared__ int32_t s_total;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -223,27 +222,33 @@ k_merge_append(const float* __restrict__ X, const int32_t* __restrict__ cand,
 // and coverage took 131 to 158 us for 128 to 2048 candidates; so 89 to 108 us. A
 // block's sweep grows with k / 1024 (139 against 183 us at 4096 candidates, no
 // gain expected at 8192), so larger rounds keep the launches.
-// So do rounds with a candidate of more conflicts than are stored: a look at it
-// tests the candidates ranked above it one by one, and one SM for all of them
-// took 9.9 ms for 4096 candidates of four cells, where the launches take 1.0 ms.
-// The block then leaves all of them undecided (dc->undecided = k).
+// Of candidates with more conflicts than are stored the line is kMergeScan: a look
+// at one of them tests the candidates ranked above it one by one. 947 candidates of
+// six cells: 302 us here, 363 us in launches; 3880: 2.0 ms here, 0.89 ms in launches
+// over all SMs. The block leaves such a round undecided (dc->undecided = k).
+// Xr lies in the modes' rows that the append writes, after the last look.
 template <int Dp>
 __global__ void __launch_bounds__(1024)
-k_merge_one(const float* __restrict__ X, const int32_t* __restrict__ cand, int k,
+k_merge_one(const float* __restrict__ X, const float* Xr, const int32_t* __restrict__ cand, int k,
             const int32_t* __restrict__ rank_cand, uint8_t* cand_state, const int32_t* __restrict__ conf_deg,
-            const int32_t* __restrict__ conf, const int32_t* __restrict__ support, float* __restrict__ modes,
-            int32_t* __restrict__ mode_support, DevCounters* dc) {
+            const int32_t* __restrict__ conf, float thr_f, double thr, const int32_t* __restrict__ support,
+            float* modes, int32_t* __restrict__ mode_support, DevCounters* dc) {
     volatile uint8_t* st = cand_state;
     bool over = false;
-    for (int a = threadIdx.x; a < k; a += 1024) over |= conf_deg[a] > kMergeCap;
-    over = __syncthreads_or(over);
+    if (k > kMergeScan) {
+        for (int a = threadIdx.x; a < k; a += 1024) over |= conf_deg[a] > kMergeCap;
+        over = __syncthreads_or(over);
+    }
     if (threadIdx.x == 0) dc->undecided = over ? k : 0;
     if (over) return;
     for (int sweep = 0; sweep < k; ++sweep) {
         bool open = false;
-        for (int a = threadIdx.x; a < k; a += 1024) {
+        for (int r = threadIdx.x; r < k; r += 1024) {
+            const int a = rank_cand[r];
             if (st[a] != kUndecided) continue;
-            const uint8_t d = merge_look(conf + (int64_t)a * kMergeCap, conf_deg[a], st);
+            const int deg = conf_deg[a];
+            const uint8_t d = deg <= kMergeCap ? merge_look(conf + (int64_t)a * kMergeCap, deg, st)
+                                               : merge_look_all<Dp>(r, Xr, rank_cand, st, thr_f, thr);
             if (d != kUndecided) st[a] = d;
             else open = true;
         }
@@ -343,14 +348,16 @@ bool merge_in_one(int32_t k) { return k <= kMergeOne; }
 
 ms_status launch_merge_one(ms_ctx* ctx, int32_t k) {
     if (k <= 0) return MS_OK;
+    const float thr_f = (float)ctx->cfg.merge_cos;
+    const double thr = ctx->cfg.merge_cos;
     if (ctx->Dp == 16)
-        k_merge_one<16><<<1, 1024, 0, ctx->stream>>>(ctx->X, ctx->cand, k, ctx->rank_cand, ctx->cand_state,
-                                                     ctx->conf_deg, ctx->conf, ctx->support, ctx->modes,
-                                                     ctx->mode_support, ctx->dc);
+        k_merge_one<16><<<1, 1024, 0, ctx->stream>>>(ctx->X, merge_xr(ctx), ctx->cand, k, ctx->rank_cand,
+                                                     ctx->cand_state, ctx->conf_deg, ctx->conf, thr_f, thr,
+                                                     ctx->support, ctx->modes, ctx->mode_support, ctx->dc);
     else
-        k_merge_one<32><<<1, 1024, 0, ctx->stream>>>(ctx->X, ctx->cand, k, ctx->rank_cand, ctx->cand_state,
-                                                     ctx->conf_deg, ctx->conf, ctx->support, ctx->modes,
-                                                     ctx->mode_support, ctx->dc);
+        k_merge_one<32><<<1, 1024, 0, ctx->stream>>>(ctx->X, merge_xr(ctx), ctx->cand, k, ctx->rank_cand,
+                                                     ctx->cand_state, ctx->conf_deg, ctx->conf, thr_f, thr,
+                                                     ctx->support, ctx->modes, ctx->mode_support, ctx->dc);
     MS_LAUNCH("k_merge_one");
     ctx->launches += 1;
     return MS_OK;

@@ -1,9 +1,9 @@
 """The merge of rounds in which candidates have up to, and more than, the 32
-stored conflicts: one block resolves the former, launches of their own the
-latter (a look at a candidate of more conflicts tests those ranked above it one
-by one). One tight cluster gives its candidate of rank r exactly r conflicts.
-Modes, supports and labels equal the oracle's on both routes; the launch count
-tells which one ran.
+stored conflicts. One block resolves up to 4096 candidates, and up to 1024 of which
+some have more conflicts (a look at such a one tests those ranked above it one by
+one); launches over all SMs the rest. One tight cluster gives its candidate of rank r
+exactly r conflicts. Modes, supports and labels equal the oracle's on each route; the
+launch count tells which one ran.
 """
 import numpy as np
 import pytest
@@ -32,10 +32,11 @@ def _run(ms_lib, emb, **kw):
 
 @pytest.mark.parametrize("precision", [0, 1])
 def test_route_follows_the_conflicts(ms_lib, precision):
-    emb = _tight(1, 400)
-    launches = {m: _run(ms_lib, emb, precision=precision, n_initial=m, max_rounds=1) for m in (2, 32, 33, 34, 200)}
-    assert launches[2] == launches[32] == launches[33]
-    assert launches[34] == launches[200] >= launches[33] + 8
+    emb = _tight(1, 1200)
+    launches = {m: _run(ms_lib, emb, precision=precision, n_initial=m, max_rounds=1) for m in (33, 34, 1024, 1025)}
+    assert launches[33] == launches[34]
+    # the selection of 1024 and of 1025 seeds may differ by three launches
+    assert launches[1025] >= launches[1024] + 8 - 3
 
 
 @pytest.mark.parametrize("precision", [0, 1])
