@@ -250,6 +250,8 @@ k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
         tmem_alloc(tmem_slot, kTmemCols);
         tmem_relinquish();
     }
+    __syncthreads();
+    grid_release();  // TMEM is held
     grid_wait();
     const int items = map.init() ? map.total() : 0;
     if (warp < 4 && (int)blockIdx.x < items) {  // the first item's seeds, while the rest is set up
@@ -262,7 +264,6 @@ k_shift_tc(const __grid_constant__ CUtensorMap pmap, const __grid_constant__ CUt
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    grid_release();  // TMEM is held
 
     if (warp == kWarpTma) {
         // ------------------------------------------------ TMA producer
