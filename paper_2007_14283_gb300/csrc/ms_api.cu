@@ -189,8 +189,7 @@ void free_ctx(ms_ctx* ctx) {
     if (!ctx) return;
     for (int i = 0; i < 64; ++i)
         if (ctx->ev[i]) cudaEventDestroy(ctx->ev[i]);
-    cudaStreamSynchronize(ctx->stream);
-    block_free(ctx->ws);
+    block_free(ctx->ws_block, ctx->stream);
     counters_free(ctx->hc);
     delete[] ctx->round_log;
     delete ctx;
@@ -257,7 +256,9 @@ ms_status ctx_alloc(const ms_config* cfg, int64_t max_pixels, cudaStream_t strea
     ctx->target_items = 2 * ctx->shift_grid;
     const Layout L = plan(max_pixels, ctx->Dp);
     ctx->ws_bytes = L.total;
-    cudaError_t e = injected_alloc_failure() ? cudaErrorMemoryAllocation : block_alloc(&ctx->ws, L.total, stream);
+    cudaError_t e = injected_alloc_failure() ? cudaErrorMemoryAllocation
+                                             : block_alloc(&ctx->ws_block, L.total, stream);
+    ctx->ws = ctx->ws_block.p;
     if (e != cudaSuccess) {
         free_ctx(ctx);
         return cuda_check(e, "cudaMalloc(workspace)");
@@ -592,9 +593,10 @@ ms_status ms_run_host(const ms_config* cfg, const float* h_emb, const uint8_t* h
     const size_t mb = h_mask ? (size_t)n_pixels : 0;
     const size_t lb = sizeof(int32_t) * (size_t)n_pixels;
     const size_t modes_b = h_modes ? sizeof(float) * (size_t)(cap > 0 ? cap : 0) * (size_t)cfg->dim : 0;
-    char* buf = nullptr;
     const size_t o_mask = align_up(eb), o_lab = o_mask + align_up(mb), o_modes = o_lab + align_up(lb);
-    MS_CUDA(block_alloc((void**)&buf, o_modes + align_up(modes_b) + kAlign, st));
+    Block block;
+    MS_CUDA(block_alloc(&block, o_modes + align_up(modes_b) + kAlign, st));
+    char* buf = (char*)block.p;
     ms_ctx* ctx = nullptr;
     int32_t k = 0;
     s = cuda_check(cudaMemcpyAsync(buf, h_emb, eb, cudaMemcpyHostToDevice, st), "copy h_emb");
@@ -609,8 +611,7 @@ ms_status ms_run_host(const ms_config* cfg, const float* h_emb, const uint8_t* h
     if (s == MS_OK && stats_out) ms_stats_get(ctx, stats_out);
     if (n_modes_out) *n_modes_out = k;
     ms_destroy(ctx);
-    cudaStreamSynchronize(st);
-    block_free(buf);
+    block_free(block, st);
     return s;
 }
 

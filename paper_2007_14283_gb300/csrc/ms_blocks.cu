@@ -132,19 +132,23 @@ cudaError_t device_malloc(void** p, size_t bytes) {
     return cudaMalloc(p, bytes);
 }
 
-cudaError_t block_alloc(void** p, size_t bytes, cudaStream_t st) {
+cudaError_t block_alloc(Block* b, size_t bytes, cudaStream_t st) {
     Pools pools;
-    *p = nullptr;
-    if (bytes > kKeepBytes || !current_pools(&pools)) return device_malloc(p, bytes);
-    const cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pools.blocks, st);
+    *b = Block{};
+    if (bytes > kKeepBytes || !current_pools(&pools)) return device_malloc(&b->p, bytes);
+    const cudaError_t e = cudaMallocFromPoolAsync(&b->p, bytes, pools.blocks, st);
+    b->pooled = e == cudaSuccess;
     if (e != cudaErrorMemoryAllocation) return e;
     give_back();
-    return cudaMalloc(p, bytes);
+    return cudaMalloc(&b->p, bytes);
 }
 
-// cudaFree hands a pool's block back to the pool, without waiting for the device.
-void block_free(void* p) {
-    if (p) cudaFree(p);
+// cudaFree hands a pool's block back to the pool without a wait, so the stream is
+// waited for first; if that fails (a stream that was destroyed already), the device.
+void block_free(const Block& b, cudaStream_t st) {
+    if (!b.p) return;
+    const bool idle = cudaStreamSynchronize(st) == cudaSuccess || cudaDeviceSynchronize() == cudaSuccess;
+    if (idle || !b.pooled) cudaFree(b.p);
 }
 
 cudaError_t scratch_malloc_async(void** p, size_t bytes, cudaStream_t st) {

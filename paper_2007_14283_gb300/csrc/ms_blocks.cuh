@@ -13,10 +13,15 @@ struct DevCounters;
 // (ms_inject_alloc_failure).
 bool injected_alloc_failure();
 // Device memory of a context or of ms_run_host, from what earlier ones left where
-// it fits. Its first use follows on `st`. Freed by block_free once no work on it is
-// left.
-cudaError_t block_alloc(void** p, size_t bytes, cudaStream_t st);
-void block_free(void* p);
+// it fits. Its first use follows on `st`.
+struct Block {
+    void* p = nullptr;
+    bool pooled = false;
+};
+cudaError_t block_alloc(Block* b, size_t bytes, cudaStream_t st);
+// Its return, once the work on `st` (all of the work on it) has ended. What cannot be
+// waited for, on a stream that is being captured, is not handed out again.
+void block_free(const Block& b, cudaStream_t st);
 // cudaMalloc that gives back what the library keeps before it reports that the
 // device is out of memory.
 cudaError_t device_malloc(void** p, size_t bytes);

@@ -113,6 +113,7 @@ struct ms_ctx {
     //    that those took;
     //  - the modes' rows from n_kept on with Xr (the merge, until it appends there);
     //  - X with label_fix (labelling, between rounds).
+    ms::Block ws_block;
     void* ws;
     size_t ws_bytes;
     float* P32;          // [n_pixels, Dp] normalised foreground
@@ -151,7 +152,7 @@ struct ms_ctx {
     int32_t last_iters;  // iterations of the frame's last round (0: none yet)
     ms_stats stats;
     // tensor-core operands
-    void* Pk;            // [n_pad, 64] bf16: [Ph | Pm | Pl | 0] per pixel
+    void* Pk;            // [n_pad, 64] bf16 split rows of the pixels (pack_split_row)
     int64_t n_pad;       // n rounded up to 128 (0 when n = 0)
     CUtensorMap pmap;    // TMA map of Pk: boxes of 128 rows x 128 bytes, 128-byte swizzle
     CUtensorMap pmap1;   // d = 32: the same for dimensions 16..31 (the second Pk array)

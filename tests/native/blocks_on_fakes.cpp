@@ -4,6 +4,7 @@
 // Prints a line for each check that fails and returns their number.
 #include <cuda.h>
 
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -32,6 +33,8 @@ std::map<void*, unsigned long long> pinned;
 std::vector<Pool*> pools;
 std::map<Pool*, unsigned long long> pool_ctx;
 uintptr_t next_addr = 0x1000;
+bool capturing = false;  // the stream of the calls
+std::atomic<int> stream_waits{0};
 int device_waits = 0, dead_uses = 0, bad_frees = 0, mallocs = 0, host_mallocs = 0, errors_left = 0;
 
 void trim(Pool* p, size_t to) {
@@ -75,7 +78,11 @@ cudaError_t cudaGetLastError() {
 }
 cudaError_t cudaDeviceSynchronize() {
     ++device_waits;
-    return cudaSuccess;
+    return capturing ? cudaErrorStreamCaptureUnsupported : cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t) {
+    ++stream_waits;
+    return capturing ? cudaErrorStreamCaptureUnsupported : cudaSuccess;
 }
 cudaError_t cudaMalloc(void** p, size_t bytes) {
     std::lock_guard<std::mutex> lk(mu);
@@ -166,57 +173,64 @@ void check(bool ok, const char* what) {
     }
 }
 constexpr size_t MB = size_t(1) << 20;
-bool take(void** p, size_t bytes) { return ms::block_alloc(p, bytes, nullptr) == cudaSuccess; }
+bool take(ms::Block* p, size_t bytes) { return ms::block_alloc(p, bytes, nullptr) == cudaSuccess; }
+void give(const ms::Block& b) {
+    const int waits = stream_waits;
+    ms::block_free(b, nullptr);
+    check(stream_waits == waits + 1, "the stream is waited for");
+}
 
 }  // namespace
 
 int main() {
-    void *a, *b, *c;
+    ms::Block a, b, c;
+    void* m;
+    void* m2;
     // kept within the bound, taken over, larger blocks not kept
     check(take(&a, 300 * MB) && take(&b, 300 * MB), "two blocks");
-    ms::block_free(a);
-    ms::block_free(b);
+    give(a);
+    give(b);
     check(device_free == 1024 * MB - 512 * MB, "512 MB are kept of 600");
     const size_t before = device_free;
     check(take(&a, 400 * MB) && device_free == before, "a block from what was left");
-    ms::block_free(a);
+    give(a);
     check(take(&a, 513 * MB), "a block larger than what may be kept, where it fits only without the kept ones");
-    ms::block_free(a);
+    give(a);
     check(device_free == 1024 * MB, "which is given back at once");
 
     // every allocation gets the kept memory, with a driver that takes it itself and one that does not
     for (int own = 0; own < 2; ++own) {
         driver_trims = own == 0;
         check(take(&a, 500 * MB), "a block");
-        ms::block_free(a);
-        check(ms::device_malloc(&b, 900 * MB) == cudaSuccess && errors_left == 0, "a batch's workspace");
-        ms::block_free(b);
+        give(a);
+        check(ms::device_malloc(&m, 900 * MB) == cudaSuccess && errors_left == 0, "a batch's workspace");
+        cudaFree(m);
         check(take(&a, 500 * MB), "a block");
-        ms::block_free(a);
-        check(ms::scratch_malloc_async(&b, 900 * MB, nullptr) == cudaSuccess && errors_left == 0, "scratch");
-        cudaFree(b);  // the scratch pool keeps it
+        give(a);
+        check(ms::scratch_malloc_async(&m, 900 * MB, nullptr) == cudaSuccess && errors_left == 0, "scratch");
+        cudaFree(m);  // the scratch pool keeps it
         check(device_free == 1024 * MB - 900 * MB, "scratch stays mapped");
         check(take(&a, 500 * MB) && errors_left == 0, "a block once the scratch is unused");
         check(!take(&c, 525 * MB) && take(&b, 500 * MB) && !take(&c, 100 * MB), "no more than there is");
-        ms::block_free(a);
-        ms::block_free(b);
-        check(ms::device_malloc(&b, 1024 * MB) == cudaSuccess, "all of it");
-        check(ms::device_malloc(&c, MB) == cudaErrorMemoryAllocation, "out of memory is said");
-        ms::block_free(b);
+        give(a);
+        give(b);
+        check(ms::device_malloc(&m, 1024 * MB) == cudaSuccess, "all of it");
+        check(ms::device_malloc(&m2, MB) == cudaErrorMemoryAllocation, "out of memory is said");
+        cudaFree(m);
     }
     driver_trims = true;
 
     // nothing kept crosses a device reset
     ms::DevCounters *h1, *h2;
     check(take(&a, 200 * MB) && ms::counters_alloc(&h1, 96) == cudaSuccess, "before the reset");
-    ms::block_free(a);
+    give(a);
     ms::counters_free(h1);
     check(ms::counters_alloc(&h2, 96) == cudaSuccess && h2 == h1 && host_mallocs == 1, "counters are taken over");
     ms::counters_free(h2);
     reset();
     check(take(&a, 200 * MB) && ms::counters_alloc(&h2, 96) == cudaSuccess && host_mallocs == 2, "after the reset");
     check(h2 != h1 && dead_uses == 0, "nothing of the dead context");
-    ms::block_free(a);
+    give(a);
     ms::counters_free(h2);
 
     // pinned counters are bounded
@@ -230,9 +244,9 @@ int main() {
     for (int t = 0; t < 8; ++t)
         ts.emplace_back([t] {
             for (int i = 0; i < 200; ++i) {
-                void* p;
+                ms::Block p;
                 ms::DevCounters* h;
-                if (ms::block_alloc(&p, (1 + (t * 7 + i) % 20) * MB, nullptr) == cudaSuccess) ms::block_free(p);
+                if (take(&p, (1 + (t * 7 + i) % 20) * MB)) ms::block_free(p, nullptr);
                 ms::counters_alloc(&h, 96);
                 ms::counters_free(h);
             }
@@ -240,5 +254,13 @@ int main() {
     for (auto& t : ts) t.join();
     check(live.empty() && device_free >= 512 * MB, "threads leave no block");
     check(bad_frees == 0 && device_waits == 0, "no foreign free, no wait for the device");
+
+    // a block whose stream is being captured is not handed out again, a larger one is freed
+    check(take(&a, 100 * MB) && take(&b, 600 * MB), "blocks");
+    capturing = true;
+    ms::block_free(a, nullptr);
+    ms::block_free(b, nullptr);
+    capturing = false;
+    check(live.size() == 1 && live.count(a.p) == 1, "the pool's block stays taken");
     return failed;
 }
